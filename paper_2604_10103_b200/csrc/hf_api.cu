@@ -5,7 +5,6 @@
 #include "k_swa_mma.cuh"
 #include "k_swa_tc5.cuh"
 #include "k_swa_tc5p.cuh"
-#include "k_swa_tc5g.cuh"
 #include "k_swa_bwd.cuh"
 #include "k_readout_bwd.cuh"
 #include "k_state_mma.cuh"
@@ -272,14 +271,16 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 // 4-D bf16 map [slots, B*H, rows, d] with a box of box_cols x box_rows, 128-byte swizzle (or none); rows past the end read as zero.
+// (the swizzle is the box's row width: 128 or 64 bytes)
 hf_status make_map_ex(hf_ctx* c, CUtensorMap* m, const void* base, long long rows, int slots, int box_cols, int box_rows, bool swizzle) {
+    const CUtensorMapSwizzle sw = box_cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
     const cuuint64_t dims[4] = {(cuuint64_t)c->d, (cuuint64_t)rows, (cuuint64_t)c->BH, (cuuint64_t)slots};
     const cuuint64_t strides[3] = {(cuuint64_t)c->d * 2, (cuuint64_t)rows * c->d * 2, (cuuint64_t)c->BH * rows * c->d * 2};
     const cuuint32_t box[4] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, 1, 1};
     const cuuint32_t es[4] = {1, 1, 1, 1};
     CUresult r = reinterpret_cast<EncodeTiledFn>(c->encode_tiled)(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims,
                                                                   strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                                                  swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                                                                  swizzle ? sw : CU_TENSOR_MAP_SWIZZLE_NONE,
                                                                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(HF_ERR_CUDA, "cuTensorMapEncodeTiled failed with %d", (int)r);
     return HF_OK;
@@ -484,27 +485,37 @@ hf_status launch_swa_mma_t(hf_ctx* c, const bf16* q, const ChunkTable& tab, cons
 }
 
 
-#ifndef HF_TC5_GROUPS
-#define HF_TC5_GROUPS 2   // softmax column groups of the tcgen05 attention kernel at head_dim 64
-#endif
-#ifndef HF_TC5_GROUPS_128
-#define HF_TC5_GROUPS_128 2   // ... and at head_dim 128
-#endif
-template <int D> struct Tc5Groups { static constexpr int N = (D == 128) ? HF_TC5_GROUPS_128 : HF_TC5_GROUPS; };
-
-template <int D>
+// The tcgen05 attention kernel.  Blocks of 16 or 64 tokens: first the kept lists of the query blocks that share a 128-row unit
+// are merged (k_union_tiles).  hist_inside: the kernel forms the history term; overlap_prev: it may be launched under the tail
+// of the kernel before it in the stream.
+template <int D, int BLK>
 hf_status launch_swa_tc5_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_cur, const bf16* v_cur, const int32_t* idx,
-                           int keep, const float* hist, bf16* o, float* lse, cudaStream_t st, bool fuse_history = false,
-                           bool overlap_prev = false) {
-    typedef SwaTc5<D, Tc5Groups<D>::N> C;
+                           int keep, const float* hist, bf16* o, float* lse, cudaStream_t st, bool hist_inside, bool overlap_prev) {
+    typedef SwaTc5<D> C;
+    constexpr int G = 128 / BLK;
+    Tc5Params p;
+    memset(&p, 0, sizeof(p));
+    p.upb = (c->Tc + 127) / 128; p.n_units = p.upb * c->BH;
+    if (BLK != 128) {
+        const int Tn = (L.n_sink + L.n_cached + 1) * c->n_b;
+        const int uni = G * keep < Tn ? G * keep : Tn;
+        const int max_tiles = (uni + G - 1) / G;
+        if (max_tiles > c->union_max_tiles) return fail(HF_ERR_SHAPE, "tile list of %d tiles exceeds the %d the context was sized for", max_tiles, c->union_max_tiles);
+        PdlLaunch pu(dim3(p.upb, c->BH), dim3(256), 0, st, true);
+        HF_CUDA(cudaLaunchKernelEx(&pu.cfg, k_union_tiles<BLK>, idx, keep, c->Tm, Tn, c->n_b, c->Tc, max_tiles, c->union_entries, c->union_tiles,
+                                   c->dev_status));
+        HF_TRY(post_launch(c, "k_union_tiles"));
+        p.entries = c->union_entries; p.tiles = c->union_tiles; p.max_tiles = max_tiles;
+        overlap_prev = true;
+    }
     CUtensorMap tq, tk, tv, to;
     HF_TRY(make_map(c, &tq, q, 1));
-    HF_TRY(make_map(c, &tk, k_cur, 1));
-    HF_TRY(make_map(c, &tv, v_cur, 1));
-    HF_TRY(make_map_ex(c, &to, o, c->Tc, 1, 64, 32, true));      // output: one warp's 32 rows x 64 columns per store
-    Tc5Params p;
+    HF_TRY(make_map_ex(c, &tk, k_cur, c->Tc, 1, 64, BLK, true));
+    HF_TRY(make_map_ex(c, &tv, v_cur, c->Tc, 1, 64, BLK, true));
+    HF_TRY(make_map_ex(c, &to, o, c->Tc, 1, C::OCOLS, 32, true));      // output: one warp's 32 rows x half of the columns per store
     p.idx = idx; p.keep = keep; p.Tc = c->Tc; p.n_b = c->n_b; p.n_cached = L.n_cached; p.ring_head = L.head; p.n_sink = L.n_sink;
-    p.P = c->R;
+    p.P = c->R; p.Tm = c->Tm;
+    p.nb_magic = c->n_b > 1 ? (uint32_t)((0x100000000ull + c->n_b - 1) / c->n_b) : 0u;
     p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D));
     p.hist = hist; p.o = o; p.lse = lse; p.dev_status = c->dev_status;
     p.heads = c->cfg.heads; p.eps = c->cfg.eps;
@@ -512,18 +523,17 @@ hf_status launch_swa_tc5_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16* 
     p.tab = make_table(c, L, k_cur, v_cur); p.sf_hi = L.sf_hi; p.sf_lo = L.sf_lo;
     const CUtensorMap& rk = c->R + c->n_sink_max > 0 ? L.tm_kring : tk;
     const CUtensorMap& rv = c->R + c->n_sink_max > 0 ? L.tm_vring : tv;
-    p.Tm = c->Tm; p.n_units = c->Tm * c->BH;
     const int grid = p.n_units < c->sm_count ? p.n_units : c->sm_count;
     PdlLaunch pl(dim3(grid), dim3(C::THREADS), C::SMEM_BYTES, st, overlap_prev);
-    if constexpr (C::FUSE) {
-        if (fuse_history) {
-            HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, Tc5Groups<D>::N, true>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
-            return post_launch(c, "k_swa_tc5 (history term inside)");
-        }
-    }
-    if (fuse_history) return fail(HF_ERR_UNSUPPORTED, "the attention kernel of this configuration cannot form the history term");
-    HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, Tc5Groups<D>::N, false>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
+    if (hist_inside) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, true>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
+    else HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, false>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
     return post_launch(c, "k_swa_tc5");
+}
+template <int D, int BLK>
+hf_status set_swa_tc5_attr() {
+    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D>::SMEM_BYTES));
+    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D>::SMEM_BYTES));
+    return HF_OK;
 }
 
 #ifndef HF_TC5P_COLGROUPS
@@ -552,60 +562,18 @@ hf_status launch_swa_tc5p_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16*
     return post_launch(c, "k_swa_tc5p");
 }
 
-// Blocks of 16 or 64 tokens on the tcgen05 path: merge the kept lists of the query blocks that share a 128-row unit
-// (k_union_tiles), then the attention kernel over 128-key tiles made of 128 / BLK key blocks each.
-template <int D, int BLK>
-hf_status launch_swa_tc5g_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_cur, const bf16* v_cur, const int32_t* idx,
-                            int keep, const float* hist, bf16* o, float* lse, cudaStream_t st) {
-    typedef SwaTc5<D, 2> C;
-    constexpr int G = 128 / BLK;
-    const int Tn = (L.n_sink + L.n_cached + 1) * c->n_b;
-    const int Tmt = (c->Tc + 127) / 128;
-    const int uni = G * keep < Tn ? G * keep : Tn;
-    const int max_tiles = (uni + G - 1) / G;
-    if (max_tiles > c->union_max_tiles) return fail(HF_ERR_SHAPE, "tile list of %d tiles exceeds the %d the context was sized for", max_tiles, c->union_max_tiles);
-    PdlLaunch pu(dim3(Tmt, c->BH), dim3(256), 0, st, true);
-    HF_CUDA(cudaLaunchKernelEx(&pu.cfg, k_union_tiles<BLK>, idx, keep, c->Tm, Tn, c->n_b, c->Tc, max_tiles, c->union_entries, c->union_tiles,
-                               c->dev_status));
-    HF_TRY(post_launch(c, "k_union_tiles"));
-    CUtensorMap tq, tk, tv, to;
-    HF_TRY(make_map(c, &tq, q, 1));
-    HF_TRY(make_map_ex(c, &tk, k_cur, c->Tc, 1, 64, BLK, true));
-    HF_TRY(make_map_ex(c, &tv, v_cur, c->Tc, 1, 64, BLK, true));
-    HF_TRY(make_map_ex(c, &to, o, c->Tc, 1, 64, 32, true));
-    Tc5GParams p;
-    memset(&p, 0, sizeof(p));
-    p.entries = c->union_entries; p.tiles = c->union_tiles; p.max_tiles = max_tiles;
-    p.Tmt = Tmt; p.n_units = Tmt * c->BH;
-    p.idx = idx; p.keep = keep; p.Tm = c->Tm;
-    p.Tc = c->Tc; p.n_b = c->n_b; p.n_cached = L.n_cached; p.ring_head = L.head; p.P = c->R; p.n_sink = L.n_sink;
-    p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D));
-    p.hist = hist; p.q = q; p.o = o; p.lse = lse; p.dev_status = c->dev_status;
-    p.tab = make_table(c, L, k_cur, v_cur);
-    const CUtensorMap& rk = c->R + c->n_sink_max > 0 ? L.tm_kring : tk;
-    const CUtensorMap& rv = c->R + c->n_sink_max > 0 ? L.tm_vring : tv;
-    const int grid = p.n_units < c->sm_count ? p.n_units : c->sm_count;
-    PdlLaunch pl(dim3(grid), dim3(C::THREADS), C::SMEM_BYTES, st, true);
-    HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5g<D, BLK>, tq, rk, rv, tk, tv, to, p));
-    return post_launch(c, "k_swa_tc5g");
-}
-
+// hist_inside: the attention kernel forms the history term itself (the tcgen05 kernel only).
 hf_status launch_swa(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_cur, const bf16* v_cur, const int32_t* idx,
-                     int keep, const float* hist, bf16* o, float* lse, cudaStream_t st) {
-    if (c->swa_kernel == HF_SWA_TCGEN05 && c->cfg.block != 128) {
+                     int keep, const float* hist, bf16* o, float* lse, cudaStream_t st, bool hist_inside = false, bool overlap_prev = false) {
+    if (c->swa_kernel == HF_SWA_TCGEN05) {
         const int b = c->cfg.block, d = c->d;
-        if (b == 64 && d == 128) return launch_swa_tc5g_t<128, 64>(c, L, q, k_cur, v_cur, idx, keep, hist, o, lse, st);
-        if (b == 64 && d == 64) return launch_swa_tc5g_t<64, 64>(c, L, q, k_cur, v_cur, idx, keep, hist, o, lse, st);
-        if (b == 16 && d == 128) return launch_swa_tc5g_t<128, 16>(c, L, q, k_cur, v_cur, idx, keep, hist, o, lse, st);
-        return launch_swa_tc5g_t<64, 16>(c, L, q, k_cur, v_cur, idx, keep, hist, o, lse, st);
+#define HF_TC5_CASE(D_, B_) if (d == D_ && b == B_) return launch_swa_tc5_t<D_, B_>(c, L, q, k_cur, v_cur, idx, keep, hist, o, lse, st, hist_inside, overlap_prev)
+        HF_TC5_CASE(128, 128); HF_TC5_CASE(128, 64); HF_TC5_CASE(128, 16); HF_TC5_CASE(64, 128); HF_TC5_CASE(64, 64); HF_TC5_CASE(64, 16);
+#undef HF_TC5_CASE
     }
     if (c->swa_kernel == HF_SWA_TCGEN05_PINGPONG) {
         if (c->d == 128) return launch_swa_tc5p_t<128>(c, L, q, k_cur, v_cur, idx, keep, hist, o, lse, st);
         return launch_swa_tc5p_t<64>(c, L, q, k_cur, v_cur, idx, keep, hist, o, lse, st);
-    }
-    if (c->swa_kernel == HF_SWA_TCGEN05) {
-        if (c->d == 128) return launch_swa_tc5_t<128>(c, L, q, k_cur, v_cur, idx, keep, hist, o, lse, st);
-        return launch_swa_tc5_t<64>(c, L, q, k_cur, v_cur, idx, keep, hist, o, lse, st);
     }
     ChunkTable tab = make_table(c, L, k_cur, v_cur);
     const int b = c->cfg.block, d = c->d;
@@ -830,17 +798,14 @@ hf_status hf_create(const hf_config* cfg, int device, hf_ctx** out) {
         if (s == HF_OK) s = set_swa_attr<64, 128>();
         if (s == HF_OK) s = set_swa_attr<128, 64>();
         if (s == HF_OK) s = set_swa_attr<128, 128>();
-        if (s == HF_OK && cudaFuncSetAttribute(k_swa_tc5<64, Tc5Groups<64>::N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<64, Tc5Groups<64>::N>::SMEM_BYTES) != cudaSuccess) s = fail(HF_ERR_CUDA, "cudaFuncSetAttribute(k_swa_tc5<64>) failed");
-        if (s == HF_OK && cudaFuncSetAttribute(k_swa_tc5<128, Tc5Groups<128>::N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<128, Tc5Groups<128>::N>::SMEM_BYTES) != cudaSuccess) s = fail(HF_ERR_CUDA, "cudaFuncSetAttribute(k_swa_tc5<128>) failed");
-        if constexpr (SwaTc5<128, Tc5Groups<128>::N>::FUSE)
-            if (s == HF_OK && cudaFuncSetAttribute(k_swa_tc5<128, Tc5Groups<128>::N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<128, Tc5Groups<128>::N>::SMEM_BYTES) != cudaSuccess) s = fail(HF_ERR_CUDA, "cudaFuncSetAttribute(k_swa_tc5<128, history>) failed");
+        if (s == HF_OK) s = set_swa_tc5_attr<64, 16>();
+        if (s == HF_OK) s = set_swa_tc5_attr<64, 64>();
+        if (s == HF_OK) s = set_swa_tc5_attr<64, 128>();
+        if (s == HF_OK) s = set_swa_tc5_attr<128, 16>();
+        if (s == HF_OK) s = set_swa_tc5_attr<128, 64>();
+        if (s == HF_OK) s = set_swa_tc5_attr<128, 128>();
         if (s == HF_OK && cudaFuncSetAttribute(k_swa_tc5p<64, HF_TC5P_COLGROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5P<64, HF_TC5P_COLGROUPS>::SMEM_BYTES) != cudaSuccess) s = fail(HF_ERR_CUDA, "cudaFuncSetAttribute(k_swa_tc5p<64>) failed");
         if (s == HF_OK && cudaFuncSetAttribute(k_swa_tc5p<128, HF_TC5P_COLGROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5P<128, HF_TC5P_COLGROUPS>::SMEM_BYTES) != cudaSuccess) s = fail(HF_ERR_CUDA, "cudaFuncSetAttribute(k_swa_tc5p<128>) failed");
-        if (s == HF_OK && (cudaFuncSetAttribute(k_swa_tc5g<64, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<64, 2>::SMEM_BYTES) != cudaSuccess ||
-                           cudaFuncSetAttribute(k_swa_tc5g<64, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<64, 2>::SMEM_BYTES) != cudaSuccess ||
-                           cudaFuncSetAttribute(k_swa_tc5g<128, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<128, 2>::SMEM_BYTES) != cudaSuccess ||
-                           cudaFuncSetAttribute(k_swa_tc5g<128, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<128, 2>::SMEM_BYTES) != cudaSuccess))
-            s = fail(HF_ERR_CUDA, "cudaFuncSetAttribute(k_swa_tc5g) failed");
         if (s == HF_OK) s = set_state_attr<64>();
         if (s == HF_OK) s = set_state_attr<128>();
     }
@@ -1219,16 +1184,18 @@ hf_status hf_linear_attn_backward_dq(hf_ctx* c, int layer, const void* q, const 
     return HF_DISPATCH_D(c, launch_readout_bwd, c, c->layers[layer], (const bf16*)q, (const bf16*)d_o, (bf16*)dq, (cudaStream_t)stream);
 }
 
+// Whether the attention kernel forms the history term itself: the tcgen05 kernel does, for the per-head and the identity
+// merge.  The rotated variant of Eq. 4 (numerator and denominator see different phi(Q)) and the full-width merge (which couples
+// the heads) keep the separate read-out.
+static bool one_kernel_forward(const hf_ctx* c) {
+    return c->swa_kernel == HF_SWA_TCGEN05 && !c->has_rope_q && c->cfg.merge != HF_MERGE_FULL_WIDTH;
+}
+
 // Eq. 6 + Eq. 4 + Eq. 7 for a selection that is already made.  after_select: the call follows launch_select in the same
 // stream directly, so the attention kernel may be launched under its tail.
 static hf_status attend_merge(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k, const bf16* v, const int32_t* idx, int keep,
                               bf16* o, cudaStream_t st, bool after_select) {
-    // At head_dim 128 the tcgen05 attention kernel forms the history term itself (three more tensor-core products per
-    // query block against the folded state, which it keeps in shared memory): no read-out kernel, no scratch buffer.
-    // The rotated variant of Eq. 4 (numerator and denominator see different phi(Q)) keeps the separate read-out.
-    if (c->swa_kernel == HF_SWA_TCGEN05 && c->d == 128 && c->cfg.block == 128 && SwaTc5<128, Tc5Groups<128>::N>::FUSE && !c->has_rope_q &&
-        c->cfg.merge != HF_MERGE_FULL_WIDTH)
-        return launch_swa_tc5_t<128>(c, L, q, k, v, idx, keep, nullptr, o, nullptr, st, true, after_select);
+    if (one_kernel_forward(c)) return launch_swa(c, L, q, k, v, idx, keep, nullptr, o, nullptr, st, true, after_select);
     // Otherwise the read-out kernel writes the history term to the context's scratch buffer and the attention kernel adds
     // it in its epilogue.
     HF_TRY(HF_DISPATCH_D(c, launch_readout, c, L, q, (bf16*)nullptr, c->hist, st));
@@ -1263,8 +1230,7 @@ hf_status hf_hybrid_forward(hf_ctx* c, int layer, const void* q, const void* k, 
     HF_TRY(check_ptr(o, "o"));
     LayerState& L = c->layers[layer];
     cudaStream_t st = (cudaStream_t)stream;
-    const bool one_kernel = c->swa_kernel == HF_SWA_TCGEN05 && c->d == 128 && c->cfg.block == 128 && SwaTc5<128, Tc5Groups<128>::N>::FUSE &&
-                            !c->has_rope_q && c->cfg.merge != HF_MERGE_FULL_WIDTH;
+    const bool one_kernel = one_kernel_forward(c);
     if (one_kernel || c->has_trope) {
         // (with the temporal rotation the selection's pooling pass also writes the rotated q and k that everything after it
         // reads, so the history read-out cannot run beside it: one stream)

@@ -62,12 +62,30 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     return mbar_wait_slow<PARKED, LIMIT>(bar, parity, abort_flag, dev_status, where);
 }
 
+// A whole warp's wait (all 32 lanes, converged): the test, a vote and a uniform branch.  A per-lane result would make the
+// compiler put a reconvergence point around every wait, ~60 clk each on the softmax warps' serial path.
+template <bool PARKED = false, long long LIMIT = WAIT_LIMIT_CYCLES>
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* dev_status, int where) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait_slow<PARKED, LIMIT>(bar, parity, abort_flag, dev_status, where));
+}
+// One arrival, by the lanes for which `on` is set, without a branch.
+__device__ __forceinline__ void mbar_arrive_if(uint32_t bar, bool on) {
+    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %1, 0;\n @p mbarrier.arrive.shared::cta.b64 _, [%0];\n}\n"
+                 ::"r"(bar), "r"((uint32_t)on) : "memory");
+}
+
 // ----------------------------------------------------------------------------------------- TMA
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3, uint32_t bar) {
     asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];\n"
                  ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar) : "memory");
 }
 
+// Untiled copy global -> shared (both addresses 16-byte aligned, size a multiple of 16 bytes).
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
 // Tile store shared -> global through a tensor map (bulk async-group completion).  The shared-memory writes that filled
 // the tile must be followed by fence_proxy_async() in the writing threads before the issuing thread is signalled.
 __device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, uint32_t src, int c0, int c1, int c2, int c3) {
@@ -138,7 +156,36 @@ __device__ __forceinline__ void mma_ts_tile(uint32_t d_tmem, uint32_t a_tmem, ui
                  HF_TS_STEP(4, "pt") HF_TS_STEP(5, "pt") HF_TS_STEP(6, "pt") HF_TS_STEP(7, "pt")
                  "}\n" ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"((uint32_t)accumulate_first) : "memory");
 }
+// ... over 64 keys (four steps).
+__device__ __forceinline__ void mma_ts_half(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi, uint32_t idesc,
+                                            bool accumulate_first) {
+    asm volatile("{\n .reg .pred pt, p0;\n .reg .b64 db;\n .reg .b32 a, b;\n"
+                 "setp.eq.u32 pt, %0, %0;\n setp.ne.b32 p0, %5, 0;\n"
+                 HF_TS_STEP(0, "p0") HF_TS_STEP(1, "pt") HF_TS_STEP(2, "pt") HF_TS_STEP(3, "pt")
+                 "}\n" ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"((uint32_t)accumulate_first) : "memory");
+}
 #undef HF_TS_STEP
+#define HF_TK_STEP(KS, BOFF, PRED)                                                                 \
+    "add.u32 a, %1, " #KS " * 8;\n add.u32 b, %2, " #BOFF ";\n mov.b64 db, {b, %3};\n"            \
+    "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], db, %4, " PRED ";\n"
+// D[tmem] = A[tmem] * B[smem] over the whole head dimension: A = bf16 rows (8 columns per 16 features), B K-major as in
+// mma_ss_tile.
+template <int D>
+__device__ __forceinline__ void mma_ts_kmajor(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi, uint32_t idesc) {
+    if constexpr (D == 128) {
+        asm volatile("{\n .reg .pred pt, pf;\n .reg .b64 db;\n .reg .b32 a, b;\n"
+                     "setp.eq.u32 pt, %0, %0;\n setp.ne.u32 pf, %0, %0;\n"
+                     HF_TK_STEP(0, 0, "pf") HF_TK_STEP(1, 2, "pt") HF_TK_STEP(2, 4, "pt") HF_TK_STEP(3, 6, "pt")
+                     HF_TK_STEP(4, 1024, "pt") HF_TK_STEP(5, 1026, "pt") HF_TK_STEP(6, 1028, "pt") HF_TK_STEP(7, 1030, "pt")
+                     "}\n" ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc) : "memory");
+    } else {
+        asm volatile("{\n .reg .pred pt, pf;\n .reg .b64 db;\n .reg .b32 a, b;\n"
+                     "setp.eq.u32 pt, %0, %0;\n setp.ne.u32 pf, %0, %0;\n"
+                     HF_TK_STEP(0, 0, "pf") HF_TK_STEP(1, 2, "pt") HF_TK_STEP(2, 4, "pt") HF_TK_STEP(3, 6, "pt")
+                     "}\n" ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc) : "memory");
+    }
+}
+#undef HF_TK_STEP
 // The same product with the A operand in two pieces: keys 0..63 at a_tmem (32 columns), keys 64..127 at a_tmem_hi.
 #define HF_TS2_STEP(KS, AOP, AOFF, PRED)                                                            \
     "add.u32 a, " AOP ", " #AOFF " * 8;\n add.u32 b, %2, " #KS " * 128;\n mov.b64 db, {b, %3};\n" \
@@ -153,6 +200,33 @@ __device__ __forceinline__ void mma_ts_tile_split(uint32_t d_tmem, uint32_t a_tm
                  : "memory");
 }
 #undef HF_TS2_STEP
+#define HF_TG_STEP(KS, AOFF, PRED)                                                                 \
+    "add.u32 a, %1, " #AOFF ";\n add.u32 b, %2, " #KS " * 128;\n mov.b64 db, {b, %3};\n"         \
+    "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], db, %4, " PRED ";\n"
+// D[tmem] (+)= A[tmem] * B[smem] over D contraction rows (B MN-major, 2048 bytes per 16 rows), A in four pieces of D / 4 rows,
+// 32 columns apart.
+template <int D>
+__device__ __forceinline__ void mma_ts_groups(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi, uint32_t idesc,
+                                              bool accumulate_first) {
+    if constexpr (D == 128) {
+        asm volatile("{\n .reg .pred pt, p0;\n .reg .b64 db;\n .reg .b32 a, b;\n"
+                     "setp.eq.u32 pt, %0, %0;\n setp.ne.b32 p0, %5, 0;\n"
+                     HF_TG_STEP(0, 0, "p0") HF_TG_STEP(1, 8, "pt") HF_TG_STEP(2, 32, "pt") HF_TG_STEP(3, 40, "pt")
+                     HF_TG_STEP(4, 64, "pt") HF_TG_STEP(5, 72, "pt") HF_TG_STEP(6, 96, "pt") HF_TG_STEP(7, 104, "pt")
+                     "}\n" ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"((uint32_t)accumulate_first) : "memory");
+    } else {
+        asm volatile("{\n .reg .pred pt, p0;\n .reg .b64 db;\n .reg .b32 a, b;\n"
+                     "setp.eq.u32 pt, %0, %0;\n setp.ne.b32 p0, %5, 0;\n"
+                     HF_TG_STEP(0, 0, "p0") HF_TG_STEP(1, 32, "pt") HF_TG_STEP(2, 64, "pt") HF_TG_STEP(3, 96, "pt")
+                     "}\n" ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"((uint32_t)accumulate_first) : "memory");
+    }
+}
+#undef HF_TG_STEP
+// Copy 128 rows x 32 bytes from shared memory (matrix descriptor) to 8 columns of tensor memory; ordered before the MMAs
+// the same thread issues afterwards.
+__device__ __forceinline__ void tmem_cp_128x256b(uint32_t d_tmem, uint64_t s_desc) {
+    asm volatile("tcgen05.cp.cta_group::1.128x256b [%0], %1;\n" ::"r"(d_tmem), "l"(s_desc) : "memory");
+}
 // 32 lanes x 32 consecutive 32-bit columns: thread t of the warp gets lane (base lane + t)
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "

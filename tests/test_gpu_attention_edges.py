@@ -1,0 +1,45 @@
+"""The attention kernel at the edges of its tiling: units of one tile (the history products share its S buffer), lists longer than
+the 32 entries of one tail window, a chunk shorter than a tile, ragged last blocks, units on the same thread block with a new
+head in between; forward (selection + both branches in one kernel) and softmax branch with lse, against the oracle."""
+import numpy as np
+import pytest
+
+from paper_2604_10103_b200 import inputs as gen
+from tests import harness as hz
+
+pytestmark = pytest.mark.gpu
+
+f64 = gen.bf16_bits_to_f64
+
+
+@pytest.mark.parametrize("d,block,tpf,wf,topk,heads,batch", [
+    (128, 128, 1000, 2, 1, 10, 2),     # one tile per unit, 160 units: two units on some thread blocks
+    (64, 128, 1000, 2, 1, 10, 2),
+    (64, 128, 100, 2, 2, 3, 1),        # one short block per chunk: every tile is a tail
+    (128, 128, 520, 7, 35, 2, 1),      # all 35 blocks kept (last one of each chunk 8 tokens): two tail windows
+    (64, 64, 130, 4, 1, 3, 1),         # small blocks, lists of one
+    (128, 64, 330, 3, 5, 2, 1),
+    (128, 16, 200, 3, 1, 2, 1),        # up to eight one-entry lists in a unit; last block 8 tokens
+    (64, 16, 90, 5, 7, 2, 2),
+])
+def test_forward_at_tile_edges(d, block, tpf, wf, topk, heads, batch):
+    w = gen.Workload("edges", batch=batch, heads=heads, head_dim=d, tokens_per_frame=tpf, chunk_frames=1, window_frames=wf, block=block,
+                     topk=topk, keep_permille=0, seed=211)
+    gpu = hz.GpuStream(w); ora = hz.make_oracle(w)
+    try:
+        for c in range(wf + 1):
+            kc, vc = gen.clean_kv(w, 0, c)
+            gpu.append(gpu.up(kc), gpu.up(vc)); ora.append(f64(kc), f64(vc))
+        qb, kb, vb = gen.qkv(w, 0, wf + 1, 0)
+        q, k, v = gpu.up(qb), gpu.up(kb), gpu.up(vb)
+        m_gpu, _, _ = gpu.select(q, k)
+        m_ref, _ = ora.select(f64(qb), f64(kb))
+        assert np.array_equal(m_gpu, m_ref)
+        o_ref, ol_ref, _ = ora.forward(f64(qb), f64(kb), f64(vb), mask=m_ref, parts=True)
+        hz.assert_close_out(gpu.forward(q, k, v), o_ref, "hybrid O")
+        o_local, lse = gpu.swa(q, k, v, want_lse=True)
+        hz.assert_close_out(o_local, ol_ref, "softmax branch")
+        assert np.isfinite(lse).all()
+        assert gpu.ctx.hf_get_device_status() == (0, 0)
+    finally:
+        gpu.close()
