@@ -201,6 +201,13 @@ hf_status set_swa_attr() {
     return HF_OK;
 }
 template <int D>
+hf_status set_select_attr() {
+    HF_CUDA(cudaFuncSetAttribute(k_select<D, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D>::smem_bytes(128)));
+    HF_CUDA(cudaFuncSetAttribute(k_select<D, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D>::smem_bytes(256)));
+    HF_CUDA(cudaFuncSetAttribute(k_select<D, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D>::smem_bytes(HF_MAX_TN)));
+    return HF_OK;
+}
+template <int D>
 hf_status set_state_attr() {
     HF_CUDA(cudaFuncSetAttribute(k_absorb_tc5<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AbsorbTc5<D>::SMEM_BYTES));
     HF_CUDA(cudaFuncSetAttribute(k_absorb_tc5<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, AbsorbTc5<D>::SMEM_BYTES));
@@ -460,15 +467,14 @@ hf_status launch_select(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_c
     const int Tn = (L.n_sink + L.n_cached + 1) * c->n_b;
     const int keep = keep_for(c, Tn);
     ChunkTable tab = make_table(c, L, k_cur, nullptr);
-    PdlLaunch pl(dim3(c->Tm, c->BH), dim3(256), 0, st, true);      // follows the pooling kernel launched above
-    // Two forms of the scoring loop, same arithmetic: the wide one keeps a pass's loads in flight (80 registers, three
-    // thread blocks per SM) and is ahead while the grid fits that; the narrow one (40 registers) fits twice the thread blocks.
-    if (c->Tm * c->BH <= 3 * c->sm_count)
-        HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_select<D, true>, tab, (const float*)c->pooled_q, c->n_b, c->Tm, Tn, keep, c->mask_words,
-                                   L.mask, L.idx, mask_out, idx_out, scores_out));
-    else
-        HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_select<D, false>, tab, (const float*)c->pooled_q, c->n_b, c->Tm, Tn, keep, c->mask_words,
-                                   L.mask, L.idx, mask_out, idx_out, scores_out));
+    typedef Select<D> S;
+    PdlLaunch pl(dim3((c->Tm + S::R - 1) / S::R, c->BH), dim3(256), S::smem_bytes(Tn), st, true);      // follows the pooling kernel launched above
+#define HF_SELECT(KPL_) cudaLaunchKernelEx(&pl.cfg, k_select<D, KPL_>, tab, (const float*)c->pooled_q, c->n_b, c->Tm, Tn, keep, c->mask_words, \
+                                           L.mask, L.idx, mask_out, idx_out, scores_out, -0.f)
+    if (Tn <= 128) HF_CUDA(HF_SELECT(4));           // (registers of the ranking warps: T_n / 32 images per lane)
+    else if (Tn <= 256) HF_CUDA(HF_SELECT(8));
+    else HF_CUDA(HF_SELECT(32));
+#undef HF_SELECT
     HF_TRY(post_launch(c, "k_select"));
     L.sel_epoch = L.cache_epoch;
     L.sel_keep = keep;
@@ -806,6 +812,8 @@ hf_status hf_create(const hf_config* cfg, int device, hf_ctx** out) {
         if (s == HF_OK) s = set_swa_tc5_attr<128, 128>();
         if (s == HF_OK && cudaFuncSetAttribute(k_swa_tc5p<64, HF_TC5P_COLGROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5P<64, HF_TC5P_COLGROUPS>::SMEM_BYTES) != cudaSuccess) s = fail(HF_ERR_CUDA, "cudaFuncSetAttribute(k_swa_tc5p<64>) failed");
         if (s == HF_OK && cudaFuncSetAttribute(k_swa_tc5p<128, HF_TC5P_COLGROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5P<128, HF_TC5P_COLGROUPS>::SMEM_BYTES) != cudaSuccess) s = fail(HF_ERR_CUDA, "cudaFuncSetAttribute(k_swa_tc5p<128>) failed");
+        if (s == HF_OK) s = set_select_attr<64>();
+        if (s == HF_OK) s = set_select_attr<128>();
         if (s == HF_OK) s = set_state_attr<64>();
         if (s == HF_OK) s = set_state_attr<128>();
     }

@@ -178,169 +178,194 @@ __global__ void __launch_bounds__(256, 6) k_pool_copy_layers(const __grid_consta
     pool_copy_block<D, false>(jb, Tc, blk, n_b, blockIdx.x, blockIdx.y, none);
 }
 
-// A[i][j] = Mean(q_i) . Mean(k_j) in the canonical order, formed by one warp: 32 partials (partial l = columns l,
-// l + 32, ... ascending, product and sum rounded separately; lane l holds partial l, so the loads of a key row are
-// coalesced), then the butterfly p[l] + p[l ^ off], off = 16 .. 1: both partners get the same value (IEEE addition
-// commutes), so lane 0 ends with the fold of the upper half onto the lower half level by level, bit for bit.
-// grid (T_m, B*H), 256 threads.  One query-block row: T_n scores, top-K under the total order (score descending, block
-// index ascending; by counting for short rows, by a bitonic sort of (score, index) keys for long ones), bit mask +
-// ascending index list.
-template <int D, bool WIDE>
+// A[i][j] = Mean(q_i) . Mean(k_j) in the canonical order, and the top-K of every row under the total order (score descending,
+// block index ascending): bit mask and ascending index list.  grid (ceil(T_m / 4), B*H), 256 threads: four query blocks of a
+// head per thread block.
+//
+// Scores: one THREAD per (query block, key block).  The butterfly of the canonical order is a plain tree, so a thread that walks
+// the columns in the order l, l + 16, l + 8, l + 24 (l = 0..3, then 4..7) needs four running values and no shuffle: 2 D - 1
+// packed fp32 operations per pair of columns.  Key rows come from shared memory (padded rows: conflict-free 16-byte reads), each
+// fetched from L2 once for four query blocks, the cached chunks' before the wait for the pooling kernel; query rows are
+// broadcast reads.  Top-K: one WARP per row, score images in registers, the keep-th largest found bit by bit (count by
+// redux; the search ends as soon as a threshold separates exactly `keep`), ties cut by ballot.
+//
+// What bounds it: latency (a trip to L2, 32 + 32 tree steps, ~16 count steps).  The form before (one warp per score with its
+// five-step butterfly, one query block per thread block, ranking by counting or a bitonic sort of the whole block):
+// pooling + selection as part of the forward, 12 heads of 128: 128-token blocks (T_n 111) 128.3 -> 125.5 us, 64-token blocks
+// (T_n 222) 171 -> 164 us, 16-token blocks at head dim 64 (T_n 246) 64.6 -> 55.1 us; this kernel alone at T_n 259, batch 4:
+// 76 -> 39 us.
+template <int D>
+struct Select {
+    static constexpr int R = 4, KT = 128;       // query blocks per thread block; key rows per pass
+    static constexpr int LD = D + 4;            // floats per key row in shared memory
+    static int smem_bytes(int Tn) { const int kt = Tn < KT ? Tn : KT; return (kt * LD + R * D + R * Tn) * (int)sizeof(float); }
+};
+struct Quad { float2 a, b; };                   // four neighbouring columns
+__device__ __forceinline__ Quad quad_add(const Quad& x, const Quad& y) { return {fadd2(x.a, y.a), fadd2(x.b, y.b)}; }
+// Products rounded separately: x y + (-0), which is the rounded product for every x y.  (The packed multiply would be contracted
+// with the packed addition that follows it, explicit rounding or not.)  nz: (-0, -0), a run-time value for the same reason.
+__device__ __forceinline__ Quad quad_mul(const float4& x, const float4& y, float2 nz) {
+    return {ffma2(make_float2(x.x, x.y), make_float2(y.x, y.y), nz), ffma2(make_float2(x.z, x.w), make_float2(y.z, y.w), nz)};
+}
+// Scores of one key row against RPT query rows (rows of D floats in shared memory).
+template <int D, int RPT>
+__device__ __forceinline__ void canonical_scores(const float* kr, const float* qr, float2 nz, float (&out)[RPT]) {
+    constexpr int M = D / 32;
+    Quad c[RPT];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {               // l = 0..3, then 4..7
+        Quad b[RPT];
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {           // columns l and l + 16, then l + 8 and l + 24
+            Quad a[RPT];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int x = 4 * h + 8 * g + 16 * e;
+                float4 kv[M];
+#pragma unroll
+                for (int m = 0; m < M; ++m) kv[m] = *reinterpret_cast<const float4*>(kr + x + 32 * m);
+#pragma unroll
+                for (int r = 0; r < RPT; ++r) {
+                    Quad part = quad_mul(*reinterpret_cast<const float4*>(qr + r * D + x), kv[0], nz);
+#pragma unroll
+                    for (int m = 1; m < M; ++m) part = quad_add(part, quad_mul(*reinterpret_cast<const float4*>(qr + r * D + x + 32 * m), kv[m], nz));
+                    a[r] = e == 0 ? part : quad_add(a[r], part);
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) b[r] = g == 0 ? a[r] : quad_add(b[r], a[r]);
+        }
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) c[r] = h == 0 ? b[r] : quad_add(c[r], b[r]);
+    }
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) {
+        const float2 dd = fadd2(c[r].a, c[r].b);
+        out[r] = __fadd_rn(dd.x, dd.y);
+    }
+}
+// Order-preserving image of a score: ascending integers = ascending floats, -0 = +0, a NaN (anywhere in the query block or the
+// key block) below every number, so that exactly `keep` blocks are kept whatever the inputs hold.
+__device__ __forceinline__ uint32_t score_image(float s) {
+    const uint32_t u = __float_as_uint(s);
+    if (s != s) return 0u;
+    if (u == 0x80000000u) return 0x80000000u;
+    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+
+// KPL: key blocks per lane of a ranking warp (T_n <= 32 KPL).
+template <int D, int KPL>
 __global__ void __launch_bounds__(256) k_select(ChunkTable tab, const float* __restrict__ pooled_q,
                                                 int n_b, int Tm, int Tn, int keep, int mask_words,
                                                 uint32_t* __restrict__ mask, int32_t* __restrict__ idx,
                                                 uint32_t* __restrict__ mask_out, int32_t* __restrict__ idx_out,
-                                                float* __restrict__ scores_out) {
-    __shared__ float sc[HF_MAX_TN];
-    __shared__ uint8_t keepf[HF_MAX_TN];
-    __shared__ unsigned long long keys[HF_MAX_TN];
-    const int i = blockIdx.x, bh = blockIdx.y;
+                                                float* __restrict__ scores_out, float neg_zero) {
+    typedef Select<D> C;
+    const float2 nz = make_float2(neg_zero, neg_zero);
+    extern __shared__ __align__(16) float sel_smem[];
+    const int kt = min(Tn, C::KT);
+    float* s_k = sel_smem;                      // [kt][LD]
+    float* s_q = s_k + kt * C::LD;              // [R][D]
+    float* s_sc = s_q + C::R * D;               // [R][Tn]
+    const int i0 = blockIdx.x * C::R, bh = blockIdx.y;
+    const int rows = min(C::R, Tm - i0);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const size_t row = (size_t)bh * Tm + i;
-    pdl_trigger();              // the attention kernel may be made resident as blocks of this grid leave
-    pdl_wait();                 // the pooled rows of the query and of the current chunk come from the kernel before
-    // One warp per score, lane l = partial l.  All loads of a pass (the lane's columns of the query row and of sixteen key
-    // rows) are issued before the first use: one trip to memory per pass, and one pass covers 128 key blocks.
-    constexpr int NW = 8, PER = 16, M = D / 32;
-    float qv[M];
-#pragma unroll
-    for (int m = 0; m < M; ++m) qv[m] = __ldg(pooled_q + row * D + lane + 32 * m);
-    for (int base = 0; base < Tn; base += NW * PER) {
-        float kv[PER][M];
-#pragma unroll
-        for (int u = 0; u < PER; ++u) {
-            const int j = min(base + warp + NW * u, Tn - 1);
-            const int c = j / n_b, jb = j - c * n_b;
-            const float* kp = tab.pooled[c] + ((size_t)bh * n_b + jb) * D + lane;
-#pragma unroll
-            for (int m = 0; m < M; ++m) kv[u][m] = __ldg(kp + 32 * m);
+    const uint32_t s_k_addr = smem_u32(s_k);
+    // key rows [j0, j1) of the pass that starts at `base`, sixteen bytes per thread and step
+    auto load_keys = [&](int base, int j0, int j1) {
+        constexpr int V = D / 4;
+        for (int e = threadIdx.x; e < (j1 - j0) * V; e += 256) {
+            const int j = j0 + e / V, part = e % V;
+            int c = 0, jb = j;
+            while (jb >= n_b) { jb -= n_b; ++c; }
+            cp_async16(s_k_addr + ((j - base) * C::LD + part * 4) * 4, tab.pooled[c] + ((size_t)bh * n_b + jb) * D + part * 4, true);
         }
-        if constexpr (WIDE) {
-            // one butterfly per key row (the compiler keeps all loads of the pass in flight in front of them: ~80 registers)
-#pragma unroll
-            for (int u = 0; u < PER; ++u) {
-                float p = __fmul_rn(qv[0], kv[u][0]);
-#pragma unroll
-                for (int m = 1; m < M; ++m) p = __fadd_rn(p, __fmul_rn(qv[m], kv[u][m]));
-#pragma unroll
-                for (int off = 16; off >= 1; off >>= 1) p = __fadd_rn(p, __shfl_xor_sync(0xffffffffu, p, off));
-                const int j = base + warp + NW * u;
-                if (lane == 0 && j < Tn) {
-                    sc[j] = p;
-                    if (scores_out) scores_out[row * Tn + j] = p;
-                }
-            }
-        } else {
-            // The sixteen butterflies side by side.  At the step with lane offset `off` a lane keeps the half of its rows
-            // that its own bit of `off` names and hands the other half to its partner, which does the opposite: every sum
-            // is still own partial + partner's partial (IEEE addition commutes, so both orders give the same bits), level
-            // by level as in the one-row butterfly, with 8 + 4 + 2 + 1 + 1 shuffles instead of 16 x 5.  After the last
-            // step lanes 2u and 2u + 1 both hold the score of row u.  (The compiler pairs this form's loads with their
-            // products: ~40 registers, twice the resident thread blocks, more trips to memory per pass.)
-            float pa[PER];
-#pragma unroll
-            for (int u = 0; u < PER; ++u) {
-                float p = __fmul_rn(qv[0], kv[u][0]);
-#pragma unroll
-                for (int m = 1; m < M; ++m) p = __fadd_rn(p, __fmul_rn(qv[m], kv[u][m]));
-                pa[u] = p;
-            }
-#pragma unroll
-            for (int half = PER / 2, off = 16; half >= 1; half >>= 1, off >>= 1) {
-                const bool upper = (lane & off) != 0;
-#pragma unroll
-                for (int x = 0; x < half; ++x) {
-                    const float mine = upper ? pa[x + half] : pa[x];
-                    const float theirs = upper ? pa[x] : pa[x + half];
-                    pa[x] = __fadd_rn(mine, __shfl_xor_sync(0xffffffffu, theirs, off));
-                }
-            }
-            static_assert(PER == 16, "one row per lane pair after four halvings");
-            const float score = __fadd_rn(pa[0], __shfl_xor_sync(0xffffffffu, pa[0], 1));
-            const int j = base + warp + NW * (lane >> 1);
-            if ((lane & 1) == 0 && j < Tn) {
-                sc[j] = score;
-                if (scores_out) scores_out[row * Tn + j] = score;
-            }
-        }
-    }
-    __syncthreads();
-    // Keep the `keep` best under a TOTAL order: score descending, then block index ascending; +0 and -0 tie; a NaN score (a
-    // NaN anywhere in the query block or the key block) compares false both ways and would otherwise rank first everywhere:
-    // here it ranks below every number, NaNs among themselves by block index, so that exactly `keep` blocks are kept whatever
-    // the inputs hold.
-    // 64-bit keys: an order-preserving image of the score (NaN lowest, -0 = +0), then the complement of the block index;
-    // all keys of a row are distinct and "comes before" is "has the larger key"
-    auto key_of = [](float s, int j) -> unsigned long long {
-        uint32_t u = __float_as_uint(s);
-        if (s != s) u = 0u;                                         // NaN: below -inf
-        else {
-            if (u == 0x80000000u) u = 0u;                           // -0 ties with +0
-            u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);         // ascending integers = ascending floats
-        }
-        return ((unsigned long long)u << 32) | (unsigned long long)(0xffffffffu - (uint32_t)j);
+        cp_async_commit();
     };
-    if (Tn <= 128) {
-        // short rows: count, for every block, the blocks that come before it.  Two threads per block, one for the even and
-        // one for the odd competitors, four comparisons in flight each.
-        for (int j = threadIdx.x; j < Tn; j += 256) keys[j] = key_of(sc[j], j);
-        __syncthreads();
-        {
-            const int j = threadIdx.x >> 1, par = threadIdx.x & 1;
-            int rank = 0;
-            if (j < Tn) {
-                const unsigned long long mine = keys[j];
-                int r0 = 0, r1 = 0, r2 = 0, r3 = 0;
-                int jj = par;
-                for (; jj + 6 < Tn; jj += 8) {
-                    r0 += keys[jj] > mine; r1 += keys[jj + 2] > mine; r2 += keys[jj + 4] > mine; r3 += keys[jj + 6] > mine;
-                }
-                for (; jj < Tn; jj += 2) r0 += keys[jj] > mine;
-                rank = (r0 + r1) + (r2 + r3);
-            }
-            rank += __shfl_xor_sync(0xffffffffu, rank, 1);
-            if (par == 0 && j < Tn) keepf[j] = rank < keep;
+    pdl_trigger();              // the attention kernel may be made resident as blocks of this grid leave
+    // The cached chunks' rows are older than the pooling kernel before this one (which has itself waited for what came before it).
+    const int old = min((tab.n_chunks - 1) * n_b, kt);
+    load_keys(0, 0, old);
+    pdl_wait();                 // the pooled rows of the queries and of the current chunk come from the kernel before
+    for (int e = threadIdx.x; e < rows * (D / 4); e += 256)
+        cp_async16(smem_u32(s_q) + e * 16, pooled_q + ((size_t)bh * Tm + i0) * D + e * 4, true);
+    load_keys(0, old, kt);
+    for (int base = 0; base < Tn; base += C::KT) {
+        const int n = min(C::KT, Tn - base);
+        if (base > 0) {
+            __syncthreads();    // the pass before has been read
+            load_keys(base, base, base + n);
         }
-    } else {
-        // long rows (counting is quadratic in T_n): sort the keys in shared memory with a bitonic network and compare every
-        // block with the keep-th key
-        int n2 = 256;
-        while (n2 < Tn) n2 <<= 1;
-        for (int j = threadIdx.x; j < n2; j += 256) keys[j] = j < Tn ? key_of(sc[j], j) : 0ull;      // padding sorts last
+        cp_async_wait<0>();
         __syncthreads();
-        for (int size = 2; size <= n2; size <<= 1) {
-            for (int stride = size >> 1; stride > 0; stride >>= 1) {
-                for (int x = threadIdx.x; x < (n2 >> 1); x += 256) {
-                    const int lo = 2 * x - (x & (stride - 1)), hi = lo + stride;      // the pair (lo, lo + stride)
-                    const bool descending = (lo & size) == 0;
-                    const unsigned long long a = keys[lo], b = keys[hi];
-                    if ((a < b) == descending) { keys[lo] = b; keys[hi] = a; }
-                }
-                __syncthreads();
+        if (n <= 64) {          // few keys: one score per thread
+            const int j = threadIdx.x & 63, r = threadIdx.x >> 6;
+            if (j < n && r < rows) {
+                float v[1];
+                canonical_scores<D, 1>(s_k + j * C::LD, s_q + r * D, nz, v);
+                s_sc[r * Tn + base + j] = v[0];
+            }
+        } else {                // two scores per thread: query blocks 2 h, 2 h + 1 (rows past T_m: stale shared memory, not stored)
+            const int j = threadIdx.x & 127, r = (threadIdx.x >> 7) * 2;
+            if (j < n && r < rows) {
+                float v[2];
+                canonical_scores<D, 2>(s_k + j * C::LD, s_q + r * D, nz, v);
+                s_sc[r * Tn + base + j] = v[0];
+                if (r + 1 < rows) s_sc[(r + 1) * Tn + base + j] = v[1];
             }
         }
-        const unsigned long long kth = keys[keep - 1];
-        for (int j = threadIdx.x; j < Tn; j += 256) keepf[j] = key_of(sc[j], j) >= kth;
     }
     __syncthreads();
-    if (warp == 0) {
-        int running = 0;
-        for (int w = 0; w < mask_words; ++w) {
-            const int j = w * 32 + lane;
-            const bool f = (j < Tn) && keepf[j];
-            const uint32_t word = __ballot_sync(0xffffffffu, f);
-            if (lane == 0) {
-                mask[row * mask_words + w] = word;
-                if (mask_out) mask_out[row * mask_words + w] = word;
+    if (scores_out)
+        for (int e = threadIdx.x; e < rows * Tn; e += 256) scores_out[((size_t)bh * Tm + i0) * Tn + e] = s_sc[e];
+    if (warp >= rows) return;
+    // ---- top-K of row `warp`: lane l holds the images of blocks l, l + 32, ... (padding: 0, and behind every block)
+    const size_t row = (size_t)bh * Tm + i0 + warp;
+    uint32_t key[KPL];
+#pragma unroll
+    for (int x = 0; x < KPL; ++x) {
+        const int j = x * 32 + lane;
+        key[x] = j < Tn ? score_image(s_sc[warp * Tn + j]) : 0u;
+    }
+    uint32_t thr = 0;           // largest value with at least `keep` images at or above it
+    bool exact = keep >= Tn;    // ... and exactly `keep`: no ties to cut (all blocks kept: every image counts)
+    for (uint32_t bit = 0x80000000u; bit != 0u && !exact; bit >>= 1) {
+        const uint32_t cand = thr | bit;
+        int n = 0;
+#pragma unroll
+        for (int x = 0; x < KPL; ++x) n += key[x] >= cand;
+        n = __reduce_add_sync(0xffffffffu, n);
+        if (n >= keep) { thr = cand; exact = n == keep; }
+    }
+    int ties = Tn;              // blocks at the threshold still to be kept, lowest index first
+    if (!exact) {
+        int n = 0;
+#pragma unroll
+        for (int x = 0; x < KPL; ++x) n += key[x] > thr;
+        ties = keep - __reduce_add_sync(0xffffffffu, n);
+    }
+    const uint32_t below = (1u << lane) - 1u;
+    int pos = 0;
+    uint32_t my_word = 0;
+#pragma unroll
+    for (int x = 0; x < KPL; ++x) {
+        const int j = x * 32 + lane;
+        const uint32_t eq = __ballot_sync(0xffffffffu, j < Tn && key[x] == thr);
+        const bool kept = j < Tn && (key[x] > thr || (key[x] == thr && __popc(eq & below) < ties));
+        ties -= __popc(eq);
+        const uint32_t word = __ballot_sync(0xffffffffu, kept);
+        if (lane == x) my_word = word;
+        if (kept) {
+            const int at = pos + __popc(word & below);
+            if (at < keep) {    // (always true under the total order above; the store never leaves the row)
+                idx[row * keep + at] = j;
+                if (idx_out) idx_out[row * keep + at] = j;
             }
-            if (f) {
-                const int pos = running + __popc(word & ((1u << lane) - 1u));
-                if (pos < keep) {       // (always true under the total order above; the store never leaves the row)
-                    idx[row * keep + pos] = j;
-                    if (idx_out) idx_out[row * keep + pos] = j;
-                }
-            }
-            running += __popc(word);
         }
+        pos += __popc(word);
+    }
+    if (lane < mask_words) {
+        mask[row * mask_words + lane] = my_word;
+        if (mask_out) mask_out[row * mask_words + lane] = my_word;
     }
 }
