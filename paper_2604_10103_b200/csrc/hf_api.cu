@@ -596,7 +596,8 @@ hf_status launch_bwd_dq(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_c
     if (c->bwd_delta == nullptr) HF_TRY(dmalloc(&c->bwd_delta, (size_t)c->BH * c->Tc));
     HF_CUDA(cudaFuncSetAttribute(k_swa_bwd_dq<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES));
     const long long rows = (long long)c->BH * c->Tc;
-    k_rowdot<D><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(d_o, o_local, c->bwd_delta, rows);
+    PdlLaunch pr(dim3((unsigned)((rows + RowDot<D>::RPB - 1) / RowDot<D>::RPB)), dim3(256), 0, st, true);
+    HF_CUDA(cudaLaunchKernelEx(&pr.cfg, k_rowdot<D>, d_o, o_local, c->bwd_delta, rows));
     HF_TRY(post_launch(c, "k_rowdot"));
     CUtensorMap tq, tdo, tk, tv;
     HF_TRY(make_map(c, &tq, q, 1));
@@ -608,11 +609,12 @@ hf_status launch_bwd_dq(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_c
     p.idx = idx; p.keep = keep; p.Tc = c->Tc; p.n_b = c->n_b; p.n_cached = L.n_cached; p.ring_head = L.head; p.P = c->R; p.n_sink = L.n_sink;
     p.Tm = c->Tm; p.n_units = c->Tm * c->BH;
     p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D)); p.scale = (float)(1.0 / std::sqrt((double)D));
+    p.nb_magic = c->n_b > 1 ? (uint32_t)((0x100000000ull + c->n_b - 1) / c->n_b) : 0u;
     p.lse = lse; p.delta = c->bwd_delta; p.dq = dq; p.dev_status = c->dev_status;
     const CUtensorMap& rk = c->R + c->n_sink_max > 0 ? L.tm_kring : tk;
     const CUtensorMap& rv = c->R + c->n_sink_max > 0 ? L.tm_vring : tv;
     const int grid = p.n_units < c->sm_count ? p.n_units : c->sm_count;
-    PdlLaunch pl(dim3(grid), dim3(C::THREADS), C::SMEM_BYTES, st, false);
+    PdlLaunch pl(dim3(grid), dim3(C::THREADS), C::SMEM_BYTES, st, true);
     HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_bwd_dq<D>, tq, tdo, rk, rv, tk, tv, p));
     return post_launch(c, "k_swa_bwd_dq");
 }
@@ -624,7 +626,8 @@ hf_status launch_bwd_dkv(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_
     if (c->bwd_delta == nullptr) HF_TRY(dmalloc(&c->bwd_delta, (size_t)c->BH * c->Tc));
     HF_CUDA(cudaFuncSetAttribute(k_swa_bwd_dkv<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES));
     const long long rows = (long long)c->BH * c->Tc;
-    k_rowdot<D><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(d_o, o_local, c->bwd_delta, rows);
+    PdlLaunch pr(dim3((unsigned)((rows + RowDot<D>::RPB - 1) / RowDot<D>::RPB)), dim3(256), 0, st, true);
+    HF_CUDA(cudaLaunchKernelEx(&pr.cfg, k_rowdot<D>, d_o, o_local, c->bwd_delta, rows));
     HF_TRY(post_launch(c, "k_rowdot"));
     CUtensorMap tq, tdo, tk, tv;
     HF_TRY(make_map(c, &tq, q, 1));
@@ -638,7 +641,7 @@ hf_status launch_bwd_dkv(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_
     p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D)); p.scale = (float)(1.0 / std::sqrt((double)D));
     p.lse = lse; p.delta = c->bwd_delta; p.dk = dk; p.dv = dv; p.dev_status = c->dev_status;
     const int grid = p.n_units < c->sm_count ? p.n_units : c->sm_count;
-    PdlLaunch pl(dim3(grid), dim3(C::THREADS), C::SMEM_BYTES, st, false);
+    PdlLaunch pl(dim3(grid), dim3(C::THREADS), C::SMEM_BYTES, st, true);
     HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_bwd_dkv<D>, tq, tdo, tk, tv, p));
     return post_launch(c, "k_swa_bwd_dkv");
 }

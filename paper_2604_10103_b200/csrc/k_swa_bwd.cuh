@@ -11,29 +11,77 @@
 //   dP = dO V_t^T         A = dO (smem, K-major),  B = V_t (smem, K-major)          -> TMEM [128, 256)
 //   dQ += dS K_t          A = dS (TMEM, bf16, written over S),  B = K_t (MN-major)   -> TMEM [256, 256 + D)
 // and between them, on the softmax warps (thread = query row x half of the 128 key columns):
-//   dS = exp2(S c - lse log2 e) * (dP - delta) / sqrt(d)        (columns past a short block's end: 0)
+//   dS = exp2(S c - lse log2 e) * (dP - delta)        (columns past a short block's end: 0; 1 / sqrt(d) is applied to dQ)
 // The two score products of tile t + 1 are issued while the softmax warps work on tile t: S has two buffers, and the
 // softmax threads free dP's one buffer as soon as their share of it is in registers.  A K tile is held from S to dS K
 // (three stages), a V tile only until dP (two); with less, the latency of the tile loads (~3 000 clk here) is what a
-// tile costs.  Every wait is bounded and reports through the device status word.
+// tile costs.  The softmax section runs in packed fp32, with the tail mask as separate code and one arrival per warp: 153 -> 132
+// us at 12 heads of 128, 4 680 queries, 28 kept blocks, against scalar code with a select per column.
+// Every wait is bounded and reports through the device status word.
 #pragma once
 #include "k_swa_tc5.cuh"
 
-// delta[r] = sum_d dO[r][d] * O[r][d], one warp per row.  grid: ceil(rows / 8), 256 threads.
+// delta[r] = sum_d dO[r][d] * O[r][d].  D / 8 lanes per row (16 bytes of each tensor per lane), four rows per lane with all
+// eight loads in flight: memory-bound (28.75 MB at 12 heads x 4 680 rows x 128: 11.5 us with one row per warp and four bytes
+// per lane, 5.7 us like this).  grid: ceil(rows / (4 * 256 / (D / 8))), 256 threads.
+template <int D>
+struct RowDot { static constexpr int LPR = D / 8, RPB = 4 * 256 / LPR; };      // lanes per row; rows per thread block
 template <int D>
 __global__ void __launch_bounds__(256) k_rowdot(const bf16* __restrict__ a, const bf16* __restrict__ b, float* __restrict__ out, long long rows) {
-    const long long r = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (r >= rows) return;
-    float acc = 0.f;
-    for (int c = lane * 2; c < D; c += 64) {
-        const float2 x = unpack_bf16(*reinterpret_cast<const uint32_t*>(a + r * D + c));
-        const float2 y = unpack_bf16(*reinterpret_cast<const uint32_t*>(b + r * D + c));
-        acc = fmaf(x.x, y.x, fmaf(x.y, y.y, acc));
+    typedef RowDot<D> C;
+    pdl_wait();
+    pdl_trigger();              // the backward kernel may set itself up; it waits for this grid before it reads delta
+    const int part = threadIdx.x % C::LPR;
+    const long long r0 = (long long)blockIdx.x * C::RPB + threadIdx.x / C::LPR;
+    uint4 x[4], y[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const long long r = r0 + i * (256 / C::LPR);
+        x[i] = y[i] = make_uint4(0, 0, 0, 0);
+        if (r < rows) {
+            x[i] = __ldg(reinterpret_cast<const uint4*>(a + r * D) + part);
+            y[i] = __ldg(reinterpret_cast<const uint4*>(b + r * D) + part);
+        }
     }
 #pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (lane == 0) out[r] = acc;
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t xs[4] = {x[i].x, x[i].y, x[i].z, x[i].w}, ys[4] = {y[i].x, y[i].y, y[i].z, y[i].w};
+        float acc = 0.f;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float2 u = unpack_bf16(xs[e]), v = unpack_bf16(ys[e]);
+            acc = fmaf(u.x, v.x, fmaf(u.y, v.y, acc));
+        }
+#pragma unroll
+        for (int off = C::LPR / 2; off >= 1; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        const long long r = r0 + i * (256 / C::LPR);
+        if (part == 0 && r < rows) out[r] = acc;
+    }
+}
+
+// dS / scale = P (dP - delta) of 32 columns of a thread's row as bf16 pairs: packed fp32, two columns per instruction; the factor
+// 1 / sqrt(d) waits for the output.  MASK: columns from nv on count nothing.
+template <bool MASK>
+__device__ __forceinline__ void bwd_ds(const uint32_t* s, const uint32_t* dp, int nv, float scale_log2, float neg_lse2, float delta, uint32_t (&pk)[16]) {
+    const float2 c2 = make_float2(scale_log2, scale_log2), l2 = make_float2(neg_lse2, neg_lse2), nd = make_float2(-delta, -delta);
+#pragma unroll
+    for (int e0 = 0; e0 < 32; e0 += 8) {
+        float2 x[4], g[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int e = e0 + 2 * v;
+            x[v] = ffma2(make_float2(__uint_as_float(s[e]), __uint_as_float(s[e + 1])), c2, l2);
+            g[v] = fadd2(make_float2(__uint_as_float(dp[e]), __uint_as_float(dp[e + 1])), nd);
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) x[v] = make_float2(fast_exp2(x[v].x), fast_exp2(x[v].y));
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int e = e0 + 2 * v;
+            x[v].x *= g[v].x; x[v].y *= g[v].y;
+            pk[e >> 1] = pack_bf16(MASK && e >= nv ? 0.f : x[v].x, MASK && e + 1 >= nv ? 0.f : x[v].y);
+        }
+    }
 }
 
 template <int D>
@@ -56,6 +104,7 @@ struct SwaBwd {
 struct SwaBwdParams {
     const int32_t* idx;      // [B*H, T_m, keep]
     int keep, Tc, n_b, n_cached, ring_head, P, n_sink, Tm, n_units;
+    uint32_t nb_magic;       // ceil(2^32 / n_b) (n_b > 1)
     float scale_log2, scale; // log2(e) / sqrt(d), 1 / sqrt(d)
     const float* lse;        // [B*H, T_c] natural log of the row's sum of exponentials (forward)
     const float* delta;      // [B*H, T_c] g . o_local
@@ -89,7 +138,7 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::KST; ++s) { mbar_init(bar_kf + 8 * s, 1); mbar_init(bar_ke + 8 * s, 1); }
         for (int s = 0; s < C::VST; ++s) { mbar_init(bar_vf + 8 * s, 1); mbar_init(bar_ve + 8 * s, 1); }
-        mbar_init(bar_qf, 1); mbar_init(bar_qe, 1); mbar_init(bar_sd, 1); mbar_init(bar_ds, 256); mbar_init(bar_dqf, 1); mbar_init(bar_dqe, 256); mbar_init(bar_dpf, 256);
+        mbar_init(bar_qf, 1); mbar_init(bar_qe, 1); mbar_init(bar_sd, 1); mbar_init(bar_ds, 8); mbar_init(bar_dqf, 1); mbar_init(bar_dqe, 8); mbar_init(bar_dpf, 8);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
@@ -207,6 +256,7 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         const int grp = warp >> 2;                          // key columns [64 grp, 64 grp + 64) of a tile
         const int row = (warp & 3) * 32 + lane;
         const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        const bool lane0 = lane == 0, ragged = p.Tc % C::BLK != 0;
         bool ok = true;
         int t = 0;
         for (int n = 0; ok && n < my_units; ++n) {
@@ -217,50 +267,47 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             const size_t g_row = (size_t)bh * p.Tc + q0 + row;
             const float neg_lse2 = row < nq ? -p.lse[g_row] * 1.4426950408889634f : 0.f;
             const float delta = row < nq ? p.delta[g_row] : 0.f;
+            uint32_t tails = 0;         // one bit per tile of the current 32: the block is a chunk's short last one
             for (int j = 0; j < keep; ++j, ++t) {
-                const int blk = __ldg(my_idx + j);
-                bool tail = false;
-#pragma unroll
-                for (int c = 1; c <= HF_MAX_CHUNKS; ++c) tail |= (blk + 1 == c * p.n_b);
-                const int nv = tail ? p.Tc - (p.n_b - 1) * C::BLK : C::BLK;
-                ok = __all_sync(0xffffffffu, mbar_wait(bar_sd, t & 1, abort_flag, p.dev_status, 89));
+                if (ragged && (j & 31) == 0) {
+                    const uint32_t x1 = j + lane < keep ? (uint32_t)__ldg(my_idx + j + lane) + 1u : 0xffffffffu;
+                    tails = __ballot_sync(0xffffffffu, x1 <= HF_MAX_TN && (p.n_b == 1 || __umulhi(x1, p.nb_magic) * p.n_b == x1));
+                }
+                ok = mbar_wait_warp(bar_sd, t & 1, abort_flag, p.dev_status, 89);
                 if (!ok) break;
                 fence_after_sync();
                 const uint32_t tS = lane_base + ((t & 1) ? C::COL_S1 : C::COL_S) + grp * 64;
-                // this thread's share of dP first, all of it: the MMA warp refills the buffer as soon as every thread has it
-                uint32_t dp[2][32], s[32];
+                // this thread's share of dP and S: the MMA warp refills dP's buffer as soon as every warp has it
+                uint32_t dp[2][32], s[2][32];
                 tmem_ld32(lane_base + C::COL_DP + grp * 64, dp[0]);
                 tmem_ld32(lane_base + C::COL_DP + grp * 64 + 32, dp[1]);
-                tmem_ld32(tS, s);
+                tmem_ld32(tS, s[0]);
+                tmem_ld32(tS + 32, s[1]);
                 tmem_wait_ld();
                 fence_before_sync();
-                mbar_arrive(bar_dpf);
+                mbar_arrive_if(bar_dpf, lane0);
+                // (all of this thread's S columns are in registers: the bf16 dS may go over them)
+                if (!((tails >> (j & 31)) & 1u)) {
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    uint32_t pk[16];
-                    if (c == 1) {
-                        tmem_ld32(tS + 32, s);
-                        tmem_wait_ld();
+                    for (int c = 0; c < 2; ++c) {
+                        uint32_t pk[16];
+                        bwd_ds<false>(s[c], dp[c], 32, p.scale_log2, neg_lse2, delta, pk);
+                        tmem_st16(tS + c * 16, pk);
                     }
+                } else {
 #pragma unroll
-                    for (int e = 0; e < 32; e += 2) {
-                        const float p0 = fast_exp2(fmaf(__uint_as_float(s[e]), p.scale_log2, neg_lse2));
-                        const float p1 = fast_exp2(fmaf(__uint_as_float(s[e + 1]), p.scale_log2, neg_lse2));
-                        float d0 = p0 * (__uint_as_float(dp[c][e]) - delta) * p.scale;
-                        float d1 = p1 * (__uint_as_float(dp[c][e + 1]) - delta) * p.scale;
-                        if (grp * 64 + c * 32 + e >= nv) d0 = 0.f;
-                        if (grp * 64 + c * 32 + e + 1 >= nv) d1 = 0.f;
-                        pk[e >> 1] = pack_bf16_alu(d0, d1);
+                    for (int c = 0; c < 2; ++c) {
+                        uint32_t pk[16];
+                        bwd_ds<true>(s[c], dp[c], p.Tc - (p.n_b - 1) * C::BLK - grp * 64 - c * 32, p.scale_log2, neg_lse2, delta, pk);
+                        tmem_st16(tS + c * 16, pk);
                     }
-                    // (all of this thread's S columns of the chunk are in registers: the bf16 dS may go over them)
-                    tmem_st16(tS + c * 16, pk);
                 }
                 tmem_wait_st();
                 fence_before_sync();
-                mbar_arrive(bar_ds);
+                mbar_arrive_if(bar_ds, lane0);
             }
             if (!ok) break;
-            ok = __all_sync(0xffffffffu, mbar_wait(bar_dqf, n & 1, abort_flag, p.dev_status, 90));
+            ok = mbar_wait_warp(bar_dqf, n & 1, abort_flag, p.dev_status, 90);
             if (!ok) break;
             fence_after_sync();
 #pragma unroll
@@ -268,6 +315,8 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
                 uint32_t o[32];
                 tmem_ld32(lane_base + C::COL_DQ + grp * (D / 2) + c * 32, o);
                 tmem_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * p.scale);
                 if (row < nq) {
                     bf16* dst = p.dq + g_row * D + grp * (D / 2) + c * 32;
 #pragma unroll
@@ -282,7 +331,7 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
                 }
             }
             fence_before_sync();
-            mbar_arrive(bar_dqe);
+            mbar_arrive_if(bar_dqe, lane0);
         }
     }
     fence_before_sync();
