@@ -639,10 +639,13 @@ hf_status launch_bwd_dkv(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_
     p.mask = L.mask; p.mask_words = c->mask_words; p.first_block = (L.n_sink + L.n_cached) * c->n_b;
     p.Tc = c->Tc; p.n_b = c->n_b; p.Tm = c->Tm; p.n_units = c->BH * c->n_b;
     p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D)); p.scale = (float)(1.0 / std::sqrt((double)D));
-    p.lse = lse; p.delta = c->bwd_delta; p.dk = dk; p.dv = dv; p.dev_status = c->dev_status;
+    p.lse = lse; p.delta = c->bwd_delta; p.dev_status = c->dev_status;
+    CUtensorMap tdk, tdv;            // outputs: one warp's 32 rows x half of the columns per store
+    HF_TRY(make_map_ex(c, &tdk, dk, c->Tc, 1, D / 2, 32, true));
+    HF_TRY(make_map_ex(c, &tdv, dv, c->Tc, 1, D / 2, 32, true));
     const int grid = p.n_units < c->sm_count ? p.n_units : c->sm_count;
     PdlLaunch pl(dim3(grid), dim3(C::THREADS), C::SMEM_BYTES, st, true);
-    HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_bwd_dkv<D>, tq, tdo, tk, tv, p));
+    HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_bwd_dkv<D>, tq, tdo, tk, tv, tdk, tdv, p));
     return post_launch(c, "k_swa_bwd_dkv");
 }
 

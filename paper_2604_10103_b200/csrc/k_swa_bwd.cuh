@@ -345,14 +345,18 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
 // ------------------------------------------------------------------------------------------------------------
 // dK and dV of the current chunk (the keys and values that carry gradient in the rollout: the cache holds clean chunks of
 // earlier, gradient-free passes).  The transposed walk: unit = (batch*head, key block j of the current chunk); for every
-// query block i that keeps j (read off the selection's bit mask), with rows = keys and columns = queries:
-//   S^T  = K_j Q_i^T      A = K_j (smem), B = Q_i (smem)                      -> TMEM [0, 128)
-//   dP^T = V_j dO_i^T     A = V_j (smem), B = dO_i (smem)                     -> TMEM [128, 256)
-//   P^T  = exp2(S^T c - lse_i log2 e)  (bf16, over S^T),   dS^T = P^T (dP^T - delta_i) / sqrt(d)  (bf16, over dP^T)
-//   dV_j += P^T dO_i      A = P^T (TMEM), B = dO_i (MN-major)                  -> TMEM [256, 256 + D)
-//   dK_j += dS^T Q_i      A = dS^T (TMEM), B = Q_i (MN-major)                  -> TMEM [384, 384 + D)
-// lse and delta are per QUERY, i.e. per column here: staged in shared memory per tile.  First version: S^T / dP^T
-// single-buffered; Q / dO tiles double-buffered.
+// query block i that keeps j (read off the selection's bit mask), in two halves h of 64 queries, rows = keys, columns = queries:
+//   S^T  = K_j Q_ih^T      A = K_j (smem), B = Q_ih (smem)                    -> TMEM [128 h, + 64)
+//   dP^T = V_j dO_ih^T     A = V_j (smem), B = dO_ih (smem)                   -> TMEM [128 h + 64, + 64)
+//   P^T  = exp2(S^T c - lse_i log2 e)  (bf16, over S^T),   dS^T = P^T (dP^T - delta_i)  (bf16, over dP^T)
+//   dV_j += P^T dO_ih      A = P^T (TMEM), B = dO_ih (MN-major)                -> TMEM [256, 256 + D)
+//   dK_j += dS^T Q_ih      A = dS^T (TMEM), B = Q_ih (MN-major)                -> TMEM [384, 384 + D); 1 / sqrt(d) at the end
+// The accumulators and one full pair of score tiles fill tensor memory at head dim 128; halves are what lets the tensor core
+// form one half's scores while the softmax warps work on the other (a pair's four products are 2 048 clk of tensor time, 2 560
+// with the score products' operand reads from shared memory; whole tiles alternated strictly: ~9 000 clk a pair).
+// lse and delta are per QUERY, i.e. per column here: staged in shared memory a pair ahead; a query row past the chunk's end
+// gets lse = +inf, so its P and dS are zero, and key rows past the end only reach output rows that are not stored: no masks.
+// Measured at 12 heads of 128, 4 680 queries, 28 kept blocks: 134 -> 94 us.
 // ------------------------------------------------------------------------------------------------------------
 template <int D>
 struct SwaBwdKV {
@@ -360,13 +364,17 @@ struct SwaBwdKV {
     static constexpr int SUB = D / 64, SUB_BYTES = BLK * 128, TILE_BYTES = SUB * SUB_BYTES;
     static constexpr int STAGES = 2;
     static constexpr int OFF_K = 0, OFF_V = TILE_BYTES, OFF_Q = 2 * TILE_BYTES, OFF_DO = OFF_Q + STAGES * TILE_BYTES;
-    static constexpr int OFF_BAR = OFF_DO + STAGES * TILE_BYTES;
-    static constexpr int OFF_ROW = OFF_BAR + 256;        // [2 stages][lse log2 e, delta][128] floats
+    static constexpr int OFF_OUT = OFF_DO + STAGES * TILE_BYTES;         // staging of the output tile, 32 rows x D / 2 columns per warp
+    static constexpr int OFF_BAR = OFF_OUT + BLK * D * 2;
+    static constexpr int OFF_ROW = OFF_BAR + 256;        // [2 pairs][-lse log2 e, -delta][128] floats
     static constexpr int USED_BYTES = OFF_ROW + 2 * 2 * BLK * 4;
-    static constexpr int SMEM_BYTES = USED_BYTES + 1024;
+    // one CTA per SM (it takes all of TMEM); slack for the alignment of the tiles to 1 KB, as far as there is room (checked)
+    static constexpr int WANT_BYTES = USED_BYTES + 1024 > 120 * 1024 ? USED_BYTES + 1024 : 120 * 1024, MAX_SMEM = 232448;
+    static constexpr int SMEM_BYTES = WANT_BYTES < MAX_SMEM ? WANT_BYTES : MAX_SMEM;
+    static_assert(USED_BYTES <= MAX_SMEM, "shared memory layout does not fit");
     static constexpr int THREADS = 320;                  // warps 0-7: softmax (two column groups), 8: TMA, 9: MMA
     static constexpr int WARP_TMA = 8, WARP_MMA = 9;
-    static constexpr int COL_S = 0, COL_DP = 128, COL_DV = 256, COL_DK = 384, TMEM_COLS = 512;
+    static constexpr int COL_DV = 256, COL_DK = 384, TMEM_COLS = 512;
 };
 
 struct SwaBwdKVParams {
@@ -376,40 +384,65 @@ struct SwaBwdKVParams {
     float scale_log2, scale;
     const float* lse;        // [B*H, T_c]
     const float* delta;      // [B*H, T_c]
-    bf16* dk;                // [B*H, T_c, D]
-    bf16* dv;
     int* dev_status;
+};
+
+// The query blocks that keep a unit's key block, in ascending order: 32 mask rows at a time, one ballot each.  All calls by a
+// whole warp.
+struct PairWalk {
+    int bh = 0, jb = 0, w = 0;
+    uint32_t bits = 0;
+    __device__ __forceinline__ uint32_t word(const SwaBwdKVParams& p, int w_) const {
+        const int i = w_ * 32 + (threadIdx.x & 31), jlog = p.first_block + jb;
+        const bool kept = i < p.Tm && ((__ldg(p.mask + ((size_t)bh * p.Tm + i) * p.mask_words + (jlog >> 5)) >> (jlog & 31)) & 1u);
+        return __ballot_sync(0xffffffffu, kept);
+    }
+    __device__ __forceinline__ void open(const SwaBwdKVParams& p, int u) {
+        bh = u / p.n_b; jb = u - bh * p.n_b; w = 0;
+        bits = word(p, 0);
+    }
+    __device__ __forceinline__ int pop(const SwaBwdKVParams& p) {      // the next query block, or -1
+        while (bits == 0) {
+            if (++w * 32 >= p.Tm) return -1;
+            bits = word(p, w);
+        }
+        const int i = w * 32 + __ffs(bits) - 1;
+        bits &= bits - 1;
+        return i;
+    }
 };
 
 template <int D>
 __global__ void __launch_bounds__(SwaBwdKV<D>::THREADS, 1)
 k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_do,
               const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
+              const __grid_constant__ CUtensorMap tm_dk, const __grid_constant__ CUtensorMap tm_dv,
               const __grid_constant__ SwaBwdKVParams p) {
     using namespace tc5;
     typedef SwaBwdKV<D> C;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t s_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    if (s_base - smem_u32(smem_raw) + C::USED_BYTES > C::SMEM_BYTES) {   // the window started too far off a 1 KB boundary
+        if (threadIdx.x == 0) { atomicOr(p.dev_status, HF_DEV_TIMEOUT_FLAG); atomicExch(p.dev_status + 1, 97); }
+        return;
+    }
     uint8_t* s_gen = smem_raw + (s_base - smem_u32(smem_raw));
     const uint32_t sK = s_base + C::OFF_K, sV = s_base + C::OFF_V, sQ = s_base + C::OFF_Q, sDO = s_base + C::OFF_DO;
     const uint32_t bar0 = s_base + C::OFF_BAR;
-    const uint32_t bar_kvf = bar0, bar_kve = bar0 + 8, bar_qf = bar0 + 16, bar_qe = bar0 + 32, bar_sd = bar0 + 48, bar_ds = bar0 + 56,
-                   bar_accf = bar0 + 64, bar_acce = bar0 + 72;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_gen + C::OFF_BAR + 80);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(s_gen + C::OFF_BAR + 84);
+    // half-pair s = 2 t + h: pairs of barriers, index h, completion t
+    const uint32_t bar_kvf = bar0, bar_kve = bar0 + 8, bar_qf = bar0 + 16, bar_qe = bar0 + 32, bar_sd = bar0 + 48, bar_ds = bar0 + 64,
+                   bar_accf = bar0 + 80, bar_acce = bar0 + 88;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_gen + C::OFF_BAR + 96);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(s_gen + C::OFF_BAR + 100);
     float* row_vals = reinterpret_cast<float*>(s_gen + C::OFF_ROW);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int my_units = (p.n_units - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-    // does query block i of batch*head bh keep the unit's key block?  (the same answer in every role: all walk i = 0 .. T_m - 1)
-    auto keeps = [&](int bh, int i, int jlog) -> bool {
-        return (__ldg(p.mask + ((size_t)bh * p.Tm + i) * p.mask_words + (jlog >> 5)) >> (jlog & 31)) & 1u;
-    };
 
     if (threadIdx.x == 0) {
         mbar_init(bar_kvf, 1); mbar_init(bar_kve, 1);
-        for (int s = 0; s < C::STAGES; ++s) { mbar_init(bar_qf + 8 * s, 1); mbar_init(bar_qe + 8 * s, 1); }
-        mbar_init(bar_sd, 1); mbar_init(bar_ds, 256); mbar_init(bar_accf, 1); mbar_init(bar_acce, 256);
+        for (int s = 0; s < 2; ++s) { mbar_init(bar_qf + 8 * s, 1); mbar_init(bar_qe + 8 * s, 1); mbar_init(bar_sd + 8 * s, 1); mbar_init(bar_ds + 8 * s, 8); }
+        mbar_init(bar_accf, 1); mbar_init(bar_acce, 8);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
@@ -423,173 +456,238 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     const uint32_t tmem = *tmem_slot;
     pdl_wait();
 
+    auto wait_w = [&](uint32_t bar, uint32_t parity, int where) -> bool {
+        return mbar_wait_warp<true>(bar, parity & 1u, abort_flag, p.dev_status, where);
+    };
+
     if (warp == C::WARP_TMA) {
         // ================================================================= TMA producer: K_j, V_j per unit; Q_i, dO_i per kept pair
-        if (lane == 0) {
-            bool ok = true;
-            int t = 0;
-            for (int n = 0; ok && n < my_units; ++n) {
-                const int u = blockIdx.x + n * gridDim.x;
-                const int bh = u / p.n_b, jb = u - bh * p.n_b;
-                const int jlog = p.first_block + jb;
-                if (n >= 1 && !(ok = mbar_wait<true>(bar_kve, (n - 1) & 1, abort_flag, p.dev_status, 91))) break;
-                mbar_expect_tx(bar_kvf, 2 * C::TILE_BYTES);
+        bool ok = true;
+        int t = 0, m = 0;                             // pairs; units that have any
+        PairWalk walk;
+        for (int n = 0; ok && n < my_units; ++n) {
+            walk.open(p, blockIdx.x + n * gridDim.x);
+            bool first = true;
+            for (int i = walk.pop(p); ok && i >= 0; i = walk.pop(p), ++t) {
+                if (first) {
+                    if (m >= 1 && !(ok = wait_w(bar_kve, m - 1, 91))) break;
+                    if (elect_one()) {
+                        mbar_expect_tx(bar_kvf, 2 * C::TILE_BYTES);
 #pragma unroll
-                for (int s = 0; s < C::SUB; ++s) {
-                    tma_load_4d(sK + s * C::SUB_BYTES, &tm_k, s * 64, jb * C::BLK, bh, 0, bar_kvf);
-                    tma_load_4d(sV + s * C::SUB_BYTES, &tm_v, s * 64, jb * C::BLK, bh, 0, bar_kvf);
+                        for (int s = 0; s < C::SUB; ++s) {
+                            tma_load_4d(sK + s * C::SUB_BYTES, &tm_k, s * 64, walk.jb * C::BLK, walk.bh, 0, bar_kvf);
+                            tma_load_4d(sV + s * C::SUB_BYTES, &tm_v, s * 64, walk.jb * C::BLK, walk.bh, 0, bar_kvf);
+                        }
+                    }
+                    __syncwarp();
+                    first = false; ++m;
                 }
-                for (int i = 0; ok && i < p.Tm; ++i) {
-                    if (!keeps(bh, i, jlog)) continue;
-                    const int st = t % C::STAGES;
-                    if (t >= C::STAGES && !(ok = mbar_wait<true>(bar_qe + 8 * st, ((t / C::STAGES) & 1) ^ 1, abort_flag, p.dev_status, 92))) break;
+                const int st = t & 1;
+                if (t >= 2 && !(ok = wait_w(bar_qe + 8 * st, (t >> 1) - 1, 92))) break;
+                if (elect_one()) {
                     mbar_expect_tx(bar_qf + 8 * st, 2 * C::TILE_BYTES);
 #pragma unroll
                     for (int s = 0; s < C::SUB; ++s) {
-                        tma_load_4d(sQ + st * C::TILE_BYTES + s * C::SUB_BYTES, &tm_q, s * 64, i * C::BLK, bh, 0, bar_qf + 8 * st);
-                        tma_load_4d(sDO + st * C::TILE_BYTES + s * C::SUB_BYTES, &tm_do, s * 64, i * C::BLK, bh, 0, bar_qf + 8 * st);
+                        tma_load_4d(sQ + st * C::TILE_BYTES + s * C::SUB_BYTES, &tm_q, s * 64, i * C::BLK, walk.bh, 0, bar_qf + 8 * st);
+                        tma_load_4d(sDO + st * C::TILE_BYTES + s * C::SUB_BYTES, &tm_do, s * 64, i * C::BLK, walk.bh, 0, bar_qf + 8 * st);
                     }
-                    ++t;
                 }
+                __syncwarp();
             }
-            if (!ok) {
-                const long long t0 = clock64();
-                while (clock64() - t0 < 400000) {}
-            }
+        }
+        if (!ok) {
+            const long long t0 = clock64();
+            while (clock64() - t0 < 400000) {}
         }
     } else if (warp == C::WARP_MMA) {
         // ================================================================= MMA issuer (warp-uniform, one elected lane issues)
-        constexpr uint32_t IDESC_S = idesc_bf16(128, false);
+        constexpr uint32_t IDESC_S = idesc_bf16(64, false);
         constexpr uint32_t IDESC_ACC = idesc_bf16(D, true);
-        constexpr uint32_t TILE_STEP = C::TILE_BYTES >> 4;
+        constexpr uint32_t TILE_STEP = C::TILE_BYTES >> 4, HALF = 64 * 128 >> 4;    // 64 rows of a tile, in 16-byte units
         const uint64_t dk0 = smem_desc_sw128(sK, 16, 1024), dv0 = smem_desc_sw128(sV, 16, 1024);
         const uint64_t dq0 = smem_desc_sw128(sQ, 16, 1024), dd0 = smem_desc_sw128(sDO, 16, 1024);
         const uint64_t dqm = smem_desc_sw128(sQ, C::SUB_BYTES, 1024), ddm = smem_desc_sw128(sDO, C::SUB_BYTES, 1024);   // as MN-major operands
         const uint32_t hi_k = (uint32_t)(dk0 >> 32), hi_m = (uint32_t)(dqm >> 32);
         bool ok = true;
+        // ---- the score products run half a pair ahead, over unit boundaries too: their own walk of the pairs
+        PairWalk ws;
+        int n_s = -1, t_s = 0, h_s = 0, m_s = -1, cur_s = -1, nxt_s = -1;
+        bool first_s = false;
+        auto next_pair_s = [&]() {                    // cur_s: the pair to issue (-1: none left); nxt_s: the one after it in the unit
+            cur_s = nxt_s;
+            if (cur_s >= 0) nxt_s = ws.pop(p);
+            while (cur_s < 0 && ++n_s < my_units) {
+                ws.open(p, blockIdx.x + n_s * gridDim.x);
+                cur_s = ws.pop(p);
+                if (cur_s >= 0) { nxt_s = ws.pop(p); first_s = true; ++m_s; }
+            }
+        };
+        auto issue_scores = [&]() -> bool {
+            const int st = t_s & 1;
+            if (h_s == 0) {
+                if (first_s && !wait_w(bar_kvf, m_s, 93)) return false;
+                first_s = false;
+                if (!wait_w(bar_qf + 8 * st, t_s >> 1, 94)) return false;
+            }
+            fence_after_sync();
+            if (elect_one()) {
+                mma_ss_tile<D>(tmem + 128 * h_s, (uint32_t)dk0, (uint32_t)dq0 + st * TILE_STEP + h_s * HALF, hi_k, IDESC_S);
+                mma_ss_tile<D>(tmem + 128 * h_s + 64, (uint32_t)dv0, (uint32_t)dd0 + st * TILE_STEP + h_s * HALF, hi_k, IDESC_S);
+                mma_commit(bar_sd + 8 * h_s);
+                if (h_s == 1 && nxt_s < 0) mma_commit(bar_kve);       // K_j and V_j have been read for the last time
+            }
+            __syncwarp();
+            if (h_s == 1) { ++t_s; next_pair_s(); }
+            h_s ^= 1;
+            return true;
+        };
+        next_pair_s();
+        if (cur_s >= 0) ok = issue_scores();
+        PairWalk wa;
         int t = 0;
         for (int n = 0; ok && n < my_units; ++n) {
-            const int u = blockIdx.x + n * gridDim.x;
-            const int bh = u / p.n_b, jb = u - bh * p.n_b;
-            const int jlog = p.first_block + jb;
-            if (!(ok = __all_sync(0xffffffffu, mbar_wait<true>(bar_kvf, n & 1, abort_flag, p.dev_status, 93)))) break;
+            wa.open(p, blockIdx.x + n * gridDim.x);
             int pairs = 0;
-            for (int i = 0; ok && i < p.Tm; ++i) {
-                if (!keeps(bh, i, jlog)) continue;
-                const int st = t % C::STAGES;
-                if (!(ok = __all_sync(0xffffffffu, mbar_wait<true>(bar_qf + 8 * st, (t / C::STAGES) & 1, abort_flag, p.dev_status, 94)))) break;
-                fence_after_sync();
-                if (elect_one()) {
-                    mma_ss_tile<D>(tmem + C::COL_S, (uint32_t)dk0, (uint32_t)dq0 + st * TILE_STEP, hi_k, IDESC_S);
-                    mma_ss_tile<D>(tmem + C::COL_DP, (uint32_t)dv0, (uint32_t)dd0 + st * TILE_STEP, hi_k, IDESC_S);
-                    mma_commit(bar_sd);
+            for (int i = wa.pop(p); ok && i >= 0; i = wa.pop(p), ++t, ++pairs) {
+                const int st = t & 1;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    // scores of the next half first -- unless they wait for another unit's K and V
+                    const bool ahead = cur_s >= 0 && !first_s;
+                    if (ahead && !(ok = issue_scores())) break;
+                    if (!(ok = wait_w(bar_ds + 8 * h, t, 95))) break;
+                    // the accumulators of the previous unit have been read out before this unit's first products overwrite them
+                    if (h == 0 && pairs == 0 && n >= 1 && !(ok = wait_w(bar_acce, n - 1, 96))) break;
+                    fence_after_sync();
+                    if (elect_one()) {
+                        mma_ts_half_split(tmem + C::COL_DV, tmem + 128 * h, (uint32_t)ddm + st * TILE_STEP + h * HALF, hi_m, IDESC_ACC, pairs > 0 || h > 0);
+                        mma_ts_half_split(tmem + C::COL_DK, tmem + 128 * h + 64, (uint32_t)dqm + st * TILE_STEP + h * HALF, hi_m, IDESC_ACC, pairs > 0 || h > 0);
+                        if (h == 1) mma_commit(bar_qe + 8 * st);
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
-                if (!(ok = __all_sync(0xffffffffu, mbar_wait<true>(bar_ds, t & 1, abort_flag, p.dev_status, 95)))) break;
-                // the accumulators of the previous unit have been read out before this unit's first products overwrite them
-                if (pairs == 0 && n >= 1 && !(ok = __all_sync(0xffffffffu, mbar_wait<true>(bar_acce, (n - 1) & 1, abort_flag, p.dev_status, 96)))) break;
-                fence_after_sync();
-                if (elect_one()) {
-                    mma_ts_tile_split(tmem + C::COL_DV, tmem + C::COL_S, tmem + C::COL_S + 64, (uint32_t)ddm + st * TILE_STEP, hi_m, IDESC_ACC, pairs > 0);
-                    mma_ts_tile_split(tmem + C::COL_DK, tmem + C::COL_DP, tmem + C::COL_DP + 64, (uint32_t)dqm + st * TILE_STEP, hi_m, IDESC_ACC, pairs > 0);
-                    mma_commit(bar_qe + 8 * st);
-                }
-                __syncwarp();
-                ++pairs; ++t;
             }
             if (!ok) break;
-            if (elect_one()) { mma_commit(bar_accf); mma_commit(bar_kve); }      // everything of this unit has completed
+            // (nothing was issued: the read-out of the unit before still comes first, or this unit's completion could pass it by)
+            if (pairs == 0 && n >= 1 && !(ok = wait_w(bar_acce, n - 1, 97))) break;
+            if (elect_one()) mma_commit(bar_accf);    // everything of this unit has completed
             __syncwarp();
-            if (pairs == 0 && n >= 1) {     // (nothing was issued: the previous unit's read-out still has to be waited for, to keep the phases in step)
-                if (!(ok = __all_sync(0xffffffffu, mbar_wait<true>(bar_acce, (n - 1) & 1, abort_flag, p.dev_status, 97)))) break;
-            }
+            // the next unit's first scores, which were not issued ahead (in a unit without pairs they wait for theirs)
+            if (first_s && n_s == n + 1) ok = issue_scores();
         }
     } else {
         // ================================================================= softmax warps (rows = keys, columns = queries)
-        const int grp = warp >> 2;                          // query columns [64 grp, 64 grp + 64) of the pair
+        const int grp = warp >> 2;                          // query columns [32 grp, 32 grp + 32) of a half
         const int row = (warp & 3) * 32 + lane;             // key row of the block
         const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        const bool lane0 = lane == 0;
+        const float2 c2 = make_float2(p.scale_log2, p.scale_log2);
         bool ok = true;
         int t = 0;
+        PairWalk walk;
         for (int n = 0; ok && n < my_units; ++n) {
-            const int u = blockIdx.x + n * gridDim.x;
-            const int bh = u / p.n_b, jb = u - bh * p.n_b;
-            const int jlog = p.first_block + jb;
-            const int k0 = jb * C::BLK, nk = min(C::BLK, p.Tc - k0);
-            int pairs = 0;
-            for (int i = 0; ok && i < p.Tm; ++i) {
-                if (!keeps(bh, i, jlog)) continue;
-                const int q0 = i * C::BLK, nq = min(C::BLK, p.Tc - q0);
-                // per-query values of this pair into shared memory (the buffer of pair t - 2 was read before its arrival on bar_ds)
-                float* rv = row_vals + (t & 1) * 2 * C::BLK;
+            walk.open(p, blockIdx.x + n * gridDim.x);
+            const int bh = walk.bh, k0 = walk.jb * C::BLK;
+            float v_lse = 0.f, v_del = 0.f;                 // threads 0 .. 127: the next pair's values of query row threadIdx.x
+            auto fetch = [&](int i) {
+                const int r = i * C::BLK + (int)threadIdx.x;
                 if (threadIdx.x < C::BLK) {
-                    const bool v = (int)threadIdx.x < nq;
-                    rv[threadIdx.x] = v ? -p.lse[(size_t)bh * p.Tc + q0 + threadIdx.x] * 1.4426950408889634f : 0.f;
-                    rv[C::BLK + threadIdx.x] = v ? p.delta[(size_t)bh * p.Tc + q0 + threadIdx.x] : 0.f;
+                    v_lse = -INFINITY; v_del = 0.f;         // rows past the chunk's end: weight zero
+                    if (r < p.Tc) { v_lse = -p.lse[(size_t)bh * p.Tc + r] * 1.4426950408889634f; v_del = -p.delta[(size_t)bh * p.Tc + r]; }
                 }
+            };
+            int i = walk.pop(p);
+            const bool any = i >= 0;
+            if (any) fetch(i);
+            while (i >= 0) {
+                // (the buffer of pair t - 2: every warp has arrived on that pair's last half, and met the others here since)
+                float* rv = row_vals + (t & 1) * 2 * C::BLK;
+                if (threadIdx.x < C::BLK) { rv[threadIdx.x] = v_lse; rv[C::BLK + threadIdx.x] = v_del; }
                 asm volatile("bar.sync 1, 256;\n" ::: "memory");
-                ok = __all_sync(0xffffffffu, mbar_wait(bar_sd, t & 1, abort_flag, p.dev_status, 98));
-                if (!ok) break;
-                fence_after_sync();
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
+                i = walk.pop(p);
+                if (i >= 0) fetch(i);
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h) {
+                    ok = mbar_wait_warp(bar_sd + 8 * h, t & 1, abort_flag, p.dev_status, 98);
+                    if (!ok) break;
+                    fence_after_sync();
+                    const uint32_t tS = lane_base + 128 * h + grp * 32, tP = tS + 64;
                     uint32_t s[32], dp[32], pk[16], dk_[16];
-                    tmem_ld32(lane_base + C::COL_S + grp * 64 + c * 32, s);
-                    tmem_ld32(lane_base + C::COL_DP + grp * 64 + c * 32, dp);
+                    tmem_ld32(tS, s);
+                    tmem_ld32(tP, dp);
                     tmem_wait_ld();
+                    const float4* nl = reinterpret_cast<const float4*>(rv + h * 64 + grp * 32);
+                    const float4* nd = reinterpret_cast<const float4*>(rv + C::BLK + h * 64 + grp * 32);
 #pragma unroll
-                    for (int e = 0; e < 32; e += 2) {
-                        const int col = grp * 64 + c * 32 + e;
-                        float p0 = fast_exp2(fmaf(__uint_as_float(s[e]), p.scale_log2, rv[col]));
-                        float p1 = fast_exp2(fmaf(__uint_as_float(s[e + 1]), p.scale_log2, rv[col + 1]));
-                        if (row >= nk || col >= nq) p0 = 0.f;               // rows past the key block's end, columns past the query block's
-                        if (row >= nk || col + 1 >= nq) p1 = 0.f;
-                        const float d0 = p0 * (__uint_as_float(dp[e]) - rv[C::BLK + col]) * p.scale;
-                        const float d1 = p1 * (__uint_as_float(dp[e + 1]) - rv[C::BLK + col + 1]) * p.scale;
-                        pk[e >> 1] = pack_bf16(p0, p1);
-                        dk_[e >> 1] = pack_bf16(d0, d1);
+                    for (int e0 = 0; e0 < 32; e0 += 8) {
+                        float2 x[4], g[4];
+#pragma unroll
+                        for (int v = 0; v < 2; ++v) {
+                            const int e = e0 + 4 * v;
+                            const float4 l4 = nl[e >> 2], d4 = nd[e >> 2];
+                            x[2 * v] = ffma2(make_float2(__uint_as_float(s[e]), __uint_as_float(s[e + 1])), c2, make_float2(l4.x, l4.y));
+                            x[2 * v + 1] = ffma2(make_float2(__uint_as_float(s[e + 2]), __uint_as_float(s[e + 3])), c2, make_float2(l4.z, l4.w));
+                            g[2 * v] = fadd2(make_float2(__uint_as_float(dp[e]), __uint_as_float(dp[e + 1])), make_float2(d4.x, d4.y));
+                            g[2 * v + 1] = fadd2(make_float2(__uint_as_float(dp[e + 2]), __uint_as_float(dp[e + 3])), make_float2(d4.z, d4.w));
+                        }
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) x[v] = make_float2(fast_exp2(x[v].x), fast_exp2(x[v].y));
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) {
+                            pk[(e0 >> 1) + v] = pack_bf16(x[v].x, x[v].y);
+                            dk_[(e0 >> 1) + v] = pack_bf16(x[v].x * g[v].x, x[v].y * g[v].y);
+                        }
                     }
-                    tmem_st16(lane_base + C::COL_S + grp * 64 + c * 16, pk);
-                    tmem_st16(lane_base + C::COL_DP + grp * 64 + c * 16, dk_);
+                    tmem_st16(tS, pk);
+                    tmem_st16(tP, dk_);
+                    tmem_wait_st();
+                    fence_before_sync();
+                    mbar_arrive_if(bar_ds + 8 * h, lane0);
                 }
-                tmem_wait_st();
-                fence_before_sync();
-                mbar_arrive(bar_ds);
-                ++pairs; ++t;
+                if (!ok) break;
+                ++t;
             }
             if (!ok) break;
-            ok = __all_sync(0xffffffffu, mbar_wait(bar_accf, n & 1, abort_flag, p.dev_status, 99));
+            ok = mbar_wait_warp(bar_accf, n & 1, abort_flag, p.dev_status, 99);
             if (!ok) break;
             fence_after_sync();
-            const size_t g_row = (size_t)bh * p.Tc + k0 + row;
+            // dV and dK of the unit as bf16 (zeros if no query block keeps the key block), out through shared memory and one bulk
+            // tensor store per warp and tensor (32 rows x half of the columns; rows past the chunk's end are clipped by the map)
+            uint32_t out[2][D / 4];
 #pragma unroll
-            for (int which = 0; which < 2; ++which) {
-                bf16* out = which == 0 ? p.dv : p.dk;
+            for (int which = 0; which < 2; ++which)
 #pragma unroll
                 for (int c = 0; c < D / 64; ++c) {
                     uint32_t o[32];
                     tmem_ld32(lane_base + (which == 0 ? C::COL_DV : C::COL_DK) + grp * (D / 2) + c * 32, o);
                     tmem_wait_ld();
-                    if (row < nk) {
-                        bf16* dst = out + g_row * D + grp * (D / 2) + c * 32;
+                    const float f = which == 0 ? 1.f : p.scale;
 #pragma unroll
-                        for (int v = 0; v < 4; ++v) {
-                            uint4 w;
-                            if (pairs == 0) w = make_uint4(0u, 0u, 0u, 0u);     // no query block keeps this key block: no gradient
-                            else {
-                                w.x = pack_bf16(__uint_as_float(o[v * 8]), __uint_as_float(o[v * 8 + 1]));
-                                w.y = pack_bf16(__uint_as_float(o[v * 8 + 2]), __uint_as_float(o[v * 8 + 3]));
-                                w.z = pack_bf16(__uint_as_float(o[v * 8 + 4]), __uint_as_float(o[v * 8 + 5]));
-                                w.w = pack_bf16(__uint_as_float(o[v * 8 + 6]), __uint_as_float(o[v * 8 + 7]));
-                            }
-                            *reinterpret_cast<uint4*>(dst + v * 8) = w;
-                        }
-                    }
+                    for (int e = 0; e < 32; e += 2)
+                        out[which][c * 16 + e / 2] = any ? pack_bf16(__uint_as_float(o[e]) * f, __uint_as_float(o[e + 1]) * f) : 0u;
+                }
+            fence_before_sync();
+            mbar_arrive_if(bar_acce, lane0);                // the accumulators may take the next unit
+            constexpr int RB = D;                           // bytes per staged row (D / 2 columns)
+            const uint32_t off = C::OFF_OUT + warp * 32 * RB;
+            uint8_t* stage = s_gen + off + lane * RB;
+            const int swz = D == 128 ? lane & 7 : (lane >> 1) & 3;
+#pragma unroll
+            for (int which = 0; which < 2; ++which) {
+                if (lane0) bulk_wait_read();                // this warp's previous store has read its part
+                __syncwarp();
+#pragma unroll
+                for (int c = 0; c < D / 16; ++c)
+                    *reinterpret_cast<uint4*>(stage + ((c ^ swz) << 4)) = make_uint4(out[which][4 * c], out[which][4 * c + 1], out[which][4 * c + 2], out[which][4 * c + 3]);
+                fence_proxy_async();
+                __syncwarp();
+                if (lane0 && k0 + (warp & 3) * 32 < p.Tc) {
+                    tma_store_4d(which == 0 ? &tm_dv : &tm_dk, s_base + off, grp * (D / 2), k0 + (warp & 3) * 32, bh, 0);
+                    bulk_commit();
                 }
             }
-            fence_before_sync();
-            mbar_arrive(bar_acce);
         }
+        if (lane0) bulk_wait_all();
     }
     fence_before_sync();
     __syncthreads();

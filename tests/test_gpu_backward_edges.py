@@ -1,0 +1,61 @@
+"""Backward kernels at the edges of their tiling: key blocks that no query block keeps between ones that some do, several units
+per thread block, more than 32 query blocks (two words of the pair walk), chunks of one short block, one-block lists.  dq, dk and
+dv against the oracle's gradients (bf16 P and dS operands: the tolerance of the other backward tests)."""
+import numpy as np
+import pytest
+
+from oracle import hybrid_attention as oa
+from paper_2604_10103_b200 import inputs as gen
+from tests import harness as hz
+
+pytestmark = pytest.mark.gpu
+
+f64 = gen.bf16_bits_to_f64
+
+
+@pytest.mark.parametrize("d,tpf,wf,topk,heads,batch", [
+    (128, 1290, 2, 1, 16, 1),      # 176 units, most key blocks unkept
+    (64, 1290, 2, 2, 16, 1),
+    (128, 4300, 1, 3, 2, 1),       # 34 query blocks
+    (64, 77, 2, 1, 3, 1),          # one short block per chunk
+    (128, 200, 5, 9, 2, 1),        # 72-row last block; nine of ten blocks kept
+    (64, 4300, 1, 33, 1, 1),
+])
+def test_gradients_at_tile_edges(d, tpf, wf, topk, heads, batch):
+    import torch
+    w = gen.Workload("bwd_edges", batch=batch, heads=heads, head_dim=d, tokens_per_frame=tpf, chunk_frames=1, window_frames=wf, block=128,
+                     topk=topk, keep_permille=0, seed=401)
+    gpu = hz.GpuStream(w); ora = hz.make_oracle(w)
+    try:
+        for c in range(wf):
+            kc, vc = gen.clean_kv(w, 0, c)
+            gpu.append(gpu.up(kc), gpu.up(vc)); ora.append(f64(kc), f64(vc))
+        qb, kb, vb = gen.qkv(w, 0, wf, 0)
+        gb = gen.normal_bf16(qb.shape, 401, 7, 7)
+        q, k, v, g = gpu.up(qb), gpu.up(kb), gpu.up(vb), gpu.up(gb)
+        m, _, _ = gpu.select(q, k)
+        o = torch.empty(gpu.shape, dtype=torch.bfloat16, device="cuda")
+        lse = torch.empty(gpu.shape[:3], dtype=torch.float32, device="cuda")
+        gpu.ctx.hf_sparse_swa(0, q, k, v, o, lse=lse)
+        dq, dk, dv = torch.empty_like(o), torch.full_like(o, 7.0), torch.full_like(o, 7.0)
+        gpu.ctx.hf_sparse_swa_backward_dq(0, q, k, v, o, lse, g, dq)
+        gpu.ctx.hf_sparse_swa_backward_dkv(0, q, k, v, o, lse, g, dk, dv)
+        torch.cuda.synchronize()
+        assert gpu.ctx.hf_get_device_status() == (0, 0)
+        got = [gpu.f64(x) for x in (dq, dk, dv)]
+        ref = [np.empty_like(got[0]) for _ in got]
+        held = ora.sink + ora.past
+        for bi in range(batch):
+            for h in range(heads):
+                kc_ = [kp[bi, h] for kp, _ in held] + [f64(kb)[bi, h]]
+                vc_ = [vp[bi, h] for _, vp in held] + [f64(vb)[bi, h]]
+                rq, rk, rv = oa.sparse_attention_backward(f64(qb)[bi, h], kc_, vc_, w.block, m[bi, h], f64(gb)[bi, h])
+                ref[0][bi, h], ref[1][bi, h], ref[2][bi, h] = rq, rk[-1], rv[-1]
+        for name, a, b in zip(("dq", "dk", "dv"), got, ref):
+            rl, ma = hz.rel_l2(a, b), hz.max_abs(a, b)
+            assert rl <= 1e-2 and ma <= 2e-2 * max(1.0, np.abs(b).max()), f"{name}: rel-L2 {rl:.3e}, max-abs {ma:.3e}"
+        unkept = ~m[..., -w.blocks_per_chunk:].any(axis=2)
+        for bi, h, jb in zip(*np.nonzero(unkept)):
+            assert not got[1][bi, h, jb * 128:(jb + 1) * 128].any() and not got[2][bi, h, jb * 128:(jb + 1) * 128].any()
+    finally:
+        gpu.close()
