@@ -95,6 +95,7 @@ struct hf_ctx {
     int* union_tiles = nullptr;          // ... and tiles per unit
     int union_max_tiles = 0;
     float* bwd_delta = nullptr;          // backward pass: g . o_local per query row [B*H, T_c]
+    int* bwd_order = nullptr;            // ... and the key blocks of the current chunk, most pairs first [B*H, n_b]
     float* partials = nullptr;       // absorb split partials
     float* partials_layers = nullptr;    // layer-batched state update: one partial per (layer, batch*head, group)
     size_t partials_layers_count = 0;
@@ -185,7 +186,7 @@ void free_all(hf_ctx* c) {
     for (auto& L : c->layers) { cudaFree(L.W_full); cudaFree(L.mask); cudaFree(L.idx); }
     cudaFree(c->ring_k_all); cudaFree(c->ring_v_all); cudaFree(c->pooled_k_all); cudaFree(c->S_all); cudaFree(c->z_all);
     cudaFree(c->sf_hi_all); cudaFree(c->sf_lo_all); cudaFree(c->W_all); cudaFree(c->bias_all);
-    cudaFree(c->union_entries); cudaFree(c->union_tiles); cudaFree(c->bwd_delta); cudaFree(c->pooled_q); cudaFree(c->pooled_kcur); cudaFree(c->hist); cudaFree(c->partials); cudaFree(c->partials_layers); cudaFree(c->x_hi); cudaFree(c->x_lo);
+    cudaFree(c->union_entries); cudaFree(c->union_tiles); cudaFree(c->bwd_delta); cudaFree(c->bwd_order); cudaFree(c->pooled_q); cudaFree(c->pooled_kcur); cudaFree(c->hist); cudaFree(c->partials); cudaFree(c->partials_layers); cudaFree(c->x_hi); cudaFree(c->x_lo);
     cudaFree(c->dev_status);
     cudaFree(c->rope_q[0]); cudaFree(c->rope_q[1]); cudaFree(c->rope_k[0]); cudaFree(c->rope_k[1]);
     cudaFree(c->trope_tab[0]); cudaFree(c->trope_tab[1]); cudaFree(c->q_rot); cudaFree(c->k_rot);
@@ -597,7 +598,7 @@ hf_status launch_bwd_dq(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_c
     HF_CUDA(cudaFuncSetAttribute(k_swa_bwd_dq<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES));
     const long long rows = (long long)c->BH * c->Tc;
     PdlLaunch pr(dim3((unsigned)((rows + RowDot<D>::RPB - 1) / RowDot<D>::RPB)), dim3(256), 0, st, true);
-    HF_CUDA(cudaLaunchKernelEx(&pr.cfg, k_rowdot<D>, d_o, o_local, c->bwd_delta, rows));
+    HF_CUDA(cudaLaunchKernelEx(&pr.cfg, k_rowdot<D>, d_o, o_local, c->bwd_delta, rows, BwdOrder{}));
     HF_TRY(post_launch(c, "k_rowdot"));
     CUtensorMap tq, tdo, tk, tv;
     HF_TRY(make_map(c, &tq, q, 1));
@@ -626,8 +627,12 @@ hf_status launch_bwd_dkv(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_
     if (c->bwd_delta == nullptr) HF_TRY(dmalloc(&c->bwd_delta, (size_t)c->BH * c->Tc));
     HF_CUDA(cudaFuncSetAttribute(k_swa_bwd_dkv<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES));
     const long long rows = (long long)c->BH * c->Tc;
-    PdlLaunch pr(dim3((unsigned)((rows + RowDot<D>::RPB - 1) / RowDot<D>::RPB)), dim3(256), 0, st, true);
-    HF_CUDA(cudaLaunchKernelEx(&pr.cfg, k_rowdot<D>, d_o, o_local, c->bwd_delta, rows));
+    if (c->bwd_order == nullptr) HF_TRY(dmalloc(&c->bwd_order, (size_t)c->BH * c->n_b));
+    BwdOrder ord;
+    ord.mask = L.mask; ord.mask_words = c->mask_words; ord.first_block = (L.n_sink + L.n_cached) * c->n_b; ord.n_b = c->n_b; ord.Tm = c->Tm;
+    ord.BH = c->BH; ord.order = c->bwd_order;
+    PdlLaunch pr(dim3((unsigned)((rows + RowDot<D>::RPB - 1) / RowDot<D>::RPB) + 1), dim3(256), 0, st, true);
+    HF_CUDA(cudaLaunchKernelEx(&pr.cfg, k_rowdot<D>, d_o, o_local, c->bwd_delta, rows, ord));
     HF_TRY(post_launch(c, "k_rowdot"));
     CUtensorMap tq, tdo, tk, tv;
     HF_TRY(make_map(c, &tq, q, 1));
@@ -639,7 +644,7 @@ hf_status launch_bwd_dkv(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_
     p.mask = L.mask; p.mask_words = c->mask_words; p.first_block = (L.n_sink + L.n_cached) * c->n_b;
     p.Tc = c->Tc; p.n_b = c->n_b; p.Tm = c->Tm; p.n_units = c->BH * c->n_b;
     p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D)); p.scale = (float)(1.0 / std::sqrt((double)D));
-    p.lse = lse; p.delta = c->bwd_delta; p.dev_status = c->dev_status;
+    p.lse = lse; p.delta = c->bwd_delta; p.order = c->bwd_order; p.dev_status = c->dev_status;
     CUtensorMap tdk, tdv;            // outputs: one warp's 32 rows x half of the columns per store
     HF_TRY(make_map_ex(c, &tdk, dk, c->Tc, 1, D / 2, 32, true));
     HF_TRY(make_map_ex(c, &tdv, dv, c->Tc, 1, D / 2, 32, true));

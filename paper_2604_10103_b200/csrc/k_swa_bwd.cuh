@@ -26,13 +26,76 @@
 // per lane, 5.7 us like this).  grid: ceil(rows / (4 * 256 / (D / 8))), 256 threads.
 template <int D>
 struct RowDot { static constexpr int LPR = D / 8, RPB = 4 * 256 / LPR; };      // lanes per row; rows per thread block
+
+// The units of the dK/dV kernel (key blocks of the current chunk) in descending order of the query blocks that keep them,
+// written by one extra thread block of the k_rowdot launch before it.  Key blocks differ in popularity (9.4 +- 2.6 of 37 at 28 of
+// 111 kept, i.i.d. or not): in natural order the busiest of 148 thread blocks has 49 pairs and unit ends against a mean of 37,
+// in this order 38.
+struct BwdOrder {
+    const uint32_t* mask;    // [B*H, T_m, mask_words], or nullptr: no ordering
+    int mask_words, first_block, n_b, Tm, BH;
+    int* order;              // [B*H * n_b]
+};
+constexpr int BWD_ORDER_MAX = 4096;              // units that are ordered; beyond that a thread block has dozens and balance comes by itself
+__device__ __noinline__ void bwd_order_units(const BwdOrder& q) {
+    __shared__ int cnt[BWD_ORDER_MAX];
+    __shared__ int at[HF_MAX_TN + 2];            // units with fewer kept pairs come later: bin b holds count Tm - b
+    const int n = q.BH * q.n_b, tid = threadIdx.x;
+    if (n > BWD_ORDER_MAX || q.Tm > HF_MAX_TN) {
+        for (int u = tid; u < n; u += 256) q.order[u] = u;
+        return;
+    }
+    for (int u = tid; u < n; u += 256) cnt[u] = 0;
+    for (int b = tid; b <= q.Tm + 1; b += 256) at[b] = 0;
+    __syncthreads();
+    const int w0 = q.first_block >> 5, nw = ((q.first_block + q.n_b - 1) >> 5) - w0 + 1, items = q.BH * q.Tm * nw;
+    for (int base = 0; base < items; base += 256 * 8) {       // eight mask words per thread in flight
+        uint32_t bits[8];
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+            const int it = base + x * 256 + tid, r = it / nw;
+            bits[x] = it < items ? __ldg(q.mask + (size_t)r * q.mask_words + w0 + (it - r * nw)) : 0u;
+        }
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+            const int it = base + x * 256 + tid, r = it / nw, bh = r / q.Tm;
+            const int j0 = (w0 + it - r * nw) * 32 - q.first_block;
+            while (bits[x]) {
+                const int j = j0 + __ffs(bits[x]) - 1;
+                bits[x] &= bits[x] - 1;
+                if (j >= 0 && j < q.n_b) atomicAdd(&cnt[bh * q.n_b + j], 1);
+            }
+        }
+    }
+    __syncthreads();
+    for (int u = tid; u < n; u += 256) atomicAdd(&at[q.Tm - cnt[u] + 1], 1);
+    __syncthreads();
+    if (tid < 32) {                              // at[b] = first position of bin b: running sums, 32 bins at a time
+        int base = 0;
+        for (int b0 = 0; b0 <= q.Tm + 1; b0 += 32) {
+            const int b = b0 + tid;
+            int v = b <= q.Tm + 1 ? at[b] : 0;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int x = __shfl_up_sync(0xffffffffu, v, off);
+                if (tid >= off) v += x;
+            }
+            if (b <= q.Tm + 1) at[b] = base + v;
+            base += __shfl_sync(0xffffffffu, v, 31);
+        }
+    }
+    __syncthreads();
+    for (int u = tid; u < n; u += 256) q.order[atomicAdd(&at[q.Tm - cnt[u]], 1)] = u;
+}
 template <int D>
-__global__ void __launch_bounds__(256) k_rowdot(const bf16* __restrict__ a, const bf16* __restrict__ b, float* __restrict__ out, long long rows) {
+__global__ void __launch_bounds__(256) k_rowdot(const bf16* __restrict__ a, const bf16* __restrict__ b, float* __restrict__ out, long long rows, BwdOrder ord) {
     typedef RowDot<D> C;
     pdl_wait();
     pdl_trigger();              // the backward kernel may set itself up; it waits for this grid before it reads delta
+    if (ord.mask && blockIdx.x == 0) { bwd_order_units(ord); return; }      // (the first thread block: it starts first and ends last)
+    const int block = blockIdx.x - (ord.mask ? 1 : 0);
     const int part = threadIdx.x % C::LPR;
-    const long long r0 = (long long)blockIdx.x * C::RPB + threadIdx.x / C::LPR;
+    const long long r0 = (long long)block * C::RPB + threadIdx.x / C::LPR;
     uint4 x[4], y[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -356,7 +419,7 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
 // with the score products' operand reads from shared memory; whole tiles alternated strictly: ~9 000 clk a pair).
 // lse and delta are per QUERY, i.e. per column here: staged in shared memory a pair ahead; a query row past the chunk's end
 // gets lse = +inf, so its P and dS are zero, and key rows past the end only reach output rows that are not stored: no masks.
-// Measured at 12 heads of 128, 4 680 queries, 28 kept blocks: 134 -> 94 us.
+// Measured at 12 heads of 128, 4 680 queries, 28 kept blocks: 134 -> 94 us, 82 with the units in order of their pairs (BwdOrder).
 // ------------------------------------------------------------------------------------------------------------
 template <int D>
 struct SwaBwdKV {
@@ -381,6 +444,7 @@ struct SwaBwdKVParams {
     const uint32_t* mask;    // [B*H, T_m, mask_words]: the forward's selection
     int mask_words, first_block;     // logical index of the current chunk's first key block
     int Tc, n_b, Tm, n_units;        // units = B*H x n_b
+    const int* order;        // [n_units]: the units, most pairs first
     float scale_log2, scale;
     const float* lse;        // [B*H, T_c]
     const float* delta;      // [B*H, T_c]
@@ -437,7 +501,11 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     float* row_vals = reinterpret_cast<float*>(s_gen + C::OFF_ROW);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int my_units = (p.n_units - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    // Unit number n of this thread block: position n * grid + c of the order, with c running backwards in odd rounds.
+    const int rounds = p.n_units / (int)gridDim.x, rest = p.n_units - rounds * (int)gridDim.x;
+    auto place = [&](int n) -> int { return (n & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x; };
+    const int my_units = rounds + (place(rounds) < rest ? 1 : 0);
+    auto unit_of = [&](int n) -> int { return __ldg(p.order + n * (int)gridDim.x + place(n)); };
 
     if (threadIdx.x == 0) {
         mbar_init(bar_kvf, 1); mbar_init(bar_kve, 1);
@@ -466,7 +534,7 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         int t = 0, m = 0;                             // pairs; units that have any
         PairWalk walk;
         for (int n = 0; ok && n < my_units; ++n) {
-            walk.open(p, blockIdx.x + n * gridDim.x);
+            walk.open(p, unit_of(n));
             bool first = true;
             for (int i = walk.pop(p); ok && i >= 0; i = walk.pop(p), ++t) {
                 if (first) {
@@ -517,7 +585,7 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             cur_s = nxt_s;
             if (cur_s >= 0) nxt_s = ws.pop(p);
             while (cur_s < 0 && ++n_s < my_units) {
-                ws.open(p, blockIdx.x + n_s * gridDim.x);
+                ws.open(p, unit_of(n_s));
                 cur_s = ws.pop(p);
                 if (cur_s >= 0) { nxt_s = ws.pop(p); first_s = true; ++m_s; }
             }
@@ -546,7 +614,7 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         PairWalk wa;
         int t = 0;
         for (int n = 0; ok && n < my_units; ++n) {
-            wa.open(p, blockIdx.x + n * gridDim.x);
+            wa.open(p, unit_of(n));
             int pairs = 0;
             for (int i = wa.pop(p); ok && i >= 0; i = wa.pop(p), ++t, ++pairs) {
                 const int st = t & 1;
@@ -586,7 +654,7 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         int t = 0;
         PairWalk walk;
         for (int n = 0; ok && n < my_units; ++n) {
-            walk.open(p, blockIdx.x + n * gridDim.x);
+            walk.open(p, unit_of(n));
             const int bh = walk.bh, k0 = walk.jb * C::BLK;
             float v_lse = 0.f, v_del = 0.f;                 // threads 0 .. 127: the next pair's values of query row threadIdx.x
             auto fetch = [&](int i) {
