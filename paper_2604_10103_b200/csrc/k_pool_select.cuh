@@ -44,26 +44,39 @@ struct TemporalRope {
     int first_pair, n_pairs, tokens_per_frame;
 };
 
-// One block of one tensor: copy (optional) and per-column mean in the canonical order.  256 threads: 16 threads per token
-// row, 16 rows per pass.
+// Turn of one thread's VEC features of a row: cosine and sine of those of its VEC / 2 pairs that turn.
+template <int VEC>
+struct PairTurn {
+    float c[VEC / 2], s[VEC / 2];
+    int frame = -1;             // of the chunk; the entries are reloaded when a row belongs to another one
+};
+template <int VEC>
+__device__ __forceinline__ void load_turn(PairTurn<VEC>& t, int first_feature, int steps, const TemporalRope& tr) {
+    const int a = steps < 0 ? -steps : steps;
+#pragma unroll
+    for (int e = 0; e < VEC / 2; ++e) {
+        const int pr = first_feature / 2 + e - tr.first_pair;
+        if (pr >= 0 && pr < tr.n_pairs) {
+            t.c[e] = __ldg(tr.cos_tab + (size_t)a * tr.n_pairs + pr);
+            const float sn = __ldg(tr.sin_tab + (size_t)a * tr.n_pairs + pr);
+            t.s[e] = steps < 0 ? -sn : sn;
+        }
+    }
+}
 template <int VEC, typename V>
-__device__ __forceinline__ V rotate_vec(const V& u, int first_feature, int steps, const TemporalRope& tr) {
+__device__ __forceinline__ V rotate_vec(const V& u, const PairTurn<VEC>& t, int first_feature, const TemporalRope& tr) {
     float f[VEC];
     VecLoad<VEC>::widen(u, f);
-    const int a = steps < 0 ? -steps : steps;
     uint32_t w[VEC / 2];
 #pragma unroll
-    for (int e = 0; e < VEC; e += 2) {
-        const int pr = (first_feature + e) / 2 - tr.first_pair;
-        float y0 = f[e], y1 = f[e + 1];
+    for (int e = 0; e < VEC / 2; ++e) {
+        const int pr = first_feature / 2 + e - tr.first_pair;
+        float y0 = f[2 * e], y1 = f[2 * e + 1];
         if (pr >= 0 && pr < tr.n_pairs) {
-            const float c = __ldg(tr.cos_tab + (size_t)a * tr.n_pairs + pr);
-            float sn = __ldg(tr.sin_tab + (size_t)a * tr.n_pairs + pr);
-            if (steps < 0) sn = -sn;
-            y0 = __fsub_rn(__fmul_rn(f[e], c), __fmul_rn(f[e + 1], sn));
-            y1 = __fadd_rn(__fmul_rn(f[e], sn), __fmul_rn(f[e + 1], c));
+            y0 = __fsub_rn(__fmul_rn(f[2 * e], t.c[e]), __fmul_rn(f[2 * e + 1], t.s[e]));
+            y1 = __fadd_rn(__fmul_rn(f[2 * e], t.s[e]), __fmul_rn(f[2 * e + 1], t.c[e]));
         }
-        w[e / 2] = pack_bf16(y0, y1);
+        w[e] = pack_bf16(y0, y1);
     }
     V out;
     if constexpr (VEC == 8) { out.x = w[0]; out.y = w[1]; out.z = w[2]; out.w = w[3]; }
@@ -71,6 +84,8 @@ __device__ __forceinline__ V rotate_vec(const V& u, int first_feature, int steps
     return out;
 }
 
+// One block of one tensor: copy (optional) and per-column mean in the canonical order.  256 threads: 16 threads per token
+// row, 16 rows per pass.
 template <int D, bool ROT>
 __device__ __forceinline__ void pool_copy_block(const PoolJob& jb, int Tc, int blk, int n_b, int b_idx, int bh, const TemporalRope& tr) {
     constexpr int VEC = D / 16;
@@ -86,6 +101,18 @@ __device__ __forceinline__ void pool_copy_block(const PoolJob& jb, int Tc, int b
     float acc[VEC];
 #pragma unroll
     for (int e = 0; e < VEC; ++e) acc[e] = 0.f;
+    // ROT: this thread's pairs are the same in every row, and a block's rows span few frames: the angles stay in registers
+    PairTurn<VEC> turn;
+    int frame_end = 0;          // first row of the block that belongs to the frame after turn.frame
+    bool turns = false;         // any of this thread's pairs turns at all
+    if (ROT) {
+        turns = jb.rot_on && cv * VEC / 2 < tr.first_pair + tr.n_pairs && (cv + 1) * VEC / 2 > tr.first_pair;
+        if (turns) {
+            turn.frame = (t0 + r) / tr.tokens_per_frame;
+            frame_end = (turn.frame + 1) * tr.tokens_per_frame - t0;
+            load_turn<VEC>(turn, cv * VEC, jb.rot_base + jb.rot_per_frame * turn.frame, tr);
+        }
+    }
 #pragma unroll
     for (int i0 = 0; i0 < MAXR; i0 += BATCH) {
         V u[BATCH];
@@ -96,8 +123,21 @@ __device__ __forceinline__ void pool_copy_block(const PoolJob& jb, int Tc, int b
                 // (the rotating instantiation may work in place: plain loads there, the read-only path elsewhere)
                 if (ROT) u[i] = *reinterpret_cast<const V*>(jb.src + base + (size_t)t * D);
                 else u[i] = __ldg(reinterpret_cast<const V*>(jb.src + base + (size_t)t * D));
-                if (ROT) {
-                    if (jb.rot_on) u[i] = rotate_vec<VEC, V>(u[i], cv * VEC, jb.rot_base + jb.rot_per_frame * ((t0 + t) / tr.tokens_per_frame), tr);
+            }
+        }
+        if (ROT) {
+            if (turns) {
+#pragma unroll
+                for (int i = 0; i < BATCH; ++i) {
+                    const int t = r + 16 * (i0 + i);
+                    if (t < n) {
+                        if (t >= frame_end) {
+                            turn.frame = (t0 + t) / tr.tokens_per_frame;
+                            frame_end = (turn.frame + 1) * tr.tokens_per_frame - t0;
+                            if (jb.rot_per_frame != 0) load_turn<VEC>(turn, cv * VEC, jb.rot_base + jb.rot_per_frame * turn.frame, tr);
+                        }
+                        u[i] = rotate_vec<VEC, V>(u[i], turn, cv * VEC, tr);
+                    }
                 }
             }
         }
@@ -140,7 +180,9 @@ __global__ void __launch_bounds__(256, 6) k_pool_copy(PoolJobs jobs, int Tc, int
     TemporalRope none = {nullptr, nullptr, 0, 0, 1};
     pool_copy_block<D, false>(jb, Tc, blk, n_b, blockIdx.x, blockIdx.y, none);
 }
-// The same with the temporal rotation applied to the jobs that ask for it (before the copy and the means).
+// The same with the temporal rotation applied to the jobs that ask for it (before the copy and the means).  The angles of a
+// thread's pairs stay in registers from row to row (22 -> 16 us for two 14 MB tensors turned and copied, against table loads
+// and a division per row).
 template <int D>
 __global__ void __launch_bounds__(256, 4) k_pool_copy_rot(PoolJobs jobs, int Tc, int blk, int n_b, TemporalRope tr) {
     pdl_wait();
