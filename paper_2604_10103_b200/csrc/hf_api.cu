@@ -527,19 +527,22 @@ hf_status launch_swa_tc5_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16* 
     p.hist = hist; p.o = o; p.lse = lse; p.dev_status = c->dev_status;
     p.heads = c->cfg.heads; p.eps = c->cfg.eps;
     p.q = q; p.z = L.z; p.bias = L.has_bias ? L.bias : nullptr;
+    p.cos_q = c->has_rope_q ? c->rope_q[0] : nullptr; p.sin_q = c->has_rope_q ? c->rope_q[1] : nullptr;
     p.tab = make_table(c, L, k_cur, v_cur); p.sf_hi = L.sf_hi; p.sf_lo = L.sf_lo;
     const CUtensorMap& rk = c->R + c->n_sink_max > 0 ? L.tm_kring : tk;
     const CUtensorMap& rv = c->R + c->n_sink_max > 0 ? L.tm_vring : tv;
     const int grid = p.n_units < c->sm_count ? p.n_units : c->sm_count;
     PdlLaunch pl(dim3(grid), dim3(C::THREADS), C::SMEM_BYTES, st, overlap_prev);
-    if (hist_inside) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, true>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
-    else HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, false>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
+    if (hist_inside && c->has_rope_q) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 2>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
+    else if (hist_inside) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 1>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
+    else HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 0>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
     return post_launch(c, "k_swa_tc5");
 }
 template <int D, int BLK>
 hf_status set_swa_tc5_attr() {
-    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D>::SMEM_BYTES));
-    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D>::SMEM_BYTES));
+    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D>::SMEM_BYTES));
+    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D>::SMEM_BYTES));
+    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D>::SMEM_BYTES));
     return HF_OK;
 }
 
@@ -1204,10 +1207,9 @@ hf_status hf_linear_attn_backward_dq(hf_ctx* c, int layer, const void* q, const 
 }
 
 // Whether the attention kernel forms the history term itself: the tcgen05 kernel does, for the per-head and the identity
-// merge.  The rotated variant of Eq. 4 (numerator and denominator see different phi(Q)) and the full-width merge (which couples
-// the heads) keep the separate read-out.
+// merge, rotated or not.  The full-width merge (which couples the heads) keeps the separate read-out.
 static bool one_kernel_forward(const hf_ctx* c) {
-    return c->swa_kernel == HF_SWA_TCGEN05 && !c->has_rope_q && c->cfg.merge != HF_MERGE_FULL_WIDTH;
+    return c->swa_kernel == HF_SWA_TCGEN05 && c->cfg.merge != HF_MERGE_FULL_WIDTH;
 }
 
 // Eq. 6 + Eq. 4 + Eq. 7 for a selection that is already made.  after_select: the call follows launch_select in the same

@@ -111,6 +111,8 @@ struct Tc5Params {
     const bf16* q;
     const float* z;
     const bf16* bias;
+    const float* cos_q;      // rotation of Eq. 4's numerator, tables [T_c, D / 2], or nullptr: none
+    const float* sin_q;
     bf16* o;
     float* lse;
     int* dev_status;
@@ -201,7 +203,7 @@ __global__ void __launch_bounds__(256) k_union_tiles(const int32_t* __restrict__
 // block, after the tile stream has drained (shared memory and the exchange buffers are free by then).  HIST: the history
 // term of Eq. 4 for the unit's rows is formed first, in fp32 on the CUDA cores, into a shared-memory tile that the
 // attention epilogue adds (Eq. 7).  Slow and rare by design.
-template <int D, int BLK, bool HIST>
+template <int D, int BLK, int HIST>
 __device__ __noinline__ void swa_redo_unit(uint8_t* s_gen, const Tc5Params& p, int u) {
     typedef SwaMma<128, D> M;          // its shared-memory window is the largest: the history tile sits behind it
     constexpr int ROWS = 128;
@@ -239,6 +241,17 @@ __device__ __noinline__ void swa_redo_unit(uint8_t* s_gen, const Tc5Params& p, i
             const float* zr = p.z + (size_t)bh * D;
             for (int a = 0; a < D; ++a) dsum = fmaf(phi_t[tid * PS + a], __ldg(zr + a), dsum);
             den_t[tid] = dsum + p.eps;
+        }
+        if constexpr (HIST == 2) {      // the numerator sees phi(q) rotated, the denominator above does not
+            sync256();
+            const int row = tid >> 1, f0 = (tid & 1) * (D / 2), r_tab = min(q0 + row, p.Tc - 1);
+            for (int a = f0; a < f0 + D / 2; a += 2) {
+                const float c = __ldg(p.cos_q + (size_t)r_tab * (D / 2) + a / 2), sn = __ldg(p.sin_q + (size_t)r_tab * (D / 2) + a / 2);
+                const float x0 = phi_t[row * PS + a], x1 = phi_t[row * PS + a + 1];
+                phi_t[row * PS + a] = fmaf(-x1, sn, x0 * c);
+                phi_t[row * PS + a + 1] = fmaf(x0, sn, x1 * c);
+            }
+            sync256();
         }
         {   // numerator phi(q) S' : thread = (output column, group of rows); S' = hi + lo halves of the folded state
             constexpr int GROUPS = 256 / D, RPT = ROWS / GROUPS;
@@ -309,8 +322,9 @@ __device__ __forceinline__ float swa_max(const uint32_t* r, int nv) {
 }
 
 // Persistent: CTA c processes units c, c + gridDim.x, ...
-// HIST: the history term is formed here; otherwise p.hist, if any, is added.
-template <int D, int BLK, bool HIST>
+// HIST 1: the history term is formed here; 2: with its numerator rotated (code of its own: as a branch it cost the plain one
+// 2 % of the call); 0: p.hist, if any, is added.
+template <int D, int BLK, int HIST>
 __global__ void __launch_bounds__(SwaTc5<D>::THREADS, 1)
 k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kring,
           const __grid_constant__ CUtensorMap tm_vring, const __grid_constant__ CUtensorMap tm_kcur,
@@ -669,11 +683,22 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                             const float4 z0 = *reinterpret_cast<const float4*>(zs + c * 8), z1 = *reinterpret_cast<const float4*>(zs + c * 8 + 4);
                             const float zz[8] = {z0.x, z0.y, z0.z, z0.w, z1.x, z1.y, z1.z, z1.w};
                             const uint32_t ws[4] = {qv.x, qv.y, qv.z, qv.w};
+                            float cs[4] = {1.f, 1.f, 1.f, 1.f}, sn[4] = {0.f, 0.f, 0.f, 0.f};
+                            if constexpr (HIST == 2) {      // the pairs' angles belong to the query's row
+                                const size_t at = (size_t)min(q0 + row, p.Tc - 1) * (D / 2) + k * (FPT / 2) + c * 4;
+                                const float4 c4 = __ldg(reinterpret_cast<const float4*>(p.cos_q + at)), s4 = __ldg(reinterpret_cast<const float4*>(p.sin_q + at));
+                                cs[0] = c4.x; cs[1] = c4.y; cs[2] = c4.z; cs[3] = c4.w;
+                                sn[0] = s4.x; sn[1] = s4.y; sn[2] = s4.z; sn[3] = s4.w;
+                            }
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
                                 const float2 xq = unpack_bf16(ws[e]);
-                                const float f0 = phi_elu1(xq.x), f1 = phi_elu1(xq.y);
-                                dsum = fmaf(f0, zz[2 * e], fmaf(f1, zz[2 * e + 1], dsum));
+                                float f0 = phi_elu1(xq.x), f1 = phi_elu1(xq.y);
+                                dsum = fmaf(f0, zz[2 * e], fmaf(f1, zz[2 * e + 1], dsum));      // (the denominator is not rotated)
+                                if constexpr (HIST == 2) {
+                                    const float r0 = fmaf(-f1, sn[e], f0 * cs[e]), r1 = fmaf(f0, sn[e], f1 * cs[e]);
+                                    f0 = r0; f1 = r1;
+                                }
                                 const uint32_t hp = pack_bf16(f0, f1);
                                 const float2 hf = unpack_bf16(hp);
                                 hi[c * 4 + e] = hp;

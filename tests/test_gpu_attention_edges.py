@@ -43,3 +43,29 @@ def test_forward_at_tile_edges(d, block, tpf, wf, topk, heads, batch):
         assert gpu.ctx.hf_get_device_status() == (0, 0)
     finally:
         gpu.close()
+
+
+@pytest.mark.parametrize("d,block", [(128, 128), (64, 128), (128, 64), (64, 16)])
+def test_rotated_history_in_both_passes(d, block):
+    """The rotated numerator of the history term inside the attention kernel, in its tile stream and in the second pass (the
+    newest keys rise ~180 nats above the first kept block for half of the queries)."""
+    w = gen.Workload("rot_edges", batch=1, heads=2, head_dim=d, tokens_per_frame=300, chunk_frames=1, window_frames=2, block=block,
+                     topk=0, keep_permille=600, seed=223)
+    gpu = hz.GpuStream(w, rope=True); ora = hz.make_oracle(w, rope=True)
+    u = gen.direction(w, 0)
+    a = (180.0 / d ** 0.5) ** 0.5
+    try:
+        for c in range(4):
+            kc, vc = gen.clean_kv(w, 0, c)
+            gpu.append(gpu.up(kc), gpu.up(vc)); ora.append(f64(kc), f64(vc))
+        qb, kb, vb = gen.qkv(w, 0, 4, 0)
+        qb = gen.shifted(qb, u, a, slice(0, 128)); kb = gen.shifted(kb, u, a, slice(256, None))
+        q, k, v = gpu.up(qb), gpu.up(kb), gpu.up(vb)
+        m_gpu, _, _ = gpu.select(q, k)
+        m_ref, _ = ora.select(f64(qb), f64(kb))
+        assert np.array_equal(m_gpu, m_ref)
+        hz.assert_close_out(gpu.forward(q, k, v), ora.forward(f64(qb), f64(kb), f64(vb), mask=m_ref), "hybrid O, rotated")
+        assert gpu.ctx.hf_slow_path_units() > 0
+        assert gpu.ctx.hf_get_device_status() == (0, 0)
+    finally:
+        gpu.close()
