@@ -105,12 +105,14 @@ def _check(status: int):
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream():
+    # the handle of the current device's current stream, without building a torch.cuda.Stream object (0.1 us instead of 3.5 us
+    # per call; a forward's own host time is 7 us)
     import torch
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def make_config(w, merge: int = HF_MERGE_PER_HEAD, swa_kernel: int = HF_SWA_AUTO, z_mode: int = HF_Z_SUM,
