@@ -614,12 +614,14 @@ hf_status launch_bwd_dq(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_c
     p.Tm = c->Tm; p.n_units = c->Tm * c->BH;
     p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D)); p.scale = (float)(1.0 / std::sqrt((double)D));
     p.nb_magic = c->n_b > 1 ? (uint32_t)((0x100000000ull + c->n_b - 1) / c->n_b) : 0u;
-    p.lse = lse; p.delta = c->bwd_delta; p.dq = dq; p.dev_status = c->dev_status;
+    p.lse = lse; p.delta = c->bwd_delta; p.dev_status = c->dev_status;
+    CUtensorMap tdq;                 // output: one warp's 32 rows x half of the columns per store
+    HF_TRY(make_map_ex(c, &tdq, dq, c->Tc, 1, D / 2, 32, true));
     const CUtensorMap& rk = c->R + c->n_sink_max > 0 ? L.tm_kring : tk;
     const CUtensorMap& rv = c->R + c->n_sink_max > 0 ? L.tm_vring : tv;
     const int grid = p.n_units < c->sm_count ? p.n_units : c->sm_count;
     PdlLaunch pl(dim3(grid), dim3(C::THREADS), C::SMEM_BYTES, st, true);
-    HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_bwd_dq<D>, tq, tdo, rk, rv, tk, tv, p));
+    HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_bwd_dq<D>, tq, tdo, rk, rv, tk, tv, tdq, p));
     return post_launch(c, "k_swa_bwd_dq");
 }
 

@@ -7,17 +7,19 @@
 // and k_rowdot forms delta; the block mask is the forward's (held fixed: the top-K choice is piecewise constant).
 //
 // Per (batch*head, query block) unit and kept key tile t, three tensor-core products:
-//   S  = Q K_t^T          A = Q  (smem, K-major),  B = K_t (smem, K-major)          -> TMEM [0, 128) / [384, 512), t even / odd
-//   dP = dO V_t^T         A = dO (smem, K-major),  B = V_t (smem, K-major)          -> TMEM [128, 256)
-//   dQ += dS K_t          A = dS (TMEM, bf16, written over S),  B = K_t (MN-major)   -> TMEM [256, 256 + D)
-// and between them, on the softmax warps (thread = query row x half of the 128 key columns):
+//   S  = Q K_t^T          A = Q  (tensor memory),  B = K_t (smem, K-major)           -> TMEM [0, 128)
+//   dP = dO V_t^T         A = dO (smem, K-major),  B = V_t (smem, K-major)           -> TMEM [128, 256)
+//   dQ += dS K_t          A = dS (TMEM [448, 512), bf16),  B = K_t (MN-major)        -> TMEM [256, 256 + D)
+// and between them, on the softmax warps (four per half g of the key columns, thread = query row):
 //   dS = exp2(S c - lse log2 e) * (dP - delta)        (columns past a short block's end: 0; 1 / sqrt(d) is applied to dQ)
-// The two score products of tile t + 1 are issued while the softmax warps work on tile t: S has two buffers, and the
-// softmax threads free dP's one buffer as soon as their share of it is in registers.  A K tile is held from S to dS K
-// (three stages), a V tile only until dP (two); with less, the latency of the tile loads (~3 000 clk here) is what a
-// tile costs.  The softmax section runs in packed fp32, with the tail mask as separate code and one arrival per warp: 153 -> 132
-// us at 12 heads of 128, 4 680 queries, 28 kept blocks, against scalar code with a select per column.
-// Every wait is bounded and reports through the device status word.
+// As in the forward kernel, the score buffers are free as soon as they are in registers, dS has slots of its own, dS K is
+// issued per half as its four warps finish, and a warp each issues the scores and dS K: the tensor core forms the next
+// tile's scores while the softmax warps work.  What bounds it: 1 536 clk of tensor time and about as much shared-memory
+// operand traffic per tile (Q in tensor memory saves 256 clk of it).  12 heads of 128, 4 680 queries, 28 kept blocks: 153 us with
+// one MMA warp, both score operands in shared memory and scalar softmax code, 128 with packed code, 109 like this.  (Score tiles of half
+// the width, which leave room for more buffers, do not pay: a 128 x 64 product takes as long as a 128 x 128 one; 126 us.)
+// A K tile is held from S to dS K (three stages), a V tile only until dP (two).  The output leaves through the tile Q came in
+// by, once the next unit's Q has been copied out of it.  Every wait is bounded and reports through the device status word.
 #pragma once
 #include "k_swa_tc5.cuh"
 
@@ -151,17 +153,15 @@ template <int D>
 struct SwaBwd {
     static constexpr int BLK = 128;
     static constexpr int SUB = D / 64, SUB_BYTES = BLK * 128, TILE_BYTES = SUB * SUB_BYTES;
-    // a K tile is held until its dS K product has completed, a V tile only until dP has: three and two stages
     static constexpr int KST = 3, VST = 2;
-    static constexpr int OFF_Q = 0, OFF_DO = TILE_BYTES, OFF_K = 2 * TILE_BYTES, OFF_V = OFF_K + KST * TILE_BYTES;
+    static constexpr int OFF_Q = 0, OFF_DO = TILE_BYTES, OFF_K = 2 * TILE_BYTES, OFF_V = OFF_K + KST * TILE_BYTES;   // (Q: also the output's staging tile)
     static constexpr int OFF_BAR = OFF_V + VST * TILE_BYTES;
-    static constexpr int USED_BYTES = OFF_BAR + 256;
-    static constexpr int SMEM_BYTES = USED_BYTES + 1024;
-    static constexpr int THREADS = 320;                  // warps 0-7: softmax (two column groups), 8: TMA, 9: MMA
-    static constexpr int WARP_TMA = 8, WARP_MMA = 9;
-    // S alternates between two buffers (tile t in buffer t % 2, the bf16 dS written over it); dP has one, which the softmax
-    // threads free as soon as they hold their share of it in registers
-    static constexpr int COL_S = 0, COL_S1 = 384, COL_DP = 128, COL_DQ = 256, TMEM_COLS = 512;
+    static constexpr int USED_BYTES = OFF_BAR + 384;
+    // one CTA per SM (it takes all of TMEM); slack for the alignment of the tiles to 1 KB
+    static constexpr int SMEM_BYTES = USED_BYTES + 1024 > 120 * 1024 ? USED_BYTES + 1024 : 120 * 1024;
+    static constexpr int THREADS = 384;                  // warps 0-7: softmax (four per half of the key columns), 8: K loads, 9: V, Q, dO loads, 10: scores, 11: dS K
+    static constexpr int WARP_LOAD_K = 8, WARP_LOAD_V = 9, WARP_S = 10, WARP_DQ = 11;
+    static constexpr int COL_DQ = 256, COL_Q = 384, COL_DS = 448, TMEM_COLS = 512;
 };
 
 struct SwaBwdParams {
@@ -171,7 +171,6 @@ struct SwaBwdParams {
     float scale_log2, scale; // log2(e) / sqrt(d), 1 / sqrt(d)
     const float* lse;        // [B*H, T_c] natural log of the row's sum of exponentials (forward)
     const float* delta;      // [B*H, T_c] g . o_local
-    bf16* dq;                // [B*H, T_c, D]
     int* dev_status;
 };
 
@@ -180,7 +179,7 @@ __global__ void __launch_bounds__(SwaBwd<D>::THREADS, 1)
 k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_do,
              const __grid_constant__ CUtensorMap tm_kring, const __grid_constant__ CUtensorMap tm_vring,
              const __grid_constant__ CUtensorMap tm_kcur, const __grid_constant__ CUtensorMap tm_vcur,
-             const __grid_constant__ SwaBwdParams p) {
+             const __grid_constant__ CUtensorMap tm_dq, const __grid_constant__ SwaBwdParams p) {
     using namespace tc5;
     typedef SwaBwd<D> C;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -188,10 +187,19 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
     uint8_t* s_gen = smem_raw + (s_base - smem_u32(smem_raw));
     const uint32_t sQ = s_base + C::OFF_Q, sDO = s_base + C::OFF_DO, sK = s_base + C::OFF_K, sV = s_base + C::OFF_V;
     const uint32_t bar0 = s_base + C::OFF_BAR;
-    const uint32_t bar_kf = bar0 + 128, bar_ke = bar0 + 152, bar_vf = bar0 + 32, bar_ve = bar0 + 48, bar_qf = bar0 + 64, bar_qe = bar0 + 72,
-                   bar_sd = bar0 + 80, bar_ds = bar0 + 88, bar_dqf = bar0 + 96, bar_dqe = bar0 + 104, bar_dpf = bar0 + 120;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_gen + C::OFF_BAR + 112);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(s_gen + C::OFF_BAR + 116);
+    // half tile s = 2 t + h: pairs of barriers, index h, completion t
+    // (ds, df: pairs, index = half; completion t, like sd and se)
+    const uint32_t bar_kf = bar0, bar_ke = bar0 + 48, bar_vf = bar0 + 96, bar_ve = bar0 + 128, bar_sd = bar0 + 160, bar_ds = bar0 + 176,
+                   bar_se = bar0 + 192,         // scores of tile t are in registers (eight warps)
+                   bar_df = bar0 + 208,         // dS K of a half of tile t complete: its dS slot is free
+                   bar_drain = bar0 + 224,      // two: each MMA warp's last operations complete
+                   bar_qf = bar0 + 240,         // unit n: Q landed
+                   bar_cp = bar0 + 248,         // unit n: ... and copied to tensor memory
+                   bar_qe = bar0 + 256,         // unit n: its output, staged where Q of unit n + 1 had been, has left
+                   bar_of = bar0 + 264, bar_oe = bar0 + 272,       // unit n: dO landed / read for the last time
+                   bar_dqf = bar0 + 280, bar_dqe = bar0 + 288;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_gen + C::OFF_BAR + 296);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(s_gen + C::OFF_BAR + 300);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int keep = p.keep;
@@ -201,11 +209,13 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::KST; ++s) { mbar_init(bar_kf + 8 * s, 1); mbar_init(bar_ke + 8 * s, 1); }
         for (int s = 0; s < C::VST; ++s) { mbar_init(bar_vf + 8 * s, 1); mbar_init(bar_ve + 8 * s, 1); }
-        mbar_init(bar_qf, 1); mbar_init(bar_qe, 1); mbar_init(bar_sd, 1); mbar_init(bar_ds, 8); mbar_init(bar_dqf, 1); mbar_init(bar_dqe, 8); mbar_init(bar_dpf, 8);
+        for (int s = 0; s < 2; ++s) { mbar_init(bar_ds + 8 * s, 4); mbar_init(bar_df + 8 * s, 1); mbar_init(bar_drain + 8 * s, 1); }
+        mbar_init(bar_sd, 1); mbar_init(bar_se, 8);
+        mbar_init(bar_qf, 1); mbar_init(bar_cp, 1); mbar_init(bar_of, 1); mbar_init(bar_oe, 1); mbar_init(bar_qe, 8); mbar_init(bar_dqf, 1); mbar_init(bar_dqe, 8);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
-    if (warp == C::WARP_MMA) {
+    if (warp == C::WARP_S) {
         tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS);
         tmem_relinquish();
     }
@@ -215,25 +225,38 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
     const uint32_t tmem = *tmem_slot;
     pdl_wait();
 
-    if (warp == C::WARP_TMA) {
-        // ================================================================= TMA producer: Q and dO per unit, K and V per tile
+    auto wait_w = [&](uint32_t bar, uint32_t parity, int where) -> bool {
+        return mbar_wait_warp<true>(bar, parity & 1u, abort_flag, p.dev_status, where);
+    };
+
+    if (warp == C::WARP_LOAD_K || warp == C::WARP_LOAD_V) {
+        // ================================================================= TMA producers: K; V, Q and dO
         if (lane == 0) {
+            const bool is_k = warp == C::WARP_LOAD_K;
             bool ok = true;
+            RingPos<C::KST> rk;
+            RingPos<C::VST> rv;
             int t = 0;
             const int Tn = (p.n_sink + p.n_cached + 1) * p.n_b;
+            auto load_q = [&](int m) {
+                const int u = blockIdx.x + m * gridDim.x, bh = u / p.Tm, i = u - bh * p.Tm;
+                mbar_expect_tx(bar_qf, C::TILE_BYTES);
+#pragma unroll
+                for (int s = 0; s < C::SUB; ++s) tma_load_4d(sQ + s * C::SUB_BYTES, &tm_q, s * 64, i * C::BLK, bh, 0, bar_qf);
+            };
+            if (!is_k && my_units > 0) load_q(0);
             for (int n = 0; ok && n < my_units; ++n) {
                 const int u = blockIdx.x + n * gridDim.x;
-                const int bh = u / p.Tm, i = u - bh * p.Tm;
+                const int bh = u / p.Tm;
                 const int32_t* my_idx = p.idx + (size_t)u * keep;
-                if (n >= 1 && !(ok = mbar_wait<true>(bar_qe, (n - 1) & 1, abort_flag, p.dev_status, 81))) break;
-                mbar_expect_tx(bar_qf, 2 * C::TILE_BYTES);
+                if (!is_k) {
+                    if (n >= 1 && !(ok = mbar_wait<true>(bar_oe, (n - 1) & 1, abort_flag, p.dev_status, 94))) break;
+                    mbar_expect_tx(bar_of, C::TILE_BYTES);
 #pragma unroll
-                for (int s = 0; s < C::SUB; ++s) {
-                    tma_load_4d(sQ + s * C::SUB_BYTES, &tm_q, s * 64, i * C::BLK, bh, 0, bar_qf);
-                    tma_load_4d(sDO + s * C::SUB_BYTES, &tm_do, s * 64, i * C::BLK, bh, 0, bar_qf);
+                    for (int s = 0; s < C::SUB; ++s) tma_load_4d(sDO + s * C::SUB_BYTES, &tm_do, s * 64, (u - bh * p.Tm) * C::BLK, bh, 0, bar_of);
                 }
-                for (int j = 0; j < keep; ++j, ++t) {
-                    const int blk = checked_block(__ldg(my_idx + j), Tn, p.dev_status, u);
+                for (int j = 0; ok && j < keep; ++j, ++t) {
+                    const int blk = checked_block(__ldg(my_idx + j), Tn, is_k ? p.dev_status : nullptr, u);
                     int c = 0, jb = blk;
                     while (jb >= p.n_b) { jb -= p.n_b; ++c; }
                     const bool cur = (c == p.n_sink + p.n_cached);
@@ -242,17 +265,24 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
                         if (c < p.n_sink) slot = p.P + c;
                         else { slot = p.ring_head + c - p.n_sink; if (slot >= p.P) slot -= p.P; }
                     }
-                    const int kst = t % C::KST, vst = t % C::VST;
-                    if (t >= C::VST && !(ok = mbar_wait<true>(bar_ve + 8 * vst, ((t / C::VST) & 1) ^ 1, abort_flag, p.dev_status, 83))) break;
-                    mbar_expect_tx(bar_vf + 8 * vst, C::TILE_BYTES);
+                    const CUtensorMap* m = is_k ? (cur ? &tm_kcur : &tm_kring) : (cur ? &tm_vcur : &tm_vring);
+                    const int st = is_k ? rk.stage : rv.stage;
+                    const uint32_t ph = is_k ? rk.phase : rv.phase;
+                    const uint32_t full = (is_k ? bar_kf : bar_vf) + 8 * st, freed = (is_k ? bar_ke : bar_ve) + 8 * st;
+                    if (t >= (is_k ? C::KST : C::VST) && !(ok = mbar_wait<true>(freed, ph ^ 1u, abort_flag, p.dev_status, is_k ? 82 : 83))) break;
+                    mbar_expect_tx(full, C::TILE_BYTES);
 #pragma unroll
                     for (int s = 0; s < C::SUB; ++s)
-                        tma_load_4d(sV + vst * C::TILE_BYTES + s * C::SUB_BYTES, cur ? &tm_vcur : &tm_vring, s * 64, jb * C::BLK, bh, slot, bar_vf + 8 * vst);
-                    if (t >= C::KST && !(ok = mbar_wait<true>(bar_ke + 8 * kst, ((t / C::KST) & 1) ^ 1, abort_flag, p.dev_status, 82))) break;
-                    mbar_expect_tx(bar_kf + 8 * kst, C::TILE_BYTES);
-#pragma unroll
-                    for (int s = 0; s < C::SUB; ++s)
-                        tma_load_4d(sK + kst * C::TILE_BYTES + s * C::SUB_BYTES, cur ? &tm_kcur : &tm_kring, s * 64, jb * C::BLK, bh, slot, bar_kf + 8 * kst);
+                        tma_load_4d((is_k ? sK : sV) + st * C::TILE_BYTES + s * C::SUB_BYTES, m, s * 64, jb * C::BLK, bh, slot, full);
+                    if (is_k) rk.advance(); else rv.advance();
+                    if (!is_k && ok && j == (keep > 2 ? 2 : keep - 1) && n + 1 < my_units) {
+                        // Q of the next unit: its tile is free once this unit's has been copied out of it and the output of the
+                        // unit before, staged there since, has left (said after this unit's first tile)
+                        if (n == 0) ok = mbar_wait<true>(bar_cp, 0, abort_flag, p.dev_status, 81);
+                        else ok = mbar_wait<true>(bar_qe, (n - 1) & 1, abort_flag, p.dev_status, 80);
+                        if (!ok) break;
+                        load_q(n + 1);
+                    }
                 }
             }
             if (!ok) {
@@ -260,63 +290,95 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
                 while (clock64() - t0 < 400000) {}
             }
         }
-    } else if (warp == C::WARP_MMA) {
-        // ================================================================= MMA issuer (warp-uniform, one elected lane issues)
+    } else if (warp == C::WARP_S) {
+        // ================================================================= scores (warp-uniform, one elected lane issues)
         constexpr uint32_t IDESC_S = idesc_bf16(128, false);
-        constexpr uint32_t IDESC_DQ = idesc_bf16(D, true);
-        constexpr uint32_t TILE_STEP = C::TILE_BYTES >> 4;
+        constexpr uint32_t STEP = C::TILE_BYTES >> 4;             // descriptor address field counts 16-byte units
         const uint64_t dq0 = smem_desc_sw128(sQ, 16, 1024), dd0 = smem_desc_sw128(sDO, 16, 1024);
         const uint64_t dk0 = smem_desc_sw128(sK, 16, 1024), dv0 = smem_desc_sw128(sV, 16, 1024);
-        const uint64_t dkm = smem_desc_sw128(sK, C::SUB_BYTES, 1024);        // the K tile again, as the MN-major operand of dS K
-        const uint32_t hi_k = (uint32_t)(dq0 >> 32), hi_m = (uint32_t)(dkm >> 32);
+        const uint32_t hi_k = (uint32_t)(dk0 >> 32);
         bool ok = true;
-        // S_t = Q K_t^T and dP_t = dO V_t^T, one tile ahead of the softmax warps: tile t + 1 is issued while they turn
-        // tile t into dS (S into the other buffer; dP as soon as they have taken tile t's out of tensor memory)
-        int n_s = 0, j_s = 0, t_s = 0;
-        auto issue_scores = [&]() -> bool {
-            if (j_s == 0 && !__all_sync(0xffffffffu, mbar_wait<true>(bar_qf, n_s & 1, abort_flag, p.dev_status, 84))) return false;
-            const int kst = t_s % C::KST, vst = t_s % C::VST;
-            if (!__all_sync(0xffffffffu, mbar_wait<true>(bar_kf + 8 * kst, (t_s / C::KST) & 1, abort_flag, p.dev_status, 85))) return false;
-            if (!__all_sync(0xffffffffu, mbar_wait<true>(bar_vf + 8 * vst, (t_s / C::VST) & 1, abort_flag, p.dev_status, 86))) return false;
-            fence_after_sync();
-            if (elect_one()) {
-                mma_ss_tile<D>(tmem + ((t_s & 1) ? C::COL_S1 : C::COL_S), (uint32_t)dq0, (uint32_t)dk0 + kst * TILE_STEP, hi_k, IDESC_S);
-                mma_ss_tile<D>(tmem + C::COL_DP, (uint32_t)dd0, (uint32_t)dv0 + vst * TILE_STEP, hi_k, IDESC_S);
-                mma_commit(bar_sd);
-                mma_commit(bar_ve + 8 * vst);
-                if (j_s == keep - 1) mma_commit(bar_qe);          // Q and dO of this unit have been read for the last time
-            }
-            __syncwarp();
-            ++t_s;
-            if (++j_s == keep) { j_s = 0; ++n_s; }
-            return true;
-        };
-        if (n_tiles > 0) ok = issue_scores();
         int t = 0;
+        RingPos<C::KST> rk;
+        RingPos<C::VST> rv;
         for (int n = 0; ok && n < my_units; ++n) {
             for (int j = 0; ok && j < keep; ++j, ++t) {
-                const int kst = t % C::KST;
-                if (t + 1 < n_tiles) {
-                    // dP of tile t is in the softmax threads' registers: the buffer may take tile t + 1
-                    if (!(ok = __all_sync(0xffffffffu, mbar_wait<true>(bar_dpf, t & 1, abort_flag, p.dev_status, 91)))) break;
-                    if (!(ok = issue_scores())) break;
+                if (j == 0) {
+                    // Q moves to tensor memory, where the previous unit's last scores have read theirs by then
+                    if (!(ok = wait_w(bar_qf, n, 84))) break;
+                    if (t >= 1 && !(ok = wait_w(bar_sd, t - 1, 92))) break;
+                    fence_after_sync();
+                    if (elect_one()) {
+#pragma unroll
+                        for (int ks = 0; ks < D / 16; ++ks)                         // 16 features = 32 bytes of a row = 8 columns
+                            tmem_cp_128x256b(tmem + C::COL_Q + 8 * ks, dq0 + (uint64_t)((ks >> 2) * (C::SUB_BYTES >> 4) + (ks & 3) * 2));
+                        mma_commit(bar_cp);
+                    }
+                    __syncwarp();
+                    if (!(ok = wait_w(bar_of, n, 95))) break;
                 }
-                if (!(ok = __all_sync(0xffffffffu, mbar_wait<true>(bar_ds, t & 1, abort_flag, p.dev_status, 87)))) break;
-                // the accumulator of the previous unit has been read out before this unit's first product overwrites it
-                if (j == 0 && n >= 1 && !(ok = __all_sync(0xffffffffu, mbar_wait<true>(bar_dqe, (n - 1) & 1, abort_flag, p.dev_status, 88)))) break;
+                if (!(ok = wait_w(bar_kf + 8 * rk.stage, rk.phase, 85))) break;
+                if (!(ok = wait_w(bar_vf + 8 * rv.stage, rv.phase, 86))) break;
+                if (t >= 1 && !(ok = wait_w(bar_se, t - 1, 91))) break;        // the tile before is in registers
                 fence_after_sync();
                 if (elect_one()) {
-                    const uint32_t tS = tmem + ((t & 1) ? C::COL_S1 : C::COL_S);
-                    mma_ts_tile_split(tmem + C::COL_DQ, tS, tS + 64, (uint32_t)dkm + kst * TILE_STEP, hi_m, IDESC_DQ, j > 0);
-                    mma_commit(bar_ke + 8 * kst);
-                    if (j == keep - 1) mma_commit(bar_dqf);
+                    // dP first: V's stage, of which there are fewer, is free earlier
+                    mma_ss_tile<D>(tmem + 128, (uint32_t)dd0, (uint32_t)dv0 + rv.stage * STEP, hi_k, IDESC_S);
+                    mma_commit(bar_ve + 8 * rv.stage);
+                    if (j == keep - 1) mma_commit(bar_oe);
+                    mma_ts_kmajor<D>(tmem, tmem + C::COL_Q, (uint32_t)dk0 + rk.stage * STEP, hi_k, IDESC_S);
+                    mma_commit(bar_sd);
                 }
                 __syncwarp();
+                rk.advance();
+                rv.advance();
             }
+        }
+        if (elect_one()) mma_commit(bar_drain);
+        __syncwarp();
+        {
+            const long long t0 = clock64();
+            while (!mbar_try_wait(bar_drain, 0) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
+        }
+    } else if (warp == C::WARP_DQ) {
+        // ================================================================= dQ += dS K
+        constexpr uint32_t IDESC_DQ = idesc_bf16(D, true);
+        constexpr uint32_t STEP = C::TILE_BYTES >> 4, HALF = 64 * 128 >> 4;  // 64 rows of a tile, in 16-byte units
+        const uint64_t dkm = smem_desc_sw128(sK, C::SUB_BYTES, 1024);        // the K tile again, as the MN-major operand
+        const uint32_t hi_m = (uint32_t)(dkm >> 32);
+        bool ok = true;
+        int t = 0;
+        RingPos<C::KST> rk;
+        for (int n = 0; ok && n < my_units; ++n) {
+            for (int j = 0; ok && j < keep; ++j, ++t) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if (!(ok = wait_w(bar_ds + 8 * h, t, 87))) break;
+                    // the accumulator of the previous unit has been read out before this unit's first product overwrites it
+                    if (h == 0 && j == 0 && n >= 1 && !(ok = wait_w(bar_dqe, n - 1, 88))) break;
+                    fence_after_sync();
+                    if (elect_one()) {
+                        mma_ts_half(tmem + C::COL_DQ, tmem + C::COL_DS + 32 * h, (uint32_t)dkm + rk.stage * STEP + h * HALF, hi_m, IDESC_DQ, j > 0 || h > 0);
+                        mma_commit(bar_df + 8 * h);
+                        if (h == 1) {
+                            mma_commit(bar_ke + 8 * rk.stage);
+                            if (j == keep - 1) mma_commit(bar_dqf);
+                        }
+                    }
+                    __syncwarp();
+                }
+                rk.advance();
+            }
+        }
+        if (elect_one()) mma_commit(bar_drain + 8);
+        __syncwarp();
+        {
+            const long long t0 = clock64();
+            while (!mbar_try_wait(bar_drain + 8, 0) && clock64() - t0 < WAIT_LIMIT_CYCLES) {}
         }
     } else {
         // ================================================================= softmax warps: dS from S and dP; dQ out at the unit's end
-        const int grp = warp >> 2;                          // key columns [64 grp, 64 grp + 64) of a tile
+        const int grp = warp >> 2;                          // the half of every tile's key columns this warp turns; then a half of dQ's columns
         const int row = (warp & 3) * 32 + lane;
         const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
         const bool lane0 = lane == 0, ragged = p.Tc % C::BLK != 0;
@@ -336,70 +398,87 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
                     const uint32_t x1 = j + lane < keep ? (uint32_t)__ldg(my_idx + j + lane) + 1u : 0xffffffffu;
                     tails = __ballot_sync(0xffffffffu, x1 <= HF_MAX_TN && (p.n_b == 1 || __umulhi(x1, p.nb_magic) * p.n_b == x1));
                 }
+                const bool tail = (tails >> (j & 31)) & 1u;
                 ok = mbar_wait_warp(bar_sd, t & 1, abort_flag, p.dev_status, 89);
                 if (!ok) break;
                 fence_after_sync();
-                const uint32_t tS = lane_base + ((t & 1) ? C::COL_S1 : C::COL_S) + grp * 64;
-                // this thread's share of dP and S: the MMA warp refills dP's buffer as soon as every warp has it
-                uint32_t dp[2][32], s[2][32];
-                tmem_ld32(lane_base + C::COL_DP + grp * 64, dp[0]);
-                tmem_ld32(lane_base + C::COL_DP + grp * 64 + 32, dp[1]);
+                const uint32_t tS = lane_base + 64 * grp;
+                uint32_t s[2][32], dp[2][32];
                 tmem_ld32(tS, s[0]);
                 tmem_ld32(tS + 32, s[1]);
+                tmem_ld32(tS + 128, dp[0]);
+                tmem_ld32(tS + 160, dp[1]);
                 tmem_wait_ld();
                 fence_before_sync();
-                mbar_arrive_if(bar_dpf, lane0);
-                // (all of this thread's S columns are in registers: the bf16 dS may go over them)
-                if (!((tails >> (j & 31)) & 1u)) {
+                mbar_arrive_if(bar_se, lane0);                  // the next tile's scores may be formed
+                auto store_ds = [&](int c, const uint32_t (&pk)[16]) {
+                    if (c == 0 && t >= 1) {                     // the half's dS slot: dS K of the tile before has read it
+                        ok = mbar_wait_warp(bar_df + 8 * grp, (t - 1) & 1, abort_flag, p.dev_status, 96);
+                        fence_after_sync();
+                    }
+                    tmem_st16(lane_base + C::COL_DS + 32 * grp + 16 * c, pk);
+                };
+                if (!tail) {
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
                         uint32_t pk[16];
                         bwd_ds<false>(s[c], dp[c], 32, p.scale_log2, neg_lse2, delta, pk);
-                        tmem_st16(tS + c * 16, pk);
+                        store_ds(c, pk);
                     }
                 } else {
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
                         uint32_t pk[16];
                         bwd_ds<true>(s[c], dp[c], p.Tc - (p.n_b - 1) * C::BLK - grp * 64 - c * 32, p.scale_log2, neg_lse2, delta, pk);
-                        tmem_st16(tS + c * 16, pk);
+                        store_ds(c, pk);
                     }
                 }
+                if (!ok) break;
                 tmem_wait_st();
                 fence_before_sync();
-                mbar_arrive_if(bar_ds, lane0);
+                mbar_arrive_if(bar_ds + 8 * grp, lane0);
+                if (j == 0 && n >= 1) {         // the previous unit's output has long left its staging tile by now
+                    if (lane0) bulk_wait_read();
+                    __syncwarp();
+                    mbar_arrive_if(bar_qe, lane0);
+                }
             }
             if (!ok) break;
             ok = mbar_wait_warp(bar_dqf, n & 1, abort_flag, p.dev_status, 90);
+            if (ok && n + 1 < my_units) ok = mbar_wait_warp(bar_cp, (n + 1) & 1, abort_flag, p.dev_status, 93);    // Q of the next unit has left the staging tile
             if (!ok) break;
             fence_after_sync();
+            uint32_t out[D / 4];
 #pragma unroll
             for (int c = 0; c < D / 64; ++c) {
                 uint32_t o[32];
                 tmem_ld32(lane_base + C::COL_DQ + grp * (D / 2) + c * 32, o);
                 tmem_wait_ld();
 #pragma unroll
-                for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * p.scale);
-                if (row < nq) {
-                    bf16* dst = p.dq + g_row * D + grp * (D / 2) + c * 32;
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        uint4 w;
-                        w.x = pack_bf16(__uint_as_float(o[v * 8]), __uint_as_float(o[v * 8 + 1]));
-                        w.y = pack_bf16(__uint_as_float(o[v * 8 + 2]), __uint_as_float(o[v * 8 + 3]));
-                        w.z = pack_bf16(__uint_as_float(o[v * 8 + 4]), __uint_as_float(o[v * 8 + 5]));
-                        w.w = pack_bf16(__uint_as_float(o[v * 8 + 6]), __uint_as_float(o[v * 8 + 7]));
-                        *reinterpret_cast<uint4*>(dst + v * 8) = w;
-                    }
-                }
+                for (int e = 0; e < 32; e += 2) out[c * 16 + e / 2] = pack_bf16(__uint_as_float(o[e]) * p.scale, __uint_as_float(o[e + 1]) * p.scale);
             }
             fence_before_sync();
             mbar_arrive_if(bar_dqe, lane0);
+            // out through shared memory and one bulk tensor store per warp (32 rows x half of the columns; the map clips)
+            constexpr int RB = D;                           // bytes per staged row (D / 2 columns)
+            const uint32_t off = C::OFF_Q + warp * 32 * RB;
+            uint8_t* stage = s_gen + off + lane * RB;
+            const int swz = D == 128 ? lane & 7 : (lane >> 1) & 3;
+#pragma unroll
+            for (int c = 0; c < D / 16; ++c)
+                *reinterpret_cast<uint4*>(stage + ((c ^ swz) << 4)) = make_uint4(out[4 * c], out[4 * c + 1], out[4 * c + 2], out[4 * c + 3]);
+            fence_proxy_async();
+            __syncwarp();
+            if (lane0 && q0 + (warp & 3) * 32 < p.Tc) {
+                tma_store_4d(&tm_dq, s_base + off, grp * (D / 2), q0 + (warp & 3) * 32, bh, 0);
+                bulk_commit();
+            }
         }
+        if (lane0) bulk_wait_all();
     }
     fence_before_sync();
     __syncthreads();
-    if (warp == C::WARP_MMA) {
+    if (warp == C::WARP_S) {
         fence_after_sync();
         tmem_dealloc(tmem, C::TMEM_COLS);
     }
