@@ -95,7 +95,7 @@ struct hf_ctx {
     int* union_tiles = nullptr;          // ... and tiles per unit
     int union_max_tiles = 0;
     float* bwd_delta = nullptr;          // backward pass: g . o_local per query row [B*H, T_c]
-    int* bwd_order = nullptr;            // ... and the key blocks of the current chunk, most pairs first [B*H, n_b]
+    int2* bwd_order = nullptr;           // ... and the key blocks of the current chunk, most pairs first, with their number [B*H, n_b]
     float* partials = nullptr;       // absorb split partials
     float* partials_layers = nullptr;    // layer-batched state update: one partial per (layer, batch*head, group)
     size_t partials_layers_count = 0;

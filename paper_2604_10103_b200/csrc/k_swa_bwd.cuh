@@ -36,7 +36,7 @@ struct RowDot { static constexpr int LPR = D / 8, RPB = 4 * 256 / LPR; };      /
 struct BwdOrder {
     const uint32_t* mask;    // [B*H, T_m, mask_words], or nullptr: no ordering
     int mask_words, first_block, n_b, Tm, BH;
-    int* order;              // [B*H * n_b]
+    int2* order;             // [B*H * n_b]: unit, its pairs (-1: not counted)
 };
 constexpr int BWD_ORDER_MAX = 4096;              // units that are ordered; beyond that a thread block has dozens and balance comes by itself
 __device__ __noinline__ void bwd_order_units(const BwdOrder& q) {
@@ -44,7 +44,7 @@ __device__ __noinline__ void bwd_order_units(const BwdOrder& q) {
     __shared__ int at[HF_MAX_TN + 2];            // units with fewer kept pairs come later: bin b holds count Tm - b
     const int n = q.BH * q.n_b, tid = threadIdx.x;
     if (n > BWD_ORDER_MAX || q.Tm > HF_MAX_TN) {
-        for (int u = tid; u < n; u += 256) q.order[u] = u;
+        for (int u = tid; u < n; u += 256) q.order[u] = make_int2(u, -1);
         return;
     }
     for (int u = tid; u < n; u += 256) cnt[u] = 0;
@@ -87,7 +87,7 @@ __device__ __noinline__ void bwd_order_units(const BwdOrder& q) {
         }
     }
     __syncthreads();
-    for (int u = tid; u < n; u += 256) q.order[atomicAdd(&at[q.Tm - cnt[u]], 1)] = u;
+    for (int u = tid; u < n; u += 256) q.order[atomicAdd(&at[q.Tm - cnt[u]], 1)] = make_int2(u, cnt[u]);
 }
 template <int D>
 __global__ void __launch_bounds__(256) k_rowdot(const bf16* __restrict__ a, const bf16* __restrict__ b, float* __restrict__ out, long long rows, BwdOrder ord) {
@@ -486,19 +486,25 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
 
 // ------------------------------------------------------------------------------------------------------------
 // dK and dV of the current chunk (the keys and values that carry gradient in the rollout: the cache holds clean chunks of
-// earlier, gradient-free passes).  The transposed walk: unit = (batch*head, key block j of the current chunk); for every
-// query block i that keeps j (read off the selection's bit mask), in two halves h of 64 queries, rows = keys, columns = queries:
-//   S^T  = K_j Q_ih^T      A = K_j (smem), B = Q_ih (smem)                    -> TMEM [128 h, + 64)
-//   dP^T = V_j dO_ih^T     A = V_j (smem), B = dO_ih (smem)                   -> TMEM [128 h + 64, + 64)
+// earlier, gradient-free passes).  The transposed walk: unit = (batch*head, key block j of the current chunk); for every query
+// block i that keeps j (read off the selection's bit mask), rows = keys, columns = queries:
+//   S^T  = K_j Q_i^T      A = K_j (smem), B = Q_i (smem)                      -> TMEM [0, 128)
+//   dP^T = V_j dO_i^T     A = V_j (smem), B = dO_i (smem)                     -> TMEM [128, 256)
 //   P^T  = exp2(S^T c - lse_i log2 e)  (bf16, over S^T),   dS^T = P^T (dP^T - delta_i)  (bf16, over dP^T)
-//   dV_j += P^T dO_ih      A = P^T (TMEM), B = dO_ih (MN-major)                -> TMEM [256, 256 + D)
-//   dK_j += dS^T Q_ih      A = dS^T (TMEM), B = Q_ih (MN-major)                -> TMEM [384, 384 + D); 1 / sqrt(d) at the end
-// The accumulators and one full pair of score tiles fill tensor memory at head dim 128; halves are what lets the tensor core
-// form one half's scores while the softmax warps work on the other (a pair's four products are 2 048 clk of tensor time, 2 560
-// with the score products' operand reads from shared memory; whole tiles alternated strictly: ~9 000 clk a pair).
-// lse and delta are per QUERY, i.e. per column here: staged in shared memory a pair ahead; a query row past the chunk's end
-// gets lse = +inf, so its P and dS are zero, and key rows past the end only reach output rows that are not stored: no masks.
-// Measured at 12 heads of 128, 4 680 queries, 28 kept blocks: 134 -> 94 us, 82 with the units in order of their pairs (BwdOrder).
+//   dV_j += P^T dO_i      A = P^T (TMEM), B = dO_i (MN-major)                  -> TMEM [256, 256 + D)
+//   dK_j += dS^T Q_i      A = dS^T (TMEM), B = Q_i (MN-major)                  -> TMEM [384, 384 + D); 1 / sqrt(d) at the end
+// Accumulators and one pair of score tiles fill tensor memory at head dim 128.  What keeps the tensor core busy all the same is
+// the order in which the one MMA warp issues: dV(t), S(t + 1), dK(t), dP(t + 1) -- the softmax warps form dS(t) during the first
+// two products and P(t + 1) during the last two.  A pair is 2 048 clk of tensor time and, with the tiles' arrival, somewhat
+// more of shared-memory traffic.  lse and delta are per QUERY, i.e. per column here: a warp of its own finds the pairs and stages
+// them a pair ahead; the others only need the number of a unit's pairs, which comes with the order.  A query row past the
+// chunk's end gets lse = +inf, so its P and dS are zero, and key rows past the end only reach output rows that are not stored:
+// no masks.
+// 12 heads of 128, 4 680 queries, 28 kept blocks (28 pairs per thread block): whole tiles that alternate strictly between
+// tensor core and (scalar) softmax 134 us; half-width score tiles, which overlap but take the tensor core twice as long (a
+// 128 x 64 product costs as much as a 128 x 128 one), 94 us, 85 with the units in order of their pairs (BwdOrder); the order
+// above 71 us.  (The two score regions as chains with an MMA warp each: 79 us, their products interleave and each region
+// is late.  Walking the mask in every warp: 1 000 clk per pair of 4 000.)
 // ------------------------------------------------------------------------------------------------------------
 template <int D>
 struct SwaBwdKV {
@@ -508,14 +514,14 @@ struct SwaBwdKV {
     static constexpr int OFF_K = 0, OFF_V = TILE_BYTES, OFF_Q = 2 * TILE_BYTES, OFF_DO = OFF_Q + STAGES * TILE_BYTES;
     static constexpr int OFF_OUT = OFF_DO + STAGES * TILE_BYTES;         // staging of the output tile, 32 rows x D / 2 columns per warp
     static constexpr int OFF_BAR = OFF_OUT + BLK * D * 2;
-    static constexpr int OFF_ROW = OFF_BAR + 256;        // [2 pairs][-lse log2 e, -delta][128] floats
+    static constexpr int OFF_ROW = OFF_BAR + 256;        // [2 pairs][2 halves of the queries][-lse log2 e, -delta][64] floats
     static constexpr int USED_BYTES = OFF_ROW + 2 * 2 * BLK * 4;
     // one CTA per SM (it takes all of TMEM); slack for the alignment of the tiles to 1 KB, as far as there is room (checked)
     static constexpr int WANT_BYTES = USED_BYTES + 1024 > 120 * 1024 ? USED_BYTES + 1024 : 120 * 1024, MAX_SMEM = 232448;
     static constexpr int SMEM_BYTES = WANT_BYTES < MAX_SMEM ? WANT_BYTES : MAX_SMEM;
     static_assert(USED_BYTES <= MAX_SMEM, "shared memory layout does not fit");
-    static constexpr int THREADS = 320;                  // warps 0-7: softmax (two column groups), 8: TMA, 9: MMA
-    static constexpr int WARP_TMA = 8, WARP_MMA = 9;
+    static constexpr int THREADS = 352;                  // warps 0-7: softmax (two halves of the queries), 8: TMA, 9: MMA,
+    static constexpr int WARP_TMA = 8, WARP_MMA = 9, WARP_ROW = 10;                 // 10: lse and delta of the queries
     static constexpr int COL_DV = 256, COL_DK = 384, TMEM_COLS = 512;
 };
 
@@ -523,7 +529,7 @@ struct SwaBwdKVParams {
     const uint32_t* mask;    // [B*H, T_m, mask_words]: the forward's selection
     int mask_words, first_block;     // logical index of the current chunk's first key block
     int Tc, n_b, Tm, n_units;        // units = B*H x n_b
-    const int* order;        // [n_units]: the units, most pairs first
+    const int2* order;       // [n_units]: the units, most pairs first, with the number of their pairs (-1: not counted)
     float scale_log2, scale;
     const float* lse;        // [B*H, T_c]
     const float* delta;      // [B*H, T_c]
@@ -543,6 +549,13 @@ struct PairWalk {
     __device__ __forceinline__ void open(const SwaBwdKVParams& p, int u) {
         bh = u / p.n_b; jb = u - bh * p.n_b; w = 0;
         bits = word(p, 0);
+    }
+    // the pairs of unit u: all of its mask words
+    __device__ __forceinline__ int count(const SwaBwdKVParams& p, int u) {
+        open(p, u);
+        int n = __popc(bits);
+        for (int x = 1; x * 32 < p.Tm; ++x) n += __popc(word(p, x));
+        return n;
     }
     __device__ __forceinline__ int pop(const SwaBwdKVParams& p) {      // the next query block, or -1
         while (bits == 0) {
@@ -572,11 +585,14 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     uint8_t* s_gen = smem_raw + (s_base - smem_u32(smem_raw));
     const uint32_t sK = s_base + C::OFF_K, sV = s_base + C::OFF_V, sQ = s_base + C::OFF_Q, sDO = s_base + C::OFF_DO;
     const uint32_t bar0 = s_base + C::OFF_BAR;
-    // half-pair s = 2 t + h: pairs of barriers, index h, completion t
-    const uint32_t bar_kvf = bar0, bar_kve = bar0 + 8, bar_qf = bar0 + 16, bar_qe = bar0 + 32, bar_sd = bar0 + 48, bar_ds = bar0 + 64,
-                   bar_accf = bar0 + 80, bar_acce = bar0 + 88;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_gen + C::OFF_BAR + 96);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(s_gen + C::OFF_BAR + 100);
+    // pair t of the thread block: Q and dO rings, stage t & 1; pd: completion t; pr, ds: index = half of the queries, completion t
+    const uint32_t bar_kvf = bar0, bar_kve = bar0 + 8,         // m-th unit with pairs: K and V landed / read for the last time
+                   bar_qf = bar0 + 16, bar_qe = bar0 + 32, bar_of = bar0 + 48, bar_oe = bar0 + 64,
+                   bar_sd = bar0 + 152, bar_pd = bar0 + 88,    // S of pair t complete and its lse and delta staged (index t & 1); dP complete
+                   bar_pr = bar0 + 96, bar_ds = bar0 + 112,    // half of P, dS written (four warps)
+                   bar_accf = bar0 + 128, bar_acce = bar0 + 136;       // unit n: dV and dK complete / read out
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_gen + C::OFF_BAR + 144);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(s_gen + C::OFF_BAR + 148);
     float* row_vals = reinterpret_cast<float*>(s_gen + C::OFF_ROW);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -584,12 +600,19 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     const int rounds = p.n_units / (int)gridDim.x, rest = p.n_units - rounds * (int)gridDim.x;
     auto place = [&](int n) -> int { return (n & 1) ? (int)gridDim.x - 1 - (int)blockIdx.x : (int)blockIdx.x; };
     const int my_units = rounds + (place(rounds) < rest ? 1 : 0);
-    auto unit_of = [&](int n) -> int { return __ldg(p.order + n * (int)gridDim.x + place(n)); };
+    auto unit_of = [&](int n) -> int2 { return n < my_units ? __ldg(p.order + n * (int)gridDim.x + place(n)) : make_int2(0, 0); };
+    auto pairs_of = [&](int2 u) -> int {
+        PairWalk walk;
+        return u.y >= 0 ? u.y : walk.count(p, u.x);
+    };
 
     if (threadIdx.x == 0) {
         mbar_init(bar_kvf, 1); mbar_init(bar_kve, 1);
-        for (int s = 0; s < 2; ++s) { mbar_init(bar_qf + 8 * s, 1); mbar_init(bar_qe + 8 * s, 1); mbar_init(bar_sd + 8 * s, 1); mbar_init(bar_ds + 8 * s, 8); }
-        mbar_init(bar_accf, 1); mbar_init(bar_acce, 8);
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(bar_qf + 8 * s, 1); mbar_init(bar_qe + 8 * s, 1); mbar_init(bar_of + 8 * s, 1); mbar_init(bar_oe + 8 * s, 1);
+            mbar_init(bar_pr + 8 * s, 4); mbar_init(bar_ds + 8 * s, 4);
+        }
+        mbar_init(bar_sd, 2); mbar_init(bar_sd + 8, 2); mbar_init(bar_pd, 1); mbar_init(bar_accf, 1); mbar_init(bar_acce, 8);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
@@ -613,7 +636,7 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         int t = 0, m = 0;                             // pairs; units that have any
         PairWalk walk;
         for (int n = 0; ok && n < my_units; ++n) {
-            walk.open(p, unit_of(n));
+            walk.open(p, unit_of(n).x);
             bool first = true;
             for (int i = walk.pop(p); ok && i >= 0; i = walk.pop(p), ++t) {
                 if (first) {
@@ -630,14 +653,21 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     first = false; ++m;
                 }
                 const int st = t & 1;
+                // dO first: its stage is free half a pair before Q's
+                if (t >= 2 && !(ok = wait_w(bar_oe + 8 * st, (t >> 1) - 1, 90))) break;
+                if (elect_one()) {
+                    mbar_expect_tx(bar_of + 8 * st, C::TILE_BYTES);
+#pragma unroll
+                    for (int s = 0; s < C::SUB; ++s)
+                        tma_load_4d(sDO + st * C::TILE_BYTES + s * C::SUB_BYTES, &tm_do, s * 64, i * C::BLK, walk.bh, 0, bar_of + 8 * st);
+                }
+                __syncwarp();
                 if (t >= 2 && !(ok = wait_w(bar_qe + 8 * st, (t >> 1) - 1, 92))) break;
                 if (elect_one()) {
-                    mbar_expect_tx(bar_qf + 8 * st, 2 * C::TILE_BYTES);
+                    mbar_expect_tx(bar_qf + 8 * st, C::TILE_BYTES);
 #pragma unroll
-                    for (int s = 0; s < C::SUB; ++s) {
+                    for (int s = 0; s < C::SUB; ++s)
                         tma_load_4d(sQ + st * C::TILE_BYTES + s * C::SUB_BYTES, &tm_q, s * 64, i * C::BLK, walk.bh, 0, bar_qf + 8 * st);
-                        tma_load_4d(sDO + st * C::TILE_BYTES + s * C::SUB_BYTES, &tm_do, s * 64, i * C::BLK, walk.bh, 0, bar_qf + 8 * st);
-                    }
                 }
                 __syncwarp();
             }
@@ -648,150 +678,201 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         }
     } else if (warp == C::WARP_MMA) {
         // ================================================================= MMA issuer (warp-uniform, one elected lane issues)
-        constexpr uint32_t IDESC_S = idesc_bf16(64, false);
+        constexpr uint32_t IDESC_S = idesc_bf16(128, false);
         constexpr uint32_t IDESC_ACC = idesc_bf16(D, true);
         constexpr uint32_t TILE_STEP = C::TILE_BYTES >> 4, HALF = 64 * 128 >> 4;    // 64 rows of a tile, in 16-byte units
-        const uint64_t dk0 = smem_desc_sw128(sK, 16, 1024), dv0 = smem_desc_sw128(sV, 16, 1024);
-        const uint64_t dq0 = smem_desc_sw128(sQ, 16, 1024), dd0 = smem_desc_sw128(sDO, 16, 1024);
-        const uint64_t dqm = smem_desc_sw128(sQ, C::SUB_BYTES, 1024), ddm = smem_desc_sw128(sDO, C::SUB_BYTES, 1024);   // as MN-major operands
-        const uint32_t hi_k = (uint32_t)(dk0 >> 32), hi_m = (uint32_t)(dqm >> 32);
+        const uint64_t kd = smem_desc_sw128(sK, 16, 1024), vd = smem_desc_sw128(sV, 16, 1024);
+        const uint64_t qd = smem_desc_sw128(sQ, 16, 1024), od = smem_desc_sw128(sDO, 16, 1024);
+        const uint64_t qm = smem_desc_sw128(sQ, C::SUB_BYTES, 1024), om = smem_desc_sw128(sDO, C::SUB_BYTES, 1024);     // as MN-major operands
+        const uint32_t hi_k = (uint32_t)(kd >> 32), hi_m = (uint32_t)(qm >> 32);
         bool ok = true;
-        // ---- the score products run half a pair ahead, over unit boundaries too: their own walk of the pairs
-        PairWalk ws;
-        int n_s = -1, t_s = 0, h_s = 0, m_s = -1, cur_s = -1, nxt_s = -1;
+        // ---- the scores run one pair ahead, over unit boundaries too: a count of pairs of their own
+        int n_s = -1, t_s = 0, m_s = -1, left_s = 0;  // left_s: pairs of the unit whose scores are still to be issued, the next one included
         bool first_s = false;
-        auto next_pair_s = [&]() {                    // cur_s: the pair to issue (-1: none left); nxt_s: the one after it in the unit
-            cur_s = nxt_s;
-            if (cur_s >= 0) nxt_s = ws.pop(p);
-            while (cur_s < 0 && ++n_s < my_units) {
-                ws.open(p, unit_of(n_s));
-                cur_s = ws.pop(p);
-                if (cur_s >= 0) { nxt_s = ws.pop(p); first_s = true; ++m_s; }
+        int2 unit_s = unit_of(0);
+        auto next_unit_s = [&]() {                    // the next unit that has pairs, if there is one
+            while (left_s == 0 && ++n_s < my_units) {
+                left_s = pairs_of(unit_s);
+                unit_s = unit_of(n_s + 1);
+                if (left_s > 0) { first_s = true; ++m_s; }
             }
         };
-        auto issue_scores = [&]() -> bool {
-            const int st = t_s & 1;
-            if (h_s == 0) {
-                if (first_s && !wait_w(bar_kvf, m_s, 93)) return false;
-                first_s = false;
-                if (!wait_w(bar_qf + 8 * st, t_s >> 1, 94)) return false;
-            }
+        auto issue_s = [&]() -> bool {                // S^T = K Q^T
+            if (first_s && !wait_w(bar_kvf, m_s, 93)) return false;
+            first_s = false;
+            if (!wait_w(bar_qf + 8 * (t_s & 1), t_s >> 1, 94)) return false;
             fence_after_sync();
             if (elect_one()) {
-                mma_ss_tile<D>(tmem + 128 * h_s, (uint32_t)dk0, (uint32_t)dq0 + st * TILE_STEP + h_s * HALF, hi_k, IDESC_S);
-                mma_ss_tile<D>(tmem + 128 * h_s + 64, (uint32_t)dv0, (uint32_t)dd0 + st * TILE_STEP + h_s * HALF, hi_k, IDESC_S);
-                mma_commit(bar_sd + 8 * h_s);
-                if (h_s == 1 && nxt_s < 0) mma_commit(bar_kve);       // K_j and V_j have been read for the last time
+                mma_ss_tile<D>(tmem, (uint32_t)kd, (uint32_t)qd + (t_s & 1) * TILE_STEP, hi_k, IDESC_S);
+                mma_commit(bar_sd + 8 * (t_s & 1));
             }
             __syncwarp();
-            if (h_s == 1) { ++t_s; next_pair_s(); }
-            h_s ^= 1;
             return true;
         };
-        next_pair_s();
-        if (cur_s >= 0) ok = issue_scores();
-        PairWalk wa;
+        auto issue_dp = [&]() -> bool {               // dP^T = V dO^T, and on to the next pair
+            if (!wait_w(bar_of + 8 * (t_s & 1), t_s >> 1, 89)) return false;
+            fence_after_sync();
+            if (elect_one()) {
+                mma_ss_tile<D>(tmem + 128, (uint32_t)vd, (uint32_t)od + (t_s & 1) * TILE_STEP, hi_k, IDESC_S);
+                mma_commit(bar_pd);
+                if (left_s == 1) mma_commit(bar_kve);                 // K_j and V_j have been read for the last time
+            }
+            __syncwarp();
+            ++t_s;
+            if (--left_s == 0) next_unit_s();
+            return true;
+        };
+        next_unit_s();
+        if (left_s > 0) ok = issue_s() && issue_dp();
         int t = 0;
+        int2 unit = unit_of(0);
         for (int n = 0; ok && n < my_units; ++n) {
-            wa.open(p, unit_of(n));
-            int pairs = 0;
-            for (int i = wa.pop(p); ok && i >= 0; i = wa.pop(p), ++t, ++pairs) {
+            const int pairs = pairs_of(unit);
+            unit = unit_of(n + 1);
+            if (pairs == 0) {
+                // no pairs: the read-out of the unit before comes first, or this unit's completion could pass it by
+                if (n >= 1 && !(ok = wait_w(bar_acce, n - 1, 97))) break;
+                if (elect_one()) mma_commit(bar_accf);
+                __syncwarp();
+                continue;
+            }
+            for (int x = 0; ok && x < pairs; ++x, ++t) {
                 const int st = t & 1;
+                // the accumulators of the previous unit have been read out before this unit's first product overwrites them
+                if (x == 0 && n >= 1 && !(ok = wait_w(bar_acce, n - 1, 96))) break;
+                bool more = false;
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    // scores of the next half first -- unless they wait for another unit's K and V
-                    const bool ahead = cur_s >= 0 && !first_s;
-                    if (ahead && !(ok = issue_scores())) break;
-                    if (!(ok = wait_w(bar_ds + 8 * h, t, 95))) break;
-                    // the accumulators of the previous unit have been read out before this unit's first products overwrite them
-                    if (h == 0 && pairs == 0 && n >= 1 && !(ok = wait_w(bar_acce, n - 1, 96))) break;
-                    fence_after_sync();
-                    if (elect_one()) {
-                        mma_ts_half_split(tmem + C::COL_DV, tmem + 128 * h, (uint32_t)ddm + st * TILE_STEP + h * HALF, hi_m, IDESC_ACC, pairs > 0 || h > 0);
-                        mma_ts_half_split(tmem + C::COL_DK, tmem + 128 * h + 64, (uint32_t)dqm + st * TILE_STEP + h * HALF, hi_m, IDESC_ACC, pairs > 0 || h > 0);
-                        if (h == 1) mma_commit(bar_qe + 8 * st);
+                for (int c = 0; c < 2; ++c) {         // dV += P^T dO, scores of the next pair; dK += dS^T Q, dP of the next pair
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        if (!(ok = wait_w((c == 0 ? bar_pr : bar_ds) + 8 * h, t, 95))) break;
+                        fence_after_sync();
+                        if (elect_one()) {
+                            mma_ts_half(tmem + (c == 0 ? C::COL_DV : C::COL_DK), tmem + 128 * c + 64 * h,
+                                        (uint32_t)(c == 0 ? om : qm) + st * TILE_STEP + h * HALF, hi_m, IDESC_ACC, x > 0 || h > 0);
+                            if (h == 1) {
+                                mma_commit((c == 0 ? bar_oe : bar_qe) + 8 * st);      // (the pair's scores completed before P, dS were formed)
+                                if (c == 1 && x == pairs - 1) mma_commit(bar_accf);   // everything of this unit has completed
+                            }
+                        }
+                        __syncwarp();
                     }
-                    __syncwarp();
+                    if (!ok) break;
+                    if (c == 0) more = left_s > 0;
+                    if (more && !(ok = c == 0 ? issue_s() : issue_dp())) break;
                 }
             }
-            if (!ok) break;
-            // (nothing was issued: the read-out of the unit before still comes first, or this unit's completion could pass it by)
-            if (pairs == 0 && n >= 1 && !(ok = wait_w(bar_acce, n - 1, 97))) break;
-            if (elect_one()) mma_commit(bar_accf);    // everything of this unit has completed
-            __syncwarp();
-            // the next unit's first scores, which were not issued ahead (in a unit without pairs they wait for theirs)
-            if (first_s && n_s == n + 1) ok = issue_scores();
+        }
+        if (!ok) {                                    // given up: nothing of this warp's is in flight when tensor memory is freed
+            const long long t0 = clock64();
+            while (clock64() - t0 < 400000) {}
+        }
+    } else if (warp == C::WARP_ROW) {
+        // ================================================================= -lse log2 e and -delta of every pair's queries, a pair ahead
+        bool ok = true;
+        int t = 0;
+        PairWalk walk;
+        for (int n = 0; ok && n < my_units; ++n) {
+            walk.open(p, unit_of(n).x);
+            for (int i = walk.pop(p); i >= 0; i = walk.pop(p), ++t) {
+                float nl[4], nd[4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const int r = i * C::BLK + x * 32 + lane;
+                    const bool in = r < p.Tc;                         // rows past the chunk's end: weight zero
+                    nl[x] = in ? -p.lse[(size_t)walk.bh * p.Tc + r] * 1.4426950408889634f : -INFINITY;
+                    nd[x] = in ? -p.delta[(size_t)walk.bh * p.Tc + r] : 0.f;
+                }
+                // dK of pair t - 2 has left the tensor core, so its values have been read
+                if (t >= 2 && !(ok = wait_w(bar_qe + 8 * (t & 1), (t >> 1) - 1, 87))) break;
+                float* slot = row_vals + (t & 1) * 256;
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    float* at = slot + (x >> 1) * 128 + (x & 1) * 32 + lane;
+                    at[0] = nl[x];
+                    at[64] = nd[x];
+                }
+                __syncwarp();
+                mbar_arrive_if(bar_sd + 8 * (t & 1), lane == 0);
+            }
         }
     } else {
         // ================================================================= softmax warps (rows = keys, columns = queries)
-        const int grp = warp >> 2;                          // query columns [32 grp, 32 grp + 32) of a half
+        const int grp = warp >> 2;                          // the half of every pair's queries this warp turns; then a half of the output columns
         const int row = (warp & 3) * 32 + lane;             // key row of the block
         const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
         const bool lane0 = lane == 0;
         const float2 c2 = make_float2(p.scale_log2, p.scale_log2);
         bool ok = true;
         int t = 0;
-        PairWalk walk;
+        int2 unit = unit_of(0);
         for (int n = 0; ok && n < my_units; ++n) {
-            walk.open(p, unit_of(n));
-            const int bh = walk.bh, k0 = walk.jb * C::BLK;
-            float v_lse = 0.f, v_del = 0.f;                 // threads 0 .. 127: the next pair's values of query row threadIdx.x
-            auto fetch = [&](int i) {
-                const int r = i * C::BLK + (int)threadIdx.x;
-                if (threadIdx.x < C::BLK) {
-                    v_lse = -INFINITY; v_del = 0.f;         // rows past the chunk's end: weight zero
-                    if (r < p.Tc) { v_lse = -p.lse[(size_t)bh * p.Tc + r] * 1.4426950408889634f; v_del = -p.delta[(size_t)bh * p.Tc + r]; }
-                }
-            };
-            int i = walk.pop(p);
-            const bool any = i >= 0;
-            if (any) fetch(i);
-            while (i >= 0) {
-                // (the buffer of pair t - 2: every warp has arrived on that pair's last half, and met the others here since)
-                float* rv = row_vals + (t & 1) * 2 * C::BLK;
-                if (threadIdx.x < C::BLK) { rv[threadIdx.x] = v_lse; rv[C::BLK + threadIdx.x] = v_del; }
-                asm volatile("bar.sync 1, 256;\n" ::: "memory");
-                i = walk.pop(p);
-                if (i >= 0) fetch(i);
-#pragma unroll 1
-                for (int h = 0; h < 2; ++h) {
-                    ok = mbar_wait_warp(bar_sd + 8 * h, t & 1, abort_flag, p.dev_status, 98);
-                    if (!ok) break;
-                    fence_after_sync();
-                    const uint32_t tS = lane_base + 128 * h + grp * 32, tP = tS + 64;
-                    uint32_t s[32], dp[32], pk[16], dk_[16];
-                    tmem_ld32(tS, s);
-                    tmem_ld32(tP, dp);
-                    tmem_wait_ld();
-                    const float4* nl = reinterpret_cast<const float4*>(rv + h * 64 + grp * 32);
-                    const float4* nd = reinterpret_cast<const float4*>(rv + C::BLK + h * 64 + grp * 32);
-#pragma unroll
-                    for (int e0 = 0; e0 < 32; e0 += 8) {
-                        float2 x[4], g[4];
-#pragma unroll
-                        for (int v = 0; v < 2; ++v) {
-                            const int e = e0 + 4 * v;
-                            const float4 l4 = nl[e >> 2], d4 = nd[e >> 2];
-                            x[2 * v] = ffma2(make_float2(__uint_as_float(s[e]), __uint_as_float(s[e + 1])), c2, make_float2(l4.x, l4.y));
-                            x[2 * v + 1] = ffma2(make_float2(__uint_as_float(s[e + 2]), __uint_as_float(s[e + 3])), c2, make_float2(l4.z, l4.w));
-                            g[2 * v] = fadd2(make_float2(__uint_as_float(dp[e]), __uint_as_float(dp[e + 1])), make_float2(d4.x, d4.y));
-                            g[2 * v + 1] = fadd2(make_float2(__uint_as_float(dp[e + 2]), __uint_as_float(dp[e + 3])), make_float2(d4.z, d4.w));
-                        }
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) x[v] = make_float2(fast_exp2(x[v].x), fast_exp2(x[v].y));
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) {
-                            pk[(e0 >> 1) + v] = pack_bf16(x[v].x, x[v].y);
-                            dk_[(e0 >> 1) + v] = pack_bf16(x[v].x * g[v].x, x[v].y * g[v].y);
-                        }
-                    }
-                    tmem_st16(tS, pk);
-                    tmem_st16(tP, dk_);
-                    tmem_wait_st();
-                    fence_before_sync();
-                    mbar_arrive_if(bar_ds + 8 * h, lane0);
-                }
+            const int pairs = pairs_of(unit), bh = unit.x / p.n_b, k0 = (unit.x - bh * p.n_b) * C::BLK;
+            const bool any = pairs > 0;
+            unit = unit_of(n + 1);
+            for (int x = 0; x < pairs; ++x) {
+                const float* rv = row_vals + ((t & 1) * 2 + grp) * 128;
+                // ---- P = exp2(S c - lse log2 e), kept in registers for dS
+                ok = mbar_wait_warp(bar_sd + 8 * (t & 1), (t >> 1) & 1, abort_flag, p.dev_status, 98);
                 if (!ok) break;
+                fence_after_sync();
+                const uint32_t tS = lane_base + 64 * grp, tP = tS + 128;
+                float2 pe[32];
+                {
+                    uint32_t s[2][32];
+                    tmem_ld32(tS, s[0]);
+                    tmem_ld32(tS + 32, s[1]);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        const float4* nl = reinterpret_cast<const float4*>(rv + c * 32);
+                        uint32_t pk[16];
+#pragma unroll
+                        for (int e = 0; e < 32; e += 4) {
+                            const float4 l4 = nl[e >> 2];
+                            float2& x0 = pe[16 * c + e / 2];
+                            float2& x1 = pe[16 * c + e / 2 + 1];
+                            x0 = ffma2(make_float2(__uint_as_float(s[c][e]), __uint_as_float(s[c][e + 1])), c2, make_float2(l4.x, l4.y));
+                            x1 = ffma2(make_float2(__uint_as_float(s[c][e + 2]), __uint_as_float(s[c][e + 3])), c2, make_float2(l4.z, l4.w));
+                            x0 = make_float2(fast_exp2(x0.x), fast_exp2(x0.y));
+                            x1 = make_float2(fast_exp2(x1.x), fast_exp2(x1.y));
+                            pk[e / 2] = pack_bf16(x0.x, x0.y);
+                            pk[e / 2 + 1] = pack_bf16(x1.x, x1.y);
+                        }
+                        tmem_st16(tS + 16 * c, pk);
+                    }
+                }
+                tmem_wait_st();
+                fence_before_sync();
+                mbar_arrive_if(bar_pr + 8 * grp, lane0);
+                // ---- dS = P (dP - delta)
+                ok = mbar_wait_warp(bar_pd, t & 1, abort_flag, p.dev_status, 88);
+                if (!ok) break;
+                fence_after_sync();
+                {
+                    uint32_t dp[2][32];
+                    tmem_ld32(tP, dp[0]);
+                    tmem_ld32(tP + 32, dp[1]);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        const float4* nd = reinterpret_cast<const float4*>(rv + 64 + c * 32);
+                        uint32_t dk_[16];
+#pragma unroll
+                        for (int e = 0; e < 32; e += 4) {
+                            const float4 d4 = nd[e >> 2];
+                            const float2 g0 = fadd2(make_float2(__uint_as_float(dp[c][e]), __uint_as_float(dp[c][e + 1])), make_float2(d4.x, d4.y));
+                            const float2 g1 = fadd2(make_float2(__uint_as_float(dp[c][e + 2]), __uint_as_float(dp[c][e + 3])), make_float2(d4.z, d4.w));
+                            const float2 x0 = pe[16 * c + e / 2], x1 = pe[16 * c + e / 2 + 1];
+                            dk_[e / 2] = pack_bf16(x0.x * g0.x, x0.y * g0.y);
+                            dk_[e / 2 + 1] = pack_bf16(x1.x * g1.x, x1.y * g1.y);
+                        }
+                        tmem_st16(tP + 16 * c, dk_);
+                    }
+                }
+                tmem_wait_st();
+                fence_before_sync();
+                mbar_arrive_if(bar_ds + 8 * grp, lane0);
                 ++t;
             }
             if (!ok) break;

@@ -186,29 +186,6 @@ __device__ __forceinline__ void mma_ts_kmajor(uint32_t d_tmem, uint32_t a_tmem, 
     }
 }
 #undef HF_TK_STEP
-// The same product with the A operand in two pieces: keys 0..63 at a_tmem (32 columns), keys 64..127 at a_tmem_hi.
-#define HF_TS2_STEP(KS, AOP, AOFF, PRED)                                                            \
-    "add.u32 a, " AOP ", " #AOFF " * 8;\n add.u32 b, %2, " #KS " * 128;\n mov.b64 db, {b, %3};\n" \
-    "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], db, %4, " PRED ";\n"
-__device__ __forceinline__ void mma_ts_tile_split(uint32_t d_tmem, uint32_t a_tmem, uint32_t a_tmem_hi, uint32_t b_lo, uint32_t b_hi,
-                                                  uint32_t idesc, bool accumulate_first) {
-    asm volatile("{\n .reg .pred pt, p0;\n .reg .b64 db;\n .reg .b32 a, b;\n"
-                 "setp.eq.u32 pt, %0, %0;\n setp.ne.b32 p0, %5, 0;\n"
-                 HF_TS2_STEP(0, "%1", 0, "p0") HF_TS2_STEP(1, "%1", 1, "pt") HF_TS2_STEP(2, "%1", 2, "pt") HF_TS2_STEP(3, "%1", 3, "pt")
-                 HF_TS2_STEP(4, "%6", 0, "pt") HF_TS2_STEP(5, "%6", 1, "pt") HF_TS2_STEP(6, "%6", 2, "pt") HF_TS2_STEP(7, "%6", 3, "pt")
-                 "}\n" ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"((uint32_t)accumulate_first), "r"(a_tmem_hi)
-                 : "memory");
-}
-// ... over 64 keys: keys 0..31 at a_tmem (16 columns), keys 32..63 at a_tmem + 32.
-__device__ __forceinline__ void mma_ts_half_split(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi, uint32_t idesc,
-                                                  bool accumulate_first) {
-    asm volatile("{\n .reg .pred pt, p0;\n .reg .b64 db;\n .reg .b32 a, b;\n"
-                 "setp.eq.u32 pt, %0, %0;\n setp.ne.b32 p0, %5, 0;\n"
-                 HF_TS2_STEP(0, "%1", 0, "p0") HF_TS2_STEP(1, "%1", 1, "pt") HF_TS2_STEP(2, "%6", 0, "pt") HF_TS2_STEP(3, "%6", 1, "pt")
-                 "}\n" ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"((uint32_t)accumulate_first), "r"(a_tmem + 32)
-                 : "memory");
-}
-#undef HF_TS2_STEP
 #define HF_TG_STEP(KS, AOFF, PRED)                                                                 \
     "add.u32 a, %1, " #AOFF ";\n add.u32 b, %2, " #KS " * 128;\n mov.b64 db, {b, %3};\n"         \
     "tcgen05.mma.cta_group::1.kind::f16 [%0], [a], db, %4, " PRED ";\n"

@@ -59,3 +59,32 @@ def test_gradients_at_tile_edges(d, tpf, wf, topk, heads, batch):
             assert not got[1][bi, h, jb * 128:(jb + 1) * 128].any() and not got[2][bi, h, jb * 128:(jb + 1) * 128].any()
     finally:
         gpu.close()
+
+
+def test_more_units_than_are_put_in_order():
+    """4 200 key blocks of the chunk: beyond the sort's capacity, each warp counts a unit's pairs itself.  A head's gradients do
+    not depend on how many others there are, so they equal, bit for bit, those of a context with six heads."""
+    import torch
+    rng = torch.Generator(device="cuda").manual_seed(5)
+    full = [torch.randn((2, 350, 700, 64), generator=rng, device="cuda").to(torch.bfloat16) for _ in range(4)]
+
+    def gradients(batch, heads):
+        w = gen.Workload("bwd_many", batch=batch, heads=heads, head_dim=64, tokens_per_frame=700, chunk_frames=1, window_frames=1, block=128,
+                         topk=2, keep_permille=0, seed=402)
+        gpu = hz.GpuStream(w)
+        try:
+            q, k, v, g = [x[:batch, :heads].contiguous() for x in full]
+            gpu.append(k, v)
+            gpu.select(q, k)
+            o, lse = torch.empty_like(q), torch.empty(q.shape[:3], dtype=torch.float32, device="cuda")
+            gpu.ctx.hf_sparse_swa(0, q, k, v, o, lse=lse)
+            dk, dv = torch.full_like(q, 7.0), torch.full_like(q, 7.0)
+            gpu.ctx.hf_sparse_swa_backward_dkv(0, q, k, v, o, lse, g, dk, dv)
+            torch.cuda.synchronize()
+            assert gpu.ctx.hf_get_device_status() == (0, 0)
+            return dk[:1, :6].cpu(), dv[:1, :6].cpu()
+        finally:
+            gpu.close()
+
+    for a, b in zip(gradients(2, 350), gradients(1, 6)):
+        assert torch.equal(a, b) and float(b.float().abs().max()) > 0
