@@ -425,13 +425,16 @@ template <int D>
 hf_status launch_readout_bwd(hf_ctx* c, LayerState& L, const bf16* q, const bf16* d_o, bf16* dq, cudaStream_t st) {
     typedef ReadoutBwd<D> R;
     HF_CUDA(cudaFuncSetAttribute(k_readout_bwd_dq<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, R::SMEM_BYTES));
-    CUtensorMap tg;
+    CUtensorMap tg, tq, tdq;
     HF_TRY(make_map(c, &tg, d_o, 1));
+    HF_TRY(make_map(c, &tq, q, 1));
+    HF_TRY(make_map_ex(c, &tdq, dq, c->Tc, 1, 64, 32, true));
     ReadoutBwdParams p;
-    p.q = q; p.z = L.z; p.dq = dq; p.Tc = c->Tc; p.Tm = (c->Tc + R::ROWS - 1) / R::ROWS; p.n_units = p.Tm * c->BH;
+    p.z = L.z; p.Tc = c->Tc; p.Tm = (c->Tc + R::ROWS - 1) / R::ROWS; p.n_units = p.Tm * c->BH;
     p.eps = c->cfg.eps; p.dev_status = c->dev_status;
     const int grid = p.n_units < c->sm_count ? p.n_units : c->sm_count;
-    k_readout_bwd_dq<D><<<grid, R::THREADS, R::SMEM_BYTES, st>>>(tg, L.tm_sfhi, L.tm_sflo, p);
+    PdlLaunch pl(dim3(grid), dim3(R::THREADS), R::SMEM_BYTES, st, true);
+    HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_readout_bwd_dq<D>, tg, tq, L.tm_sfhi, L.tm_sflo, tdq, p));
     return post_launch(c, "k_readout_bwd_dq");
 }
 
