@@ -401,11 +401,13 @@ hf_status launch_readout(hf_ctx* c, LayerState& L, const bf16* q, bf16* out_bf16
     p.cos_q = c->rope_q[0]; p.sin_q = c->rope_q[1];
     p.z = L.z; p.bias = (L.has_bias && !full) ? L.bias : nullptr; p.heads = c->cfg.heads; p.Tc = c->Tc;
     p.Tm = (c->Tc + R::ROWS - 1) / R::ROWS; p.n_units = p.Tm * c->BH; p.eps = c->cfg.eps;
-    p.out_bf16 = full ? c->x_hi : out_bf16; p.out_f32 = full ? nullptr : out_f32; p.out_lo = full ? c->x_lo : nullptr;
+    p.out_bf16 = full ? c->x_hi : nullptr; p.out_f32 = full ? nullptr : out_f32; p.out_lo = full ? c->x_lo : nullptr;
     p.dev_status = c->dev_status;
     const int grid = p.n_units < c->sm_count ? p.n_units : c->sm_count;
-    if (c->has_rope_q) k_readout_tc5<D, true><<<grid, R::THREADS, R::SMEM_BYTES, st>>>(tq, L.tm_sfhi, L.tm_sflo, p);
-    else k_readout_tc5<D, false><<<grid, R::THREADS, R::SMEM_BYTES, st>>>(tq, L.tm_sfhi, L.tm_sflo, p);
+    CUtensorMap tout = tq;           // a bf16 result: one warp's 32 rows x 64 columns per store
+    if (!full && out_f32 == nullptr) HF_TRY(make_map_ex(c, &tout, out_bf16, c->Tc, 1, 64, 32, true));
+    PdlLaunch pr(dim3(grid), dim3(R::THREADS), R::SMEM_BYTES, st, true);
+    HF_CUDA(cudaLaunchKernelEx(&pr.cfg, c->has_rope_q ? k_readout_tc5<D, true> : k_readout_tc5<D, false>, tq, L.tm_sfhi, L.tm_sflo, tout, p));
     HF_TRY(post_launch(c, "k_readout_tc5"));
     if (!full) return HF_OK;
     typedef MergeFull<D> M;

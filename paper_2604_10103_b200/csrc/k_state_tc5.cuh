@@ -280,20 +280,24 @@ k_absorb_tc5(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ C
 // ------------------------------------------------------------------------------------------------------------
 // Read-out.  Unit = (batch*head, tile of 128 query rows).  A = phi(Q): M = query row (lane), K = key feature.
 // B = S' [a][c] (N = c contiguous, MN-major), hi and lo halves.  D = A_hi S'_hi + A_lo S'_hi + A_hi S'_lo.
-// A thread block takes a contiguous run of units, so that S' is fetched once per (batch, head) it touches
-// ("epoch"), into one of two buffers.
+// A thread block takes a contiguous run of units, so that S' is fetched once per (batch, head) it touches ("epoch").
+// A bf16 result takes q's place in its tile and leaves by bulk tensor store (rows past the chunk's end are clipped by the map).
+// Memory-bound by its bytes (28.8 MB at 12 heads x 4 680 x 128 = 4.3 us) but short: three units per thread block, so the latency
+// of start-up and of each unit's chain weigh most.  Seven chunks absorbed and read: 76.6 us when z and bias came through
+// registers and a barrier per unit and a lane stored a row, 70.6 like this.
 // ------------------------------------------------------------------------------------------------------------
 template <int D>
 struct ReadoutTc5 {
     static constexpr int ROWS = 128;
-    static constexpr int NST = 2;                        // Q stages; S' {hi, lo} buffers likewise two
+    static constexpr int QST = 3;                        // Q stages (held until the result has left); accumulators and A operands: two
     static constexpr int SUB = D / 64;
     static constexpr int QSUB_BYTES = ROWS * 128, Q_BYTES = SUB * QSUB_BYTES;
     static constexpr int SSUB_BYTES = D * 128, S_BYTES = SUB * SSUB_BYTES;
-    static constexpr int OFF_Q = 0, OFF_S = NST * Q_BYTES;   // S' buffer e at OFF_S + e * 2 * S_BYTES: hi then lo
-    static constexpr int OFF_VEC = OFF_S + 2 * 2 * S_BYTES;  // per stage: z [D] floats, bias [D] floats
-    static constexpr int OFF_DEN = OFF_VEC + NST * 2 * D * 4;   // per stage: denominator partials [2][128] floats
-    static constexpr int OFF_BAR = OFF_DEN + NST * 2 * ROWS * 4;
+    static constexpr int OFF_Q = 0, OFF_S = QST * Q_BYTES;   // S': hi then lo
+    static constexpr int OFF_Z = OFF_S + 2 * S_BYTES;        // per Q stage: z [D] floats
+    static constexpr int OFF_BIAS = OFF_Z + QST * D * 4;     // per Q stage: bias [D] bf16 (zeros without one)
+    static constexpr int OFF_DEN = OFF_BIAS + QST * D * 2;   // per accumulator: denominator partials [2][128] floats
+    static constexpr int OFF_BAR = OFF_DEN + 2 * 2 * ROWS * 4;
     static constexpr int SMEM_BYTES = OFF_BAR + 256 + 1024;
     static constexpr int THREADS = 320;                  // warps 0-7: phi / epilogue (two per TMEM lane quadrant), warp 8: TMA, warp 9: MMA
     static constexpr int WARP_TMA = 8, WARP_MMA = 9;
@@ -307,26 +311,28 @@ struct ReadoutTc5Params {
     const bf16* bias;         // [H, D] or nullptr
     int heads, Tc, Tm, n_units;
     float eps;
-    bf16* out_bf16;           // exactly one of out_bf16 / out_f32 is non-null: [B*H, T_c, D]
+    // the result, [B*H, T_c, D]: fp32 here, or bf16 here with its bf16 residual (value = out_bf16 + out_lo to ~16 bits), or
+    // neither: bf16 through tm_out
     float* out_f32;
-    bf16* out_lo;             // with out_bf16: the bf16 residual of the result (value = out_bf16 + out_lo to ~16 bits), or nullptr
+    bf16 *out_bf16, *out_lo;
     int* dev_status;
 };
 
 // CTA c processes units [c * upc, (c + 1) * upc), upc = ceil(n_units / gridDim.x).  tm_q: [D, T_c, B*H, 1] box {64, 128};
-// tm_sh, tm_sl: [D, D, B*H, 1] box {64, D}; all 128B swizzle.
+// tm_sh, tm_sl: [D, D, B*H, 1] box {64, D}; tm_out: as tm_q, box {64, 32}; all 128B swizzle.
 template <int D, bool ROPE>
 __global__ void __launch_bounds__(ReadoutTc5<D>::THREADS, 1)
 k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_sh,
-              const __grid_constant__ CUtensorMap tm_sl, const ReadoutTc5Params p) {
+              const __grid_constant__ CUtensorMap tm_sl, const __grid_constant__ CUtensorMap tm_out,
+              const __grid_constant__ ReadoutTc5Params p) {
     using namespace tc5;
     typedef ReadoutTc5<D> C;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t s_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* s_gen = smem_raw + (s_base - smem_u32(smem_raw));
     const uint32_t bar0 = s_base + C::OFF_BAR;
-    const uint32_t bar_full = bar0, bar_qfree = bar0 + 16, bar_sfree = bar0 + 32, bar_afull = bar0 + 48, bar_afree = bar0 + 64,
-                   bar_dfull = bar0 + 80, bar_dfree = bar0 + 96, bar_vec = bar0 + 112, bar_sfull = bar0 + 128;
+    const uint32_t bar_full = bar0, bar_qfree = bar0 + 24, bar_sfull = bar0 + 48, bar_sfree = bar0 + 56, bar_afull = bar0 + 64,
+                   bar_afree = bar0 + 80, bar_dfull = bar0 + 96, bar_dfree = bar0 + 112;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_gen + C::OFF_BAR + 144);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(s_gen + C::OFF_BAR + 148);
 
@@ -336,11 +342,12 @@ k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     const int my_units = min(upc, p.n_units - u0);
 
     if (threadIdx.x == 0) {
+        for (int s = 0; s < C::QST; ++s) { mbar_init(bar_full + 8 * s, 1); mbar_init(bar_qfree + 8 * s, 8); }
         for (int s = 0; s < 2; ++s) {
-            mbar_init(bar_full + 8 * s, 1); mbar_init(bar_qfree + 8 * s, 256); mbar_init(bar_sfree + 8 * s, 1);
             mbar_init(bar_afull + 8 * s, 256); mbar_init(bar_afree + 8 * s, 1); mbar_init(bar_dfull + 8 * s, 1);
-            mbar_init(bar_dfree + 8 * s, 256); mbar_init(bar_vec + 8 * s, 256); mbar_init(bar_sfull + 8 * s, 1);
+            mbar_init(bar_dfree + 8 * s, 256);
         }
+        mbar_init(bar_sfull, 1); mbar_init(bar_sfree, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
@@ -348,38 +355,42 @@ k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS);
         tmem_relinquish();
     }
+    if (p.bias == nullptr)
+        for (int e = threadIdx.x; e < C::QST * D / 2; e += C::THREADS) reinterpret_cast<uint32_t*>(s_gen + C::OFF_BIAS)[e] = 0u;
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    pdl_wait();
+    pdl_trigger();
 
     if (warp == C::WARP_TMA) {
         // ================================================================= TMA producer
         if (lane == 0) {
             bool ok = true;
             int epoch = -1, bh_prev = -1;
-            for (int n = 0; ok && n < my_units; ++n) {
+            for (int n = 0, st = 0, ph = 1; ok && n < my_units; ++n) {
                 const int u = u0 + n;
                 const int bh = u / p.Tm, i = u - bh * p.Tm;
-                const int s = n & 1;
-                if (bh != bh_prev) {                 // new (batch, head): its folded state, hi and lo halves
-                    bh_prev = bh; ++epoch;
-                    const int e = epoch & 1;
-                    if (epoch >= 2 && !(ok = mbar_wait<true>(bar_sfree + 8 * e, ((epoch >> 1) & 1) ^ 1, abort_flag, p.dev_status, 42))) break;
-                    const uint32_t sb = s_base + C::OFF_S + e * 2 * C::S_BYTES;
-                    mbar_expect_tx(bar_sfull + 8 * e, 2 * C::S_BYTES);
-#pragma unroll
-                    for (int v = 0; v < C::SUB; ++v) {
-                        tma_load_4d(sb + v * C::SSUB_BYTES, &tm_sh, v * 64, 0, bh, 0, bar_sfull + 8 * e);
-                        tma_load_4d(sb + C::S_BYTES + v * C::SSUB_BYTES, &tm_sl, v * 64, 0, bh, 0, bar_sfull + 8 * e);
-                    }
-                }
-                if (n >= 2 && !(ok = mbar_wait<true>(bar_qfree + 8 * s, ((n >> 1) & 1) ^ 1, abort_flag, p.dev_status, 41))) break;
-                const uint32_t st = s_base + C::OFF_Q + s * C::Q_BYTES;
-                mbar_expect_tx(bar_full + 8 * s, C::Q_BYTES);
+                if (n >= C::QST && !(ok = mbar_wait<true>(bar_qfree + 8 * st, ph, abort_flag, p.dev_status, 41))) break;
+                const uint32_t full = bar_full + 8 * st;
+                mbar_expect_tx(full, C::Q_BYTES + D * 4 + (p.bias ? D * 2 : 0));
 #pragma unroll
                 for (int v = 0; v < C::SUB; ++v)
-                    tma_load_4d(st + v * C::QSUB_BYTES, &tm_q, v * 64, i * C::ROWS, bh, 0, bar_full + 8 * s);
+                    tma_load_4d(s_base + C::OFF_Q + st * C::Q_BYTES + v * C::QSUB_BYTES, &tm_q, v * 64, i * C::ROWS, bh, 0, full);
+                bulk_load(s_base + C::OFF_Z + st * D * 4, p.z + (size_t)bh * D, D * 4, full);
+                if (p.bias) bulk_load(s_base + C::OFF_BIAS + st * D * 2, p.bias + (size_t)(bh % p.heads) * D, D * 2, full);
+                if (++st == C::QST) { st = 0; ph ^= 1; }
+                if (bh != bh_prev) {                 // new (batch, head): its folded state, hi and lo halves
+                    bh_prev = bh; ++epoch;
+                    if (epoch >= 1 && !(ok = mbar_wait<true>(bar_sfree, (epoch - 1) & 1, abort_flag, p.dev_status, 42))) break;
+                    mbar_expect_tx(bar_sfull, 2 * C::S_BYTES);
+#pragma unroll
+                    for (int v = 0; v < C::SUB; ++v) {
+                        tma_load_4d(s_base + C::OFF_S + v * C::SSUB_BYTES, &tm_sh, v * 64, 0, bh, 0, bar_sfull);
+                        tma_load_4d(s_base + C::OFF_S + C::S_BYTES + v * C::SSUB_BYTES, &tm_sl, v * 64, 0, bh, 0, bar_sfull);
+                    }
+                }
             }
             if (!ok) {
                 const long long t0 = clock64();
@@ -397,7 +408,7 @@ k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             const int bh = (u0 + n) / p.Tm;
             if (bh != bh_prev) {
                 bh_prev = bh; ++epoch;
-                if (!(ok = __all_sync(0xffffffffu, mbar_wait<true>(bar_sfull + 8 * (epoch & 1), (epoch >> 1) & 1, abort_flag, p.dev_status, 45)))) break;
+                if (!(ok = __all_sync(0xffffffffu, mbar_wait<true>(bar_sfull, epoch & 1, abort_flag, p.dev_status, 45)))) break;
             }
             const bool last_of_epoch = (n + 1 == my_units) || ((u0 + n + 1) / p.Tm != bh);
             if (!(ok = __all_sync(0xffffffffu, mbar_wait<true>(bar_afull + 8 * s, par, abort_flag, p.dev_status, 43)))) break;
@@ -405,7 +416,7 @@ k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             fence_after_sync();
             if (elect_one()) {
                 const uint32_t tD = tmem + s * D, tA = tmem + 2 * D + s * D;
-                const uint32_t sb = s_base + C::OFF_S + (epoch & 1) * 2 * C::S_BYTES;
+                const uint32_t sb = s_base + C::OFF_S;
                 const uint64_t dsh = smem_desc_sw128(sb, C::SSUB_BYTES, 1024);
                 const uint64_t dsl = smem_desc_sw128(sb + C::S_BYTES, C::SSUB_BYTES, 1024);
 #pragma unroll
@@ -417,7 +428,7 @@ k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 }
                 mma_commit(bar_dfull + 8 * s);
                 mma_commit(bar_afree + 8 * s);
-                if (last_of_epoch) mma_commit(bar_sfree + 8 * (epoch & 1));
+                if (last_of_epoch) mma_commit(bar_sfree);
             }
             __syncwarp();
         }
@@ -430,6 +441,7 @@ k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         const int row = (warp & 3) * 32 + lane;                 // query row of the tile = TMEM lane
         const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
         constexpr int PASSES = D / 64;                          // 32-feature (and 32-column) passes per thread
+        const bool lane0 = lane == 0, staged = p.out_f32 == nullptr && p.out_bf16 == nullptr, storer = C::SUB == 2 || half == 0;
         bool ok = true;
         auto convert = [&](int n) -> bool {                     // A operand of unit n; denominator partial of the half
             const int u = u0 + n;
@@ -437,23 +449,17 @@ k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             const int s = n & 1;
             const uint32_t par = (n >> 1) & 1;
             const int r_tab = min((u - bh * p.Tm) * C::ROWS + row, p.Tc - 1);     // row of the rotation tables
-            // z and bias of the unit's head, staged by these threads once every thread has left the epilogue that read
-            // the stage's buffers last (two units ago)
-            float* vec = reinterpret_cast<float*>(s_gen + C::OFF_VEC + s * 2 * D * 4);
+            const int qs = n % C::QST;
+            const float* z_s = reinterpret_cast<const float*>(s_gen + C::OFF_Z + qs * D * 4);
             float* den_x = reinterpret_cast<float*>(s_gen + C::OFF_DEN + s * 2 * C::ROWS * 4);
+            // (every thread has left the epilogue that read the denominators of two units ago)
             if (n >= 2 && !__all_sync(0xffffffffu, mbar_wait(bar_dfree + 8 * s, par ^ 1u, abort_flag, p.dev_status, 50))) return false;
-            if (threadIdx.x < D) {
-                vec[threadIdx.x] = p.z[(size_t)bh * D + threadIdx.x];
-                vec[D + threadIdx.x] = p.bias ? __bfloat162float(p.bias[(size_t)(bh % p.heads) * D + threadIdx.x]) : 0.f;
-            }
-            mbar_arrive(bar_vec + 8 * s);
-            if (!__all_sync(0xffffffffu, mbar_wait(bar_vec + 8 * s, par, abort_flag, p.dev_status, 46))) return false;
-            if (!__all_sync(0xffffffffu, mbar_wait(bar_full + 8 * s, par, abort_flag, p.dev_status, 47))) return false;
+            if (!__all_sync(0xffffffffu, mbar_wait(bar_full + 8 * qs, (n / C::QST) & 1, abort_flag, p.dev_status, 47))) return false;
             if (n >= 2) {
                 if (!__all_sync(0xffffffffu, mbar_wait(bar_afree + 8 * s, par ^ 1u, abort_flag, p.dev_status, 48))) return false;
                 fence_after_sync();
             }
-            const uint8_t* qt = s_gen + C::OFF_Q + s * C::Q_BYTES + row * 128;
+            const uint8_t* qt = s_gen + C::OFF_Q + qs * C::Q_BYTES + row * 128;
             const uint32_t tA = lane_base + 2 * D + s * D;
             float dsum = 0.f;
 #pragma unroll 1
@@ -478,7 +484,7 @@ k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                         const float2 x = unpack_bf16(ws[e]);
                         float f0 = phi_elu1(x.x), f1 = phi_elu1(x.y);
                         const int feat = chunk * 8 + 2 * e;
-                        dsum = fmaf(f0, vec[feat], fmaf(f1, vec[feat + 1], dsum));     // denominator: unrotated
+                        dsum = fmaf(f0, z_s[feat], fmaf(f1, z_s[feat + 1], dsum));     // denominator: unrotated
                         if (ROPE) {
                             const float r0 = fmaf(-f1, sn[e], f0 * cs[e]), r1 = fmaf(f0, sn[e], f1 * cs[e]);
                             f0 = r0; f1 = r1;
@@ -496,7 +502,6 @@ k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             tmem_wait_st();
             fence_before_sync();
             mbar_arrive(bar_afull + 8 * s);
-            mbar_arrive(bar_qfree + 8 * s);
             return true;
         };
         auto epilogue = [&](int n) -> bool {
@@ -507,7 +512,13 @@ k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             // published its denominator partial), so the partials of both halves are visible here
             if (!__all_sync(0xffffffffu, mbar_wait(bar_dfull + 8 * s, (n >> 1) & 1, abort_flag, p.dev_status, 49))) return false;
             fence_after_sync();
-            const float* vec = reinterpret_cast<const float*>(s_gen + C::OFF_VEC + s * 2 * D * 4);
+            const int qs = n % C::QST;
+            const uint32_t* bias_s = reinterpret_cast<const uint32_t*>(s_gen + C::OFF_BIAS + qs * D * 2);
+            if (staged && n >= 1 && storer && lane0) {          // the result of the unit before has left its tile
+                bulk_wait_read();
+                mbar_arrive(bar_qfree + 8 * ((n - 1) % C::QST));
+            }
+            uint8_t* ot = s_gen + C::OFF_Q + qs * C::Q_BYTES + row * 128;
             const float* den_x = reinterpret_cast<const float*>(s_gen + C::OFF_DEN + s * 2 * C::ROWS * 4);
             const float inv = 1.f / (den_x[row] + den_x[C::ROWS + row] + p.eps);
             const int r_glob = i * C::ROWS + row;
@@ -519,10 +530,22 @@ k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 uint32_t r[32];
                 tmem_ld32(lane_base + s * D + col, r);
                 tmem_wait_ld();
-                if (valid) {
-                    float x[32];
+                float x[32];
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) x[e] = fmaf(__uint_as_float(r[e]), inv, vec[D + col + e]);
+                for (int e = 0; e < 32; e += 2) {
+                    const float2 b2 = unpack_bf16(bias_s[(col + e) >> 1]);
+                    x[e] = fmaf(__uint_as_float(r[e]), inv, b2.x);
+                    x[e + 1] = fmaf(__uint_as_float(r[e + 1]), inv, b2.y);
+                }
+                if (staged) {
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        const int chunk = (col >> 3) + v;
+                        *reinterpret_cast<uint4*>(ot + (chunk >> 3) * C::QSUB_BYTES + (((chunk & 7) ^ (row & 7)) << 4)) =
+                            make_uint4(pack_bf16(x[8 * v], x[8 * v + 1]), pack_bf16(x[8 * v + 2], x[8 * v + 3]),
+                                       pack_bf16(x[8 * v + 4], x[8 * v + 5]), pack_bf16(x[8 * v + 6], x[8 * v + 7]));
+                    }
+                } else if (valid) {
                     if (p.out_f32) {
                         float4* dst = reinterpret_cast<float4*>(p.out_f32 + g + col);
 #pragma unroll
@@ -534,22 +557,33 @@ k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                         for (int e = 0; e < 16; ++e) hp[e] = pack_bf16(x[2 * e], x[2 * e + 1]);
 #pragma unroll
                         for (int v = 0; v < 4; ++v) dst[v] = make_uint4(hp[4 * v], hp[4 * v + 1], hp[4 * v + 2], hp[4 * v + 3]);
-                        if (p.out_lo) {
-                            uint4* dlo = reinterpret_cast<uint4*>(p.out_lo + g + col);
-                            uint32_t lp[16];
+                        uint4* dlo = reinterpret_cast<uint4*>(p.out_lo + g + col);
+                        uint32_t lp[16];
 #pragma unroll
-                            for (int e = 0; e < 16; ++e) {
-                                const float2 hf = unpack_bf16(hp[e]);
-                                lp[e] = pack_bf16(x[2 * e] - hf.x, x[2 * e + 1] - hf.y);
-                            }
-#pragma unroll
-                            for (int v = 0; v < 4; ++v) dlo[v] = make_uint4(lp[4 * v], lp[4 * v + 1], lp[4 * v + 2], lp[4 * v + 3]);
+                        for (int e = 0; e < 16; ++e) {
+                            const float2 hf = unpack_bf16(hp[e]);
+                            lp[e] = pack_bf16(x[2 * e] - hf.x, x[2 * e + 1] - hf.y);
                         }
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) dlo[v] = make_uint4(lp[4 * v], lp[4 * v + 1], lp[4 * v + 2], lp[4 * v + 3]);
                     }
                 }
             }
             fence_before_sync();
             mbar_arrive(bar_dfree + 8 * s);
+            if (staged) fence_proxy_async();
+            if (C::SUB == 2 || !staged) __syncwarp();
+            else asm volatile("bar.sync %0, 64;\n" ::"r"(1 + (warp & 3)) : "memory");     // 64 columns are both halves' here
+            if (lane0) {
+                if (staged && storer) {
+                    if (i * C::ROWS + (warp & 3) * 32 < p.Tc)
+                        tma_store_4d(&tm_out, s_base + C::OFF_Q + qs * C::Q_BYTES + (C::SUB == 2 ? half * C::QSUB_BYTES : 0) + (warp & 3) * 32 * 128,
+                                     C::SUB == 2 ? half * 64 : 0, i * C::ROWS + (warp & 3) * 32, bh, 0);
+                    bulk_commit();
+                } else {
+                    mbar_arrive(bar_qfree + 8 * qs);
+                }
+            }
             return true;
         };
         if (my_units > 0) ok = convert(0);
@@ -557,6 +591,7 @@ k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             if (n + 1 < my_units && !(ok = convert(n + 1))) break;
             ok = epilogue(n);
         }
+        if (lane0) bulk_wait_all();
     }
     fence_before_sync();
     __syncthreads();

@@ -94,7 +94,7 @@ def test_more_units_than_are_put_in_order():
     (128, 2330, 24, 1),            # four tiles per thread block: every buffer used again; heads change within a range; 26-row last tile
     (64, 1025, 30, 2),             # the same at head_dim 64, one-row last tile
 ])
-def test_read_out_gradient_at_tile_edges(d, tpf, heads, batch):
+def test_read_out_and_its_gradient_at_tile_edges(d, tpf, heads, batch):
     import torch
     w = gen.Workload("bwdh_edges", batch=batch, heads=heads, head_dim=d, tokens_per_frame=tpf, chunk_frames=1, window_frames=1, block=128,
                      topk=1, keep_permille=0, seed=403)
@@ -106,16 +106,20 @@ def test_read_out_gradient_at_tile_edges(d, tpf, heads, batch):
         qb, _, _ = gen.qkv(w, 0, 2, 0)
         gb = gen.normal_bf16(qb.shape, 403, 7, 7)
         q, g = gpu.up(qb), gpu.up(gb)
-        dq = torch.empty_like(q)
+        dq, y = torch.empty_like(q), torch.empty_like(q)
+        gpu.ctx.hf_linear_attn(0, q, y)
         gpu.ctx.hf_linear_attn_backward_dq(0, q, g, dq)
         torch.cuda.synchronize()
         assert gpu.ctx.hf_get_device_status() == (0, 0)
-        got, qf, gf = gpu.f64(dq), f64(qb), f64(gb)
+        got, got_y, qf, gf = gpu.f64(dq), gpu.f64(y), f64(qb), f64(gb)
         for bi in range(batch):
             for h in range(heads):
                 ref = oa.linear_readout_backward(qf[bi, h], ora.S[bi, h], ora.z[bi, h], gf[bi, h],
                                                  W=None if ora.W is None else ora.W[h], eps=ora.eps)[0]
-                rl, ma = hz.rel_l2(got[bi, h], ref), hz.max_abs(got[bi, h], ref)
-                assert rl <= 1e-2 and ma <= 2e-2 * max(1.0, np.abs(ref).max()), f"({bi}, {h}): rel-L2 {rl:.3e}, max-abs {ma:.3e}"
+                out = oa.linear_readout(qf[bi, h], ora.S[bi, h], ora.z[bi, h], W=None if ora.W is None else ora.W[h],
+                                        bias=None if ora.bias is None else ora.bias[h], eps=ora.eps)
+                for name, a, b in (("dq", got[bi, h], ref), ("y", got_y[bi, h], out)):
+                    rl, ma = hz.rel_l2(a, b), hz.max_abs(a, b)
+                    assert rl <= 1e-2 and ma <= 2e-2 * max(1.0, np.abs(b).max()), f"{name} ({bi}, {h}): rel-L2 {rl:.3e}, max-abs {ma:.3e}"
     finally:
         gpu.close()
