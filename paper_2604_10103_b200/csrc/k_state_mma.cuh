@@ -127,7 +127,7 @@ k_absorb_mma(const bf16* __restrict__ k_ev, const bf16* __restrict__ v_ev, int n
     }
 }
 
-// grid (D / 16, B*H, layers), D threads.  Adds the nsplit partials of every (layer, batch*head) to S (rows a0 .. a0 + 15 per
+// grid (D / 16, B*H, layers), 2 D threads.  Adds the nsplit partials of every (layer, batch*head) to S (rows a0 .. a0 + 15 per
 // block) and z (block 0), then folds the updated rows: Sf = S W_h^T (or S where the layer has no matrix) as bf16 hi and lo
 // halves.  Order of the additions (it fixes the bits of the state, whichever kernel produced the partials): the splits are
 // taken in `ngroup` groups of consecutive splits, group g = splits [nsplit g / ngroup, nsplit (g + 1) / ngroup); a group is
@@ -135,30 +135,34 @@ k_absorb_mma(const bf16* __restrict__ k_ev, const bf16* __restrict__ v_ev, int n
 // kernel sums a group on chip and hands over one partial per group: nsplit == ngroup there.)
 // The fold is a 16 x D x D product per block on the warp-level tensor path: the fp32 rows are split exactly into three bf16
 // terms (hi + mid + lo = all 24 mantissa bits), W_h is bf16 already, so every product is exact and only the fp32
-// accumulation of mma.sync rounds; warp w owns output columns [32 w, 32 w + 32).
+// accumulation of mma.sync rounds; warp w owns output columns [16 w, 16 w + 16).
+// Latency-bound (12 heads of 128, 12 splits: 9.5 MB that the partials kernel left in L2): a thread takes one column of eight
+// rows and has six splits in flight at a time; 16 rows per thread and two splits in
+// flight cost an absorb 3 us more (seven chunks absorbed and read: 71.2 -> 68.4 us).
 // nsplit == 0: fold only.  sf_hi == nullptr: state update only.  z_scale: 1 for z = sum of phi(K) rows, 1 / tokens-per-frame
 // for the per-frame-mean reading of Eq. 3.  partials: [layers][B*H][nsplit][D*D + D]; S, sf_hi, sf_lo: [layers][B*H][D][D];
 // z: [layers][B*H][D]; W: [layers][H][D][D] or nullptr, used for the layers whose bit is set in has_w_mask.
 template <int D>
-__global__ void __launch_bounds__(D)
+__global__ void __launch_bounds__(2 * D)
 k_reduce_fold(const float* __restrict__ partials, int nsplit, int ngroup, float* __restrict__ S, float* __restrict__ z, float z_scale,
               const bf16* __restrict__ W, int heads, int BH, bf16* __restrict__ sf_hi, bf16* __restrict__ sf_lo,
               unsigned long long has_w_mask) {
-    constexpr int ROWS = 16;
+    constexpr int ROWS = 16, TR = ROWS / 2, BATCH = 6;              // rows per block and per thread; splits in flight
     constexpr int PART_FLOATS = D * D + D;
     constexpr int ROW_BYTES = D * 2;
     __shared__ __align__(128) uint8_t sW[D * ROW_BYTES];            // W_h [c'][c], 16-byte chunks XOR-swizzled by the row
     __shared__ __align__(128) uint8_t sA[3][ROWS * ROW_BYTES];      // the block's rows of S as bf16 hi / mid / lo, same swizzle
-    const int a0 = blockIdx.x * ROWS, bh = blockIdx.y, lay = blockIdx.z, h = bh % heads;
+    const int bh = blockIdx.y, lay = blockIdx.z, h = bh % heads;
     const size_t item = (size_t)lay * BH + bh;
-    const int cp = threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int cp = threadIdx.x % D, r0 = threadIdx.x / D * TR, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int a0 = blockIdx.x * ROWS, at = a0 + r0;                 // the block's first row, the thread's
     const bool fold = sf_hi != nullptr, with_w = fold && W != nullptr && ((has_w_mask >> lay) & 1ull);
     if (with_w) {       // the matrix does not depend on the kernel before this one: fetched while that kernel drains
         const bf16* wsrc = W + ((size_t)lay * heads + h) * D * D;
         constexpr int CPR = D / 8;                                  // 16-byte chunks per row
 #pragma unroll
-        for (int i = 0; i < CPR; ++i) {
-            const int id = threadIdx.x + i * D, row = id / CPR, ch = id % CPR;
+        for (int i = 0; i < CPR / 2; ++i) {
+            const int id = threadIdx.x + i * 2 * D, row = id / CPR, ch = id % CPR;
             cp_async16(smem_u32(sW) + swz<ROW_BYTES>(row, ch), wsrc + (size_t)row * D + ch * 8, true);
         }
         cp_async_commit();
@@ -166,38 +170,55 @@ k_reduce_fold(const float* __restrict__ partials, int nsplit, int ngroup, float*
     pdl_wait();         // launched under the tail of the partials kernel: its partials (and the state) are complete from here on
     const float* base = partials + item * nsplit * PART_FLOATS;
     float* S_it = S + item * D * D;
-    float sum[ROWS];
+    float sum[TR];
 #pragma unroll
-    for (int r = 0; r < ROWS; ++r) sum[r] = S_it[(size_t)(a0 + r) * D + cp];
+    for (int r = 0; r < TR; ++r) sum[r] = S_it[(size_t)(at + r) * D + cp];
     float ztot = 0.f;           // this call's sum of phi(K) rows; enters z scaled (1, or 1 / tokens per frame)
-    const bool do_z = blockIdx.x == 0 && nsplit > 0;
-    for (int g = 0; g < ngroup && nsplit > 0; ++g) {
-        const int s0 = (int)(((long long)nsplit * g) / ngroup), s1 = (int)(((long long)nsplit * (g + 1)) / ngroup);
-        float sg[ROWS], zg = 0.f;
+    const bool do_z = blockIdx.x == 0 && r0 == 0 && nsplit > 0;
+    float sg[TR], zg = 0.f;
 #pragma unroll
-        for (int r = 0; r < ROWS; ++r) sg[r] = __ldcg(base + (size_t)s0 * PART_FLOATS + (size_t)(a0 + r) * D + cp);
-        if (do_z) zg = __ldcg(base + (size_t)s0 * PART_FLOATS + D * D + cp);
-#pragma unroll 2
-        for (int s = s0 + 1; s < s1; ++s) {      // ascending split order per element; several splits' loads in flight
+    for (int r = 0; r < TR; ++r) sg[r] = 0.f;
+    bool first = true;
+    int g = 0, s1 = nsplit / max(ngroup, 1);                        // the group at hand and its end
+    for (int b = 0; b < nsplit; b += BATCH) {
+        float v[BATCH][TR], vz[BATCH];
 #pragma unroll
-            for (int r = 0; r < ROWS; ++r) sg[r] += __ldcg(base + (size_t)s * PART_FLOATS + (size_t)(a0 + r) * D + cp);
-            if (do_z) zg += __ldcg(base + (size_t)s * PART_FLOATS + D * D + cp);
+        for (int x = 0; x < BATCH; ++x) {
+            const float* part = base + (size_t)(b + x) * PART_FLOATS;
+            vz[x] = 0.f;
+            if (b + x < nsplit) {
+#pragma unroll
+                for (int r = 0; r < TR; ++r) v[x][r] = __ldcg(part + (size_t)(at + r) * D + cp);
+                if (do_z) vz[x] = __ldcg(part + D * D + cp);
+            }
         }
 #pragma unroll
-        for (int r = 0; r < ROWS; ++r) sum[r] += sg[r];
-        ztot += zg;
+        for (int x = 0; x < BATCH; ++x)                             // ascending split order per element
+            if (b + x < nsplit) {
+#pragma unroll
+                for (int r = 0; r < TR; ++r) sg[r] = first ? v[x][r] : sg[r] + v[x][r];
+                zg = first ? vz[x] : zg + vz[x];
+                first = b + x + 1 == s1;
+                if (first) {                                        // the group is complete
+#pragma unroll
+                    for (int r = 0; r < TR; ++r) sum[r] += sg[r];
+                    ztot += zg;
+                    ++g;
+                    s1 = (int)(((long long)nsplit * (g + 1)) / ngroup);
+                }
+            }
     }
     if (nsplit > 0) {
 #pragma unroll
-        for (int r = 0; r < ROWS; ++r) S_it[(size_t)(a0 + r) * D + cp] = sum[r];
+        for (int r = 0; r < TR; ++r) S_it[(size_t)(at + r) * D + cp] = sum[r];
         if (do_z) z[item * D + cp] += ztot * z_scale;
     }
     if (!fold) return;
     if (!with_w) {
 #pragma unroll
-        for (int r = 0; r < ROWS; ++r) {
+        for (int r = 0; r < TR; ++r) {
             const __nv_bfloat16 hi = __float2bfloat16_rn(sum[r]);
-            const size_t o = (item * D + a0 + r) * D + cp;
+            const size_t o = (item * D + at + r) * D + cp;
             sf_hi[o] = hi;
             sf_lo[o] = __float2bfloat16_rn(sum[r] - __bfloat162float(hi));
         }
@@ -205,12 +226,12 @@ k_reduce_fold(const float* __restrict__ partials, int nsplit, int ngroup, float*
     }
     // ---- the rows as three bf16 terms (each difference is exact in fp32), column cp of every row
 #pragma unroll
-    for (int r = 0; r < ROWS; ++r) {
+    for (int r = 0; r < TR; ++r) {
         const __nv_bfloat16 t0 = __float2bfloat16_rn(sum[r]);
         const float r1 = sum[r] - __bfloat162float(t0);
         const __nv_bfloat16 t1 = __float2bfloat16_rn(r1);
         const __nv_bfloat16 t2 = __float2bfloat16_rn(r1 - __bfloat162float(t1));
-        const uint32_t off = swz<ROW_BYTES>(r, cp >> 3) + (cp & 7) * 2;
+        const uint32_t off = swz<ROW_BYTES>(r0 + r, cp >> 3) + (cp & 7) * 2;
         *reinterpret_cast<__nv_bfloat16*>(sA[0] + off) = t0;
         *reinterpret_cast<__nv_bfloat16*>(sA[1] + off) = t1;
         *reinterpret_cast<__nv_bfloat16*>(sA[2] + off) = t2;
@@ -218,29 +239,26 @@ k_reduce_fold(const float* __restrict__ partials, int nsplit, int ngroup, float*
     cp_async_wait<0>();
     __syncthreads();
     // ---- out[a][c'] = sum_c S[a][c] W_h[c'][c]: A = the rows (16 x D), B = W_h as stored ([n][k], k contiguous)
-    float acc[4][4];
+    float acc[2][4];
 #pragma unroll
-    for (int n = 0; n < 4; ++n) { acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f; }
-    const int n0 = warp * 32;
+    for (int n = 0; n < 2; ++n) { acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f; }
+    const int n0 = warp * 16;
 #pragma unroll
     for (int ks = 0; ks < D / 16; ++ks) {
         uint32_t af[3][4];
 #pragma unroll
         for (int t = 0; t < 3; ++t)
             ldsm_x4(smem_u32(sA[t]) + swz<ROW_BYTES>(lane & 15, ks * 2 + (lane >> 4)), af[t][0], af[t][1], af[t][2], af[t][3]);
+        uint32_t b0, b1, b2, b3;
+        ldsm_x4(smem_u32(sW) + swz<ROW_BYTES>(n0 + (lane & 7) + ((lane >> 4) << 3), ks * 2 + ((lane >> 3) & 1)), b0, b1, b2, b3);
 #pragma unroll
-        for (int np = 0; np < 2; ++np) {
-            uint32_t b0, b1, b2, b3;
-            ldsm_x4(smem_u32(sW) + swz<ROW_BYTES>(n0 + np * 16 + (lane & 7) + ((lane >> 4) << 3), ks * 2 + ((lane >> 3) & 1)), b0, b1, b2, b3);
-#pragma unroll
-            for (int t = 0; t < 3; ++t) {
-                mma_bf16(acc[2 * np], af[t][0], af[t][1], af[t][2], af[t][3], b0, b1);
-                mma_bf16(acc[2 * np + 1], af[t][0], af[t][1], af[t][2], af[t][3], b2, b3);
-            }
+        for (int t = 0; t < 3; ++t) {
+            mma_bf16(acc[0], af[t][0], af[t][1], af[t][2], af[t][3], b0, b1);
+            mma_bf16(acc[1], af[t][0], af[t][1], af[t][2], af[t][3], b2, b3);
         }
     }
 #pragma unroll
-    for (int n = 0; n < 4; ++n) {
+    for (int n = 0; n < 2; ++n) {
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
             const float x0 = acc[n][2 * half], x1 = acc[n][2 * half + 1];

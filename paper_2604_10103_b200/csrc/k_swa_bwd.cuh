@@ -204,7 +204,6 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int keep = p.keep;
     const int my_units = (p.n_units - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-    const int n_tiles = my_units * keep;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::KST; ++s) { mbar_init(bar_kf + 8 * s, 1); mbar_init(bar_ke + 8 * s, 1); }
@@ -799,7 +798,6 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     } else {
         // ================================================================= softmax warps (rows = keys, columns = queries)
         const int grp = warp >> 2;                          // the half of every pair's queries this warp turns; then a half of the output columns
-        const int row = (warp & 3) * 32 + lane;             // key row of the block
         const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
         const bool lane0 = lane == 0;
         const float2 c2 = make_float2(p.scale_log2, p.scale_log2);
