@@ -602,12 +602,7 @@ template <int D>
 hf_status launch_bwd_dq(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_cur, const bf16* v_cur, const int32_t* idx, int keep,
                                const bf16* o_local, const float* lse, const bf16* d_o, bf16* dq, cudaStream_t st) {
     typedef SwaBwd<D> C;
-    if (c->bwd_delta == nullptr) HF_TRY(dmalloc(&c->bwd_delta, (size_t)c->BH * c->Tc));
     HF_CUDA(cudaFuncSetAttribute(k_swa_bwd_dq<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES));
-    const long long rows = (long long)c->BH * c->Tc;
-    PdlLaunch pr(dim3((unsigned)((rows + RowDot<D>::RPB - 1) / RowDot<D>::RPB)), dim3(256), 0, st, true);
-    HF_CUDA(cudaLaunchKernelEx(&pr.cfg, k_rowdot<D>, d_o, o_local, c->bwd_delta, rows, BwdOrder{}));
-    HF_TRY(post_launch(c, "k_rowdot"));
     CUtensorMap tq, tdo, tk, tv;
     HF_TRY(make_map(c, &tq, q, 1));
     HF_TRY(make_map(c, &tdo, d_o, 1));
@@ -619,7 +614,7 @@ hf_status launch_bwd_dq(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_c
     p.Tm = c->Tm; p.n_units = c->Tm * c->BH;
     p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D)); p.scale = (float)(1.0 / std::sqrt((double)D));
     p.nb_magic = c->n_b > 1 ? (uint32_t)((0x100000000ull + c->n_b - 1) / c->n_b) : 0u;
-    p.lse = lse; p.delta = c->bwd_delta; p.dev_status = c->dev_status;
+    p.lse = lse; p.d_o = d_o; p.o = o_local; p.dev_status = c->dev_status;
     CUtensorMap tdq;                 // output: one warp's 32 rows x half of the columns per store
     HF_TRY(make_map_ex(c, &tdq, dq, c->Tc, 1, D / 2, 32, true));
     const CUtensorMap& rk = c->R + c->n_sink_max > 0 ? L.tm_kring : tk;

@@ -4,7 +4,7 @@
 // With p = softmax(s) over the kept keys of a query row, s = q k^T / sqrt(d), and g = dL/dO_local:
 //     dq = (1 / sqrt(d)) * sum_c p_c (g . v_c - delta) k_c,     delta = g . o_local     (= sum_c p_c g . v_c)
 // The forward pass leaves lse = log sum_c exp(s_c) per row (hf_sparse_swa), so p = exp(s - lse) needs no running maximum,
-// and k_rowdot forms delta; the block mask is the forward's (held fixed: the top-K choice is piecewise constant).
+// and delta is formed per unit here, by k_rowdot for dK and dV; the block mask is the forward's (held fixed: the top-K choice is piecewise constant).
 //
 // Per (batch*head, query block) unit and kept key tile t, three tensor-core products:
 //   S  = Q K_t^T          A = Q  (tensor memory),  B = K_t (smem, K-major)           -> TMEM [0, 128)
@@ -26,6 +26,16 @@
 // delta[r] = sum_d dO[r][d] * O[r][d].  D / 8 lanes per row (16 bytes of each tensor per lane), four rows per lane with all
 // eight loads in flight: memory-bound (28.75 MB at 12 heads x 4 680 rows x 128: 11.5 us with one row per warp and four bytes
 // per lane, 5.7 us like this).  grid: ceil(rows / (4 * 256 / (D / 8))), 256 threads.
+__device__ __forceinline__ float dot8(const uint4& x, const uint4& y) {
+    const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
+    float acc = 0.f;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float2 u = unpack_bf16(xs[e]), v = unpack_bf16(ys[e]);
+        acc = fmaf(u.x, v.x, fmaf(u.y, v.y, acc));
+    }
+    return acc;
+}
 template <int D>
 struct RowDot { static constexpr int LPR = D / 8, RPB = 4 * 256 / LPR; };      // lanes per row; rows per thread block
 
@@ -110,13 +120,7 @@ __global__ void __launch_bounds__(256) k_rowdot(const bf16* __restrict__ a, cons
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const uint32_t xs[4] = {x[i].x, x[i].y, x[i].z, x[i].w}, ys[4] = {y[i].x, y[i].y, y[i].z, y[i].w};
-        float acc = 0.f;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float2 u = unpack_bf16(xs[e]), v = unpack_bf16(ys[e]);
-            acc = fmaf(u.x, v.x, fmaf(u.y, v.y, acc));
-        }
+        float acc = dot8(x[i], y[i]);
 #pragma unroll
         for (int off = C::LPR / 2; off >= 1; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
         const long long r = r0 + i * (256 / C::LPR);
@@ -156,7 +160,8 @@ struct SwaBwd {
     static constexpr int KST = 3, VST = 2;
     static constexpr int OFF_Q = 0, OFF_DO = TILE_BYTES, OFF_K = 2 * TILE_BYTES, OFF_V = OFF_K + KST * TILE_BYTES;   // (Q: also the output's staging tile)
     static constexpr int OFF_BAR = OFF_V + VST * TILE_BYTES;
-    static constexpr int USED_BYTES = OFF_BAR + 384;
+    static constexpr int OFF_DELTA = OFF_BAR + 384;      // [2 units][128 rows]
+    static constexpr int USED_BYTES = OFF_DELTA + 2 * BLK * 4;
     // one CTA per SM (it takes all of TMEM); slack for the alignment of the tiles to 1 KB
     static constexpr int SMEM_BYTES = USED_BYTES + 1024 > 120 * 1024 ? USED_BYTES + 1024 : 120 * 1024;
     static constexpr int THREADS = 384;                  // warps 0-7: softmax (four per half of the key columns), 8: K loads, 9: V, Q, dO loads, 10: scores, 11: dS K
@@ -170,7 +175,7 @@ struct SwaBwdParams {
     uint32_t nb_magic;       // ceil(2^32 / n_b) (n_b > 1)
     float scale_log2, scale; // log2(e) / sqrt(d), 1 / sqrt(d)
     const float* lse;        // [B*H, T_c] natural log of the row's sum of exponentials (forward)
-    const float* delta;      // [B*H, T_c] g . o_local
+    const bf16 *d_o, *o;     // [B*H, T_c, D] g, o_local
     int* dev_status;
 };
 
@@ -390,7 +395,33 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             const int q0 = i * C::BLK, nq = min(C::BLK, p.Tc - q0);
             const size_t g_row = (size_t)bh * p.Tc + q0 + row;
             const float neg_lse2 = row < nq ? -p.lse[g_row] * 1.4426950408889634f : 0.f;
-            const float delta = row < nq ? p.delta[g_row] : 0.f;
+            // delta = g . o_local of the unit's rows: a warp takes 16 rows, all its loads in flight, and the two warps of a row
+            // exchange.  About 1 000 clk per unit, against a launch before this kernel: the step with gradient at 12 heads of 128,
+            // 4 680 queries 363 -> 358 us, at 2 x 8 heads of 64, 1 300 queries 96.1 -> 94.6 us.
+            float* delta_s = reinterpret_cast<float*>(s_gen + C::OFF_DELTA) + (n & 1) * C::BLK;
+            {
+                constexpr int LPR = D / 8, RPS = 32 / LPR, STEPS = 16 / RPS;        // lanes per row, rows per step
+                const int r0 = (warp & 3) * 32 + grp * 16 + lane / LPR;
+                uint4 x[STEPS], y[STEPS];
+#pragma unroll
+                for (int v = 0; v < STEPS; ++v) {
+                    x[v] = y[v] = make_uint4(0, 0, 0, 0);
+                    if (r0 + v * RPS < nq) {
+                        const size_t at = ((size_t)bh * p.Tc + q0 + r0 + v * RPS) * D + (lane % LPR) * 8;
+                        x[v] = __ldg(reinterpret_cast<const uint4*>(p.d_o + at));
+                        y[v] = __ldg(reinterpret_cast<const uint4*>(p.o + at));
+                    }
+                }
+#pragma unroll
+                for (int v = 0; v < STEPS; ++v) {
+                    float acc = dot8(x[v], y[v]);
+#pragma unroll
+                    for (int off = LPR / 2; off >= 1; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+                    if (lane % LPR == 0) delta_s[r0 + v * RPS] = acc;
+                }
+            }
+            asm volatile("bar.sync %0, 64;\n" ::"r"(1 + (warp & 3)) : "memory");
+            const float delta = delta_s[row];           // (rows past the chunk's end: 0)
             uint32_t tails = 0;         // one bit per tile of the current 32: the block is a chunk's short last one
             for (int j = 0; j < keep; ++j, ++t) {
                 if (ragged && (j & 31) == 0) {
