@@ -137,17 +137,18 @@ k_absorb_mma(const bf16* __restrict__ k_ev, const bf16* __restrict__ v_ev, int n
 // terms (hi + mid + lo = all 24 mantissa bits), W_h is bf16 already, so every product is exact and only the fp32
 // accumulation of mma.sync rounds; warp w owns output columns [16 w, 16 w + 16).
 // Latency-bound (12 heads of 128, 12 splits: 9.5 MB that the partials kernel left in L2): a thread takes one column of eight
-// rows and has six splits in flight at a time; 16 rows per thread and two splits in
-// flight cost an absorb 3 us more (seven chunks absorbed and read: 71.2 -> 68.4 us).
+// rows and has BATCH splits in flight; 16 rows per thread and two splits in flight cost an absorb of one chunk 8 us more (22.8 ->
+// 14.6; 2 heads, 32 splits: 25.7 -> 15.3).  BATCH = 6, or 3 with three thread blocks per SM where the grid is large and the
+// splits few: 30 layers of 12 heads, two group sums each, 201 us either way against 214 with BATCH = 6.
 // nsplit == 0: fold only.  sf_hi == nullptr: state update only.  z_scale: 1 for z = sum of phi(K) rows, 1 / tokens-per-frame
 // for the per-frame-mean reading of Eq. 3.  partials: [layers][B*H][nsplit][D*D + D]; S, sf_hi, sf_lo: [layers][B*H][D][D];
 // z: [layers][B*H][D]; W: [layers][H][D][D] or nullptr, used for the layers whose bit is set in has_w_mask.
-template <int D>
-__global__ void __launch_bounds__(2 * D)
+template <int D, int BATCH>
+__global__ void __launch_bounds__(2 * D, BATCH <= 3 ? 384 / D : 1)
 k_reduce_fold(const float* __restrict__ partials, int nsplit, int ngroup, float* __restrict__ S, float* __restrict__ z, float z_scale,
               const bf16* __restrict__ W, int heads, int BH, bf16* __restrict__ sf_hi, bf16* __restrict__ sf_lo,
               unsigned long long has_w_mask) {
-    constexpr int ROWS = 16, TR = ROWS / 2, BATCH = 6;              // rows per block and per thread; splits in flight
+    constexpr int ROWS = 16, TR = ROWS / 2;                         // rows per block and per thread
     constexpr int PART_FLOATS = D * D + D;
     constexpr int ROW_BYTES = D * 2;
     __shared__ __align__(128) uint8_t sW[D * ROW_BYTES];            // W_h [c'][c], 16-byte chunks XOR-swizzled by the row
