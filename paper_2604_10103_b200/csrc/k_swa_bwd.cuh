@@ -11,7 +11,7 @@
 //   dP = dO V_t^T         A = dO (smem, K-major),  B = V_t (smem, K-major)           -> TMEM [128, 256)
 //   dQ += dS K_t          A = dS (TMEM [448, 512), bf16),  B = K_t (MN-major)        -> TMEM [256, 256 + D)
 // and between them, on the softmax warps (four per half g of the key columns, thread = query row):
-//   dS = exp2(S c - lse log2 e) * (dP - delta)        (columns past a short block's end: 0; 1 / sqrt(d) is applied to dQ)
+//   dS = exp2(S c - lse log2 e) * (dP - delta) / sqrt(d)        (columns past a short block's end: 0)
 // As in the forward kernel, the score buffers are free as soon as they are in registers, dS has slots of its own, dS K is
 // issued per half as its four warps finish, and a warp each issues the scores and dS K: the tensor core forms the next
 // tile's scores while the softmax warps work.  What bounds it: 1 536 clk of tensor time and about as much shared-memory
@@ -128,11 +128,13 @@ __global__ void __launch_bounds__(256) k_rowdot(const bf16* __restrict__ a, cons
     }
 }
 
-// dS / scale = P (dP - delta) of 32 columns of a thread's row as bf16 pairs: packed fp32, two columns per instruction; the factor
-// 1 / sqrt(d) waits for the output.  MASK: columns from nv on count nothing.
+// dS = P (dP - delta) / sqrt(d) of 32 columns of a thread's row as bf16 pairs: packed fp32, two columns per instruction.  The factor
+// 1 / sqrt(d) comes before the rounding to bf16 (at head dim 128 it is no power of two: after it, half of the values of dQ are
+// other bf16 numbers); it rides in the fused multiply-add that takes delta off.  MASK: columns from nv on count nothing.
 template <bool MASK>
-__device__ __forceinline__ void bwd_ds(const uint32_t* s, const uint32_t* dp, int nv, float scale_log2, float neg_lse2, float delta, uint32_t (&pk)[16]) {
-    const float2 c2 = make_float2(scale_log2, scale_log2), l2 = make_float2(neg_lse2, neg_lse2), nd = make_float2(-delta, -delta);
+__device__ __forceinline__ void bwd_ds(const uint32_t* s, const uint32_t* dp, int nv, float scale_log2, float scale, float neg_lse2, float delta, uint32_t (&pk)[16]) {
+    const float2 c2 = make_float2(scale_log2, scale_log2), l2 = make_float2(neg_lse2, neg_lse2);
+    const float2 f2 = make_float2(scale, scale), nd = make_float2(-delta * scale, -delta * scale);
 #pragma unroll
     for (int e0 = 0; e0 < 32; e0 += 8) {
         float2 x[4], g[4];
@@ -140,14 +142,14 @@ __device__ __forceinline__ void bwd_ds(const uint32_t* s, const uint32_t* dp, in
         for (int v = 0; v < 4; ++v) {
             const int e = e0 + 2 * v;
             x[v] = ffma2(make_float2(__uint_as_float(s[e]), __uint_as_float(s[e + 1])), c2, l2);
-            g[v] = fadd2(make_float2(__uint_as_float(dp[e]), __uint_as_float(dp[e + 1])), nd);
+            g[v] = ffma2(make_float2(__uint_as_float(dp[e]), __uint_as_float(dp[e + 1])), f2, nd);
         }
 #pragma unroll
         for (int v = 0; v < 4; ++v) x[v] = make_float2(fast_exp2(x[v].x), fast_exp2(x[v].y));
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             const int e = e0 + 2 * v;
-            x[v].x *= g[v].x; x[v].y *= g[v].y;
+            x[v] = fmul2(x[v], g[v]);
             pk[e >> 1] = pack_bf16(MASK && e >= nv ? 0.f : x[v].x, MASK && e + 1 >= nv ? 0.f : x[v].y);
         }
     }
@@ -452,14 +454,14 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
                         uint32_t pk[16];
-                        bwd_ds<false>(s[c], dp[c], 32, p.scale_log2, neg_lse2, delta, pk);
+                        bwd_ds<false>(s[c], dp[c], 32, p.scale_log2, p.scale, neg_lse2, delta, pk);
                         store_ds(c, pk);
                     }
                 } else {
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
                         uint32_t pk[16];
-                        bwd_ds<true>(s[c], dp[c], p.Tc - (p.n_b - 1) * C::BLK - grp * 64 - c * 32, p.scale_log2, neg_lse2, delta, pk);
+                        bwd_ds<true>(s[c], dp[c], p.Tc - (p.n_b - 1) * C::BLK - grp * 64 - c * 32, p.scale_log2, p.scale, neg_lse2, delta, pk);
                         store_ds(c, pk);
                     }
                 }
@@ -485,7 +487,7 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
                 tmem_ld32(lane_base + C::COL_DQ + grp * (D / 2) + c * 32, o);
                 tmem_wait_ld();
 #pragma unroll
-                for (int e = 0; e < 32; e += 2) out[c * 16 + e / 2] = pack_bf16(__uint_as_float(o[e]) * p.scale, __uint_as_float(o[e + 1]) * p.scale);
+                for (int e = 0; e < 32; e += 2) out[c * 16 + e / 2] = pack_bf16(__uint_as_float(o[e]), __uint_as_float(o[e + 1]));
             }
             fence_before_sync();
             mbar_arrive_if(bar_dqe, lane0);
@@ -520,9 +522,9 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
 // block i that keeps j (read off the selection's bit mask), rows = keys, columns = queries:
 //   S^T  = K_j Q_i^T      A = K_j (smem), B = Q_i (smem)                      -> TMEM [0, 128)
 //   dP^T = V_j dO_i^T     A = V_j (smem), B = dO_i (smem)                     -> TMEM [128, 256)
-//   P^T  = exp2(S^T c - lse_i log2 e)  (bf16, over S^T),   dS^T = P^T (dP^T - delta_i)  (bf16, over dP^T)
+//   P^T  = exp2(S^T c - lse_i log2 e)  (bf16, over S^T),   dS^T = P^T (dP^T - delta_i) / sqrt(d)  (bf16, over dP^T)
 //   dV_j += P^T dO_i      A = P^T (TMEM), B = dO_i (MN-major)                  -> TMEM [256, 256 + D)
-//   dK_j += dS^T Q_i      A = dS^T (TMEM), B = Q_i (MN-major)                  -> TMEM [384, 384 + D); 1 / sqrt(d) at the end
+//   dK_j += dS^T Q_i      A = dS^T (TMEM), B = Q_i (MN-major)                  -> TMEM [384, 384 + D)
 // Accumulators and one pair of score tiles fill tensor memory at head dim 128.  What keeps the tensor core busy all the same is
 // the order in which the one MMA warp issues: dV(t), S(t + 1), dK(t), dP(t + 1) -- the softmax warps form dS(t) during the first
 // two products and P(t + 1) during the last two.  A pair is 2 048 clk of tensor time and, with the tiles' arrival, somewhat
@@ -544,7 +546,7 @@ struct SwaBwdKV {
     static constexpr int OFF_K = 0, OFF_V = TILE_BYTES, OFF_Q = 2 * TILE_BYTES, OFF_DO = OFF_Q + STAGES * TILE_BYTES;
     static constexpr int OFF_OUT = OFF_DO + STAGES * TILE_BYTES;         // staging of the output tile, 32 rows x D / 2 columns per warp
     static constexpr int OFF_BAR = OFF_OUT + BLK * D * 2;
-    static constexpr int OFF_ROW = OFF_BAR + 256;        // [2 pairs][2 halves of the queries][-lse log2 e, -delta][64] floats
+    static constexpr int OFF_ROW = OFF_BAR + 256;        // [2 pairs][2 halves of the queries][-lse log2 e, -delta / sqrt(d)][64] floats
     static constexpr int USED_BYTES = OFF_ROW + 2 * 2 * BLK * 4;
     // one CTA per SM (it takes all of TMEM); slack for the alignment of the tiles to 1 KB, as far as there is room (checked)
     static constexpr int WANT_BYTES = USED_BYTES + 1024 > 120 * 1024 ? USED_BYTES + 1024 : 120 * 1024, MAX_SMEM = 232448;
@@ -798,7 +800,7 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             while (clock64() - t0 < 400000) {}
         }
     } else if (warp == C::WARP_ROW) {
-        // ================================================================= -lse log2 e and -delta of every pair's queries, a pair ahead
+        // ================================================================= -lse log2 e and -delta / sqrt(d) of every pair's queries, a pair ahead
         bool ok = true;
         int t = 0;
         PairWalk walk;
@@ -811,7 +813,7 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     const int r = i * C::BLK + x * 32 + lane;
                     const bool in = r < p.Tc;                         // rows past the chunk's end: weight zero
                     nl[x] = in ? -p.lse[(size_t)walk.bh * p.Tc + r] * 1.4426950408889634f : -INFINITY;
-                    nd[x] = in ? -p.delta[(size_t)walk.bh * p.Tc + r] : 0.f;
+                    nd[x] = in ? -p.delta[(size_t)walk.bh * p.Tc + r] * p.scale : 0.f;
                 }
                 // dK of pair t - 2 has left the tensor core, so its values have been read
                 if (t >= 2 && !(ok = wait_w(bar_qe + 8 * (t & 1), (t >> 1) - 1, 87))) break;
@@ -831,7 +833,7 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
         const int grp = warp >> 2;                          // the half of every pair's queries this warp turns; then a half of the output columns
         const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
         const bool lane0 = lane == 0;
-        const float2 c2 = make_float2(p.scale_log2, p.scale_log2);
+        const float2 c2 = make_float2(p.scale_log2, p.scale_log2), f2 = make_float2(p.scale, p.scale);
         bool ok = true;
         int t = 0;
         int2 unit = unit_of(0);
@@ -874,7 +876,7 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                 tmem_wait_st();
                 fence_before_sync();
                 mbar_arrive_if(bar_pr + 8 * grp, lane0);
-                // ---- dS = P (dP - delta)
+                // ---- dS = P (dP - delta) / sqrt(d)
                 ok = mbar_wait_warp(bar_pd, t & 1, abort_flag, p.dev_status, 88);
                 if (!ok) break;
                 fence_after_sync();
@@ -890,11 +892,11 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
 #pragma unroll
                         for (int e = 0; e < 32; e += 4) {
                             const float4 d4 = nd[e >> 2];
-                            const float2 g0 = fadd2(make_float2(__uint_as_float(dp[c][e]), __uint_as_float(dp[c][e + 1])), make_float2(d4.x, d4.y));
-                            const float2 g1 = fadd2(make_float2(__uint_as_float(dp[c][e + 2]), __uint_as_float(dp[c][e + 3])), make_float2(d4.z, d4.w));
-                            const float2 x0 = pe[16 * c + e / 2], x1 = pe[16 * c + e / 2 + 1];
-                            dk_[e / 2] = pack_bf16(x0.x * g0.x, x0.y * g0.y);
-                            dk_[e / 2 + 1] = pack_bf16(x1.x * g1.x, x1.y * g1.y);
+                            const float2 g0 = ffma2(make_float2(__uint_as_float(dp[c][e]), __uint_as_float(dp[c][e + 1])), f2, make_float2(d4.x, d4.y));
+                            const float2 g1 = ffma2(make_float2(__uint_as_float(dp[c][e + 2]), __uint_as_float(dp[c][e + 3])), f2, make_float2(d4.z, d4.w));
+                            const float2 x0 = fmul2(pe[16 * c + e / 2], g0), x1 = fmul2(pe[16 * c + e / 2 + 1], g1);
+                            dk_[e / 2] = pack_bf16(x0.x, x0.y);
+                            dk_[e / 2 + 1] = pack_bf16(x1.x, x1.y);
                         }
                         tmem_st16(tP + 16 * c, dk_);
                     }
@@ -918,10 +920,9 @@ k_swa_bwd_dkv(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     uint32_t o[32];
                     tmem_ld32(lane_base + (which == 0 ? C::COL_DV : C::COL_DK) + grp * (D / 2) + c * 32, o);
                     tmem_wait_ld();
-                    const float f = which == 0 ? 1.f : p.scale;
 #pragma unroll
                     for (int e = 0; e < 32; e += 2)
-                        out[which][c * 16 + e / 2] = any ? pack_bf16(__uint_as_float(o[e]) * f, __uint_as_float(o[e + 1]) * f) : 0u;
+                        out[which][c * 16 + e / 2] = any ? pack_bf16(__uint_as_float(o[e]), __uint_as_float(o[e + 1])) : 0u;
                 }
             fence_before_sync();
             mbar_arrive_if(bar_acce, lane0);                // the accumulators may take the next unit

@@ -61,6 +61,35 @@ def test_gradients_at_tile_edges(d, tpf, wf, topk, heads, batch):
         gpu.close()
 
 
+@pytest.mark.parametrize("d", [64, 128])
+def test_ds_is_rounded_with_its_factor(d):
+    """dS = P (dP - delta) / sqrt(d) is rounded to bf16 as a whole.  The same products in 64 bits with that one rounding give the
+    same bf16 numbers but for a few (float32 against 64-bit sums in front of a rounding: 2^-24 against 2^-9, a few per mille);
+    with the factor applied after the rounding every other value of dq and dk is a neighbouring number at d = 128."""
+    import torch
+    w = gen.Workload("bwd_rounding", batch=1, heads=2, head_dim=d, tokens_per_frame=512, chunk_frames=1, window_frames=1, block=128, topk=4,
+                     keep_permille=0, seed=409)
+    gpu = hz.GpuStream(w)
+    try:
+        q, k, v = (gpu.up(x) for x in gen.qkv(w, 0, 0, 0))
+        g = gpu.up(gen.normal_bf16((1, 2, 512, d), 409, 7, 7))
+        gpu.select(q, k)
+        o, dq, dk, dv = (torch.empty_like(q) for _ in range(4))
+        lse = torch.empty(gpu.shape[:3], dtype=torch.float32, device="cuda")
+        gpu.ctx.hf_sparse_swa(0, q, k, v, o, lse=lse)
+        gpu.ctx.hf_sparse_swa_backward_dq(0, q, k, v, o, lse, g, dq)
+        gpu.ctx.hf_sparse_swa_backward_dkv(0, q, k, v, o, lse, g, dk, dv)
+        torch.cuda.synchronize()
+        Q, K, V, G, O = (x.cpu().double() for x in (q, k, v, g, o))
+        P = torch.exp(Q @ K.mT / d ** 0.5 - lse.cpu().double()[..., None])
+        dS = (P * (G @ V.mT - (G * O).sum(-1, keepdim=True)) / d ** 0.5).to(torch.bfloat16).double()
+        for name, got, ref in (("dq", dq, dS @ K), ("dk", dk, dS.mT @ Q)):
+            differ = float((got.cpu() != ref.to(torch.bfloat16)).double().mean())
+            assert differ < 0.05, f"{name}: {100 * differ:.1f} % of the values are other bf16 numbers"
+    finally:
+        gpu.close()
+
+
 def test_more_units_than_are_put_in_order():
     """4 200 key blocks of the chunk: beyond the sort's capacity, each warp counts a unit's pairs itself.  A head's gradients do
     not depend on how many others there are, so they equal, bit for bit, those of a context with six heads."""
