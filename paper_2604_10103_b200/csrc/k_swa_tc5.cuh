@@ -351,7 +351,10 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                    bar_pf = bar0 + 64,                     // two: half g of P_t written (4 warps); completion t
                    bar_pv = bar0 + 80,                     // P V of tile t complete, second half (so its V stage is free)
                    bar_ph = bar0 + 216,                    // ... first half
-                   bar_qf = bar0 + 96, bar_qe = bar0 + 104,    // unit n: Q landed / its shared-memory tile is free
+                   // unit n: Q landed / its shared-memory tile is free, which takes the word of both its readers: the copy to tensor
+                   // memory (a commit behind it) and, for HIST, the phi pass of every softmax warp at the unit's last tile.  Neither
+                   // implies the other: in a unit of one tile nothing else orders the phi pass behind the copy, which waits for K.
+                   bar_qf = bar0 + 96, bar_qe = bar0 + 104,
                    bar_hf = bar0 + 112, bar_he = bar0 + 120,   // unit n: S W^T and z landed / free
                    bar_af = bar0 + 128,                    // unit n: phi(Q) operand written
                    bar_ud = bar0 + 136,                    // unit n: history products complete
@@ -381,7 +384,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             mbar_init(bar_se + 8 * s, C::NSW); mbar_init(bar_pf + 8 * s, C::NSW / 2); mbar_init(bar_ph + 8 * s, 1); mbar_init(bar_drain + 8 * s, 1);
         }
         for (int s = 0; s < 4; ++s) mbar_init(bar_x + 8 * s, C::NG);
-        mbar_init(bar_qf, 1); mbar_init(bar_qe, C::NSW); mbar_init(bar_hf, 1); mbar_init(bar_he, C::NSW);
+        mbar_init(bar_qf, 1); mbar_init(bar_qe, HIST ? C::NSW + 1 : 1); mbar_init(bar_hf, 1); mbar_init(bar_he, C::NSW);
         mbar_init(bar_af, C::NSW); mbar_init(bar_ud, 1); mbar_init(bar_dr, C::NSW);
         *abort_flag = 0;
         *redo_cnt = 0; *redo_last = -1;
@@ -508,6 +511,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
 #pragma unroll
                         for (int ks = 0; ks < D / 16; ++ks)      // 16 features = 32 bytes of a row = 8 columns
                             tmem_cp_128x256b(tmem + C::COL_Q + 8 * ks, dq0 + (uint64_t)((ks >> 2) * (C::SUB_BYTES >> 4) + (ks & 3) * 2));
+                        mma_commit(bar_qe);
                     }
                     mma_ts_kmajor<D>(tmem + st * 128, tmem + C::COL_Q, k_lo + st * TILE_STEP, k_hi, IDESC_S);
                     mma_commit(bar_sf + 8 * st);
@@ -721,7 +725,6 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
 #pragma unroll
                 for (int c = 0; c < C::SCOLS / 32; ++c) tmem_ld32(lane_base + st * 128 + grp * C::SCOLS + c * 32, *reinterpret_cast<uint32_t(*)[32]>(r + 32 * c));
                 tmem_wait_ld();
-                if (!HIST && j == 0) arrive_t(bar_qe);      // S is complete, so Q is in tensor memory
                 // ---- columns of this thread that count: all, or the first nv of a segment (a short block; 0: its row group does not
                 // keep the block).  Full and masked segments are separate code: selects on 32 registers in every tile cost 9 us of
                 // a 134 us forward.

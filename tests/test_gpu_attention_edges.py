@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 
 from paper_2604_10103_b200 import inputs as gen
+from paper_2604_10103_b200.binding import HF_SWA_MMA
 from tests import harness as hz
 
 pytestmark = pytest.mark.gpu
@@ -43,6 +44,45 @@ def test_forward_at_tile_edges(d, block, tpf, wf, topk, heads, batch):
         assert gpu.ctx.hf_get_device_status() == (0, 0)
     finally:
         gpu.close()
+
+
+@pytest.mark.parametrize("d,block", [(128, 128), (64, 128), (128, 64), (64, 64), (64, 16)])
+@pytest.mark.parametrize("rope", [False, True])
+def test_units_of_one_tile_whatever_arrives_first(d, block, rope):
+    """Lists of one block, several units per thread block, and keys that arrive late (caches flushed, the queries touched again,
+    copies beside the call): the next unit's queries must not take the place of a unit's that are still to be read.  Every call
+    gives the same bits, and the warp-level kernel's results."""
+    import torch
+    w = gen.Workload("late_keys", batch=1, heads=12, head_dim=d, tokens_per_frame=1560, chunk_frames=2, window_frames=6, block=block,
+                     topk=1, keep_permille=0, seed=227)
+    gpu, ref = hz.GpuStream(w, rope=rope), hz.GpuStream(w, rope=rope, swa_kernel=HF_SWA_MMA)
+    rng = torch.Generator(device="cuda").manual_seed(3)
+    rand = lambda: torch.randn(gpu.shape, generator=rng, device="cuda").to(torch.bfloat16)
+    try:
+        for _ in range(4):
+            kc, vc = rand(), rand()
+            gpu.append(kc, vc); ref.append(kc, vc)
+        q, k, v, o = rand(), rand(), rand(), torch.empty(gpu.shape, dtype=torch.bfloat16, device="cuda")
+        hz.assert_close_out(gpu.forward(q, k, v), ref.forward(q, k, v), "against the warp-level kernel")
+        gpu.ctx.hf_sparse_swa_merged(0, q, k, v, o)
+        torch.cuda.synchronize()
+        first, side = o.clone(), torch.cuda.Stream()
+        big = [torch.zeros(1 << 27, dtype=torch.int32, device="cuda") for _ in range(2)]
+        wrong = 0
+        for it in range(60):
+            big[0].fill_(it)
+            q.add_(0)
+            torch.cuda.synchronize()
+            if it % 2:
+                with torch.cuda.stream(side):
+                    big[1].copy_(big[0])
+            gpu.ctx.hf_sparse_swa_merged(0, q, k, v, o)
+            torch.cuda.synchronize()
+            wrong += not torch.equal(o, first)
+        assert wrong == 0, f"{wrong} of 60 calls gave other results"
+        assert gpu.ctx.hf_get_device_status() == (0, 0)
+    finally:
+        gpu.close(); ref.close()
 
 
 @pytest.mark.parametrize("d,block", [(128, 128), (64, 128), (128, 64), (64, 16)])
