@@ -44,6 +44,12 @@ struct TemporalRope {
     int first_pair, n_pairs, tokens_per_frame;
 };
 
+// The frame of the chunk that row r of a block of n tokens starting at token t0 belongs to, or -1: no such row (a chunk's last
+// block may hold fewer tokens than there are rows of threads, and past the chunk's end the tables have no angles).
+__host__ __device__ inline int turn_frame(int t0, int r, int n, int tokens_per_frame) {
+    return r < n ? (t0 + r) / tokens_per_frame : -1;
+}
+
 // Turn of one thread's VEC features of a row: cosine and sine of those of its VEC / 2 pairs that turn.
 template <int VEC>
 struct PairTurn {
@@ -106,9 +112,9 @@ __device__ __forceinline__ void pool_copy_block(const PoolJob& jb, int Tc, int b
     int frame_end = 0;          // first row of the block that belongs to the frame after turn.frame
     bool turns = false;         // any of this thread's pairs turns at all
     if (ROT) {
-        turns = jb.rot_on && cv * VEC / 2 < tr.first_pair + tr.n_pairs && (cv + 1) * VEC / 2 > tr.first_pair;
+        turn.frame = turn_frame(t0, r, n, tr.tokens_per_frame);
+        turns = jb.rot_on && turn.frame >= 0 && cv * VEC / 2 < tr.first_pair + tr.n_pairs && (cv + 1) * VEC / 2 > tr.first_pair;
         if (turns) {
-            turn.frame = (t0 + r) / tr.tokens_per_frame;
             frame_end = (turn.frame + 1) * tr.tokens_per_frame - t0;
             load_turn<VEC>(turn, cv * VEC, jb.rot_base + jb.rot_per_frame * turn.frame, tr);
         }
@@ -132,7 +138,7 @@ __device__ __forceinline__ void pool_copy_block(const PoolJob& jb, int Tc, int b
                     const int t = r + 16 * (i0 + i);
                     if (t < n) {
                         if (t >= frame_end) {
-                            turn.frame = (t0 + t) / tr.tokens_per_frame;
+                            turn.frame = turn_frame(t0, t, n, tr.tokens_per_frame);
                             frame_end = (turn.frame + 1) * tr.tokens_per_frame - t0;
                             if (jb.rot_per_frame != 0) load_turn<VEC>(turn, cv * VEC, jb.rot_base + jb.rot_per_frame * turn.frame, tr);
                         }

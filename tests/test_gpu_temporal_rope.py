@@ -17,6 +17,7 @@ f64 = gen.bf16_bits_to_f64
     (64, 16, 20, 3, 6, 1, 6, 4, 10, 0, 7),          # small blocks, a sink chunk, temporal pairs in the middle of the head
     (128, 64, 96, 1, 3, 0, 4, 0, 22, 0, 8),         # one-frame chunks
     (128, 128, 130, 2, 2, 0, 4, 0, None, 0, 5),     # window == chunk: nothing cached, chunks go straight to the state
+    (128, 128, 130, 1, 3, 0, 3, 0, None, 0, 7),     # last block 2 tokens: most rows of threads have none
     (64, 128, 150, 3, 6, 0, 6, 0, None, 3, 6),      # ping-pong kernel, head_dim 64
     (128, 128, 100, 3, 9, 0, 9, 0, None, 1, 6),     # warp-level kernel
 ])
