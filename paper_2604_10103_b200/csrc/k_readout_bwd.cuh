@@ -30,7 +30,7 @@ struct ReadoutBwd {
     static constexpr int OFF_G = 0, OFF_Q = GST * G_BYTES, OFF_S = OFF_Q + QST * G_BYTES, OFF_Z = OFF_S + 2 * S_BYTES;
     static constexpr int OFF_DOT = OFF_Z + QST * D * 4;            // [2 units][2 halves][128 rows] (f . u, f . z)
     static constexpr int OFF_BAR = OFF_DOT + 2 * 2 * ROWS * 8;
-    static constexpr int USED_BYTES = OFF_BAR + 128;
+    static constexpr int USED_BYTES = OFF_BAR + 160;
     static constexpr int SMEM_BYTES = USED_BYTES + 1024;
     static constexpr int THREADS = 320, WARP_TMA = 8, WARP_MMA = 9;
     static constexpr int STORERS = SUB == 2 ? 8 : 4;               // warps that store: 64 columns each
@@ -58,7 +58,8 @@ k_readout_bwd_dq(const __grid_constant__ CUtensorMap tm_g, const __grid_constant
     uint8_t* s_gen = smem_raw + (s_base - smem_u32(smem_raw));
     const uint32_t bar0 = s_base + C::OFF_BAR;
     const uint32_t bar_gfull = bar0, bar_gfree = bar0 + 16, bar_ufull = bar0 + 32, bar_ufree = bar0 + 48, bar_sfull = bar0 + 64,
-                   bar_qfull = bar0 + 72, bar_qfree = bar0 + 96;
+                   bar_qfull = bar0 + 72, bar_qfree = bar0 + 96,
+                   bar_x = bar0 + 128;                             // four: the two warps that share 32 rows meet
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_gen + C::OFF_BAR + 120);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(s_gen + C::OFF_BAR + 124);
 
@@ -73,6 +74,7 @@ k_readout_bwd_dq(const __grid_constant__ CUtensorMap tm_g, const __grid_constant
             mbar_init(bar_ufull + 8 * s, 1); mbar_init(bar_ufree + 8 * s, 8);
         }
         for (int s = 0; s < C::QST; ++s) { mbar_init(bar_qfull + 8 * s, 1); mbar_init(bar_qfree + 8 * s, C::STORERS); }
+        for (int s = 0; s < 4; ++s) mbar_init(bar_x + 8 * s, 2);
         mbar_init(bar_sfull, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -173,6 +175,8 @@ k_readout_bwd_dq(const __grid_constant__ CUtensorMap tm_g, const __grid_constant
         bool ok = true;
         RingPos<C::QST> rq;
         int prev = 0;                                              // Q stage of the unit before
+        uint32_t met = 0;                                          // meetings with the warp of the rows' other half
+        auto meet = [&](int where) -> bool { return mbar_meet_warp(bar_x + 8 * quad, met++, lane0, abort_flag, p.dev_status, where); };
         for (int n = 0; ok && n < my_units; ++n, rq.advance()) {
             const int u = u0 + n;
             const int bh = u / p.Tm, i = u - bh * p.Tm;
@@ -216,7 +220,7 @@ k_readout_bwd_dq(const __grid_constant__ CUtensorMap tm_g, const __grid_constant
             // ---- the row's other half: f . u and f . z of all columns
             float2* dots = reinterpret_cast<float2*>(s_gen + C::OFF_DOT) + (n & 1) * 2 * C::ROWS + row;
             dots[half * C::ROWS] = make_float2(fu, fz);
-            asm volatile("bar.sync %0, 64;\n" ::"r"(1 + quad) : "memory");
+            if (!(ok = meet(69))) break;
             const float2 d0 = dots[0], d1 = dots[C::ROWS];
             const float inv = 1.f / (d0.y + d1.y + p.eps);
             const float ratio = (d0.x + d1.x) * inv;
@@ -237,7 +241,7 @@ k_readout_bwd_dq(const __grid_constant__ CUtensorMap tm_g, const __grid_constant
             }
             fence_proxy_async();
             if (C::SUB == 2) __syncwarp();
-            else asm volatile("bar.sync %0, 64;\n" ::"r"(1 + quad) : "memory");        // 64 columns are both halves' here
+            else if (!(ok = meet(60))) break;                      // 64 columns are both halves' here
             if (storer && lane0) {
                 if (i * C::ROWS + quad * 32 < p.Tc)
                     tma_store_4d(&tm_dq, s_base + q_off + quad * 32 * 128, C::SUB == 2 ? half * 64 : 0, i * C::ROWS + quad * 32, bh, 0);

@@ -332,7 +332,8 @@ k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     uint8_t* s_gen = smem_raw + (s_base - smem_u32(smem_raw));
     const uint32_t bar0 = s_base + C::OFF_BAR;
     const uint32_t bar_full = bar0, bar_qfree = bar0 + 24, bar_sfull = bar0 + 48, bar_sfree = bar0 + 56, bar_afull = bar0 + 64,
-                   bar_afree = bar0 + 80, bar_dfull = bar0 + 96, bar_dfree = bar0 + 112;
+                   bar_afree = bar0 + 80, bar_dfull = bar0 + 96, bar_dfree = bar0 + 112,
+                   bar_x = bar0 + 160;          // four: unit n's result, between the two warps that share 32 rows (head dim 64)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_gen + C::OFF_BAR + 144);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(s_gen + C::OFF_BAR + 148);
 
@@ -347,6 +348,7 @@ k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             mbar_init(bar_afull + 8 * s, 256); mbar_init(bar_afree + 8 * s, 1); mbar_init(bar_dfull + 8 * s, 1);
             mbar_init(bar_dfree + 8 * s, 256);
         }
+        for (int s = 0; s < 4; ++s) mbar_init(bar_x + 8 * s, 2);
         mbar_init(bar_sfull, 1); mbar_init(bar_sfree, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -573,7 +575,7 @@ k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
             mbar_arrive(bar_dfree + 8 * s);
             if (staged) fence_proxy_async();
             if (C::SUB == 2 || !staged) __syncwarp();
-            else asm volatile("bar.sync %0, 64;\n" ::"r"(1 + (warp & 3)) : "memory");     // 64 columns are both halves' here
+            else if (!mbar_meet_warp(bar_x + 8 * (warp & 3), n, lane0, abort_flag, p.dev_status, 51)) return false;     // 64 columns are both halves' here
             if (lane0) {
                 if (staged && storer) {
                     if (i * C::ROWS + (warp & 3) * 32 < p.Tc)

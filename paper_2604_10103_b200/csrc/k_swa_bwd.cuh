@@ -204,7 +204,8 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
                    bar_cp = bar0 + 248,         // unit n: ... and copied to tensor memory
                    bar_qe = bar0 + 256,         // unit n: its output, staged where Q of unit n + 1 had been, has left
                    bar_of = bar0 + 264, bar_oe = bar0 + 272,       // unit n: dO landed / read for the last time
-                   bar_dqf = bar0 + 280, bar_dqe = bar0 + 288;
+                   bar_dqf = bar0 + 280, bar_dqe = bar0 + 288,
+                   bar_x = bar0 + 304;          // four: unit n's delta, between the two warps that share 32 rows
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_gen + C::OFF_BAR + 296);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(s_gen + C::OFF_BAR + 300);
 
@@ -216,6 +217,7 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         for (int s = 0; s < C::KST; ++s) { mbar_init(bar_kf + 8 * s, 1); mbar_init(bar_ke + 8 * s, 1); }
         for (int s = 0; s < C::VST; ++s) { mbar_init(bar_vf + 8 * s, 1); mbar_init(bar_ve + 8 * s, 1); }
         for (int s = 0; s < 2; ++s) { mbar_init(bar_ds + 8 * s, 4); mbar_init(bar_df + 8 * s, 1); mbar_init(bar_drain + 8 * s, 1); }
+        for (int s = 0; s < 4; ++s) mbar_init(bar_x + 8 * s, 2);
         mbar_init(bar_sd, 1); mbar_init(bar_se, 8);
         mbar_init(bar_qf, 1); mbar_init(bar_cp, 1); mbar_init(bar_of, 1); mbar_init(bar_oe, 1); mbar_init(bar_qe, 8); mbar_init(bar_dqf, 1); mbar_init(bar_dqe, 8);
         *abort_flag = 0;
@@ -422,7 +424,8 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
                     if (lane % LPR == 0) delta_s[r0 + v * RPS] = acc;
                 }
             }
-            asm volatile("bar.sync %0, 64;\n" ::"r"(1 + (warp & 3)) : "memory");
+            ok = mbar_meet_warp(bar_x + 8 * (warp & 3), n, lane0, abort_flag, p.dev_status, 97);
+            if (!ok) break;
             const float delta = delta_s[row];           // (rows past the chunk's end: 0)
             uint32_t tails = 0;         // one bit per tile of the current 32: the block is a chunk's short last one
             for (int j = 0; j < keep; ++j, ++t) {

@@ -74,6 +74,14 @@ __device__ __forceinline__ void mbar_arrive_if(uint32_t bar, bool on) {
     asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %1, 0;\n @p mbarrier.arrive.shared::cta.b64 _, [%0];\n}\n"
                  ::"r"(bar), "r"((uint32_t)on) : "memory");
 }
+// Meeting of the warps that share a barrier (count: one arrival each; the phase of meeting e is e & 1): what each wrote to shared
+// memory before is visible to the others after.  Bounded like every other wait, which a named barrier is not: a partner that
+// has given up elsewhere would never come.
+__device__ __forceinline__ bool mbar_meet_warp(uint32_t bar, uint32_t parity, bool lane0, volatile int* abort_flag, int* dev_status, int where) {
+    __syncwarp();
+    mbar_arrive_if(bar, lane0);
+    return mbar_wait_warp(bar, parity & 1u, abort_flag, dev_status, where);
+}
 
 // ----------------------------------------------------------------------------------------- TMA
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3, uint32_t bar) {

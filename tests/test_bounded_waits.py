@@ -1,0 +1,27 @@
+"""Waits between the roles of a kernel are bounded: a warp may leave its loop when a wait runs out, so no other warp may wait for it
+on a barrier without a limit.  Named barriers (which have none) are for code in which nobody can have left."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2604_10103_b200", "csrc")
+
+# file: named barriers, and why nobody can be missing there
+NAMED = {
+    "k_swa_mma.cuh": 1,     # a unit's warps: no role of it has a wait that can run out
+    "k_swa_tc5.cuh": 1,     # the second pass: entered by all its threads, after the roles have met and none has given up
+}
+
+
+def sources():
+    return {f: open(os.path.join(CSRC, f)).read() for f in sorted(os.listdir(CSRC)) if f.endswith((".cu", ".cuh"))}
+
+
+def test_no_named_barrier_between_roles():
+    found = {f: len(re.findall(r"\b(?:bar|barrier)(?:\.cta)?\.(?:sync|arrive|red)", s)) for f, s in sources().items()}
+    assert {f: n for f, n in found.items() if n} == NAMED
+
+
+def test_every_polling_loop_has_a_limit():
+    for f, s in sources().items():
+        for m in re.finditer(r"while \(!mbar_try_wait[^;{]*", s):
+            assert "clock64() - t0 <" in m.group(0), f"{f}: {m.group(0)}"
