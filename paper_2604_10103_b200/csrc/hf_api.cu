@@ -632,10 +632,8 @@ template <int D>
 hf_status launch_bwd_dkv(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_cur, const bf16* v_cur, const bf16* o_local,
                          const float* lse, const bf16* d_o, bf16* dk, bf16* dv, cudaStream_t st) {
     typedef SwaBwdKV<D> C;
-    if (c->bwd_delta == nullptr) HF_TRY(dmalloc(&c->bwd_delta, (size_t)c->BH * c->Tc));
     HF_CUDA(cudaFuncSetAttribute(k_swa_bwd_dkv<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES));
     const long long rows = (long long)c->BH * c->Tc;
-    if (c->bwd_order == nullptr) HF_TRY(dmalloc(&c->bwd_order, (size_t)c->BH * c->n_b));
     BwdOrder ord;
     ord.mask = L.mask; ord.mask_words = c->mask_words; ord.first_block = (L.n_sink + L.n_cached) * c->n_b; ord.n_b = c->n_b; ord.Tm = c->Tm;
     ord.BH = c->BH; ord.order = c->bwd_order;
@@ -800,6 +798,9 @@ hf_status hf_create(const hf_config* cfg, int device, hf_ctx** out) {
         s = dmalloc(&c->union_entries, (size_t)c->BH * Tmt * c->union_max_tiles * G);
         if (s == HF_OK) s = dmalloc(&c->union_tiles, (size_t)c->BH * Tmt);
     }
+    // the backward calls' buffers (they take 128-token blocks): here, so that either call can be captured into a graph
+    if (s == HF_OK && cfg->block == 128) s = dmalloc(&c->bwd_delta, (size_t)c->BH * c->Tc);
+    if (s == HF_OK && cfg->block == 128) s = dmalloc(&c->bwd_order, (size_t)c->BH * c->n_b);
     if (s == HF_OK) s = dmalloc(&c->pooled_q, c->pooled_elems);
     if (s == HF_OK) s = dmalloc(&c->pooled_kcur, c->pooled_elems);
     if (s == HF_OK) s = dmalloc(&c->hist, c->chunk_elems);

@@ -152,3 +152,36 @@ def test_read_out_and_its_gradient_at_tile_edges(d, tpf, heads, batch):
                     assert rl <= 1e-2 and ma <= 2e-2 * max(1.0, np.abs(b).max()), f"{name} ({bi}, {h}): rel-L2 {rl:.3e}, max-abs {ma:.3e}"
     finally:
         gpu.close()
+
+
+@pytest.mark.parametrize("first,then", [("dq", "dkv"), ("dkv", "dq"), (None, "dq"), (None, "dkv")])
+def test_backward_into_a_graph(first, then):
+    """Neither backward call allocates: each can be captured, after the other or as the first, and the replay gives its bits."""
+    import torch
+    w = gen.Workload("bwd_graph", batch=1, heads=2, head_dim=128, tokens_per_frame=300, chunk_frames=1, window_frames=2, block=128, topk=2,
+                     keep_permille=0, seed=419)
+    gpu = hz.GpuStream(w)
+    try:
+        q, k, v = (gpu.up(x) for x in gen.qkv(w, 0, 0, 0))
+        g = gpu.up(gen.normal_bf16(tuple(gpu.shape), 419, 7, 7))
+        gpu.select(q, k)
+        o, dq, dk, dv = (torch.empty_like(q) for _ in range(4))
+        lse = torch.empty(gpu.shape[:3], dtype=torch.float32, device="cuda")
+        gpu.ctx.hf_sparse_swa(0, q, k, v, o, lse=lse)
+        calls = {"dq": (lambda: gpu.ctx.hf_sparse_swa_backward_dq(0, q, k, v, o, lse, g, dq), [dq]),
+                 "dkv": (lambda: gpu.ctx.hf_sparse_swa_backward_dkv(0, q, k, v, o, lse, g, dk, dv), [dk, dv])}
+        if first:
+            calls[first][0]()
+        torch.cuda.synchronize()
+        call, outs = calls[then]
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            call()
+        graph.replay()
+        torch.cuda.synchronize()
+        replayed = [t.clone() for t in outs]
+        call()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(replayed, outs))
+    finally:
+        gpu.close()
