@@ -529,7 +529,7 @@ hf_status launch_swa_tc5_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16* 
     HF_TRY(make_map_ex(c, &tv, v_cur, c->Tc, 1, 64, BLK, true));
     HF_TRY(make_map_ex(c, &to, o, c->Tc, 1, C::OCOLS, 32, true));      // output: one warp's 32 rows x half of the columns per store
     p.idx = idx; p.keep = keep; p.Tc = c->Tc; p.n_b = c->n_b; p.n_cached = L.n_cached; p.ring_head = L.head; p.n_sink = L.n_sink;
-    p.P = c->R; p.Tm = c->Tm;
+    p.P = c->R; p.Tm = c->Tm; p.Tn = (L.n_sink + L.n_cached + 1) * c->n_b;
     p.nb_magic = c->n_b > 1 ? (uint32_t)((0x100000000ull + c->n_b - 1) / c->n_b) : 0u;
     p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D));
     p.hist = hist; p.o = o; p.lse = lse; p.dev_status = c->dev_status;
@@ -614,7 +614,7 @@ hf_status launch_bwd_dq(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_c
     SwaBwdParams p;
     memset(&p, 0, sizeof(p));
     p.idx = idx; p.keep = keep; p.Tc = c->Tc; p.n_b = c->n_b; p.n_cached = L.n_cached; p.ring_head = L.head; p.P = c->R; p.n_sink = L.n_sink;
-    p.Tm = c->Tm; p.n_units = c->Tm * c->BH;
+    p.Tm = c->Tm; p.n_units = c->Tm * c->BH; p.Tn = (L.n_sink + L.n_cached + 1) * c->n_b;
     p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)D)); p.scale = (float)(1.0 / std::sqrt((double)D));
     p.nb_magic = c->n_b > 1 ? (uint32_t)((0x100000000ull + c->n_b - 1) / c->n_b) : 0u;
     p.lse = lse; p.d_o = d_o; p.o = o_local; p.dev_status = c->dev_status;

@@ -173,7 +173,7 @@ struct SwaBwd {
 
 struct SwaBwdParams {
     const int32_t* idx;      // [B*H, T_m, keep]
-    int keep, Tc, n_b, n_cached, ring_head, P, n_sink, Tm, n_units;
+    int keep, Tc, n_b, n_cached, ring_head, P, n_sink, Tm, n_units, Tn;
     uint32_t nb_magic;       // ceil(2^32 / n_b) (n_b > 1)
     float scale_log2, scale; // log2(e) / sqrt(d), 1 / sqrt(d)
     const float* lse;        // [B*H, T_c] natural log of the row's sum of exponentials (forward)
@@ -245,7 +245,7 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             RingPos<C::KST> rk;
             RingPos<C::VST> rv;
             int t = 0;
-            const int Tn = (p.n_sink + p.n_cached + 1) * p.n_b;
+            const int Tn = p.Tn;
             auto load_q = [&](int m) {
                 const int u = blockIdx.x + m * gridDim.x, bh = u / p.Tm, i = u - bh * p.Tm;
                 mbar_expect_tx(bar_qf, C::TILE_BYTES);
@@ -430,8 +430,9 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             uint32_t tails = 0;         // one bit per tile of the current 32: the block is a chunk's short last one
             for (int j = 0; j < keep; ++j, ++t) {
                 if (ragged && (j & 31) == 0) {
-                    const uint32_t x1 = j + lane < keep ? (uint32_t)__ldg(my_idx + j + lane) + 1u : 0xffffffffu;
-                    tails = __ballot_sync(0xffffffffu, x1 <= HF_MAX_TN && (p.n_b == 1 || __umulhi(x1, p.nb_magic) * p.n_b == x1));
+                    const uint32_t e = j + lane < keep ? (uint32_t)__ldg(my_idx + j + lane) : 0u;
+                    const uint32_t x1 = (e < (uint32_t)p.Tn ? e : 0u) + 1u;     // (an entry outside [0, T_n) is block 0, as for the loader)
+                    tails = __ballot_sync(0xffffffffu, p.n_b == 1 || __umulhi(x1, p.nb_magic) * p.n_b == x1);
                 }
                 const bool tail = (tails >> (j & 31)) & 1u;
                 ok = mbar_wait_warp(bar_sd, t & 1, abort_flag, p.dev_status, 89);

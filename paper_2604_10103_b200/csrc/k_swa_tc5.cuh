@@ -97,6 +97,7 @@ struct Tc5Params {
     const int32_t* idx;      // [B*H, T_m, keep]
     int keep, Tc, n_b, n_cached, ring_head, P;   // P: physical ring slots (one more than the window holds); the sink slots follow them
     int n_sink;              // sink chunks held (logical chunks 0 .. n_sink - 1)
+    int Tn;                  // key blocks of the window: (n_sink + n_cached + 1) n_b
     uint32_t nb_magic;       // ceil(2^32 / n_b) (n_b > 1): x / n_b = high word of x * nb_magic for x <= 1024
     int Tm, n_units;         // query blocks per batch*head; units in all (unit u = bh * upb + i)
     int upb;                 // units per batch*head: T_m, or ceil(T_c / 128) with 16- / 64-token blocks
@@ -416,7 +417,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             const bool is_k = (warp == C::WARP_LOAD_K);
             bool ok = true;
             int t = 0;
-            const int Tn = (p.n_sink + p.n_cached + 1) * p.n_b;
+            const int Tn = p.Tn;
             const uint32_t tiles = is_k ? sK : sV, full = is_k ? bar_kf : bar_vf, freed = is_k ? bar_sf : bar_pv;
             // one box of BLK rows of key block blk
             auto load_block = [&](int blk, uint32_t dst, uint32_t bar, int bh) {
@@ -620,7 +621,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         const uint32_t bar_own = grp == 0 ? bar_ph : bar_pv;       // product of this group's half of P
         // BLK 16, 64: list entries, read one tile ahead.  BLK 128: all that matters here is whether a tile is a chunk's short last
         // block; one bit per tile from a ballot over 32 list entries at a time (lane = entry), read one window ahead.  An entry
-        // outside [0, T_n) -- the loader reads block 0 for it and reports it -- is simply none.
+        // outside [0, T_n) is block 0 here as for the loader, which reports it.
         auto entries_of = [&](int unit) -> const uint32_t* {
             if constexpr (BLK == 128) return reinterpret_cast<const uint32_t*>(p.idx + (size_t)unit * p.keep);
             else return p.entries + (size_t)unit * p.max_tiles * G + grp * EPT;
@@ -655,8 +656,8 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                 uint32_t e_cur[EPT];
                 if constexpr (BLK == 128) {
                     if (ragged && (j & 31) == 0) {
-                        const uint32_t x1 = e_next[0] + 1u;     // last block of a chunk: its index + 1 is a multiple of n_b (no division)
-                        tails = __ballot_sync(0xffffffffu, p.n_b == 1 || (x1 <= HF_MAX_TN && __umulhi(x1, p.nb_magic) * p.n_b == x1));
+                        const uint32_t x1 = (e_next[0] < (uint32_t)p.Tn ? e_next[0] : 0u) + 1u;     // last block of a chunk: its index + 1 is a multiple of n_b (no division)
+                        tails = __ballot_sync(0xffffffffu, p.n_b == 1 || __umulhi(x1, p.nb_magic) * p.n_b == x1);
                         const int j2 = j + 32 < cnt ? j + 32 : 0;
                         if (j2 + lane < p.keep) e_next[0] = __ldg(entries_of(j2 || n + 1 >= my_units ? u : u + (int)gridDim.x) + j2 + lane);
                     }

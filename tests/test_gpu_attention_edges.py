@@ -109,3 +109,44 @@ def test_rotated_history_in_both_passes(d, block):
         assert gpu.ctx.hf_get_device_status() == (0, 0)
     finally:
         gpu.close()
+
+
+@pytest.mark.parametrize("d,tpf", [(128, 300), (64, 300), (128, 100)])
+def test_an_entry_outside_the_window_is_block_0(d, tpf):
+    """A list entry outside [0, T_n) is reported, and read as block 0, a full one or (one block per chunk) a short one: forward
+    and dq give what the same list with 0 in its place gives.  -1, the entry behind the last block and one whose index + 1 is a
+    multiple of the blocks per chunk are told apart from a chunk's short last block."""
+    import torch
+    w = gen.Workload("bad_entry", batch=1, heads=2, head_dim=d, tokens_per_frame=tpf, chunk_frames=1, window_frames=3, block=128,
+                     topk=3, keep_permille=0, seed=229)
+    gpu = hz.GpuStream(w)
+    try:
+        for c in range(3):
+            kc, vc = gen.clean_kv(w, 0, c)
+            gpu.append(gpu.up(kc), gpu.up(vc))
+        q, k, v = (gpu.up(x) for x in gen.qkv(w, 0, 3, 0))
+        g = gpu.up(gen.normal_bf16(tuple(gpu.shape), 229, 7, 7))
+        tn, nb = gpu.ctx.hf_query(0, gpu.hf.HF_Q_KEY_BLOCKS), w.blocks_per_chunk
+        _, idx0, _ = gpu.select(q, k)
+        for bad in (-1, tn, tn + nb - 1, 2 ** 30):
+            lists = {}
+            for value in (0, bad):
+                idx = idx0.copy()
+                idx[0, :, :, 1] = value
+                lists[value] = torch.from_numpy(idx).cuda()
+            outs = {}
+            for value, idx in lists.items():
+                o, lse = gpu.swa(q, k, v, idx=idx, want_lse=True)
+                ot, lt = torch.from_numpy(o).to(torch.bfloat16).cuda(), torch.from_numpy(lse).cuda()
+                dq = torch.empty_like(q)
+                gpu.ctx.hf_sparse_swa_backward_dq(0, q, k, v, ot, lt, g, dq, idx=idx)
+                outs[value] = (o, lse, gpu.f64(dq))
+                if value == 0:
+                    assert gpu.ctx.hf_get_device_status() == (0, 0)
+                else:
+                    with pytest.raises(gpu.hf.HFError, match="HF_ERR_INVALID_ARG"):
+                        gpu.ctx.hf_get_device_status()
+            for a, b in zip(outs[0], outs[bad]):
+                assert np.array_equal(a, b), f"entry {bad}"
+    finally:
+        gpu.close()
