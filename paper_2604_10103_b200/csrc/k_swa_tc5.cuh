@@ -77,7 +77,11 @@ struct SwaTc5 {
     // (the second pass keeps its fp32 history tile behind the operand tiles of swa_mma_unit, in front of the barriers)
     static constexpr int OFF_BAR = OFF_H + 2 * H_BYTES > SwaMma<128, D>::SMEM_BYTES + 128 * D * 4 ? OFF_H + 2 * H_BYTES
                                                                                                     : SwaMma<128, D>::SMEM_BYTES + 128 * D * 4;
-    static constexpr int OFF_Z = OFF_BAR + 256;        // z [D] of the unit's head
+    // units whose rows left the range of the fixed reference: count, last unit listed, up to REDO_CAP local unit numbers
+    // (more than that: every unit of the thread block is computed again)
+    static constexpr int OFF_REDO = OFF_BAR + 256, REDO_CAP = 8;
+    static constexpr int OFF_Z = OFF_REDO + 64;        // z [D] of the unit's head
+    static_assert((2 + REDO_CAP) * 4 <= OFF_Z - OFF_REDO, "the list must fit");
     static constexpr int OFF_XM = OFF_Z + 512;         // row maxima of the column groups [NG][128]
     static constexpr int USED_BYTES = OFF_XM + NG * 128 * 4;
     // row sums and shares of Eq. 4's denominator [2][NG][128] at a unit's end: beside the staging tile of the output
@@ -364,13 +368,9 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                    bar_drain = bar0 + 232;                 // two: each MMA warp's last operations complete
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_gen + C::OFF_BAR + 184);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(s_gen + C::OFF_BAR + 188);
-    // units whose rows left the range of the fixed reference: count, last unit listed, up to REDO_CAP local unit numbers
-    // (more than that: every unit of this thread block is computed again)
-    constexpr int REDO_CAP = 4;
-    int* redo_cnt = reinterpret_cast<int*>(s_gen + C::OFF_BAR + 192);
+    int* redo_cnt = reinterpret_cast<int*>(s_gen + C::OFF_REDO);
     int* redo_last = redo_cnt + 1;
     int* redo_list = redo_cnt + 2;
-    static_assert(192 + (2 + REDO_CAP) * 4 <= 216, "the list must fit in front of the barriers that follow it");
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int my_units = (p.n_units - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
@@ -611,7 +611,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         auto note_redo = [&](int n) {                       // list unit n once
             if (atomicMax(redo_last, n) < n) {
                 const int slot = atomicAdd(redo_cnt, 1);
-                if (slot < REDO_CAP) redo_list[slot] = n;
+                if (slot < C::REDO_CAP) redo_list[slot] = n;
             }
         };
         // (batch*head, position) of a unit without a division per unit; the tile count and the first list entries of the next
@@ -924,9 +924,9 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
     const int n_redo = *redo_cnt;
     if (n_redo > 0 && *abort_flag == 0 && threadIdx.x < 256) {
         fence_proxy_async();                                  // the tile stream's bulk stores of these rows came first
-        const int total = n_redo > REDO_CAP ? my_units : n_redo;
+        const int total = n_redo > C::REDO_CAP ? my_units : n_redo;
         for (int r = 0; r < total; ++r) {
-            const int n = n_redo > REDO_CAP ? r : redo_list[r];
+            const int n = n_redo > C::REDO_CAP ? r : redo_list[r];
             swa_redo_unit<D, BLK, HIST>(s_gen, p, (int)blockIdx.x + n * (int)gridDim.x);
         }
     }

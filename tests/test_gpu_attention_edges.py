@@ -150,3 +150,38 @@ def test_an_entry_outside_the_window_is_block_0(d, tpf):
                 assert np.array_equal(a, b), f"entry {bad}"
     finally:
         gpu.close()
+
+
+@pytest.mark.parametrize("units", [1, 5, 8, 9])
+def test_only_the_listed_units_are_computed_again(units):
+    """Ten units on one thread block, some with a block ~180 nats above the first kept one: up to eight of them are computed again
+    and nothing else is; with a ninth all ten are.  Results are those of the warp-level kernel."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    d, n_b = 128, 21
+    heads = -(-9 * sms // n_b) + 1
+    w = gen.Workload("redo_list", batch=1, heads=heads, head_dim=d, tokens_per_frame=128 * n_b, chunk_frames=1, window_frames=1, block=128,
+                     topk=2, keep_permille=0, seed=233)
+    gpu = hz.GpuStream(w, merge=False)
+    ref = hz.GpuStream(w, merge=False, swa_kernel=HF_SWA_MMA)
+    rng = torch.Generator(device="cuda").manual_seed(7)
+    rand = lambda: torch.randn(gpu.shape, generator=rng, device="cuda")
+    try:
+        q, k, v = rand(), rand(), rand().to(torch.bfloat16)
+        a = (180.0 / d ** 0.5) ** 0.5               # a^2 d / sqrt(d) = 180
+        k[:, :, -128:] += a                         # the last block: a few nats for queries that do not look for it
+        total = heads * n_b
+        mine = list(range(0, total, sms))           # units of the first thread block
+        assert len(mine) == 10
+        for u in mine[:units]:
+            h, i = divmod(u, n_b)
+            assert i != n_b - 1
+            q[0, h, 128 * i:128 * (i + 1)] += a
+        q, k = q.to(torch.bfloat16), k.to(torch.bfloat16)
+        _, idx, _ = gpu.select(q, k); ref.select(q, k)
+        o, r = gpu.swa(q, k, v), ref.swa(q, k, v)
+        assert gpu.ctx.hf_slow_path_units() == (units if units <= 8 else len(mine))
+        hz.assert_close_out(o, r, "against the warp-level kernel")
+        assert gpu.ctx.hf_get_device_status() == (0, 0)
+    finally:
+        gpu.close(); ref.close()
