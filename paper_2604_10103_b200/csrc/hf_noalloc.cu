@@ -49,6 +49,13 @@ hf_status setup_device(int dev, unsigned char** scratch) {
     return HF_OK;
 }
 
+// Which form of k_reduce_fold adds the partials: six splits in flight where there is more than one trip's worth of them and the
+// D / 16 thread blocks per (batch, head) all run at once, three (and the residency of that form) otherwise.  Both sides of the line,
+// us per call: head_dim 128, 1 000 tokens, 12 batch*heads (96 thread blocks) 17.4 with six, 18.4 with three; 16 of them 19.5, 18.2;
+// 48 28.7, 26.6; 192 85.4, 72.1.  Head_dim 64, 4 680 tokens, 36 (144 thread blocks) 26.7, 27.6; 40 27.3, 26.7; 224 86.4, 84.7.
+template <int D>
+constexpr bool six_in_flight(int nsplit, int bh) { return nsplit > (D == 128 ? 3 : 2) && D / 16 * bh <= (D == 128 ? 104 : 148); }
+
 template <int D>
 hf_status run(const bf16* k, const bf16* v, int bh, int n_tokens, float* S, float* z, unsigned char* scratch, cudaStream_t st) {
     typedef AbsorbMma<D> A;
@@ -65,7 +72,8 @@ hf_status run(const bf16* k, const bf16* v, int bh, int n_tokens, float* S, floa
     k_absorb_mma<D><<<dim3(nsplit, bh), A::THREADS, A::SMEM_BYTES, st>>>(k, v, n_tokens, partials);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) {
-        k_reduce_fold<D, 6><<<dim3(D / 16, bh), 2 * D, 0, st>>>(partials, nsplit, nsplit < 2 ? nsplit : 2, S, z, 1.f, nullptr, 1, bh, nullptr, nullptr, 0ull);
+        auto fold = six_in_flight<D>(nsplit, bh) ? k_reduce_fold<D, 6> : k_reduce_fold<D, 3>;
+        fold<<<dim3(D / 16, bh), 2 * D, 0, st>>>(partials, nsplit, nsplit < 2 ? nsplit : 2, S, z, 1.f, nullptr, 1, bh, nullptr, nullptr, 0ull);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return nfail(HF_ERR_CUDA, "kernel launch failed with error %lld", (long long)e);

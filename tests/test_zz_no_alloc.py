@@ -10,7 +10,9 @@ from tests import harness as hz
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("d,bh_shape,n", [(128, (1, 12), 4680), (64, (2, 3), 333)])
+@pytest.mark.parametrize("d,bh_shape,n", [(128, (1, 12), 4680), (64, (2, 3), 333),
+                                          (128, (2, 7), 500), (64, (2, 19), 400),     # several splits, more thread blocks than run at once
+                                          (128, (1, 3), 190), (64, (1, 3), 128)])     # the most splits that are one trip
 def test_noalloc_absorb_matches_context_absorb_twice_in_a_row(d, bh_shape, n):
     import torch
     from oracle import hybrid_attention as oa
