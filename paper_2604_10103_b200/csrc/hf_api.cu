@@ -196,6 +196,17 @@ void free_all(hf_ctx* c) {
     for (auto& s : c->stage) cudaFree(s);
 }
 
+#ifndef HF_TC5P_COLGROUPS
+#define HF_TC5P_COLGROUPS 1   // column groups per tile group of the ping-pong attention kernel
+#endif
+
+template <int D, int BLK>
+hf_status set_swa_tc5_attr() {
+    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D>::SMEM_BYTES));
+    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D>::SMEM_BYTES));
+    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D>::SMEM_BYTES));
+    return HF_OK;
+}
 template <int BLK, int D>
 hf_status set_swa_attr() {
     HF_CUDA(cudaFuncSetAttribute(k_swa_mma<BLK, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaMma<BLK, D>::SMEM_BYTES));
@@ -217,6 +228,23 @@ hf_status set_state_attr() {
     HF_CUDA(cudaFuncSetAttribute(k_absorb_items<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AbsorbItems<D>::SMEM_BYTES));
     HF_CUDA(cudaFuncSetAttribute(k_absorb_items<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, AbsorbItems<D>::SMEM_BYTES));
     return HF_OK;
+}
+
+// Shared-memory limits of the kernels that a context of this head_dim, block and attention kernel launches: touching a kernel
+// loads it, and the first context of a process would pay for all of them.
+template <int D>
+hf_status set_attrs(const hf_ctx* c) {
+    const int b = c->cfg.block;
+    if (c->swa_kernel == HF_SWA_TCGEN05_PINGPONG)
+        HF_CUDA(cudaFuncSetAttribute(k_swa_tc5p<D, HF_TC5P_COLGROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5P<D, HF_TC5P_COLGROUPS>::SMEM_BYTES));
+    else if (c->swa_kernel == HF_SWA_TCGEN05)
+        HF_TRY((b == 128 ? set_swa_tc5_attr<D, 128>() : b == 64 ? set_swa_tc5_attr<D, 64>() : set_swa_tc5_attr<D, 16>()));
+    else
+        HF_TRY((b == 128 ? set_swa_attr<128, D>() : b == 64 ? set_swa_attr<64, D>() : set_swa_attr<16, D>()));
+    if (c->cfg.merge == HF_MERGE_FULL_WIDTH)
+        HF_CUDA(cudaFuncSetAttribute(k_merge_full<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, MergeFull<D>::SMEM_BYTES));
+    HF_TRY(set_select_attr<D>());
+    return set_state_attr<D>();
 }
 
 #define HF_DISPATCH_D(c, FN, ...) ((c)->d == 128 ? FN<128>(__VA_ARGS__) : FN<64>(__VA_ARGS__))
@@ -546,17 +574,6 @@ hf_status launch_swa_tc5_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16* 
     else HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 0>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
     return post_launch(c, "k_swa_tc5");
 }
-template <int D, int BLK>
-hf_status set_swa_tc5_attr() {
-    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D>::SMEM_BYTES));
-    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D>::SMEM_BYTES));
-    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D>::SMEM_BYTES));
-    return HF_OK;
-}
-
-#ifndef HF_TC5P_COLGROUPS
-#define HF_TC5P_COLGROUPS 1   // column groups per tile group of the ping-pong attention kernel
-#endif
 
 template <int D>
 hf_status launch_swa_tc5p_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_cur, const bf16* v_cur, const int32_t* idx,
@@ -806,10 +823,6 @@ hf_status hf_create(const hf_config* cfg, int device, hf_ctx** out) {
     if (s == HF_OK) s = dmalloc(&c->hist, c->chunk_elems);
     if (s == HF_OK && cfg->merge == HF_MERGE_FULL_WIDTH) s = dmalloc(&c->x_hi, c->chunk_elems);
     if (s == HF_OK && cfg->merge == HF_MERGE_FULL_WIDTH) s = dmalloc(&c->x_lo, c->chunk_elems);
-    if (s == HF_OK && cfg->merge == HF_MERGE_FULL_WIDTH &&
-        (cudaFuncSetAttribute(k_merge_full<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, MergeFull<64>::SMEM_BYTES) != cudaSuccess ||
-         cudaFuncSetAttribute(k_merge_full<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, MergeFull<128>::SMEM_BYTES) != cudaSuccess))
-        s = fail(HF_ERR_CUDA, "cudaFuncSetAttribute(k_merge_full) failed");
     if (s == HF_OK) s = dmalloc(&c->partials, (size_t)c->BH * c->nsplit_max * ((size_t)c->d * c->d + c->d));
     if (s == HF_OK) s = dmalloc(&c->dev_status, (size_t)8);     // status word [4] + self-test results [4]
     if (s == HF_OK && (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
@@ -818,24 +831,7 @@ hf_status hf_create(const hf_config* cfg, int device, hf_ctx** out) {
         s = fail(HF_ERR_CUDA, "could not create the context's side stream / events");
     if (s == HF_OK) {
         cudaMemset(c->dev_status, 0, 32);
-        s = set_swa_attr<16, 64>();
-        if (s == HF_OK) s = set_swa_attr<16, 128>();
-        if (s == HF_OK) s = set_swa_attr<64, 64>();
-        if (s == HF_OK) s = set_swa_attr<64, 128>();
-        if (s == HF_OK) s = set_swa_attr<128, 64>();
-        if (s == HF_OK) s = set_swa_attr<128, 128>();
-        if (s == HF_OK) s = set_swa_tc5_attr<64, 16>();
-        if (s == HF_OK) s = set_swa_tc5_attr<64, 64>();
-        if (s == HF_OK) s = set_swa_tc5_attr<64, 128>();
-        if (s == HF_OK) s = set_swa_tc5_attr<128, 16>();
-        if (s == HF_OK) s = set_swa_tc5_attr<128, 64>();
-        if (s == HF_OK) s = set_swa_tc5_attr<128, 128>();
-        if (s == HF_OK && cudaFuncSetAttribute(k_swa_tc5p<64, HF_TC5P_COLGROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5P<64, HF_TC5P_COLGROUPS>::SMEM_BYTES) != cudaSuccess) s = fail(HF_ERR_CUDA, "cudaFuncSetAttribute(k_swa_tc5p<64>) failed");
-        if (s == HF_OK && cudaFuncSetAttribute(k_swa_tc5p<128, HF_TC5P_COLGROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5P<128, HF_TC5P_COLGROUPS>::SMEM_BYTES) != cudaSuccess) s = fail(HF_ERR_CUDA, "cudaFuncSetAttribute(k_swa_tc5p<128>) failed");
-        if (s == HF_OK) s = set_select_attr<64>();
-        if (s == HF_OK) s = set_select_attr<128>();
-        if (s == HF_OK) s = set_state_attr<64>();
-        if (s == HF_OK) s = set_state_attr<128>();
+        s = HF_DISPATCH_D(c, set_attrs, c);
     }
     if (s == HF_OK && cudaDeviceSynchronize() != cudaSuccess) s = fail(HF_ERR_CUDA, "device synchronize failed in hf_create");
     if (s != HF_OK) { free_all(c); delete c; return s; }
