@@ -77,3 +77,16 @@ def test_create_without_a_device_fails_loudly(lib):
         pytest.skip("a device is present")
     with pytest.raises(hf.HFError, match="HF_ERR_CUDA|HF_ERR_INVALID_ARG"):
         hf.Context(hf.make_config(gen.tiny()))
+
+
+@pytest.mark.parametrize("missing", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_the_stream_handle_without_torchs_raw_getters(monkeypatch, missing):
+    """The raw getters are private to torch: where one is missing the public stream object is asked."""
+    import types
+    import torch
+    for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"):
+        monkeypatch.setattr(torch._C, name, lambda *a: 5, raising=False)
+    assert hf._stream() == 5
+    monkeypatch.delattr(torch._C, missing)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=77))
+    assert hf._stream() == 77
