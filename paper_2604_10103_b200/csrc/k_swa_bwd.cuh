@@ -1,5 +1,6 @@
-// Gradient of the block-sparse attention (Eq. 6) with respect to the queries, on the Blackwell tensor path: the first
-// piece of the backward pass that the training rollout needs for its step with gradient (Alg. 1).  128-token blocks.
+// Gradients of the block-sparse attention (Eq. 6) on the Blackwell tensor path, for the training rollout's step with gradient
+// (Alg. 1): with respect to the queries here, to the current chunk's keys and values in the second half of this file.  128-token
+// blocks.
 //
 // With p = softmax(s) over the kept keys of a query row, s = q k^T / sqrt(d), and g = dL/dO_local:
 //     dq = (1 / sqrt(d)) * sum_c p_c (g . v_c - delta) k_c,     delta = g . o_local     (= sum_c p_c g . v_c)
@@ -25,7 +26,8 @@
 
 // delta[r] = sum_d dO[r][d] * O[r][d].  D / 8 lanes per row (16 bytes of each tensor per lane), four rows per lane with all
 // eight loads in flight: memory-bound (28.75 MB at 12 heads x 4 680 rows x 128: 11.5 us with one row per warp and four bytes
-// per lane, 5.7 us like this).  grid: ceil(rows / (4 * 256 / (D / 8))), 256 threads.
+// per lane, 5.7 us like this).  grid: 1 + ceil(rows / (4 * 256 / (D / 8))), 256 threads; thread block 0 orders
+// the units of the kernel that follows.
 __device__ __forceinline__ float dot8(const uint4& x, const uint4& y) {
     const uint32_t xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
     float acc = 0.f;
@@ -44,7 +46,7 @@ struct RowDot { static constexpr int LPR = D / 8, RPB = 4 * 256 / LPR; };      /
 // 111 kept, i.i.d. or not): in natural order the busiest of 148 thread blocks has 49 pairs and unit ends against a mean of 37,
 // in this order 38.
 struct BwdOrder {
-    const uint32_t* mask;    // [B*H, T_m, mask_words], or nullptr: no ordering
+    const uint32_t* mask;    // [B*H, T_m, mask_words]
     int mask_words, first_block, n_b, Tm, BH;
     int2* order;             // [B*H * n_b]: unit, its pairs (-1: not counted)
 };
@@ -104,8 +106,8 @@ __global__ void __launch_bounds__(256) k_rowdot(const bf16* __restrict__ a, cons
     typedef RowDot<D> C;
     pdl_wait();
     pdl_trigger();              // the backward kernel may set itself up; it waits for this grid before it reads delta
-    if (ord.mask && blockIdx.x == 0) { bwd_order_units(ord); return; }      // (the first thread block: it starts first and ends last)
-    const int block = blockIdx.x - (ord.mask ? 1 : 0);
+    if (blockIdx.x == 0) { bwd_order_units(ord); return; }      // (the first thread block: it starts first and ends last)
+    const int block = blockIdx.x - 1;
     const int part = threadIdx.x % C::LPR;
     const long long r0 = (long long)block * C::RPB + threadIdx.x / C::LPR;
     uint4 x[4], y[4];
@@ -194,8 +196,9 @@ k_swa_bwd_dq(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
     uint8_t* s_gen = smem_raw + (s_base - smem_u32(smem_raw));
     const uint32_t sQ = s_base + C::OFF_Q, sDO = s_base + C::OFF_DO, sK = s_base + C::OFF_K, sV = s_base + C::OFF_V;
     const uint32_t bar0 = s_base + C::OFF_BAR;
-    // half tile s = 2 t + h: pairs of barriers, index h, completion t
-    // (ds, df: pairs, index = half; completion t, like sd and se)
+    // Tile t of the thread block's stream.  K and V rings (kf, ke, vf, ve): index = stage, completion t / stages.  sd (both score
+    // products of tile t complete) and se: completion t.  ds (dS written, four warps) and df: index = half of the key columns,
+    // completion t.
     const uint32_t bar_kf = bar0, bar_ke = bar0 + 48, bar_vf = bar0 + 96, bar_ve = bar0 + 128, bar_sd = bar0 + 160, bar_ds = bar0 + 176,
                    bar_se = bar0 + 192,         // scores of tile t are in registers (eight warps)
                    bar_df = bar0 + 208,         // dS K of a half of tile t complete: its dS slot is free
