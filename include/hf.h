@@ -216,9 +216,10 @@ hf_status hf_linear_attn(hf_ctx* ctx, int layer, const void* q, void* o_hist, vo
 
 /* Eq. 6 + Eq. 4 + Eq. 7 for a selection that is already made (idx as for hf_sparse_swa; NULL = the context's last
  * selection): o = o_local + o_history, rounded once to bf16 [B,H,T_c,d].  hf_hybrid_forward is hf_block_select followed
- * by this call.  With 128-token blocks at head_dim 128 and no rotation tables it is ONE kernel: the attention kernel
- * forms the history term on the tensor cores at the end of each query block; otherwise the read-out kernel runs first
- * and the attention kernel adds its result. */
+ * by this call.  With the tcgen05 attention kernel and the per-head or identity merge, rotated or not, the attention kernel
+ * forms the history term on the tensor cores at the end of each unit of 128 query rows (blocks of 16 and 64 tokens: after a
+ * small kernel that merges the kept lists of a unit); otherwise the read-out kernel runs first and the attention kernel adds
+ * its result. */
 hf_status hf_sparse_swa_merged(hf_ctx* ctx, int layer, const void* q, const void* k_cur, const void* v_cur, const int32_t* idx,
                                void* o, void* stream);
 
