@@ -94,8 +94,11 @@ struct hf_ctx {
     uint32_t* union_entries = nullptr;   // small-block tcgen05 attention: merged kept lists [B*H * units, max tiles, G] ...
     int* union_tiles = nullptr;          // ... and tiles per unit
     int union_max_tiles = 0;
-    float* bwd_delta = nullptr;          // backward pass: g . o_local per query row [B*H, T_c]
-    int2* bwd_order = nullptr;           // ... and the key blocks of the current chunk, most pairs first, with their number [B*H, n_b]
+    // dK / dV: g . o_local per query row [B*H, T_c], and the key blocks of the current chunk, most pairs first, with their number
+    // [B*H, n_b].  Both live in `hist`, which no call holds across another (one stream per context): nothing is allocated by a
+    // backward call, so it can be captured into a graph.
+    float* bwd_delta = nullptr;
+    int2* bwd_order = nullptr;
     float* partials = nullptr;       // absorb split partials
     float* partials_layers = nullptr;    // layer-batched state update: one partial per (layer, batch*head, group)
     size_t partials_layers_count = 0;
@@ -186,7 +189,7 @@ void free_all(hf_ctx* c) {
     for (auto& L : c->layers) { cudaFree(L.W_full); cudaFree(L.mask); cudaFree(L.idx); }
     cudaFree(c->ring_k_all); cudaFree(c->ring_v_all); cudaFree(c->pooled_k_all); cudaFree(c->S_all); cudaFree(c->z_all);
     cudaFree(c->sf_hi_all); cudaFree(c->sf_lo_all); cudaFree(c->W_all); cudaFree(c->bias_all);
-    cudaFree(c->union_entries); cudaFree(c->union_tiles); cudaFree(c->bwd_delta); cudaFree(c->bwd_order); cudaFree(c->pooled_q); cudaFree(c->pooled_kcur); cudaFree(c->hist); cudaFree(c->partials); cudaFree(c->partials_layers); cudaFree(c->x_hi); cudaFree(c->x_lo);
+    cudaFree(c->union_entries); cudaFree(c->union_tiles); cudaFree(c->pooled_q); cudaFree(c->pooled_kcur); cudaFree(c->hist); cudaFree(c->partials); cudaFree(c->partials_layers); cudaFree(c->x_hi); cudaFree(c->x_lo);
     cudaFree(c->dev_status);
     cudaFree(c->rope_q[0]); cudaFree(c->rope_q[1]); cudaFree(c->rope_k[0]); cudaFree(c->rope_k[1]);
     cudaFree(c->trope_tab[0]); cudaFree(c->trope_tab[1]); cudaFree(c->q_rot); cudaFree(c->k_rot);
@@ -815,12 +818,13 @@ hf_status hf_create(const hf_config* cfg, int device, hf_ctx** out) {
         s = dmalloc(&c->union_entries, (size_t)c->BH * Tmt * c->union_max_tiles * G);
         if (s == HF_OK) s = dmalloc(&c->union_tiles, (size_t)c->BH * Tmt);
     }
-    // the backward calls' buffers (they take 128-token blocks): here, so that either call can be captured into a graph
-    if (s == HF_OK && cfg->block == 128) s = dmalloc(&c->bwd_delta, (size_t)c->BH * c->Tc);
-    if (s == HF_OK && cfg->block == 128) s = dmalloc(&c->bwd_order, (size_t)c->BH * c->n_b);
     if (s == HF_OK) s = dmalloc(&c->pooled_q, c->pooled_elems);
     if (s == HF_OK) s = dmalloc(&c->pooled_kcur, c->pooled_elems);
     if (s == HF_OK) s = dmalloc(&c->hist, c->chunk_elems);
+    if (s == HF_OK) {       // (d >= 64 floats per query row: room for its delta and, per 128 rows, a key block's entry)
+        c->bwd_delta = c->hist;
+        c->bwd_order = reinterpret_cast<int2*>(c->hist + ((size_t)c->BH * c->Tc + 3) / 4 * 4);
+    }
     if (s == HF_OK && cfg->merge == HF_MERGE_FULL_WIDTH) s = dmalloc(&c->x_hi, c->chunk_elems);
     if (s == HF_OK && cfg->merge == HF_MERGE_FULL_WIDTH) s = dmalloc(&c->x_lo, c->chunk_elems);
     if (s == HF_OK) s = dmalloc(&c->partials, (size_t)c->BH * c->nsplit_max * ((size_t)c->d * c->d + c->d));
