@@ -215,11 +215,11 @@ hf_status set_swa_attr() {
     HF_CUDA(cudaFuncSetAttribute(k_swa_mma<BLK, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaMma<BLK, D>::SMEM_BYTES));
     return HF_OK;
 }
-template <int D>
+template <int D, int G>
 hf_status set_select_attr() {
-    HF_CUDA(cudaFuncSetAttribute(k_select<D, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D>::smem_bytes(128)));
-    HF_CUDA(cudaFuncSetAttribute(k_select<D, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D>::smem_bytes(256)));
-    HF_CUDA(cudaFuncSetAttribute(k_select<D, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D>::smem_bytes(HF_MAX_TN)));
+    HF_CUDA(cudaFuncSetAttribute(k_select<D, 4, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G>::smem_bytes(128)));
+    HF_CUDA(cudaFuncSetAttribute(k_select<D, 8, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G>::smem_bytes(256)));
+    HF_CUDA(cudaFuncSetAttribute(k_select<D, 32, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G>::smem_bytes(HF_MAX_TN)));
     return HF_OK;
 }
 template <int D>
@@ -231,6 +231,14 @@ hf_status set_state_attr() {
     HF_CUDA(cudaFuncSetAttribute(k_absorb_items<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AbsorbItems<D>::SMEM_BYTES));
     HF_CUDA(cudaFuncSetAttribute(k_absorb_items<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, AbsorbItems<D>::SMEM_BYTES));
     return HF_OK;
+}
+
+// The attention kernel walks merged lists (k_union.cuh), which a forward call's selection forms beside the lists themselves.
+inline bool forward_lists(const hf_ctx* c) { return c->swa_kernel == HF_SWA_TCGEN05 && c->cfg.block != 128; }
+// Tiles of a unit's merged list, at most.
+inline int union_tiles_max(const hf_ctx* c, int keep, int Tn) {
+    const int G = 128 / c->cfg.block, uni = G * keep < Tn ? G * keep : Tn;
+    return (uni + G - 1) / G;
 }
 
 // Shared-memory limits of the kernels that a context of this head_dim, block and attention kernel launches: touching a kernel
@@ -246,7 +254,8 @@ hf_status set_attrs(const hf_ctx* c) {
         HF_TRY((b == 128 ? set_swa_attr<128, D>() : b == 64 ? set_swa_attr<64, D>() : set_swa_attr<16, D>()));
     if (c->cfg.merge == HF_MERGE_FULL_WIDTH)
         HF_CUDA(cudaFuncSetAttribute(k_merge_full<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, MergeFull<D>::SMEM_BYTES));
-    HF_TRY(set_select_attr<D>());
+    HF_TRY((set_select_attr<D, 1>()));
+    if (forward_lists(c)) HF_TRY((b == 64 ? set_select_attr<D, 2>() : set_select_attr<D, 8>()));
     return set_state_attr<D>();
 }
 
@@ -491,9 +500,23 @@ ChunkTable make_table(hf_ctx* c, LayerState& L, const bf16* k_cur, const bf16* v
     return t;
 }
 
+template <int D, int G>
+cudaError_t launch_select_kernel(hf_ctx* c, LayerState& L, const ChunkTable& tab, int Tn, int keep, uint32_t* mask_out, int32_t* idx_out,
+                                 float* scores_out, const UnionOut& lists, cudaStream_t st) {
+    typedef Select<D, G> S;
+    PdlLaunch pl(dim3((c->Tm + S::R - 1) / S::R, c->BH), dim3(S::THREADS), S::smem_bytes(Tn), st, true);      // follows the pooling kernel
+#define HF_SELECT(KPL_) cudaLaunchKernelEx(&pl.cfg, k_select<D, KPL_, G>, tab, (const float*)c->pooled_q, c->n_b, c->Tm, Tn, keep, c->mask_words, \
+                                           L.mask, L.idx, mask_out, idx_out, scores_out, -0.f, lists)
+    if (Tn <= 128) return HF_SELECT(4);             // (registers of the ranking warps: T_n / 32 images per lane)
+    if (Tn <= 256) return HF_SELECT(8);
+    return HF_SELECT(32);
+#undef HF_SELECT
+}
+
+// merged: the attention kernel follows in the same call and takes its merged lists from here.
 template <int D>
 hf_status launch_select(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_cur,
-                        uint32_t* mask_out, int32_t* idx_out, float* scores_out, cudaStream_t st) {
+                        uint32_t* mask_out, int32_t* idx_out, float* scores_out, cudaStream_t st, bool merged = false) {
     PoolJobs jobs;
     memset(&jobs, 0, sizeof(jobs));
     jobs.job[0].src = q;     jobs.job[0].pooled = c->pooled_q;
@@ -507,14 +530,14 @@ hf_status launch_select(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_c
     const int Tn = (L.n_sink + L.n_cached + 1) * c->n_b;
     const int keep = keep_for(c, Tn);
     ChunkTable tab = make_table(c, L, k_cur, nullptr);
-    typedef Select<D> S;
-    PdlLaunch pl(dim3((c->Tm + S::R - 1) / S::R, c->BH), dim3(256), S::smem_bytes(Tn), st, true);      // follows the pooling kernel launched above
-#define HF_SELECT(KPL_) cudaLaunchKernelEx(&pl.cfg, k_select<D, KPL_>, tab, (const float*)c->pooled_q, c->n_b, c->Tm, Tn, keep, c->mask_words, \
-                                           L.mask, L.idx, mask_out, idx_out, scores_out, -0.f)
-    if (Tn <= 128) HF_CUDA(HF_SELECT(4));           // (registers of the ranking warps: T_n / 32 images per lane)
-    else if (Tn <= 256) HF_CUDA(HF_SELECT(8));
-    else HF_CUDA(HF_SELECT(32));
-#undef HF_SELECT
+    UnionOut lists = {nullptr, nullptr, 0, c->Tc};
+    if (!merged) HF_CUDA((launch_select_kernel<D, 1>(c, L, tab, Tn, keep, mask_out, idx_out, scores_out, lists, st)));
+    else {
+        lists.entries = c->union_entries; lists.tiles = c->union_tiles; lists.max_tiles = union_tiles_max(c, keep, Tn);
+        if (lists.max_tiles > c->union_max_tiles) return fail(HF_ERR_SHAPE, "tile list of %d tiles exceeds the %d the context was sized for", lists.max_tiles, c->union_max_tiles);
+        if (c->cfg.block == 64) HF_CUDA((launch_select_kernel<D, 2>(c, L, tab, Tn, keep, mask_out, idx_out, scores_out, lists, st)));
+        else HF_CUDA((launch_select_kernel<D, 8>(c, L, tab, Tn, keep, mask_out, idx_out, scores_out, lists, st)));
+    }
     HF_TRY(post_launch(c, "k_select"));
     L.sel_epoch = L.cache_epoch;
     L.sel_keep = keep;
@@ -532,27 +555,27 @@ hf_status launch_swa_mma_t(hf_ctx* c, const bf16* q, const ChunkTable& tab, cons
 
 
 // The tcgen05 attention kernel.  Blocks of 16 or 64 tokens: first the kept lists of the query blocks that share a 128-row unit
-// are merged (k_union_tiles).  hist_inside: the kernel forms the history term; overlap_prev: it may be launched under the tail
+// are merged (k_union_tiles), unless the selection of the same call has done that (merged).  hist_inside: the kernel forms the history term; overlap_prev: it may be launched under the tail
 // of the kernel before it in the stream.
 template <int D, int BLK>
 hf_status launch_swa_tc5_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_cur, const bf16* v_cur, const int32_t* idx,
-                           int keep, const float* hist, bf16* o, float* lse, cudaStream_t st, bool hist_inside, bool overlap_prev) {
+                           int keep, const float* hist, bf16* o, float* lse, cudaStream_t st, bool hist_inside, bool overlap_prev, bool merged) {
     typedef SwaTc5<D> C;
-    constexpr int G = 128 / BLK;
     Tc5Params p;
     memset(&p, 0, sizeof(p));
     p.upb = (c->Tc + 127) / 128; p.n_units = p.upb * c->BH;
     if (BLK != 128) {
         const int Tn = (L.n_sink + L.n_cached + 1) * c->n_b;
-        const int uni = G * keep < Tn ? G * keep : Tn;
-        const int max_tiles = (uni + G - 1) / G;
+        const int max_tiles = union_tiles_max(c, keep, Tn);
         if (max_tiles > c->union_max_tiles) return fail(HF_ERR_SHAPE, "tile list of %d tiles exceeds the %d the context was sized for", max_tiles, c->union_max_tiles);
-        PdlLaunch pu(dim3(p.upb, c->BH), dim3(256), 0, st, true);
-        HF_CUDA(cudaLaunchKernelEx(&pu.cfg, k_union_tiles<BLK>, idx, keep, c->Tm, Tn, c->n_b, c->Tc, max_tiles, c->union_entries, c->union_tiles,
-                                   c->dev_status));
-        HF_TRY(post_launch(c, "k_union_tiles"));
+        if (!merged) {
+            const UnionOut lists = {c->union_entries, c->union_tiles, max_tiles, c->Tc};
+            PdlLaunch pu(dim3(p.upb, c->BH), dim3(256), 0, st, true);
+            HF_CUDA(cudaLaunchKernelEx(&pu.cfg, k_union_tiles<BLK>, idx, keep, c->Tm, Tn, c->n_b, lists, c->dev_status));
+            HF_TRY(post_launch(c, "k_union_tiles"));
+            overlap_prev = true;
+        }
         p.entries = c->union_entries; p.tiles = c->union_tiles; p.max_tiles = max_tiles;
-        overlap_prev = true;
     }
     CUtensorMap tq, tk, tv, to;
     HF_TRY(make_map(c, &tq, q, 1));
@@ -602,10 +625,10 @@ hf_status launch_swa_tc5p_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16*
 
 // hist_inside: the attention kernel forms the history term itself (the tcgen05 kernel only).
 hf_status launch_swa(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_cur, const bf16* v_cur, const int32_t* idx,
-                     int keep, const float* hist, bf16* o, float* lse, cudaStream_t st, bool hist_inside = false, bool overlap_prev = false) {
+                     int keep, const float* hist, bf16* o, float* lse, cudaStream_t st, bool hist_inside = false, bool overlap_prev = false, bool merged = false) {
     if (c->swa_kernel == HF_SWA_TCGEN05) {
         const int b = c->cfg.block, d = c->d;
-#define HF_TC5_CASE(D_, B_) if (d == D_ && b == B_) return launch_swa_tc5_t<D_, B_>(c, L, q, k_cur, v_cur, idx, keep, hist, o, lse, st, hist_inside, overlap_prev)
+#define HF_TC5_CASE(D_, B_) if (d == D_ && b == B_) return launch_swa_tc5_t<D_, B_>(c, L, q, k_cur, v_cur, idx, keep, hist, o, lse, st, hist_inside, overlap_prev, merged)
         HF_TC5_CASE(128, 128); HF_TC5_CASE(128, 64); HF_TC5_CASE(128, 16); HF_TC5_CASE(64, 128); HF_TC5_CASE(64, 64); HF_TC5_CASE(64, 16);
 #undef HF_TC5_CASE
     }
@@ -1219,14 +1242,14 @@ static bool one_kernel_forward(const hf_ctx* c) {
 }
 
 // Eq. 6 + Eq. 4 + Eq. 7 for a selection that is already made.  after_select: the call follows launch_select in the same
-// stream directly, so the attention kernel may be launched under its tail.
+// stream directly, so the attention kernel may be launched under its tail.  merged: that selection has formed the merged lists.
 static hf_status attend_merge(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k, const bf16* v, const int32_t* idx, int keep,
-                              bf16* o, cudaStream_t st, bool after_select) {
-    if (one_kernel_forward(c)) return launch_swa(c, L, q, k, v, idx, keep, nullptr, o, nullptr, st, true, after_select);
+                              bf16* o, cudaStream_t st, bool after_select, bool merged = false) {
+    if (one_kernel_forward(c)) return launch_swa(c, L, q, k, v, idx, keep, nullptr, o, nullptr, st, true, after_select, merged);
     // Otherwise the read-out kernel writes the history term to the context's scratch buffer and the attention kernel adds
     // it in its epilogue.
     HF_TRY(HF_DISPATCH_D(c, launch_readout, c, L, q, (bf16*)nullptr, c->hist, st));
-    return launch_swa(c, L, q, k, v, idx, keep, c->hist, o, nullptr, st);
+    return launch_swa(c, L, q, k, v, idx, keep, c->hist, o, nullptr, st, false, false, merged);
 }
 
 hf_status hf_sparse_swa_merged(hf_ctx* c, int layer, const void* q, const void* k_cur, const void* v_cur, const int32_t* idx,
@@ -1257,13 +1280,13 @@ hf_status hf_hybrid_forward(hf_ctx* c, int layer, const void* q, const void* k, 
     HF_TRY(check_ptr(o, "o"));
     LayerState& L = c->layers[layer];
     cudaStream_t st = (cudaStream_t)stream;
-    const bool one_kernel = one_kernel_forward(c);
+    const bool one_kernel = one_kernel_forward(c), merged = forward_lists(c);
     if (one_kernel || c->has_trope) {
         // (with the temporal rotation the selection's pooling pass also writes the rotated q and k that everything after it
         // reads, so the history read-out cannot run beside it: one stream)
-        HF_TRY(HF_DISPATCH_D(c, launch_select, c, L, (const bf16*)q, (const bf16*)k, (uint32_t*)nullptr, (int32_t*)nullptr, (float*)nullptr, st));
+        HF_TRY(HF_DISPATCH_D(c, launch_select, c, L, (const bf16*)q, (const bf16*)k, (uint32_t*)nullptr, (int32_t*)nullptr, (float*)nullptr, st, merged));
         if (c->has_trope) { q = c->q_rot; k = c->k_rot; }
-        return attend_merge(c, L, (const bf16*)q, (const bf16*)k, (const bf16*)v, L.idx, L.sel_keep, (bf16*)o, st, one_kernel);
+        return attend_merge(c, L, (const bf16*)q, (const bf16*)k, (const bf16*)v, L.idx, L.sel_keep, (bf16*)o, st, one_kernel, merged);
     }
     // Otherwise the history term depends on q and the state only: it runs on the context's side stream while pooling and
     // selection run on the caller's stream; the attention kernel, which adds it in its epilogue, waits for both.
@@ -1273,9 +1296,9 @@ hf_status hf_hybrid_forward(hf_ctx* c, int layer, const void* q, const void* k, 
     HF_CUDA(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
     HF_TRY(HF_DISPATCH_D(c, launch_readout, c, L, (const bf16*)q, (bf16*)nullptr, c->hist, c->side));
     HF_CUDA(cudaEventRecord(c->ev_join, c->side));
-    HF_TRY(HF_DISPATCH_D(c, launch_select, c, L, (const bf16*)q, (const bf16*)k, (uint32_t*)nullptr, (int32_t*)nullptr, (float*)nullptr, st));
+    HF_TRY(HF_DISPATCH_D(c, launch_select, c, L, (const bf16*)q, (const bf16*)k, (uint32_t*)nullptr, (int32_t*)nullptr, (float*)nullptr, st, merged));
     HF_CUDA(cudaStreamWaitEvent(st, c->ev_join, 0));
-    return launch_swa(c, L, (const bf16*)q, (const bf16*)k, (const bf16*)v, L.idx, L.sel_keep, c->hist, (bf16*)o, nullptr, st);
+    return launch_swa(c, L, (const bf16*)q, (const bf16*)k, (const bf16*)v, L.idx, L.sel_keep, c->hist, (bf16*)o, nullptr, st, false, false, merged);
 }
 
 hf_status hf_hybrid_forward_host(hf_ctx* c, int layer, const void* q_host, const void* k_host, const void* v_host,

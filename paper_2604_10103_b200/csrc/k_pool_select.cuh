@@ -7,6 +7,7 @@
 //   (multiply and add rounded separately, never fused); partials folded as a butterfly +16, +8, +4, +2, +1.
 #pragma once
 #include "hf_common.cuh"
+#include "k_union.cuh"
 
 template <int VEC> struct VecLoad;
 template <> struct VecLoad<8> {
@@ -242,9 +243,13 @@ __global__ void __launch_bounds__(256, 6) k_pool_copy_layers(const __grid_consta
 // pooling + selection as part of the forward, 12 heads of 128: 128-token blocks (T_n 111) 128.3 -> 125.5 us, 64-token blocks
 // (T_n 222) 171 -> 164 us, 16-token blocks at head dim 64 (T_n 246) 64.6 -> 55.1 us; this kernel alone at T_n 259, batch 4:
 // 76 -> 39 us.
-template <int D>
+// G: the query blocks that share a unit of the attention kernel (blocks of 64 tokens: 2, of 16: 8), whose merged list is formed here
+// from the masks in shared memory, or 1: none is asked for.  A kernel of its own behind this one costs a launch (k_union.cuh).  G = 8
+// takes eight query blocks, one unit, per thread block, with as many threads per score.
+template <int D, int G = 1>
 struct Select {
-    static constexpr int R = 4, KT = 128;       // query blocks per thread block; key rows per pass
+    static constexpr int R = G == 8 ? 8 : 4, KT = 128;       // query blocks per thread block; key rows per pass
+    static constexpr int THREADS = 64 * R;
     static constexpr int LD = D + 4;            // floats per key row in shared memory
     static int smem_bytes(int Tn) { const int kt = Tn < KT ? Tn : KT; return (kt * LD + R * D + R * Tn) * (int)sizeof(float); }
 };
@@ -302,19 +307,20 @@ __device__ __forceinline__ uint32_t score_image(float s) {
 }
 
 // KPL: key blocks per lane of a ranking warp (T_n <= 32 KPL).
-template <int D, int KPL>
-__global__ void __launch_bounds__(256) k_select(ChunkTable tab, const float* __restrict__ pooled_q,
+template <int D, int KPL, int G>
+__global__ void __launch_bounds__(Select<D, G>::THREADS) k_select(ChunkTable tab, const float* __restrict__ pooled_q,
                                                 int n_b, int Tm, int Tn, int keep, int mask_words,
                                                 uint32_t* __restrict__ mask, int32_t* __restrict__ idx,
                                                 uint32_t* __restrict__ mask_out, int32_t* __restrict__ idx_out,
-                                                float* __restrict__ scores_out, float neg_zero) {
-    typedef Select<D> C;
+                                                float* __restrict__ scores_out, float neg_zero, UnionOut lists) {
+    typedef Select<D, G> C;
     const float2 nz = make_float2(neg_zero, neg_zero);
     extern __shared__ __align__(16) float sel_smem[];
     const int kt = min(Tn, C::KT);
     float* s_k = sel_smem;                      // [kt][LD]
     float* s_q = s_k + kt * C::LD;              // [R][D]
     float* s_sc = s_q + C::R * D;               // [R][Tn]
+    __shared__ uint32_t s_mask[G > 1 ? C::R : 1][32];
     const int i0 = blockIdx.x * C::R, bh = blockIdx.y;
     const int rows = min(C::R, Tm - i0);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -322,7 +328,7 @@ __global__ void __launch_bounds__(256) k_select(ChunkTable tab, const float* __r
     // key rows [j0, j1) of the pass that starts at `base`, sixteen bytes per thread and step
     auto load_keys = [&](int base, int j0, int j1) {
         constexpr int V = D / 4;
-        for (int e = threadIdx.x; e < (j1 - j0) * V; e += 256) {
+        for (int e = threadIdx.x; e < (j1 - j0) * V; e += C::THREADS) {
             const int j = j0 + e / V, part = e % V;
             int c = 0, jb = j;
             while (jb >= n_b) { jb -= n_b; ++c; }
@@ -335,7 +341,7 @@ __global__ void __launch_bounds__(256) k_select(ChunkTable tab, const float* __r
     const int old = min((tab.n_chunks - 1) * n_b, kt);
     load_keys(0, 0, old);
     pdl_wait();                 // the pooled rows of the queries and of the current chunk come from the kernel before
-    for (int e = threadIdx.x; e < rows * (D / 4); e += 256)
+    for (int e = threadIdx.x; e < rows * (D / 4); e += C::THREADS)
         cp_async16(smem_u32(s_q) + e * 16, pooled_q + ((size_t)bh * Tm + i0) * D + e * 4, true);
     load_keys(0, old, kt);
     for (int base = 0; base < Tn; base += C::KT) {
@@ -365,55 +371,69 @@ __global__ void __launch_bounds__(256) k_select(ChunkTable tab, const float* __r
     }
     __syncthreads();
     if (scores_out)
-        for (int e = threadIdx.x; e < rows * Tn; e += 256) scores_out[((size_t)bh * Tm + i0) * Tn + e] = s_sc[e];
-    if (warp >= rows) return;
-    // ---- top-K of row `warp`: lane l holds the images of blocks l, l + 32, ... (padding: 0, and behind every block)
-    const size_t row = (size_t)bh * Tm + i0 + warp;
-    uint32_t key[KPL];
-#pragma unroll
-    for (int x = 0; x < KPL; ++x) {
-        const int j = x * 32 + lane;
-        key[x] = j < Tn ? score_image(s_sc[warp * Tn + j]) : 0u;
+        for (int e = threadIdx.x; e < rows * Tn; e += C::THREADS) scores_out[((size_t)bh * Tm + i0) * Tn + e] = s_sc[e];
+    if constexpr (G == 1) {
+        if (warp >= rows) return;
+    } else {
+        if (warp < C::R) s_mask[warp][lane] = 0;        // (query blocks past T_m keep nothing)
     }
-    uint32_t thr = 0;           // largest value with at least `keep` images at or above it
-    bool exact = keep >= Tn;    // ... and exactly `keep`: no ties to cut (all blocks kept: every image counts)
-    for (uint32_t bit = 0x80000000u; bit != 0u && !exact; bit >>= 1) {
-        const uint32_t cand = thr | bit;
-        int n = 0;
+    if (warp < rows) {
+        // ---- top-K of row `warp`: lane l holds the images of blocks l, l + 32, ... (padding: 0, and behind every block)
+        const size_t row = (size_t)bh * Tm + i0 + warp;
+        uint32_t key[KPL];
 #pragma unroll
-        for (int x = 0; x < KPL; ++x) n += key[x] >= cand;
-        n = __reduce_add_sync(0xffffffffu, n);
-        if (n >= keep) { thr = cand; exact = n == keep; }
-    }
-    int ties = Tn;              // blocks at the threshold still to be kept, lowest index first
-    if (!exact) {
-        int n = 0;
-#pragma unroll
-        for (int x = 0; x < KPL; ++x) n += key[x] > thr;
-        ties = keep - __reduce_add_sync(0xffffffffu, n);
-    }
-    const uint32_t below = (1u << lane) - 1u;
-    int pos = 0;
-    uint32_t my_word = 0;
-#pragma unroll
-    for (int x = 0; x < KPL; ++x) {
-        const int j = x * 32 + lane;
-        const uint32_t eq = __ballot_sync(0xffffffffu, j < Tn && key[x] == thr);
-        const bool kept = j < Tn && (key[x] > thr || (key[x] == thr && __popc(eq & below) < ties));
-        ties -= __popc(eq);
-        const uint32_t word = __ballot_sync(0xffffffffu, kept);
-        if (lane == x) my_word = word;
-        if (kept) {
-            const int at = pos + __popc(word & below);
-            if (at < keep) {    // (always true under the total order above; the store never leaves the row)
-                idx[row * keep + at] = j;
-                if (idx_out) idx_out[row * keep + at] = j;
-            }
+        for (int x = 0; x < KPL; ++x) {
+            const int j = x * 32 + lane;
+            key[x] = j < Tn ? score_image(s_sc[warp * Tn + j]) : 0u;
         }
-        pos += __popc(word);
+        uint32_t thr = 0;           // largest value with at least `keep` images at or above it
+        bool exact = keep >= Tn;    // ... and exactly `keep`: no ties to cut (all blocks kept: every image counts)
+        for (uint32_t bit = 0x80000000u; bit != 0u && !exact; bit >>= 1) {
+            const uint32_t cand = thr | bit;
+            int n = 0;
+#pragma unroll
+            for (int x = 0; x < KPL; ++x) n += key[x] >= cand;
+            n = __reduce_add_sync(0xffffffffu, n);
+            if (n >= keep) { thr = cand; exact = n == keep; }
+        }
+        int ties = Tn;              // blocks at the threshold still to be kept, lowest index first
+        if (!exact) {
+            int n = 0;
+#pragma unroll
+            for (int x = 0; x < KPL; ++x) n += key[x] > thr;
+            ties = keep - __reduce_add_sync(0xffffffffu, n);
+        }
+        const uint32_t below = (1u << lane) - 1u;
+        int pos = 0;
+        uint32_t my_word = 0;
+#pragma unroll
+        for (int x = 0; x < KPL; ++x) {
+            const int j = x * 32 + lane;
+            const uint32_t eq = __ballot_sync(0xffffffffu, j < Tn && key[x] == thr);
+            const bool kept = j < Tn && (key[x] > thr || (key[x] == thr && __popc(eq & below) < ties));
+            ties -= __popc(eq);
+            const uint32_t word = __ballot_sync(0xffffffffu, kept);
+            if (lane == x) my_word = word;
+            if (kept) {
+                const int at = pos + __popc(word & below);
+                if (at < keep) {    // (always true under the total order above; the store never leaves the row)
+                    idx[row * keep + at] = j;
+                    if (idx_out) idx_out[row * keep + at] = j;
+                }
+            }
+            pos += __popc(word);
+        }
+        if (lane < mask_words) {
+            mask[row * mask_words + lane] = my_word;
+            if (mask_out) mask_out[row * mask_words + lane] = my_word;
+        }
+        if constexpr (G > 1) s_mask[warp][lane] = my_word;      // (lanes past the words of T_n: 0)
     }
-    if (lane < mask_words) {
-        mask[row * mask_words + lane] = my_word;
-        if (mask_out) mask_out[row * mask_words + lane] = my_word;
+    if constexpr (G > 1) {
+        // ---- the merged lists of the units of these query blocks, the warps shared out among them
+        constexpr int UNITS = C::R / G, WPU = C::THREADS / 32 / UNITS;
+        __syncthreads();
+        const int x = warp / WPU, mt = (int)blockIdx.x * UNITS + x, upb = (Tm + G - 1) / G;
+        if (mt < upb) union_lists<G>(s_mask + x * G, warp % WPU, WPU, Tn, n_b, bh * upb + mt, lists);
     }
 }

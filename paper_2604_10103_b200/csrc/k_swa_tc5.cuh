@@ -54,6 +54,7 @@
 #pragma once
 #include "tc5_common.cuh"
 #include "k_swa_mma.cuh"
+#include "k_union.cuh"
 
 template <int D>
 struct SwaTc5 {
@@ -134,75 +135,6 @@ struct RingPos {
     uint32_t phase = 0;
     __device__ __forceinline__ void advance() { if (++stage == N) { stage = 0; phase ^= 1u; } }
 };
-
-// One list entry: key block index (10 bits) | row groups that keep it (8 bits) << 10 | valid tokens in the block << 18.
-__host__ __device__ __forceinline__ uint32_t union_entry(int blk, uint32_t rows, int nv) { return (uint32_t)blk | (rows << 10) | ((uint32_t)nv << 18); }
-
-// grid (units per batch*head, B*H), 256 threads.  idx: [B*H, T_m, keep] kept lists (ascending).  Out: entries
-// [B*H * units, max_tiles, G] and tiles [B*H * units]; slots past the union in a unit's last tile repeat its first block with
-// no row group (they are loaded -- every box of a tile must hold finite numbers -- and fully masked).
-template <int BLK>
-__global__ void __launch_bounds__(256) k_union_tiles(const int32_t* __restrict__ idx, int keep, int Tm, int Tn, int n_b, int Tc, int max_tiles,
-                                                     uint32_t* __restrict__ entries, int* __restrict__ tiles, int* dev_status) {
-    constexpr int G = 128 / BLK;
-    __shared__ uint32_t rows[HF_MAX_TN];          // bits 0..7: row groups keeping the block; bit 8: some row group's first kept block
-    __shared__ int warp_tot[2][8];
-    const int mt = blockIdx.x, bh = blockIdx.y, units = gridDim.x;
-    const int unit = bh * units + mt;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int j = threadIdx.x; j < Tn; j += 256) rows[j] = 0;
-    __syncthreads();
-    pdl_wait();                 // the lists come from the selection kernel launched before this one
-    pdl_trigger();
-    for (int e = threadIdx.x; e < G * keep; e += 256) {
-        const int r = e / keep, jj = e - r * keep, qb = mt * G + r;
-        if (qb < Tm) {
-            const int j = checked_block(__ldg(idx + ((size_t)bh * Tm + qb) * keep + jj), Tn, dev_status, bh * Tm + qb);
-            atomicOr(&rows[j], (1u << r) | (jj == 0 ? 0x100u : 0u));
-        }
-    }
-    __syncthreads();
-    // compaction: the first-kept blocks (ascending), then the rest of the union (ascending); thread t looks at blocks 4t .. 4t+3
-    uint32_t w[4];
-    int nA = 0, nB = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int j = threadIdx.x * 4 + i;
-        w[i] = j < Tn ? rows[j] : 0u;
-        nA += (w[i] & 0x100u) != 0;
-        nB += (w[i] & 0xffu) != 0 && !(w[i] & 0x100u);
-    }
-    int pA = nA, pB = nB;       // inclusive scans inside the warp
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const int a = __shfl_up_sync(0xffffffffu, pA, off), b = __shfl_up_sync(0xffffffffu, pB, off);
-        if (lane >= off) { pA += a; pB += b; }
-    }
-    if (lane == 31) { warp_tot[0][warp] = pA; warp_tot[1][warp] = pB; }
-    __syncthreads();
-    int baseA = 0, baseB = 0, totA = 0, totB = 0;
-#pragma unroll
-    for (int x = 0; x < 8; ++x) {
-        if (x < warp) { baseA += warp_tot[0][x]; baseB += warp_tot[1][x]; }
-        totA += warp_tot[0][x]; totB += warp_tot[1][x];
-    }
-    int posA = baseA + pA - nA, posB = totA + baseB + pB - nB;
-    uint32_t* out = entries + (size_t)unit * max_tiles * G;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int j = threadIdx.x * 4 + i;
-        if ((w[i] & 0xffu) == 0) continue;
-        int jb = j;
-        while (jb >= n_b) jb -= n_b;
-        const int nv = jb == n_b - 1 ? Tc - jb * BLK : BLK;
-        const uint32_t ent = union_entry(j, w[i] & 0xffu, nv);
-        if (w[i] & 0x100u) out[posA++] = ent; else out[posB++] = ent;
-    }
-    __syncthreads();
-    const int total = totA + totB, n_tiles = (total + G - 1) / G;
-    if (threadIdx.x < n_tiles * G - total) out[total + threadIdx.x] = union_entry((int)(out[0] & 1023u), 0u, BLK);
-    if (threadIdx.x == 0) tiles[unit] = n_tiles;
-}
 
 // One unit again, the way Alg. 3 prints it (running maximum m, rescaling of l and O), by threads 0 .. 255 of the thread
 // block, after the tile stream has drained (shared memory and the exchange buffers are free by then).  HIST: the history
