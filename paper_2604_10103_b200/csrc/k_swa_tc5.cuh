@@ -327,6 +327,12 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS);
         tmem_relinquish();
     }
+    if (warp == C::WARP_LOAD_K && lane == 0) { tma_prefetch_map(&tm_kring); tma_prefetch_map(&tm_kcur); }
+    if (warp == C::WARP_LOAD_V && lane == 0) {
+        tma_prefetch_map(&tm_q); tma_prefetch_map(&tm_vring); tma_prefetch_map(&tm_vcur);
+        if (HIST) { tma_prefetch_map(&tm_sh); tma_prefetch_map(&tm_sl); }
+    }
+    if (warp == 0 && lane == 0) tma_prefetch_map(&tm_o);
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
@@ -345,14 +351,40 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
 
     if (warp == C::WARP_LOAD_K || warp == C::WARP_LOAD_V) {
         // ================================================================= TMA producers
-        if (lane == 0) {
-            const bool is_k = (warp == C::WARP_LOAD_K);
-            bool ok = true;
-            int t = 0;
-            const int Tn = p.Tn;
-            const uint32_t tiles = is_k ? sK : sV, full = is_k ? bar_kf : bar_vf, freed = is_k ? bar_sf : bar_pv;
-            // one box of BLK rows of key block blk
-            auto load_block = [&](int blk, uint32_t dst, uint32_t bar, int bh) {
+        // One lane copies a tile of a 128-token block; blocks of 16 or 64 tokens have a lane each (G boxes a tile: one after the other, with
+        // their list entries' loads between them, they bounded the tile loop: 16-token blocks, 12 heads, 1 300 queries, 62 of 246 blocks
+        // kept 53 -> 32.5 us at head dim 64, 69 -> 41 at 128).  The loops are the warp's.
+        const bool is_k = (warp == C::WARP_LOAD_K);
+        const int box = lane < G ? lane : 0;
+        bool ok = true;
+        int t = 0;
+        const int Tn = p.Tn;
+        const uint32_t tiles = is_k ? sK : sV, full = is_k ? bar_kf : bar_vf, freed = is_k ? bar_sf : bar_pv;
+        auto list_of = [&](int u) -> const uint32_t* {
+            if constexpr (BLK == 128) return reinterpret_cast<const uint32_t*>(p.idx + (size_t)u * p.keep);
+            else return p.entries + (size_t)u * p.max_tiles * G + box;
+        };
+        uint32_t e_next = my_units > 0 ? __ldg(list_of(blockIdx.x)) : 0u;      // list entry, read one tile ahead
+        for (int n = 0; ok && n < my_units; ++n) {
+            const int u = blockIdx.x + n * gridDim.x;
+            const int bh = u / p.upb, i = u - bh * p.upb;
+            const int cnt = tiles_of(n);
+            if (!is_k) {   // Q of this unit, once the softmax warps are done with the previous one
+                if (n >= 1 && !(ok = wait_w(bar_qe, n - 1, 1))) break;
+                if (lane == 0) {
+                    mbar_expect_tx(bar_qf, C::TILE_BYTES);
+#pragma unroll
+                    for (int s = 0; s < C::SUB; ++s) tma_load_4d(sQ + s * C::SUB_BYTES, &tm_q, s * 64, i * 128, bh, 0, bar_qf);
+                }
+                __syncwarp();
+            }
+            const uint32_t* list = list_of(u);
+            for (int j = 0; j < cnt; ++j, ++t) {
+                const uint32_t st = t & 1, dst = tiles + st * C::TILE_BYTES + box * BLK * 128, bar = full + 8 * st;
+                int blk;
+                if constexpr (BLK == 128) blk = checked_block((int)e_next, Tn, is_k && lane == 0 ? p.dev_status : nullptr, u);
+                else { blk = (int)(e_next & 1023u); if (blk >= Tn) blk = 0; }          // (the list builder has checked every entry already)
+                e_next = __ldg(j + 1 < cnt ? list + (j + 1) * G : list_of(n + 1 < my_units ? u + (int)gridDim.x : u));
                 int c = 0, jb = blk;
                 while (jb >= p.n_b) { jb -= p.n_b; ++c; }          // at most HF_MAX_CHUNKS - 1 steps; no XU-pipe division
                 // logical chunk order: sink chunks (slots P, P + 1, ...), cached chunks oldest first (ring), current chunk
@@ -363,41 +395,20 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                     else { slot = p.ring_head + c - p.n_sink; if (slot >= p.P) slot -= p.P; }
                 }
                 const CUtensorMap* m = is_k ? (cur ? &tm_kcur : &tm_kring) : (cur ? &tm_vcur : &tm_vring);
+                if (t >= 2 && !(ok = wait_w(freed + 8 * st, (t >> 1) - 1, 2))) break;
+                if (lane == 0) mbar_expect_tx(bar, C::TILE_BYTES);
+                __syncwarp();
+                if (lane < G) {
 #pragma unroll
-                for (int s = 0; s < C::SUB; ++s) tma_load_4d(dst + s * C::SUB_BYTES, m, s * 64, jb * BLK, bh, slot, bar);
-            };
-            for (int n = 0; ok && n < my_units; ++n) {
-                const int u = blockIdx.x + n * gridDim.x;
-                const int bh = u / p.upb, i = u - bh * p.upb;
-                const int cnt = tiles_of(n);
-                if (!is_k) {   // Q of this unit, once the softmax warps are done with the previous one
-                    if (n >= 1 && !(ok = mbar_wait<true>(bar_qe, (n - 1) & 1, abort_flag, p.dev_status, 1))) break;
-                    mbar_expect_tx(bar_qf, C::TILE_BYTES);
-#pragma unroll
-                    for (int s = 0; s < C::SUB; ++s) tma_load_4d(sQ + s * C::SUB_BYTES, &tm_q, s * 64, i * 128, bh, 0, bar_qf);
+                    for (int s = 0; s < C::SUB; ++s) tma_load_4d(dst + s * C::SUB_BYTES, m, s * 64, jb * BLK, bh, slot, bar);
                 }
-                for (int j = 0; j < cnt; ++j, ++t) {
-                    const uint32_t st = t & 1, dst = tiles + st * C::TILE_BYTES, bar = full + 8 * st;
-                    if constexpr (BLK == 128) {
-                        const int blk = checked_block(__ldg(p.idx + (size_t)u * p.keep + j), Tn, is_k ? p.dev_status : nullptr, u);
-                        if (t >= 2 && !(ok = mbar_wait<true>(freed + 8 * st, ((t >> 1) & 1) ^ 1, abort_flag, p.dev_status, 2))) break;
-                        mbar_expect_tx(bar, C::TILE_BYTES);
-                        load_block(blk, dst, bar, bh);
-                    } else {
-                        const uint32_t* ent = p.entries + ((size_t)u * p.max_tiles + j) * G;
-                        if (t >= 2 && !(ok = mbar_wait<true>(freed + 8 * st, ((t >> 1) & 1) ^ 1, abort_flag, p.dev_status, 3))) break;
-                        mbar_expect_tx(bar, C::TILE_BYTES);
-#pragma unroll
-                        for (int g = 0; g < G; ++g) {
-                            const int blk = (int)(__ldg(ent + g) & 1023u);
-                            load_block(blk < Tn ? blk : 0, dst + g * BLK * 128, bar, bh);   // (the list builder has checked every entry already)
-                        }
-                    }
-                    if (HIST && !is_k && j == (cnt > 1 ? 1 : 0)) {
-                        // For the history term at the unit's end: the head's folded state and z.  The buffer is free once the
-                        // previous unit's output, which was staged in it, has been read by the bulk stores.  (Two V tiles of
-                        // this unit are on their way by now; the third needs P V of the first, which comes after that.)
-                        if (n >= 1 && !(ok = mbar_wait<true>(bar_he, (n - 1) & 1, abort_flag, p.dev_status, 13))) break;
+                __syncwarp();
+                if (HIST && !is_k && j == (cnt > 1 ? 1 : 0)) {
+                    // For the history term at the unit's end: the head's folded state and z.  The buffer is free once the
+                    // previous unit's output, which was staged in it, has been read by the bulk stores.  (Two V tiles of
+                    // this unit are on their way by now; the third needs P V of the first, which comes after that.)
+                    if (n >= 1 && !(ok = wait_w(bar_he, n - 1, 13))) break;
+                    if (lane == 0) {
                         mbar_expect_tx(bar_hf, 2 * C::H_BYTES + D * 4);
 #pragma unroll
                         for (int s = 0; s < C::SUB; ++s) {
@@ -406,12 +417,13 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                         }
                         bulk_load(s_base + C::OFF_Z, p.z + (size_t)bh * D, D * 4, bar_hf);
                     }
+                    __syncwarp();
                 }
             }
-            if (!ok) {   // gave up: let the copies already in flight land before the CTA leaves
-                const long long t0 = clock64();
-                while (clock64() - t0 < 400000) {}
-            }
+        }
+        if (!ok) {   // gave up: let the copies already in flight land before the CTA leaves
+            const long long t0 = clock64();
+            while (clock64() - t0 < 400000) {}
         }
     } else if (warp == C::WARP_S) {
         // ================================================================= S = Q K^T
@@ -759,6 +771,8 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                 if (HIST && n >= 1 && j == 0 && cnt > 1) release_h();
             }
             if (!ok) break;
+            // (a thread block that leaves room beside it lets the next kernel in only now: that one waits, but its blocks take slots)
+            if (C::SMEM_BYTES <= 200 * 1024 && n + 1 == my_units) pdl_trigger();
             // ---- end of the unit: row sums (and the shares of Eq. 4's denominator) of the column groups, range test, output
             const bf16* bias_row = (HIST && p.bias) ? p.bias + (size_t)(bh % p.heads) * D + grp * C::OCOLS : nullptr;
             uint4 bw[C::OCOLS / 8];
@@ -844,7 +858,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             if (i >= p.upb) { i -= p.upb; ++bh; }
         }
     }
-    if (warp < C::NSW && lane == 0) bulk_wait_all();     // output tiles still on their way out of shared memory
+    if (warp < C::NSW && lane == 0) bulk_wait_read();    // output tiles still on their way out of shared memory
     fence_before_sync();
     __syncthreads();
     if (warp == C::WARP_S) {
@@ -855,7 +869,8 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
     // of the tile stream has completed (the roles above drain before the barrier), so shared memory is free.
     const int n_redo = *redo_cnt;
     if (n_redo > 0 && *abort_flag == 0 && threadIdx.x < 256) {
-        fence_proxy_async();                                  // the tile stream's bulk stores of these rows came first
+        if (lane == 0) bulk_wait_all();                       // the tile stream's bulk stores of these rows come first
+        fence_proxy_async();
         const int total = n_redo > C::REDO_CAP ? my_units : n_redo;
         for (int r = 0; r < total; ++r) {
             const int n = n_redo > C::REDO_CAP ? r : redo_list[r];
