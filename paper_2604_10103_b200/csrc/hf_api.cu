@@ -241,6 +241,14 @@ inline int union_tiles_max(const hf_ctx* c, int keep, int Tn) {
     return (uni + G - 1) / G;
 }
 
+// Whether pooling and selection are one launch: where a head's blocks are few, so that a thread block per query block (128 tokens) or one
+// for all (16 tokens) has little to pool and the launch it spares weighs more.  Forward calls with it and without: 12 heads of 128,
+// 640 queries 15.9 / 16.7 us, 1 000 queries (T_m 8) 19.9 / 19.5, 1 300 (T_m 11) 27.9 / 25.9; 2 heads of 64 queries, 16-token blocks
+// 11.0 / 11.8 us, 12 heads of 300 queries (T_m 19) 29.1 / 28.1.
+inline bool pools_and_selects(const hf_ctx* c) {
+    return !c->has_trope && ((c->cfg.block == 128 && c->Tm <= 5) || (c->cfg.block == 16 && c->Tm <= 8));
+}
+
 // Shared-memory limits of the kernels that a context of this head_dim, block and attention kernel launches: touching a kernel
 // loads it, and the first context of a process would pay for all of them.
 template <int D>
@@ -255,6 +263,8 @@ hf_status set_attrs(const hf_ctx* c) {
     if (c->cfg.merge == HF_MERGE_FULL_WIDTH)
         HF_CUDA(cudaFuncSetAttribute(k_merge_full<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, MergeFull<D>::SMEM_BYTES));
     HF_TRY((set_select_attr<D, 1>()));
+    if (b == 128 && c->Tm <= 5) HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 128, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect<D, 128, 1>::smem_bytes(5 * HF_MAX_CHUNKS, 5)));
+    if (b == 16 && c->Tm <= 8) HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 16, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect<D, 16, 8>::smem_bytes(8 * HF_MAX_CHUNKS, 8)));
     if (forward_lists(c)) HF_TRY((b == 64 ? set_select_attr<D, 2>() : set_select_attr<D, 8>()));
     return set_state_attr<D>();
 }
@@ -265,13 +275,18 @@ hf_status set_attrs(const hf_ctx* c) {
 // dependent launch); the kernel calls pdl_wait() before it touches anything that kernel wrote.
 struct PdlLaunch {
     cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr[1];
-    PdlLaunch(dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool overlap) {
+    cudaLaunchAttribute attr[2];
+    PdlLaunch(dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool overlap, int cluster = 1) {
         memset(&cfg, 0, sizeof(cfg));
         cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr; cfg.numAttrs = overlap ? 1 : 0;
+        if (cluster > 1) {
+            cudaLaunchAttribute& a = attr[cfg.numAttrs++];
+            a.id = cudaLaunchAttributeClusterDimension;
+            a.val.clusterDim.x = cluster; a.val.clusterDim.y = 1; a.val.clusterDim.z = 1;
+        }
     }
 };
 
@@ -501,12 +516,10 @@ ChunkTable make_table(hf_ctx* c, LayerState& L, const bf16* k_cur, const bf16* v
 }
 
 template <int D, int G>
-cudaError_t launch_select_kernel(hf_ctx* c, LayerState& L, const ChunkTable& tab, int Tn, int keep, uint32_t* mask_out, int32_t* idx_out,
-                                 float* scores_out, const UnionOut& lists, cudaStream_t st) {
+cudaError_t launch_select_kernel(hf_ctx* c, const ChunkTable& tab, int Tn, int keep, const SelectOut& o, const UnionOut& lists, cudaStream_t st) {
     typedef Select<D, G> S;
     PdlLaunch pl(dim3((c->Tm + S::R - 1) / S::R, c->BH), dim3(S::THREADS), S::smem_bytes(Tn), st, true);      // follows the pooling kernel
-#define HF_SELECT(KPL_) cudaLaunchKernelEx(&pl.cfg, k_select<D, KPL_, G>, tab, (const float*)c->pooled_q, c->n_b, c->Tm, Tn, keep, c->mask_words, \
-                                           L.mask, L.idx, mask_out, idx_out, scores_out, -0.f, lists)
+#define HF_SELECT(KPL_) cudaLaunchKernelEx(&pl.cfg, k_select<D, KPL_, G>, tab, (const float*)c->pooled_q, c->n_b, c->Tm, Tn, keep, -0.f, o, lists)
     if (Tn <= 128) return HF_SELECT(4);             // (registers of the ranking warps: T_n / 32 images per lane)
     if (Tn <= 256) return HF_SELECT(8);
     return HF_SELECT(32);
@@ -514,31 +527,49 @@ cudaError_t launch_select_kernel(hf_ctx* c, LayerState& L, const ChunkTable& tab
 }
 
 // merged: the attention kernel follows in the same call and takes its merged lists from here.
+// Pooling and selection in one launch (k_pool_select).
+template <int D, int BLK, int R>
+hf_status launch_pool_select(hf_ctx* c, const bf16* q, const bf16* k_cur, const ChunkTable& tab, int Tn, int keep, const SelectOut& o,
+                             const UnionOut& lists, cudaStream_t st) {
+    typedef PoolSelect<D, BLK, R> S;
+    const int nc = (c->Tm + R - 1) / R;
+    PdlLaunch pl(dim3(nc, c->BH), dim3(S::THREADS), S::smem_bytes(Tn, c->n_b), st, true, nc);
+    HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_pool_select<D, BLK, R>, tab, q, k_cur, c->Tc, c->Tm, Tn, keep, -0.f, o, lists));
+    return post_launch(c, "k_pool_select");
+}
+
+// merged: the attention kernel follows in the same call and takes its merged lists from here.
 template <int D>
 hf_status launch_select(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_cur,
                         uint32_t* mask_out, int32_t* idx_out, float* scores_out, cudaStream_t st, bool merged = false) {
-    PoolJobs jobs;
-    memset(&jobs, 0, sizeof(jobs));
-    jobs.job[0].src = q;     jobs.job[0].pooled = c->pooled_q;
-    jobs.job[1].src = k_cur; jobs.job[1].pooled = c->pooled_kcur;
-    if (c->has_trope) {     // the block means are those of the rotated tensors, which the attention kernel reads afterwards
-        const int base = trope_top(c, L.frames) - c->cfg.chunk_frames + 1;
-        jobs.job[0].copy_dst = c->q_rot; jobs.job[1].copy_dst = c->k_rot;
-        for (int i = 0; i < 2; ++i) { jobs.job[i].rot_on = 1; jobs.job[i].rot_base = base; jobs.job[i].rot_per_frame = 1; }
-    }
-    HF_TRY(launch_pool<D>(c, jobs, 2, st));
     const int Tn = (L.n_sink + L.n_cached + 1) * c->n_b;
     const int keep = keep_for(c, Tn);
     ChunkTable tab = make_table(c, L, k_cur, nullptr);
+    const SelectOut o = {L.mask, L.idx, mask_out, idx_out, scores_out, c->mask_words};
     UnionOut lists = {nullptr, nullptr, 0, c->Tc};
-    if (!merged) HF_CUDA((launch_select_kernel<D, 1>(c, L, tab, Tn, keep, mask_out, idx_out, scores_out, lists, st)));
-    else {
+    if (merged) {
         lists.entries = c->union_entries; lists.tiles = c->union_tiles; lists.max_tiles = union_tiles_max(c, keep, Tn);
         if (lists.max_tiles > c->union_max_tiles) return fail(HF_ERR_SHAPE, "tile list of %d tiles exceeds the %d the context was sized for", lists.max_tiles, c->union_max_tiles);
-        if (c->cfg.block == 64) HF_CUDA((launch_select_kernel<D, 2>(c, L, tab, Tn, keep, mask_out, idx_out, scores_out, lists, st)));
-        else HF_CUDA((launch_select_kernel<D, 8>(c, L, tab, Tn, keep, mask_out, idx_out, scores_out, lists, st)));
     }
-    HF_TRY(post_launch(c, "k_select"));
+    if (pools_and_selects(c)) {
+        if (c->cfg.block == 128) HF_TRY((launch_pool_select<D, 128, 1>(c, q, k_cur, tab, Tn, keep, o, lists, st)));
+        else HF_TRY((launch_pool_select<D, 16, 8>(c, q, k_cur, tab, Tn, keep, o, lists, st)));
+    } else {
+        PoolJobs jobs;
+        memset(&jobs, 0, sizeof(jobs));
+        jobs.job[0].src = q;     jobs.job[0].pooled = c->pooled_q;
+        jobs.job[1].src = k_cur; jobs.job[1].pooled = c->pooled_kcur;
+        if (c->has_trope) {     // the block means are those of the rotated tensors, which the attention kernel reads afterwards
+            const int base = trope_top(c, L.frames) - c->cfg.chunk_frames + 1;
+            jobs.job[0].copy_dst = c->q_rot; jobs.job[1].copy_dst = c->k_rot;
+            for (int i = 0; i < 2; ++i) { jobs.job[i].rot_on = 1; jobs.job[i].rot_base = base; jobs.job[i].rot_per_frame = 1; }
+        }
+        HF_TRY(launch_pool<D>(c, jobs, 2, st));
+        if (!merged) HF_CUDA((launch_select_kernel<D, 1>(c, tab, Tn, keep, o, lists, st)));
+        else if (c->cfg.block == 64) HF_CUDA((launch_select_kernel<D, 2>(c, tab, Tn, keep, o, lists, st)));
+        else HF_CUDA((launch_select_kernel<D, 8>(c, tab, Tn, keep, o, lists, st)));
+        HF_TRY(post_launch(c, "k_select"));
+    }
     L.sel_epoch = L.cache_epoch;
     L.sel_keep = keep;
     return HF_OK;

@@ -306,13 +306,117 @@ __device__ __forceinline__ uint32_t score_image(float s) {
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// KPL: key blocks per lane of a ranking warp (T_n <= 32 KPL).
+// Where a selection goes: per layer, and copies a caller asks for.
+struct SelectOut {
+    uint32_t* mask;              // [B*H, T_m, mask_words]
+    int32_t* idx;                // [B*H, T_m, keep]
+    uint32_t *mask_out;          // (nullptr: not wanted)
+    int32_t* idx_out;
+    float* scores_out;
+    int mask_words;
+};
+// Top-K of one row by one warp: the row's scores in shared memory; its mask and ascending list are stored, the mask's word number
+// `lane` is returned.  KPL: key blocks per lane (T_n <= 32 KPL).
+template <int KPL>
+__device__ __forceinline__ uint32_t rank_row(const float* sc, size_t row, int Tn, int keep, const SelectOut& o) {
+    const int lane = threadIdx.x & 31;
+    // lane l holds the images of blocks l, l + 32, ... (padding: 0, and behind every block)
+    uint32_t key[KPL];
+#pragma unroll
+    for (int x = 0; x < KPL; ++x) {
+        const int j = x * 32 + lane;
+        key[x] = j < Tn ? score_image(sc[j]) : 0u;
+    }
+    uint32_t thr = 0;           // largest value with at least `keep` images at or above it
+    bool exact = keep >= Tn;    // ... and exactly `keep`: no ties to cut (all blocks kept: every image counts)
+    for (uint32_t bit = 0x80000000u; bit != 0u && !exact; bit >>= 1) {
+        const uint32_t cand = thr | bit;
+        int n = 0;
+#pragma unroll
+        for (int x = 0; x < KPL; ++x) n += key[x] >= cand;
+        n = __reduce_add_sync(0xffffffffu, n);
+        if (n >= keep) { thr = cand; exact = n == keep; }
+    }
+    int ties = Tn;              // blocks at the threshold still to be kept, lowest index first
+    if (!exact) {
+        int n = 0;
+#pragma unroll
+        for (int x = 0; x < KPL; ++x) n += key[x] > thr;
+        ties = keep - __reduce_add_sync(0xffffffffu, n);
+    }
+    const uint32_t below = (1u << lane) - 1u;
+    int pos = 0;
+    uint32_t my_word = 0;
+#pragma unroll
+    for (int x = 0; x < KPL; ++x) {
+        const int j = x * 32 + lane;
+        const uint32_t eq = __ballot_sync(0xffffffffu, j < Tn && key[x] == thr);
+        const bool kept = j < Tn && (key[x] > thr || (key[x] == thr && __popc(eq & below) < ties));
+        ties -= __popc(eq);
+        const uint32_t word = __ballot_sync(0xffffffffu, kept);
+        if (lane == x) my_word = word;
+        if (kept) {
+            const int at = pos + __popc(word & below);
+            if (at < keep) {    // (always true under the total order above; the store never leaves the row)
+                o.idx[row * keep + at] = j;
+                if (o.idx_out) o.idx_out[row * keep + at] = j;
+            }
+        }
+        pos += __popc(word);
+    }
+    if (lane < o.mask_words) {
+        o.mask[row * o.mask_words + lane] = my_word;
+        if (o.mask_out) o.mask_out[row * o.mask_words + lane] = my_word;
+    }
+    return my_word;
+}
+
+// Scores of n key rows of a pass (key_row(j): their D floats in shared memory) against `rows` query rows, sc[r * Tn + j].  R: query rows
+// a thread block may have; 256 threads, 512 for eight.
+template <int D, int R, typename KeyRow>
+__device__ __forceinline__ void score_pass(KeyRow key_row, int n, const float* s_q, int rows, float* sc, int Tn, float2 nz) {
+    constexpr int THREADS = R == 8 ? 512 : 256, W = THREADS / R < 128 ? THREADS / R : 128;
+    if (n <= W) {               // few keys: one score per thread
+        const int j = threadIdx.x % W, r = threadIdx.x / W;
+        if (j < n && r < rows) {
+            float v[1];
+            canonical_scores<D, 1>(key_row(j), s_q + r * D, nz, v);
+            sc[r * Tn + j] = v[0];
+        }
+    } else {                    // two scores per thread: query blocks 2 h, 2 h + 1 (rows past T_m: stale shared memory, not stored)
+        const int j = threadIdx.x & 127, r = (threadIdx.x >> 7) * 2;
+        if (j < n && r < rows) {
+            float v[2];
+            canonical_scores<D, 2>(key_row(j), s_q + r * D, nz, v);
+            sc[r * Tn + j] = v[0];
+            if (r + 1 < rows) sc[(r + 1) * Tn + j] = v[1];
+        }
+    }
+}
+// The end of a selection: scores out, top-K of every row, and (G > 1, lists.entries set) the merged lists of the units of these rows.
+template <int KPL, int G, int R>
+__device__ __forceinline__ void finish_rows(const float* s_sc, uint32_t (*s_mask)[32], int bh, int i0, int rows, int Tm, int Tn, int n_b, int keep,
+                                            const SelectOut& o, const UnionOut& lists) {
+    constexpr int THREADS = R == 8 ? 512 : 256;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (o.scores_out)
+        for (int e = threadIdx.x; e < rows * Tn; e += THREADS) o.scores_out[((size_t)bh * Tm + i0) * Tn + e] = s_sc[e];
+    if (warp < R) {
+        const uint32_t word = warp < rows ? rank_row<KPL>(s_sc + warp * Tn, (size_t)bh * Tm + i0 + warp, Tn, keep, o) : 0u;
+        if constexpr (G > 1) s_mask[warp][lane] = word;         // (query blocks past T_m, lanes past the words of T_n: 0)
+    }
+    if constexpr (G > 1) {
+        if (lists.entries == nullptr) return;
+        constexpr int UNITS = R / G, WPU = THREADS / 32 / UNITS;
+        __syncthreads();
+        const int x = warp / WPU, mt = i0 / G + x, upb = (Tm + G - 1) / G;
+        if (mt < upb) union_lists<G>(s_mask + x * G, warp % WPU, WPU, Tn, n_b, bh * upb + mt, lists);
+    }
+}
+
 template <int D, int KPL, int G>
 __global__ void __launch_bounds__(Select<D, G>::THREADS) k_select(ChunkTable tab, const float* __restrict__ pooled_q,
-                                                int n_b, int Tm, int Tn, int keep, int mask_words,
-                                                uint32_t* __restrict__ mask, int32_t* __restrict__ idx,
-                                                uint32_t* __restrict__ mask_out, int32_t* __restrict__ idx_out,
-                                                float* __restrict__ scores_out, float neg_zero, UnionOut lists) {
+                                                int n_b, int Tm, int Tn, int keep, float neg_zero, SelectOut o, UnionOut lists) {
     typedef Select<D, G> C;
     const float2 nz = make_float2(neg_zero, neg_zero);
     extern __shared__ __align__(16) float sel_smem[];
@@ -323,7 +427,6 @@ __global__ void __launch_bounds__(Select<D, G>::THREADS) k_select(ChunkTable tab
     __shared__ uint32_t s_mask[G > 1 ? C::R : 1][32];
     const int i0 = blockIdx.x * C::R, bh = blockIdx.y;
     const int rows = min(C::R, Tm - i0);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t s_k_addr = smem_u32(s_k);
     // key rows [j0, j1) of the pass that starts at `base`, sixteen bytes per thread and step
     auto load_keys = [&](int base, int j0, int j1) {
@@ -352,88 +455,156 @@ __global__ void __launch_bounds__(Select<D, G>::THREADS) k_select(ChunkTable tab
         }
         cp_async_wait<0>();
         __syncthreads();
-        if (n <= 64) {          // few keys: one score per thread
-            const int j = threadIdx.x & 63, r = threadIdx.x >> 6;
-            if (j < n && r < rows) {
-                float v[1];
-                canonical_scores<D, 1>(s_k + j * C::LD, s_q + r * D, nz, v);
-                s_sc[r * Tn + base + j] = v[0];
-            }
-        } else {                // two scores per thread: query blocks 2 h, 2 h + 1 (rows past T_m: stale shared memory, not stored)
-            const int j = threadIdx.x & 127, r = (threadIdx.x >> 7) * 2;
-            if (j < n && r < rows) {
-                float v[2];
-                canonical_scores<D, 2>(s_k + j * C::LD, s_q + r * D, nz, v);
-                s_sc[r * Tn + base + j] = v[0];
-                if (r + 1 < rows) s_sc[(r + 1) * Tn + base + j] = v[1];
-            }
-        }
+        score_pass<D, C::R>([&](int j) { return s_k + j * C::LD; }, n, s_q, rows, s_sc + base, Tn, nz);
     }
     __syncthreads();
-    if (scores_out)
-        for (int e = threadIdx.x; e < rows * Tn; e += C::THREADS) scores_out[((size_t)bh * Tm + i0) * Tn + e] = s_sc[e];
-    if constexpr (G == 1) {
-        if (warp >= rows) return;
-    } else {
-        if (warp < C::R) s_mask[warp][lane] = 0;        // (query blocks past T_m keep nothing)
+    finish_rows<KPL, G, C::R>(s_sc, s_mask, bh, i0, rows, Tm, Tn, n_b, keep, o, lists);
+}
+
+// Pooling and selection of one call in one launch, for heads of few blocks.  The thread blocks of a head form a cluster (BLK 128: one per
+// query block, at most five; BLK 16: one for the up to eight query blocks of a unit), pool the query blocks they select for and a
+// share of the current chunk's key blocks each, and hand the key means to one another through distributed shared memory.
+// grid (c, B*H), cluster (c), c = ceil(T_m / R); R: query blocks per thread block.
+//
+// Latency alone: against k_pool_copy + k_select it spares a launch and the means' way through L2 (two heads of 64 queries, 16-token
+// blocks 11.65 -> 10.5 us a forward; 8 heads of 128, 300 queries, selection alone 7.0 -> 4.9).  With more blocks a head the thread
+// blocks are too few for the pooling, which the other form spreads over the device (dispatch: pools_and_selects).
+template <int D, int BLK, int R>
+struct PoolSelect {
+    static constexpr int THREADS = R == 8 ? 512 : 256;
+    static constexpr int G = 128 / BLK, LD = D + 4;
+    static constexpr int NB = 2;                            // blocks in flight (BLK 128: one query block, one key block)
+    static constexpr int PART = BLK == 16 ? 0 : NB * 16 * D;
+    static_assert(BLK == 16 || THREADS == 256, "sixteen threads a row, sixteen rows");
+    // key rows, query rows, chains, scores
+    static int smem_bytes(int Tn, int n_b) { return (Tn * LD + R * D + R * Tn + PART) * (int)sizeof(float); }
+};
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
+// A float into the same place of thread block `rank`'s shared memory.
+__device__ __forceinline__ void cluster_store(uint32_t addr, int rank, float v) {
+    asm volatile("{\n.reg .b32 a;\nmapa.shared::cluster.u32 a, %0, %1;\nst.shared::cluster.f32 [a], %2;\n}\n" ::"r"(addr), "r"(rank), "f"(v) : "memory");
+}
+
+template <int D, int BLK, int R>
+__global__ void __launch_bounds__(PoolSelect<D, BLK, R>::THREADS) k_pool_select(ChunkTable tab, const bf16* __restrict__ q, const bf16* __restrict__ k,
+                                                int Tc, int Tm, int Tn, int keep, float neg_zero, SelectOut o, UnionOut lists) {
+    typedef PoolSelect<D, BLK, R> C;
+    constexpr int VEC = D / 16, KPL = 2;        // (T_n <= 8 chunks of 8 blocks)
+    typedef typename VecLoad<VEC>::T V;
+    const float2 nz = make_float2(neg_zero, neg_zero);
+    extern __shared__ __align__(16) float sel_smem[];
+    const int n_b = Tm, n_old = Tn - n_b;
+    float* s_k = sel_smem;                      // [T_n][LD]: key rows, cached chunks' first
+    float* s_q = s_k + Tn * C::LD;              // [R][D]
+    float* s_part = s_q + R * D;                // chains of the blocks in flight
+    float* s_sc = s_part + C::PART;             // [R][Tn]
+    __shared__ uint32_t s_mask[C::G > 1 ? R : 1][32];
+    const int nc = gridDim.x, rank = blockIdx.x, bh = blockIdx.y, i0 = rank * R;
+    const int rows = min(R, Tm - i0);
+    if (nc > 1) cluster_arrive();               // (no thread block writes to another's shared memory before that one has started)
+    pdl_wait();
+    pdl_trigger();              // the attention kernel may be made resident as blocks of this grid leave
+    // cached rows, sixteen bytes per thread and step
+    for (int e = threadIdx.x; e < n_old * (D / 4); e += C::THREADS) {
+        const int j = e / (D / 4), part = e % (D / 4);
+        int c = 0, jb = j;
+        while (jb >= n_b) { jb -= n_b; ++c; }
+        cp_async16(smem_u32(s_k) + (j * C::LD + part * 4) * 4, tab.pooled[c] + ((size_t)bh * n_b + jb) * D + part * 4, true);
     }
-    if (warp < rows) {
-        // ---- top-K of row `warp`: lane l holds the images of blocks l, l + 32, ... (padding: 0, and behind every block)
-        const size_t row = (size_t)bh * Tm + i0 + warp;
-        uint32_t key[KPL];
+    cp_async_commit();
+    // ---- block means in the canonical order: the blocks of this thread block, its query blocks first, then key blocks rank, rank + nc, ...
+    const int n_mine = rows + (n_b - rank + nc - 1) / nc;
+    auto block_of = [&](int w, bool& is_q) -> int { is_q = w < rows; return is_q ? i0 + w : rank + (w - rows) * nc; };
+    auto put = [&](bool is_q, int b, int col, float mean) {
+        if (is_q) { s_q[(b - i0) * D + col] = mean; return; }
+        float* at = s_k + (n_old + b) * C::LD + col;
+        if (nc == 1) *at = mean;
+        else for (int x = 0; x < nc; ++x) cluster_store(smem_u32(at), x, mean);
+    };
+    bool started = nc == 1;
+    if constexpr (BLK == 16) {
+        // sixteen chains of one token: a thread takes a block's pair of columns, sixteen loads in flight
+        constexpr int TPB = D / 2, BPS = C::THREADS / TPB;
+        for (int w0 = 0; w0 < n_mine; w0 += BPS) {
+            const int w = w0 + threadIdx.x / TPB, col = (threadIdx.x % TPB) * 2;
+            if (w >= n_mine) continue;
+            bool is_q;
+            const int b = block_of(w, is_q), n = min(BLK, Tc - b * BLK);
+            const bf16* src = (is_q ? q : k) + ((size_t)bh * Tc + (size_t)b * BLK) * D + col;
+            uint32_t u[16];
 #pragma unroll
-        for (int x = 0; x < KPL; ++x) {
-            const int j = x * 32 + lane;
-            key[x] = j < Tn ? score_image(s_sc[warp * Tn + j]) : 0u;
+            for (int t = 0; t < 16; ++t) u[t] = t < n ? __ldg(reinterpret_cast<const uint32_t*>(src + (size_t)t * D)) : 0u;
+            float2 tot;
+#pragma unroll
+            for (int t = 0; t < 16; ++t) {
+                const float2 f = unpack_bf16(u[t]);
+                const float x0 = __fadd_rn(0.f, f.x), x1 = __fadd_rn(0.f, f.y);
+                tot.x = t == 0 ? x0 : __fadd_rn(tot.x, x0);
+                tot.y = t == 0 ? x1 : __fadd_rn(tot.y, x1);
+            }
+            put(is_q, b, col, __fdiv_rn(tot.x, (float)n));
+            put(is_q, b, col + 1, __fdiv_rn(tot.y, (float)n));
         }
-        uint32_t thr = 0;           // largest value with at least `keep` images at or above it
-        bool exact = keep >= Tn;    // ... and exactly `keep`: no ties to cut (all blocks kept: every image counts)
-        for (uint32_t bit = 0x80000000u; bit != 0u && !exact; bit >>= 1) {
-            const uint32_t cand = thr | bit;
-            int n = 0;
+    } else {
+        constexpr int MAXR = BLK / 16;          // rows per chain
+        const int r = threadIdx.x >> 4, cv = threadIdx.x & 15;
+        for (int w0 = 0; w0 < n_mine; w0 += C::NB) {
+            V u[C::NB][MAXR];
+            int n[C::NB];
 #pragma unroll
-            for (int x = 0; x < KPL; ++x) n += key[x] >= cand;
-            n = __reduce_add_sync(0xffffffffu, n);
-            if (n >= keep) { thr = cand; exact = n == keep; }
-        }
-        int ties = Tn;              // blocks at the threshold still to be kept, lowest index first
-        if (!exact) {
-            int n = 0;
+            for (int x = 0; x < C::NB; ++x) {
+                bool is_q;
+                const int w = w0 + x, b = w < n_mine ? block_of(w, is_q) : 0;
+                n[x] = w < n_mine ? min(BLK, Tc - b * BLK) : 0;
+                if (n[x] > 0) {
+                    const bf16* src = (is_q ? q : k) + ((size_t)bh * Tc + (size_t)b * BLK) * D + cv * VEC;
 #pragma unroll
-            for (int x = 0; x < KPL; ++x) n += key[x] > thr;
-            ties = keep - __reduce_add_sync(0xffffffffu, n);
-        }
-        const uint32_t below = (1u << lane) - 1u;
-        int pos = 0;
-        uint32_t my_word = 0;
-#pragma unroll
-        for (int x = 0; x < KPL; ++x) {
-            const int j = x * 32 + lane;
-            const uint32_t eq = __ballot_sync(0xffffffffu, j < Tn && key[x] == thr);
-            const bool kept = j < Tn && (key[x] > thr || (key[x] == thr && __popc(eq & below) < ties));
-            ties -= __popc(eq);
-            const uint32_t word = __ballot_sync(0xffffffffu, kept);
-            if (lane == x) my_word = word;
-            if (kept) {
-                const int at = pos + __popc(word & below);
-                if (at < keep) {    // (always true under the total order above; the store never leaves the row)
-                    idx[row * keep + at] = j;
-                    if (idx_out) idx_out[row * keep + at] = j;
+                    for (int i = 0; i < MAXR; ++i) {
+                        const int t = r + 16 * i;
+                        if (t < n[x]) u[x][i] = __ldg(reinterpret_cast<const V*>(src + (size_t)t * D));
+                    }
                 }
             }
-            pos += __popc(word);
+            if (w0 > 0) __syncthreads();        // the chains of the step before have been added up
+#pragma unroll
+            for (int x = 0; x < C::NB; ++x) {
+                float acc[VEC];
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) acc[e] = 0.f;
+#pragma unroll
+                for (int i = 0; i < MAXR; ++i) {
+                    if (r + 16 * i < n[x]) {
+                        float f[VEC];
+                        VecLoad<VEC>::widen(u[x][i], f);
+#pragma unroll
+                        for (int e = 0; e < VEC; ++e) acc[e] = __fadd_rn(acc[e], f[e]);
+                    }
+                }
+                float* part = s_part + (x * 16 + r) * D + cv * VEC;
+#pragma unroll
+                for (int e = 0; e < VEC; e += 4) *reinterpret_cast<float4*>(part + e) = make_float4(acc[e], acc[e + 1], acc[e + 2], acc[e + 3]);
+            }
+            __syncthreads();
+            if (!started) { cluster_wait(); started = true; }
+            for (int e = threadIdx.x; e < C::NB * D; e += C::THREADS) {
+                const int x = e / D, col = e % D, w = w0 + x;
+                if (w < n_mine) {
+                    bool is_q;
+                    const int b = block_of(w, is_q);
+                    const float* part = s_part + x * 16 * D + col;
+                    float tot = part[0];
+#pragma unroll
+                    for (int rr = 1; rr < 16; ++rr) tot = __fadd_rn(tot, part[rr * D]);
+                    put(is_q, b, col, __fdiv_rn(tot, (float)min(BLK, Tc - b * BLK)));
+                }
+            }
         }
-        if (lane < mask_words) {
-            mask[row * mask_words + lane] = my_word;
-            if (mask_out) mask_out[row * mask_words + lane] = my_word;
-        }
-        if constexpr (G > 1) s_mask[warp][lane] = my_word;      // (lanes past the words of T_n: 0)
     }
-    if constexpr (G > 1) {
-        // ---- the merged lists of the units of these query blocks, the warps shared out among them
-        constexpr int UNITS = C::R / G, WPU = C::THREADS / 32 / UNITS;
-        __syncthreads();
-        const int x = warp / WPU, mt = (int)blockIdx.x * UNITS + x, upb = (Tm + G - 1) / G;
-        if (mt < upb) union_lists<G>(s_mask + x * G, warp % WPU, WPU, Tn, n_b, bh * upb + mt, lists);
-    }
+    cp_async_wait<0>();
+    if (nc > 1) { cluster_arrive(); cluster_wait(); }       // every key mean is in place in every thread block
+    else __syncthreads();
+    score_pass<D, R>([&](int j) { return s_k + j * C::LD; }, Tn, s_q, rows, s_sc, Tn, nz);
+    __syncthreads();
+    finish_rows<KPL, C::G, R>(s_sc, s_mask, bh, i0, rows, Tm, Tn, n_b, keep, o, lists);
 }
