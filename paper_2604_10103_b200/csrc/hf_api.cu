@@ -440,6 +440,19 @@ hf_status launch_absorb_layers(hf_ctx* c, int first_layer, int n_layers, const C
     return post_launch(c, "k_reduce_fold (layers)");
 }
 
+// Whether Eq. 3 of several layers goes in one persistent launch (k_absorb_items: a thread block sums half of an item's token tiles) or
+// layer by layer (k_absorb_tc5: an item cut over several thread blocks, but three launches and the side stream's events per layer).
+// As many items as SMs fill the device either way.  With fewer, in units of a 64-token tile: rounds x tiles of a unit against tiles of a
+// split, plus what a call costs beside its tiles, about ten tiles' time (8 us) either way.  Same bits either way.  The commit of four
+// layers of 8 heads of 128, 300 tokens: 60 us layer by layer, 21 in one launch.
+inline bool layers_in_one_launch(const hf_ctx* c, int n_layers, int n_tokens) {
+    if (n_layers < 2) return false;
+    if ((long long)n_layers * c->BH >= c->sm_count) return true;
+    const long long tiles = (n_tokens + 63) / 64, split = tiles < c->nsplit_max ? tiles : c->nsplit_max, groups = absorb_groups((int)split);
+    const long long rounds = (n_layers * c->BH * groups + c->sm_count - 1) / c->sm_count, rounds_one = (c->BH * split + c->sm_count - 1) / c->sm_count, fixed = 10;
+    return rounds * ((tiles + groups - 1) / groups) + fixed <= n_layers * (rounds_one * ((tiles + split - 1) / split) + fixed);
+}
+
 template <int D>
 hf_status launch_pool_layers(hf_ctx* c, const PoolLayersParams& p, int n_layers, cudaStream_t st) {
     PdlLaunch pl(dim3(c->n_b, c->BH, 2 * n_layers), dim3(256), 0, st, false);
@@ -882,6 +895,11 @@ hf_status hf_create(const hf_config* cfg, int device, hf_ctx** out) {
     if (s == HF_OK && cfg->merge == HF_MERGE_FULL_WIDTH) s = dmalloc(&c->x_hi, c->chunk_elems);
     if (s == HF_OK && cfg->merge == HF_MERGE_FULL_WIDTH) s = dmalloc(&c->x_lo, c->chunk_elems);
     if (s == HF_OK) s = dmalloc(&c->partials, (size_t)c->BH * c->nsplit_max * ((size_t)c->d * c->d + c->d));
+    if (s == HF_OK && c->cfg.layers > 1) {      // the layer-batched update of up to as many items as SMs allocates nothing; larger calls grow it
+        const size_t items = (size_t)c->cfg.layers * c->BH < (size_t)c->sm_count ? (size_t)c->cfg.layers * c->BH : (size_t)c->sm_count;
+        c->partials_layers_count = items * 2 * ((size_t)c->d * c->d + c->d);
+        s = dmalloc(&c->partials_layers, c->partials_layers_count);
+    }
     if (s == HF_OK) s = dmalloc(&c->dev_status, (size_t)8);     // status word [4] + self-test results [4]
     if (s == HF_OK && (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
                        cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
@@ -1107,9 +1125,7 @@ hf_status hf_state_absorb_layers(hf_ctx* c, int first_layer, int n_layers, const
         return fail(HF_ERR_SHAPE, "with HF_Z_FRAME_MEAN n_tokens must be a multiple of tokens_per_frame (%d)", c->cfg.tokens_per_frame);
     cudaStream_t st = (cudaStream_t)stream;
     const size_t per_layer = (size_t)c->BH * n_tokens * c->d;
-    // One persistent launch pays when there are at least as many (layer, batch*head) items as SMs; below that the
-    // per-layer kernel, which cuts every item over several thread blocks, fills the device better.  Same bits either way.
-    if ((long long)n_layers * c->BH < c->sm_count) {
+    if (!layers_in_one_launch(c, n_layers < HF_MAX_BATCH_LAYERS ? n_layers : HF_MAX_BATCH_LAYERS, n_tokens)) {
         for (int l = 0; l < n_layers; ++l)
             HF_TRY(HF_DISPATCH_D(c, launch_absorb, c, c->layers[first_layer + l], (const bf16*)k_ev + l * per_layer,
                                  (const bf16*)v_ev + l * per_layer, n_tokens, st));
@@ -1139,10 +1155,10 @@ hf_status hf_kv_append_layers(hf_ctx* c, int first_layer, int n_layers, const vo
     }
     cudaStream_t st = (cudaStream_t)stream;
     // The batched launches need every layer of the call in the same phase of Alg. 2's protocol (all still filling their
-    // sink, all filling the window, or all evicting) and enough (layer, batch*head) items to fill the device; anything
-    // else goes layer by layer.  The state gets the same bits either way.
+    // sink, all filling the window, or all evicting); anything else goes layer by layer.  The state gets the same bits either way.
     const LayerState& L0 = c->layers[first_layer];
-    bool uniform = c->P > 0 && !c->has_trope && n_layers <= HF_MAX_BATCH_LAYERS && (long long)n_layers * c->BH >= c->sm_count;
+    bool uniform = c->P > 0 && !c->has_trope && n_layers <= HF_MAX_BATCH_LAYERS &&
+                   (L0.n_sink < c->n_sink_max || L0.n_cached < c->P ? n_layers > 1 : layers_in_one_launch(c, n_layers, c->Tc));
     for (int l = 1; uniform && l < n_layers; ++l) {
         const LayerState& L = c->layers[first_layer + l];
         uniform = (L.n_sink < c->n_sink_max) == (L0.n_sink < c->n_sink_max) && (L.n_cached == c->P) == (L0.n_cached == c->P);
