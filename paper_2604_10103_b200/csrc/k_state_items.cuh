@@ -280,3 +280,12 @@ k_absorb_items(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         tmem_dealloc(tmem, C::TMEM_COLS);
     }
 }
+
+// S and z of a layer to the caller: n_S + n_z float4.
+__global__ void __launch_bounds__(256) k_copy_state(const float4* __restrict__ S, float4* __restrict__ S_out, int n_S, const float4* __restrict__ z,
+                                                    float4* __restrict__ z_out, int n_z) {
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    pdl_wait();
+    if (i < n_S) S_out[i] = S[i];
+    else if (i - n_S < n_z) z_out[i - n_S] = z[i - n_S];
+}
