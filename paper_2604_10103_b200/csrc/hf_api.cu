@@ -217,9 +217,10 @@ hf_status set_swa_attr() {
 }
 template <int D, int G>
 hf_status set_select_attr() {
-    HF_CUDA(cudaFuncSetAttribute(k_select<D, 4, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G>::smem_bytes(128)));
-    HF_CUDA(cudaFuncSetAttribute(k_select<D, 8, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G>::smem_bytes(256)));
-    HF_CUDA(cudaFuncSetAttribute(k_select<D, 32, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G>::smem_bytes(HF_MAX_TN)));
+    HF_CUDA(cudaFuncSetAttribute(k_select<D, 4, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G, 4>::smem_bytes(128)));
+    HF_CUDA(cudaFuncSetAttribute(k_select<D, 8, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G, 8>::smem_bytes(256)));
+    HF_CUDA(cudaFuncSetAttribute(k_select<D, 16, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G, 16>::smem_bytes(512)));
+    HF_CUDA(cudaFuncSetAttribute(k_select<D, 32, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G, 32>::smem_bytes(HF_MAX_TN)));
     return HF_OK;
 }
 template <int D>
@@ -530,12 +531,14 @@ ChunkTable make_table(hf_ctx* c, LayerState& L, const bf16* k_cur, const bf16* v
 
 template <int D, int G>
 cudaError_t launch_select_kernel(hf_ctx* c, const ChunkTable& tab, int Tn, int keep, const SelectOut& o, const UnionOut& lists, cudaStream_t st) {
-    typedef Select<D, G> S;
-    PdlLaunch pl(dim3((c->Tm + S::R - 1) / S::R, c->BH), dim3(S::THREADS), S::smem_bytes(Tn), st, true);      // follows the pooling kernel
-#define HF_SELECT(KPL_) cudaLaunchKernelEx(&pl.cfg, k_select<D, KPL_, G>, tab, (const float*)c->pooled_q, c->n_b, c->Tm, Tn, keep, -0.f, o, lists)
-    if (Tn <= 128) return HF_SELECT(4);             // (registers of the ranking warps: T_n / 32 images per lane)
-    if (Tn <= 256) return HF_SELECT(8);
-    return HF_SELECT(32);
+    // follows the pooling kernel
+#define HF_SELECT(KPL_) do { typedef Select<D, G, KPL_> S; \
+        PdlLaunch pl(dim3((c->Tm + S::R - 1) / S::R, c->BH), dim3(S::THREADS), S::smem_bytes(Tn), st, true); \
+        return cudaLaunchKernelEx(&pl.cfg, k_select<D, KPL_, G>, tab, (const float*)c->pooled_q, c->n_b, c->Tm, Tn, keep, -0.f, o, lists); } while (0)
+    if (Tn <= 128) HF_SELECT(4);                    // (registers of the ranking warps: T_n / 32 images per lane)
+    if (Tn <= 256) HF_SELECT(8);
+    if (Tn <= 512) HF_SELECT(16);
+    HF_SELECT(32);
 #undef HF_SELECT
 }
 

@@ -246,9 +246,12 @@ __global__ void __launch_bounds__(256, 6) k_pool_copy_layers(const __grid_consta
 // G: the query blocks that share a unit of the attention kernel (blocks of 64 tokens: 2, of 16: 8), whose merged list is formed here
 // from the masks in shared memory, or 1: none is asked for.  A kernel of its own behind this one costs a launch (k_union.cuh).  G = 8
 // takes eight query blocks, one unit, per thread block, with as many threads per score.
-template <int D, int G = 1>
+// KPL: key blocks per lane of a ranking warp (T_n <= 32 KPL).  Rows of more than 256 key blocks come in several passes of key rows, and such
+// grids are large: there, too, eight query blocks share a key row's trip through L2 (T_n 259, 48 heads, behind the pooling: 42 us
+// with four query blocks and KPL 32, 24.5 like this).
+template <int D, int G, int KPL>
 struct Select {
-    static constexpr int R = G == 8 ? 8 : 4, KT = 128;       // query blocks per thread block; key rows per pass
+    static constexpr int R = G == 8 || KPL > 8 ? 8 : 4, KT = 128;        // query blocks per thread block; key rows per pass
     static constexpr int THREADS = 64 * R;
     static constexpr int LD = D + 4;            // floats per key row in shared memory
     static int smem_bytes(int Tn) { const int kt = Tn < KT ? Tn : KT; return (kt * LD + R * D + R * Tn) * (int)sizeof(float); }
@@ -415,9 +418,9 @@ __device__ __forceinline__ void finish_rows(const float* s_sc, uint32_t (*s_mask
 }
 
 template <int D, int KPL, int G>
-__global__ void __launch_bounds__(Select<D, G>::THREADS) k_select(ChunkTable tab, const float* __restrict__ pooled_q,
+__global__ void __launch_bounds__(Select<D, G, KPL>::THREADS) k_select(ChunkTable tab, const float* __restrict__ pooled_q,
                                                 int n_b, int Tm, int Tn, int keep, float neg_zero, SelectOut o, UnionOut lists) {
-    typedef Select<D, G> C;
+    typedef Select<D, G, KPL> C;
     const float2 nz = make_float2(neg_zero, neg_zero);
     extern __shared__ __align__(16) float sel_smem[];
     const int kt = min(Tn, C::KT);
