@@ -106,7 +106,7 @@ struct hf_ctx {
     float z_scale = 1.f;             // 1 (z = sum of phi(K)) or 1 / tokens_per_frame (per-frame means)
     bf16* stage[4] = {nullptr, nullptr, nullptr, nullptr};   // q, k, v, o staging of the *_host calls
     int* dev_status = nullptr;
-    float* rope_q[2] = {nullptr, nullptr};   // cos / sin tables [T_c, d/2] of Eq. 4's numerator (nullptr: no rotation)
+    float* rope_q[2] = {nullptr, nullptr};   // cos / sin of Eq. 4's numerator, [d/8][T_c][4]: four pairs of a token side by side (nullptr: no rotation)
     float* rope_k[2] = {nullptr, nullptr};   // ... of Eq. 3, applied to a chunk when it is absorbed
     bool has_rope_q = false, has_rope_k = false;
     // relative temporal RoPE of the softmax branch (Eq. 8): tables over index steps 0 .. t0, rotated copies of q / k_cur
@@ -978,7 +978,12 @@ hf_status hf_set_rope(hf_ctx* c, const float* cos_q, const float* sin_q, const f
         if (src[i] == nullptr) continue;
         HF_TRY(check_ptr(src[i], "rotation table"));
         if (*dst[i] == nullptr) HF_TRY(dmalloc(dst[i], count));
-        HF_CUDA(cudaMemcpyAsync(*dst[i], src[i], count * sizeof(float), cudaMemcpyDeviceToDevice, st));
+        if (i >= 2) { HF_CUDA(cudaMemcpyAsync(*dst[i], src[i], count * sizeof(float), cudaMemcpyDeviceToDevice, st)); continue; }
+        // the read-out's threads own a query row each: four pairs of neighbouring rows side by side (k_rope_chunks), by way of the history scratch
+        HF_CUDA(cudaMemcpyAsync(c->hist, src[i], count * sizeof(float), cudaMemcpyDeviceToDevice, st));
+        const int n4 = (int)(count / 4);
+        k_rope_chunks<<<(n4 + 255) / 256, 256, 0, st>>>(reinterpret_cast<const float4*>(c->hist), reinterpret_cast<float4*>(*dst[i]), c->Tc, c->d / 8);
+        HF_TRY(post_launch(c, "k_rope_chunks"));
     }
     c->has_rope_q = cos_q != nullptr;
     c->has_rope_k = cos_k != nullptr;

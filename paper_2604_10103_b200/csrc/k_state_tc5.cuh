@@ -305,7 +305,7 @@ struct ReadoutTc5 {
 };
 
 struct ReadoutTc5Params {
-    const float* cos_q;       // rotation tables of Eq. 4's numerator, [T_c, D/2] each (ROPE instantiation only)
+    const float* cos_q;       // rotation tables of Eq. 4's numerator, [D/8][T_c][4] each (ROPE instantiation only)
     const float* sin_q;
     const float* z;           // [B*H, D]
     const bf16* bias;         // [H, D] or nullptr
@@ -476,8 +476,8 @@ k_readout_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
                     const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
                     float cs[4] = {1.f, 1.f, 1.f, 1.f}, sn[4] = {0.f, 0.f, 0.f, 0.f};
                     if (ROPE) {
-                        const float4 c4 = __ldg(reinterpret_cast<const float4*>(p.cos_q + (size_t)r_tab * (D / 2)) + chunk);
-                        const float4 s4 = __ldg(reinterpret_cast<const float4*>(p.sin_q + (size_t)r_tab * (D / 2)) + chunk);
+                        const float4 c4 = __ldg(reinterpret_cast<const float4*>(p.cos_q) + chunk * p.Tc + r_tab);
+                        const float4 s4 = __ldg(reinterpret_cast<const float4*>(p.sin_q) + chunk * p.Tc + r_tab);
                         cs[0] = c4.x; cs[1] = c4.y; cs[2] = c4.z; cs[3] = c4.w;
                         sn[0] = s4.x; sn[1] = s4.y; sn[2] = s4.z; sn[3] = s4.w;
                     }

@@ -117,7 +117,7 @@ struct Tc5Params {
     const bf16* q;
     const float* z;
     const bf16* bias;
-    const float* cos_q;      // rotation of Eq. 4's numerator, tables [T_c, D / 2], or nullptr: none
+    const float* cos_q;      // rotation of Eq. 4's numerator, tables [D / 8][T_c][4], or nullptr: none
     const float* sin_q;
     bf16* o;
     float* lse;
@@ -183,7 +183,8 @@ __device__ __noinline__ void swa_redo_unit(uint8_t* s_gen, const Tc5Params& p, i
             sync256();
             const int row = tid >> 1, f0 = (tid & 1) * (D / 2), r_tab = min(q0 + row, p.Tc - 1);
             for (int a = f0; a < f0 + D / 2; a += 2) {
-                const float c = __ldg(p.cos_q + (size_t)r_tab * (D / 2) + a / 2), sn = __ldg(p.sin_q + (size_t)r_tab * (D / 2) + a / 2);
+                const size_t at = ((size_t)(a / 8) * p.Tc + r_tab) * 4 + a / 2 % 4;
+                const float c = __ldg(p.cos_q + at), sn = __ldg(p.sin_q + at);
                 const float x0 = phi_t[row * PS + a], x1 = phi_t[row * PS + a + 1];
                 phi_t[row * PS + a] = fmaf(-x1, sn, x0 * c);
                 phi_t[row * PS + a + 1] = fmaf(x0, sn, x1 * c);
@@ -634,8 +635,8 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                             const uint32_t ws[4] = {qv.x, qv.y, qv.z, qv.w};
                             float cs[4] = {1.f, 1.f, 1.f, 1.f}, sn[4] = {0.f, 0.f, 0.f, 0.f};
                             if constexpr (HIST == 2) {      // the pairs' angles belong to the query's row
-                                const size_t at = (size_t)min(q0 + row, p.Tc - 1) * (D / 2) + k * (FPT / 2) + c * 4;
-                                const float4 c4 = __ldg(reinterpret_cast<const float4*>(p.cos_q + at)), s4 = __ldg(reinterpret_cast<const float4*>(p.sin_q + at));
+                                const int at = (k * (FPT / 8) + c) * p.Tc + min(q0 + row, p.Tc - 1);
+                                const float4 c4 = __ldg(reinterpret_cast<const float4*>(p.cos_q) + at), s4 = __ldg(reinterpret_cast<const float4*>(p.sin_q) + at);
                                 cs[0] = c4.x; cs[1] = c4.y; cs[2] = c4.z; cs[3] = c4.w;
                                 sn[0] = s4.x; sn[1] = s4.y; sn[2] = s4.z; sn[3] = s4.w;
                             }
