@@ -62,25 +62,33 @@ __device__ __noinline__ void bwd_order_units(const BwdOrder& q) {
     for (int u = tid; u < n; u += 256) cnt[u] = 0;
     for (int b = tid; b <= q.Tm + 1; b += 256) at[b] = 0;
     __syncthreads();
-    const int w0 = q.first_block >> 5, nw = ((q.first_block + q.n_b - 1) >> 5) - w0 + 1, items = q.BH * q.Tm * nw;
-    for (int base = 0; base < items; base += 256 * 8) {       // eight mask words per thread in flight
-        uint32_t bits[8];
+    // a thread takes mask rows tid, tid + 256, ..., four of them and two words of each in flight: a division per row.  (Three per word, the
+    // words of all rows in one range: the launch took 13.1 us behind dq at 12 heads of 37 units, 10.0 like this; 6.7 without the ordering.)
+    const int w0 = q.first_block >> 5, nw = ((q.first_block + q.n_b - 1) >> 5) - w0 + 1, rows = q.BH * q.Tm;
+    for (int r0 = tid; r0 < rows; r0 += 4 * 256)
+        for (int x0 = 0; x0 < nw; x0 += 2) {
+            uint32_t bits[4][2];
 #pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            const int it = base + x * 256 + tid, r = it / nw;
-            bits[x] = it < items ? __ldg(q.mask + (size_t)r * q.mask_words + w0 + (it - r * nw)) : 0u;
-        }
+            for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            const int it = base + x * 256 + tid, r = it / nw, bh = r / q.Tm;
-            const int j0 = (w0 + it - r * nw) * 32 - q.first_block;
-            while (bits[x]) {
-                const int j = j0 + __ffs(bits[x]) - 1;
-                bits[x] &= bits[x] - 1;
-                if (j >= 0 && j < q.n_b) atomicAdd(&cnt[bh * q.n_b + j], 1);
+                for (int x = 0; x < 2; ++x)
+                    bits[i][x] = r0 + 256 * i < rows && x0 + x < nw ? __ldg(q.mask + (size_t)(r0 + 256 * i) * q.mask_words + w0 + x0 + x) : 0u;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (r0 + 256 * i >= rows) break;
+                int* mine = cnt + (r0 + 256 * i) / q.Tm * q.n_b;
+#pragma unroll
+                for (int x = 0; x < 2; ++x) {
+                    const int j0 = (w0 + x0 + x) * 32 - q.first_block;
+                    uint32_t left = bits[i][x];
+                    while (left) {
+                        const int j = j0 + __ffs(left) - 1;
+                        left &= left - 1;
+                        if (j >= 0 && j < q.n_b) atomicAdd(mine + j, 1);
+                    }
+                }
             }
         }
-    }
     __syncthreads();
     for (int u = tid; u < n; u += 256) atomicAdd(&at[q.Tm - cnt[u] + 1], 1);
     __syncthreads();
