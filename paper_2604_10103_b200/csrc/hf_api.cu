@@ -203,11 +203,11 @@ void free_all(hf_ctx* c) {
 #define HF_TC5P_COLGROUPS 1   // column groups per tile group of the ping-pong attention kernel
 #endif
 
-template <int D, int BLK>
+template <int D, int BLK, int NG>
 hf_status set_swa_tc5_attr() {
-    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D>::SMEM_BYTES));
-    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D>::SMEM_BYTES));
-    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D>::SMEM_BYTES));
+    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 0, NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D, NG>::SMEM_BYTES));
+    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 1, NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D, NG>::SMEM_BYTES));
+    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 2, NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D, NG>::SMEM_BYTES));
     return HF_OK;
 }
 template <int BLK, int D>
@@ -257,9 +257,10 @@ hf_status set_attrs(const hf_ctx* c) {
     const int b = c->cfg.block;
     if (c->swa_kernel == HF_SWA_TCGEN05_PINGPONG)
         HF_CUDA(cudaFuncSetAttribute(k_swa_tc5p<D, HF_TC5P_COLGROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5P<D, HF_TC5P_COLGROUPS>::SMEM_BYTES));
-    else if (c->swa_kernel == HF_SWA_TCGEN05)
-        HF_TRY((b == 128 ? set_swa_tc5_attr<D, 128>() : b == 64 ? set_swa_tc5_attr<D, 64>() : set_swa_tc5_attr<D, 16>()));
-    else
+    else if (c->swa_kernel == HF_SWA_TCGEN05) {
+        HF_TRY((b == 128 ? set_swa_tc5_attr<D, 128, 2>() : b == 64 ? set_swa_tc5_attr<D, 64, 2>() : set_swa_tc5_attr<D, 16, 2>()));
+        if (D == 64 && b == 128) HF_TRY((set_swa_tc5_attr<64, 128, 4>()));
+    } else
         HF_TRY((b == 128 ? set_swa_attr<128, D>() : b == 64 ? set_swa_attr<64, D>() : set_swa_attr<16, D>()));
     if (c->cfg.merge == HF_MERGE_FULL_WIDTH)
         HF_CUDA(cudaFuncSetAttribute(k_merge_full<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, MergeFull<D>::SMEM_BYTES));
@@ -335,9 +336,9 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 // 4-D bf16 map [slots, B*H, rows, d] with a box of box_cols x box_rows, 128-byte swizzle (or none); rows past the end read as zero.
-// (the swizzle is the box's row width: 128 or 64 bytes)
+// (the swizzle is the box's row width: 128, 64 or 32 bytes)
 hf_status make_map_ex(hf_ctx* c, CUtensorMap* m, const void* base, long long rows, int slots, int box_cols, int box_rows, bool swizzle) {
-    const CUtensorMapSwizzle sw = box_cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
+    const CUtensorMapSwizzle sw = box_cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : box_cols == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
     const cuuint64_t dims[4] = {(cuuint64_t)c->d, (cuuint64_t)rows, (cuuint64_t)c->BH, (cuuint64_t)slots};
     const cuuint64_t strides[3] = {(cuuint64_t)c->d * 2, (cuuint64_t)rows * c->d * 2, (cuuint64_t)c->BH * rows * c->d * 2};
     const cuuint32_t box[4] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, 1, 1};
@@ -604,10 +605,10 @@ hf_status launch_swa_mma_t(hf_ctx* c, const bf16* q, const ChunkTable& tab, cons
 // The tcgen05 attention kernel.  Blocks of 16 or 64 tokens: first the kept lists of the query blocks that share a 128-row unit
 // are merged (k_union_tiles), unless the selection of the same call has done that (merged).  hist_inside: the kernel forms the history term; overlap_prev: it may be launched under the tail
 // of the kernel before it in the stream.
-template <int D, int BLK>
+template <int D, int BLK, int NG>
 hf_status launch_swa_tc5_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_cur, const bf16* v_cur, const int32_t* idx,
                            int keep, const float* hist, bf16* o, float* lse, cudaStream_t st, bool hist_inside, bool overlap_prev, bool merged) {
-    typedef SwaTc5<D> C;
+    typedef SwaTc5<D, NG> C;
     Tc5Params p;
     memset(&p, 0, sizeof(p));
     p.upb = (c->Tc + 127) / 128; p.n_units = p.upb * c->BH;
@@ -642,9 +643,9 @@ hf_status launch_swa_tc5_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16* 
     const CUtensorMap& rv = c->R + c->n_sink_max > 0 ? L.tm_vring : tv;
     const int grid = p.n_units < c->sm_count ? p.n_units : c->sm_count;
     PdlLaunch pl(dim3(grid), dim3(C::THREADS), C::SMEM_BYTES, st, overlap_prev);
-    if (hist_inside && c->has_rope_q) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 2>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
-    else if (hist_inside) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 1>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
-    else HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 0>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
+    if (hist_inside && c->has_rope_q) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 2, NG>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
+    else if (hist_inside) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 1, NG>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
+    else HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 0, NG>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
     return post_launch(c, "k_swa_tc5");
 }
 
@@ -675,7 +676,8 @@ hf_status launch_swa(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_cur,
                      int keep, const float* hist, bf16* o, float* lse, cudaStream_t st, bool hist_inside = false, bool overlap_prev = false, bool merged = false) {
     if (c->swa_kernel == HF_SWA_TCGEN05) {
         const int b = c->cfg.block, d = c->d;
-#define HF_TC5_CASE(D_, B_) if (d == D_ && b == B_) return launch_swa_tc5_t<D_, B_>(c, L, q, k_cur, v_cur, idx, keep, hist, o, lse, st, hist_inside, overlap_prev, merged)
+        if (swa_groups(d, b, keep) == 4) return launch_swa_tc5_t<64, 128, 4>(c, L, q, k_cur, v_cur, idx, keep, hist, o, lse, st, hist_inside, overlap_prev, merged);
+#define HF_TC5_CASE(D_, B_) if (d == D_ && b == B_) return launch_swa_tc5_t<D_, B_, 2>(c, L, q, k_cur, v_cur, idx, keep, hist, o, lse, st, hist_inside, overlap_prev, merged)
         HF_TC5_CASE(128, 128); HF_TC5_CASE(128, 64); HF_TC5_CASE(128, 16); HF_TC5_CASE(64, 128); HF_TC5_CASE(64, 64); HF_TC5_CASE(64, 16);
 #undef HF_TC5_CASE
     }

@@ -13,9 +13,9 @@
 //                   that keep a random quarter each, ~100 % when neighbouring query blocks keep the same blocks.  A unit's
 //                   first tile holds the first kept block of every row group, so that every row has a finite maximum there.
 //
-// Roles (12 warps):
-//   softmax warps 0-7   two column groups of four warps; thread (group g, row r) owns S columns [64 g, 64 g + 64) of row r
-//                       (TMEM lane = row) and half of the O columns.  It takes its share of S into registers (the S buffer is
+// Roles (12 warps, 20 with four column groups):
+//   softmax warps       two column groups of four warps (four at head dim 64, see swa_groups); thread (group g, row r) owns S columns
+//                       [64 g, 64 g + 64) of row r (TMEM lane = row) and half of the O columns.  It takes its share of S into registers (the S buffer is
 //                       free from then on), forms P = exp2(S c - m) and writes it as bf16 to the P buffer.
 //   K loader, V loader  TMA: K tiles (ring of two), V tiles (ring of two), Q, and for HIST the folded state S W^T and z
 //   S warp, P V warp    tcgen05.mma issue, one warp per product.
@@ -36,7 +36,7 @@
 //     arrivals): every instruction the convergence unit has to serve costs, so waits are warp-uniform, arrivals predicated, a
 //     tile's tail flag comes from one ballot over 32 list entries, and full, masked and empty tiles are separate code (selects in
 //     every tile: +9 us of a 134 us forward).  Four groups of 32 columns instead of two (16 warps) cover more of it and pay it
-//     twice as often: 132 against 130 us.
+//     twice as often: 132 against 130 us at head dim 128; at 64 they pay (swa_groups).
 //   - power: back to back the kernel runs at the board's limit (990 W, SM clock 1 965 -> 1 610 MHz), where time follows energy;
 //     packing P with one conversion instead of two adds and a permute is worth 2 % there.
 // Measured against the version with one MMA warp, Q in shared memory, three S buffers and a second kernel (plus a separate
@@ -56,10 +56,17 @@
 #include "k_swa_mma.cuh"
 #include "k_union.cuh"
 
-template <int D>
+// NGROUPS: softmax column groups (four warps each), two or four.  At head dim 64 the products leave the softmax warps' chain between two
+// tiles' exponentials as the bound, and four groups of 32 columns overlap more of it: 444 units of 12 heads, 28 kept blocks of 128
+// tokens 85.6 -> 79.7 us, 10 kept 36.7 -> 34.4.  Below five tiles their meetings at a unit's ends weigh more (24 units of one tile 6.4 ->
+// 6.8 us, of three 8.2 either way), and so do the masked segments of smaller blocks (64-token blocks 117 -> 119 us), and head dim 128
+// has no registers for it: two there.
+inline constexpr int swa_groups(int d, int blk, int tiles) { return d == 64 && blk == 128 && tiles >= 5 ? 4 : 2; }
+
+template <int D, int NGROUPS>
 struct SwaTc5 {
-    static constexpr int NG = 2, NSW = 4 * NG;         // softmax column groups (four warps each); softmax warps
-    static constexpr long long SKEW_CLK = 700;         // offset between the column groups, in clocks (see the softmax warps)
+    static constexpr int NG = NGROUPS, NSW = 4 * NG;   // softmax column groups; softmax warps
+    static constexpr long long SKEW_CLK = NG == 2 ? 700 : 300;       // offset between the column groups, in clocks (see the softmax warps)
     static constexpr int SCOLS = 128 / NG;             // S columns per softmax thread
     static constexpr int OCOLS = D / NG;               // O columns per softmax thread
     static constexpr int SUB = D / 64;                 // 64-column (128-byte) sub-tiles per operand tile
@@ -156,7 +163,7 @@ __device__ __noinline__ void swa_redo_unit(uint8_t* s_gen, const Tc5Params& p, i
         float* den_t = phi_t + ROWS * PS;                                   // [128]
         float* hist_t = reinterpret_cast<float*>(s_gen + M::SMEM_BYTES);    // [128][D], behind the attention tiles
         static_assert(M::TILE_BYTES + (ROWS * PS + ROWS) * 4 <= M::SMEM_BYTES, "phi(Q) tile must fit in the K / V stages");
-        static_assert(M::SMEM_BYTES + ROWS * D * 4 <= SwaTc5<D>::OFF_BAR, "history tile must fit");
+        static_assert(M::SMEM_BYTES + ROWS * D * 4 <= SwaTc5<D, 2>::OFF_BAR, "history tile must fit");
         {   // phi(q) of the unit's rows (zero past the chunk's end): thread = (row, half of the features)
             const int row = tid >> 1, f0 = (tid & 1) * (D / 2);
             const bf16* src = p.q + ((size_t)bh * p.Tc + q0 + row) * D + f0;
@@ -262,15 +269,15 @@ __device__ __forceinline__ float swa_max(const uint32_t* r, int nv) {
 // Persistent: CTA c processes units c, c + gridDim.x, ...
 // HIST 1: the history term is formed here; 2: with its numerator rotated (code of its own: as a branch it cost the plain one
 // 2 % of the call); 0: p.hist, if any, is added.
-template <int D, int BLK, int HIST>
-__global__ void __launch_bounds__(SwaTc5<D>::THREADS, 1)
+template <int D, int BLK, int HIST, int NGROUPS>
+__global__ void __launch_bounds__(SwaTc5<D, NGROUPS>::THREADS, 1)
 k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kring,
           const __grid_constant__ CUtensorMap tm_vring, const __grid_constant__ CUtensorMap tm_kcur,
           const __grid_constant__ CUtensorMap tm_vcur, const __grid_constant__ CUtensorMap tm_sh,
           const __grid_constant__ CUtensorMap tm_sl, const __grid_constant__ CUtensorMap tm_o,
           const __grid_constant__ Tc5Params p) {
     using namespace tc5;
-    typedef SwaTc5<D> C;
+    typedef SwaTc5<D, NGROUPS> C;
     constexpr int G = 128 / BLK;                       // key blocks per tile = row groups per unit
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t s_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -286,7 +293,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
     const uint32_t bar_kf = bar0, bar_vf = bar0 + 16,      // K / V tile t landed
                    bar_sf = bar0 + 32,                     // S_t complete (its K stage is free)
                    bar_se = bar0 + 48,                     // S_t is in the softmax warps' registers (all of them)
-                   bar_pf = bar0 + 64,                     // two: half g of P_t written (4 warps); completion t
+                   bar_pf = bar0 + 64,                     // two: a half of P_t written (half of the softmax warps); completion t
                    bar_pv = bar0 + 80,                     // P V of tile t complete, second half (so its V stage is free)
                    bar_ph = bar0 + 216,                    // ... first half
                    // unit n: Q landed / its shared-memory tile is free, which takes the word of both its readers: the copy to tensor
@@ -528,12 +535,13 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         }
     } else {
         // ================================================================= softmax / epilogue
-        const int grp = warp >> 2;                          // column group: key columns [64 grp, 64 grp + 64) of a tile, half grp of P
+        const int grp = warp >> 2;                          // column group: key columns [SCOLS grp, SCOLS grp + SCOLS) of a tile
+        const int half = grp * 2 / C::NG;                   // the half of P they are in
         const int row = (warp & 3) * 32 + lane;             // query row of the unit = TMEM lane
         const int rg = row / BLK;                           // row group (query block within the unit)
         const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-        constexpr int EPT = BLK == 128 ? 1 : C::SCOLS / BLK;       // list entries (key blocks) under this thread's columns
-        const int col0 = BLK == 128 ? grp * C::SCOLS : 0;          // first column within its key block
+        constexpr int EPT = BLK >= C::SCOLS ? 1 : C::SCOLS / BLK;  // list entries (key blocks) under this thread's columns
+        const int col0 = grp * C::SCOLS % BLK;                     // first column within its key block (0 where it has several)
         const uint32_t bar_xw = bar_x + 8 * (warp & 3);     // partners: the warps with the same rows in the other groups
         float* x_m = reinterpret_cast<float*>(s_gen + C::OFF_XM);
         float* x_l = reinterpret_cast<float*>(s_gen + C::OFF_XS);
@@ -563,13 +571,13 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         // unit are read during the current one
         const int dbh = gridDim.x / p.upb, di = gridDim.x - dbh * p.upb;
         int u = blockIdx.x, bh = u / p.upb, i = u - bh * p.upb, cnt_next = tiles_of(0);
-        const uint32_t bar_own = grp == 0 ? bar_ph : bar_pv;       // product of this group's half of P
+        const uint32_t bar_own = half == 0 ? bar_ph : bar_pv;      // product of its half of P
         // BLK 16, 64: list entries, read one tile ahead.  BLK 128: all that matters here is whether a tile is a chunk's short last
         // block; one bit per tile from a ballot over 32 list entries at a time (lane = entry), read one window ahead.  An entry
         // outside [0, T_n) is block 0 here as for the loader, which reports it.
         auto entries_of = [&](int unit) -> const uint32_t* {
             if constexpr (BLK == 128) return reinterpret_cast<const uint32_t*>(p.idx + (size_t)unit * p.keep);
-            else return p.entries + (size_t)unit * p.max_tiles * G + grp * EPT;
+            else return p.entries + (size_t)unit * p.max_tiles * G + grp * C::SCOLS / BLK;
         };
         uint32_t e_next[EPT], tails = 0;
 #pragma unroll
@@ -710,7 +718,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                         // special-function unit would idle through the latter.  Set back by part of a tile, one group's waits
                         // fall into the other's exponentials.  Nothing couples the groups until the end of the unit.
                         const long long t_skew = clock64();
-                        while (clock64() - t_skew < C::SKEW_CLK) {}
+                        while (clock64() - t_skew < grp * C::SKEW_CLK) {}
                     }
                 }
                 // ---- P = exp2(S*c - m), row sum, bf16 pairs, 32 columns at a time
@@ -768,7 +776,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                 l_run += ((rsum[0].x + rsum[0].y) + (rsum[1].x + rsum[1].y)) + ((rsum[2].x + rsum[2].y) + (rsum[3].x + rsum[3].y));
                 tmem_wait_st();
                 fence_before_sync();
-                arrive_t(bar_pf + 8 * grp);
+                arrive_t(bar_pf + 8 * half);
                 if (HIST && n >= 1 && j == 0 && cnt > 1) release_h();
             }
             if (!ok) break;
@@ -806,7 +814,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             // history products have completed, or were never asked for); in the map's swizzle of the row width.
             const uint32_t stage_off = C::OFF_H + warp * (32 * C::OCOLS * 2);
             uint8_t* stage = s_gen + stage_off + lane * (C::OCOLS * 2);
-            const int swz = C::OCOLS == 64 ? lane & 7 : (lane >> 1) & 3;
+            const int swz = C::OCOLS == 64 ? lane & 7 : C::OCOLS == 32 ? (lane >> 1) & 3 : (lane >> 2) & 1;
             if (!HIST && n >= 1) {
                 if (lane == 0) bulk_wait_read();            // this warp's previous store has read its part
                 __syncwarp();
