@@ -330,22 +330,41 @@ __device__ __forceinline__ uint32_t rank_row(const float* sc, size_t row, int Tn
         const int j = x * 32 + lane;
         key[x] = j < Tn ? score_image(sc[j]) : 0u;
     }
-    uint32_t thr = 0;           // largest value with at least `keep` images at or above it
-    bool exact = keep >= Tn;    // ... and exactly `keep`: no ties to cut (all blocks kept: every image counts)
-    for (uint32_t bit = 0x80000000u; bit != 0u && !exact; bit >>= 1) {
-        const uint32_t cand = thr | bit;
-        int n = 0;
+    // Few keys: every lane counts the images in front of its own (greater, or equal with a lower index; no image is 2^32 - 1, so one more
+    // does not wrap).  Sixty-four shuffles at most, against a chain of ten to twenty votes: a forward of two heads of 64 queries, 16-token
+    // blocks 9.3 -> 8.9 us; 16 forwards of 8 heads of 128, 300 queries and their commit 258.8 -> 253.6.
+    int ahead[KPL <= 2 ? KPL : 1];
+    uint32_t thr = 0;           // more keys: largest value with at least `keep` images at or above it
+    int ties = Tn;              // ... and blocks at the threshold still to be kept, lowest index first
+    if constexpr (KPL <= 2) {
 #pragma unroll
-        for (int x = 0; x < KPL; ++x) n += key[x] >= cand;
-        n = __reduce_add_sync(0xffffffffu, n);
-        if (n >= keep) { thr = cand; exact = n == keep; }
-    }
-    int ties = Tn;              // blocks at the threshold still to be kept, lowest index first
-    if (!exact) {
-        int n = 0;
+        for (int x = 0; x < KPL; ++x) ahead[x] = 0;
 #pragma unroll
-        for (int x = 0; x < KPL; ++x) n += key[x] > thr;
-        ties = keep - __reduce_add_sync(0xffffffffu, n);
+        for (int y = 0; y < KPL; ++y) {
+            const int n = min(32, Tn - 32 * y);
+#pragma unroll 8
+            for (int l = 0; l < n; ++l) {
+                const uint32_t other = __shfl_sync(0xffffffffu, key[y], l);
+#pragma unroll
+                for (int x = 0; x < KPL; ++x) ahead[x] += other + (32 * y + l < 32 * x + lane ? 1u : 0u) > key[x];
+            }
+        }
+    } else {
+        bool exact = keep >= Tn;    // exactly `keep` images at or above the threshold: no ties to cut (all blocks kept: every image counts)
+        for (uint32_t bit = 0x80000000u; bit != 0u && !exact; bit >>= 1) {
+            const uint32_t cand = thr | bit;
+            int n = 0;
+#pragma unroll
+            for (int x = 0; x < KPL; ++x) n += key[x] >= cand;
+            n = __reduce_add_sync(0xffffffffu, n);
+            if (n >= keep) { thr = cand; exact = n == keep; }
+        }
+        if (!exact) {
+            int n = 0;
+#pragma unroll
+            for (int x = 0; x < KPL; ++x) n += key[x] > thr;
+            ties = keep - __reduce_add_sync(0xffffffffu, n);
+        }
     }
     const uint32_t below = (1u << lane) - 1u;
     int pos = 0;
@@ -353,9 +372,14 @@ __device__ __forceinline__ uint32_t rank_row(const float* sc, size_t row, int Tn
 #pragma unroll
     for (int x = 0; x < KPL; ++x) {
         const int j = x * 32 + lane;
-        const uint32_t eq = __ballot_sync(0xffffffffu, j < Tn && key[x] == thr);
-        const bool kept = j < Tn && (key[x] > thr || (key[x] == thr && __popc(eq & below) < ties));
-        ties -= __popc(eq);
+        bool kept;
+        if constexpr (KPL <= 2) {
+            kept = j < Tn && ahead[x] < keep;
+        } else {
+            const uint32_t eq = __ballot_sync(0xffffffffu, j < Tn && key[x] == thr);
+            kept = j < Tn && (key[x] > thr || (key[x] == thr && __popc(eq & below) < ties));
+            ties -= __popc(eq);
+        }
         const uint32_t word = __ballot_sync(0xffffffffu, kept);
         if (lane == x) my_word = word;
         if (kept) {
