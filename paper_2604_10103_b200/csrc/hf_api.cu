@@ -265,8 +265,8 @@ hf_status set_attrs(const hf_ctx* c) {
     if (c->cfg.merge == HF_MERGE_FULL_WIDTH)
         HF_CUDA(cudaFuncSetAttribute(k_merge_full<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, MergeFull<D>::SMEM_BYTES));
     HF_TRY((set_select_attr<D, 1>()));
-    if (b == 128 && c->Tm <= 5) HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 128, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect<D, 128, 1>::smem_bytes(5 * HF_MAX_CHUNKS, 5)));
-    if (b == 16 && c->Tm <= 8) HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 16, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect<D, 16, 8>::smem_bytes(8 * HF_MAX_CHUNKS, 8)));
+    if (b == 128 && c->Tm <= 5) HF_CUDA(cudaFuncSetAttribute(k_pool_select<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 128, 5 * HF_MAX_CHUNKS)));
+    if (b == 16 && c->Tm <= 8) HF_CUDA(cudaFuncSetAttribute(k_pool_select16<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 16, 8 * HF_MAX_CHUNKS)));
     if (forward_lists(c)) HF_TRY((b == 64 ? set_select_attr<D, 2>() : set_select_attr<D, 8>()));
     return set_state_attr<D>();
 }
@@ -544,17 +544,6 @@ cudaError_t launch_select_kernel(hf_ctx* c, const ChunkTable& tab, int Tn, int k
 }
 
 // merged: the attention kernel follows in the same call and takes its merged lists from here.
-// Pooling and selection in one launch (k_pool_select).
-template <int D, int BLK, int R>
-hf_status launch_pool_select(hf_ctx* c, const bf16* q, const bf16* k_cur, const ChunkTable& tab, int Tn, int keep, const SelectOut& o,
-                             const UnionOut& lists, cudaStream_t st) {
-    typedef PoolSelect<D, BLK, R> S;
-    const int nc = (c->Tm + R - 1) / R;
-    PdlLaunch pl(dim3(nc, c->BH), dim3(S::THREADS), S::smem_bytes(Tn, c->n_b), st, true, nc);
-    HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_pool_select<D, BLK, R>, tab, q, k_cur, c->Tc, c->Tm, Tn, keep, -0.f, o, lists));
-    return post_launch(c, "k_pool_select");
-}
-
 // merged: the attention kernel follows in the same call and takes its merged lists from here.
 template <int D>
 hf_status launch_select(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_cur,
@@ -569,8 +558,11 @@ hf_status launch_select(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_c
         if (lists.max_tiles > c->union_max_tiles) return fail(HF_ERR_SHAPE, "tile list of %d tiles exceeds the %d the context was sized for", lists.max_tiles, c->union_max_tiles);
     }
     if (pools_and_selects(c)) {
-        if (c->cfg.block == 128) HF_TRY((launch_pool_select<D, 128, 1>(c, q, k_cur, tab, Tn, keep, o, lists, st)));
-        else HF_TRY((launch_pool_select<D, 16, 8>(c, q, k_cur, tab, Tn, keep, o, lists, st)));
+        const bool one = c->cfg.block == 16;
+        PdlLaunch pl(dim3(one ? 1 : c->Tm, c->BH), dim3(PoolSelect::THREADS), PoolSelect::smem_bytes(D, c->cfg.block, Tn), st, true, one ? 1 : c->Tm);
+        if (one) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_pool_select16<D>, tab, q, k_cur, c->Tc, c->Tm, Tn, keep, -0.f, o, lists));
+        else HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_pool_select<D>, tab, q, k_cur, c->Tc, c->Tm, Tn, keep, -0.f, o));
+        HF_TRY(post_launch(c, "k_pool_select"));
     } else {
         PoolJobs jobs;
         memset(&jobs, 0, sizeof(jobs));

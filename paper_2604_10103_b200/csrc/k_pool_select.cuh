@@ -399,10 +399,10 @@ __device__ __forceinline__ uint32_t rank_row(const float* sc, size_t row, int Tn
 }
 
 // Scores of n key rows of a pass (key_row(j): their D floats in shared memory) against `rows` query rows, sc[r * Tn + j].  R: query rows
-// a thread block may have; 256 threads, 512 for eight.
+// a thread block may have; 512 threads for eight and for one, otherwise 256.
 template <int D, int R, typename KeyRow>
 __device__ __forceinline__ void score_pass(KeyRow key_row, int n, const float* s_q, int rows, float* sc, int Tn, float2 nz) {
-    constexpr int THREADS = R == 8 ? 512 : 256, W = THREADS / R < 128 ? THREADS / R : 128;
+    constexpr int THREADS = R == 8 || R == 1 ? 512 : 256, W = THREADS / R < 128 ? THREADS / R : 128;
     if (n <= W) {               // few keys: one score per thread
         const int j = threadIdx.x % W, r = threadIdx.x / W;
         if (j < n && r < rows) {
@@ -424,7 +424,7 @@ __device__ __forceinline__ void score_pass(KeyRow key_row, int n, const float* s
 template <int KPL, int G, int R>
 __device__ __forceinline__ void finish_rows(const float* s_sc, uint32_t (*s_mask)[32], int bh, int i0, int rows, int Tm, int Tn, int n_b, int keep,
                                             const SelectOut& o, const UnionOut& lists) {
-    constexpr int THREADS = R == 8 ? 512 : 256;
+    constexpr int THREADS = R == 8 || R == 1 ? 512 : 256;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (o.scores_out)
         for (int e = threadIdx.x; e < rows * Tn; e += THREADS) o.scores_out[((size_t)bh * Tm + i0) * Tn + e] = s_sc[e];
@@ -488,23 +488,19 @@ __global__ void __launch_bounds__(Select<D, G, KPL>::THREADS) k_select(ChunkTabl
     finish_rows<KPL, G, C::R>(s_sc, s_mask, bh, i0, rows, Tm, Tn, n_b, keep, o, lists);
 }
 
-// Pooling and selection of one call in one launch, for heads of few blocks.  The thread blocks of a head form a cluster (BLK 128: one per
-// query block, at most five; BLK 16: one for the up to eight query blocks of a unit), pool the query blocks they select for and a
-// share of the current chunk's key blocks each, and hand the key means to one another through distributed shared memory.
-// grid (c, B*H), cluster (c), c = ceil(T_m / R); R: query blocks per thread block.
-//
-// Latency alone: against k_pool_copy + k_select it spares a launch and the means' way through L2 (two heads of 64 queries, 16-token
-// blocks 11.65 -> 10.5 us a forward; 8 heads of 128, 300 queries, selection alone 7.0 -> 4.9).  With more blocks a head the thread
-// blocks are too few for the pooling, which the other form spreads over the device (dispatch: pools_and_selects).
-template <int D, int BLK, int R>
+// Pooling and selection of one call in one launch, for heads of few blocks: latency alone.  Against k_pool_copy + k_select it spares a launch
+// and the means' way through L2 (two heads of 64 queries, 16-token blocks 11.65 -> 10.5 us a forward; 8 heads of 128, 300 queries,
+// selection alone 7.0 -> 4.9).  With more blocks a head the thread blocks are too few for the pooling, which the other form spreads
+// over the device (dispatch: pools_and_selects).  512 threads, and little code, which a thread block runs once, so that fetching it
+// counts: with 256 threads that took a block of queries and one of keys each, and one kernel for both block sizes, 16 forwards of that
+// shape and their commit took 253 us (1 300 clk from the rows' arrival to their sums), 242.5 like this; the two heads 9.2 -> 8.9.
 struct PoolSelect {
-    static constexpr int THREADS = R == 8 ? 512 : 256;
-    static constexpr int G = 128 / BLK, LD = D + 4;
-    static constexpr int NB = 2;                            // blocks in flight (BLK 128: one query block, one key block)
-    static constexpr int PART = BLK == 16 ? 0 : NB * 16 * D;
-    static_assert(BLK == 16 || THREADS == 256, "sixteen threads a row, sixteen rows");
-    // key rows, query rows, chains, scores
-    static int smem_bytes(int Tn, int n_b) { return (Tn * LD + R * D + R * Tn + PART) * (int)sizeof(float); }
+    static constexpr int THREADS = 512;
+    // key rows, query rows, scores, chains (128-token blocks: of one query block and one key block)
+    static int smem_bytes(int d, int block, int Tn) {
+        const int rows = block == 16 ? 8 : 1, part = block == 16 ? 0 : 2 * 16 * d;
+        return (Tn * (d + 4) + rows * d + rows * Tn + part) * (int)sizeof(float);
+    }
 };
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
@@ -513,125 +509,115 @@ __device__ __forceinline__ void cluster_store(uint32_t addr, int rank, float v) 
     asm volatile("{\n.reg .b32 a;\nmapa.shared::cluster.u32 a, %0, %1;\nst.shared::cluster.f32 [a], %2;\n}\n" ::"r"(addr), "r"(rank), "f"(v) : "memory");
 }
 
-template <int D, int BLK, int R>
-__global__ void __launch_bounds__(PoolSelect<D, BLK, R>::THREADS) k_pool_select(ChunkTable tab, const bf16* __restrict__ q, const bf16* __restrict__ k,
-                                                int Tc, int Tm, int Tn, int keep, float neg_zero, SelectOut o, UnionOut lists) {
-    typedef PoolSelect<D, BLK, R> C;
-    constexpr int VEC = D / 16, KPL = 2;        // (T_n <= 8 chunks of 8 blocks)
-    typedef typename VecLoad<VEC>::T V;
-    const float2 nz = make_float2(neg_zero, neg_zero);
-    extern __shared__ __align__(16) float sel_smem[];
-    const int n_b = Tm, n_old = Tn - n_b;
-    float* s_k = sel_smem;                      // [T_n][LD]: key rows, cached chunks' first
-    float* s_q = s_k + Tn * C::LD;              // [R][D]
-    float* s_part = s_q + R * D;                // chains of the blocks in flight
-    float* s_sc = s_part + C::PART;             // [R][Tn]
-    __shared__ uint32_t s_mask[C::G > 1 ? R : 1][32];
-    const int nc = gridDim.x, rank = blockIdx.x, bh = blockIdx.y, i0 = rank * R;
-    const int rows = min(R, Tm - i0);
-    if (nc > 1) cluster_arrive();               // (no thread block writes to another's shared memory before that one has started)
-    pdl_wait();
-    pdl_trigger();              // the attention kernel may be made resident as blocks of this grid leave
-    // cached rows, sixteen bytes per thread and step
-    for (int e = threadIdx.x; e < n_old * (D / 4); e += C::THREADS) {
+// The cached chunks' key means of a head, rows of LD floats, on their way to shared memory.
+template <int D, int LD>
+__device__ __forceinline__ void load_cached_keys(float* s_k, const ChunkTable& tab, int n_old, int n_b, int bh) {
+    for (int e = threadIdx.x; e < n_old * (D / 4); e += PoolSelect::THREADS) {
         const int j = e / (D / 4), part = e % (D / 4);
         int c = 0, jb = j;
         while (jb >= n_b) { jb -= n_b; ++c; }
-        cp_async16(smem_u32(s_k) + (j * C::LD + part * 4) * 4, tab.pooled[c] + ((size_t)bh * n_b + jb) * D + part * 4, true);
+        cp_async16(smem_u32(s_k) + (j * LD + part * 4) * 4, tab.pooled[c] + ((size_t)bh * n_b + jb) * D + part * 4, true);
     }
     cp_async_commit();
-    // ---- block means in the canonical order: the blocks of this thread block, its query blocks first, then key blocks rank, rank + nc, ...
-    const int n_mine = rows + (n_b - rank + nc - 1) / nc;
-    auto block_of = [&](int w, bool& is_q) -> int { is_q = w < rows; return is_q ? i0 + w : rank + (w - rows) * nc; };
-    auto put = [&](bool is_q, int b, int col, float mean) {
-        if (is_q) { s_q[(b - i0) * D + col] = mean; return; }
-        float* at = s_k + (n_old + b) * C::LD + col;
-        if (nc == 1) *at = mean;
-        else for (int x = 0; x < nc; ++x) cluster_store(smem_u32(at), x, mean);
-    };
-    bool started = nc == 1;
-    if constexpr (BLK == 16) {
-        // sixteen chains of one token: a thread takes a block's pair of columns, sixteen loads in flight
-        constexpr int TPB = D / 2, BPS = C::THREADS / TPB;
-        for (int w0 = 0; w0 < n_mine; w0 += BPS) {
-            const int w = w0 + threadIdx.x / TPB, col = (threadIdx.x % TPB) * 2;
-            if (w >= n_mine) continue;
-            bool is_q;
-            const int b = block_of(w, is_q), n = min(BLK, Tc - b * BLK);
-            const bf16* src = (is_q ? q : k) + ((size_t)bh * Tc + (size_t)b * BLK) * D + col;
-            uint32_t u[16];
+}
+
+// 128-token blocks, at most five a head.  grid (T_m, B*H), cluster (T_m): a thread block pools its query block (threads 0 .. 255) and the key
+// block of the same number (the others), hands the key mean round the cluster through distributed shared memory, and ranks its row.
+template <int D>
+__global__ void __launch_bounds__(PoolSelect::THREADS) k_pool_select(ChunkTable tab, const bf16* __restrict__ q, const bf16* __restrict__ k, int Tc,
+                                                                     int Tm, int Tn, int keep, float neg_zero, SelectOut o) {
+    constexpr int VEC = D / 16, MAXR = 8, LD = D + 4;       // MAXR: rows per chain
+    typedef typename VecLoad<VEC>::T V;
+    extern __shared__ __align__(16) float sel_smem[];
+    float* s_k = sel_smem;                      // [T_n][LD]: key rows, cached chunks' first
+    float* s_q = s_k + Tn * LD;                 // [D]
+    float* s_part = s_q + D;                    // [2][16][D]: chains of the two blocks
+    float* s_sc = s_part + 2 * 16 * D;          // [Tn]
+    const int b = blockIdx.x, bh = blockIdx.y, n_old = Tn - Tm, n = min(128, Tc - b * 128);
+    if (Tm > 1) cluster_arrive();               // (no thread block writes to another's shared memory before that one has started)
+    pdl_wait();
+    pdl_trigger();              // the attention kernel may be made resident as blocks of this grid leave
+    const int x = threadIdx.x >> 8, r = (threadIdx.x & 255) >> 4, cv = threadIdx.x & 15;
+    const bf16* src = (x == 0 ? q : k) + ((size_t)bh * Tc + (size_t)b * 128 + r) * D + cv * VEC;
+    V u[MAXR];
 #pragma unroll
-            for (int t = 0; t < 16; ++t) u[t] = t < n ? __ldg(reinterpret_cast<const uint32_t*>(src + (size_t)t * D)) : 0u;
-            float2 tot;
+    for (int i = 0; i < MAXR; ++i)
+        if (r + 16 * i < n) u[i] = __ldg(reinterpret_cast<const V*>(src + (size_t)(16 * i) * D));
+    load_cached_keys<D, LD>(s_k, tab, n_old, Tm, bh);
+    // ---- the block's mean in the canonical order
+    float acc[VEC];
 #pragma unroll
-            for (int t = 0; t < 16; ++t) {
-                const float2 f = unpack_bf16(u[t]);
-                const float x0 = __fadd_rn(0.f, f.x), x1 = __fadd_rn(0.f, f.y);
-                tot.x = t == 0 ? x0 : __fadd_rn(tot.x, x0);
-                tot.y = t == 0 ? x1 : __fadd_rn(tot.y, x1);
-            }
-            put(is_q, b, col, __fdiv_rn(tot.x, (float)n));
-            put(is_q, b, col + 1, __fdiv_rn(tot.y, (float)n));
-        }
-    } else {
-        constexpr int MAXR = BLK / 16;          // rows per chain
-        const int r = threadIdx.x >> 4, cv = threadIdx.x & 15;
-        for (int w0 = 0; w0 < n_mine; w0 += C::NB) {
-            V u[C::NB][MAXR];
-            int n[C::NB];
+    for (int e = 0; e < VEC; ++e) acc[e] = 0.f;
 #pragma unroll
-            for (int x = 0; x < C::NB; ++x) {
-                bool is_q;
-                const int w = w0 + x, b = w < n_mine ? block_of(w, is_q) : 0;
-                n[x] = w < n_mine ? min(BLK, Tc - b * BLK) : 0;
-                if (n[x] > 0) {
-                    const bf16* src = (is_q ? q : k) + ((size_t)bh * Tc + (size_t)b * BLK) * D + cv * VEC;
+    for (int i = 0; i < MAXR; ++i) {
+        if (r + 16 * i < n) {
+            float f[VEC];
+            VecLoad<VEC>::widen(u[i], f);
 #pragma unroll
-                    for (int i = 0; i < MAXR; ++i) {
-                        const int t = r + 16 * i;
-                        if (t < n[x]) u[x][i] = __ldg(reinterpret_cast<const V*>(src + (size_t)t * D));
-                    }
-                }
-            }
-            if (w0 > 0) __syncthreads();        // the chains of the step before have been added up
-#pragma unroll
-            for (int x = 0; x < C::NB; ++x) {
-                float acc[VEC];
-#pragma unroll
-                for (int e = 0; e < VEC; ++e) acc[e] = 0.f;
-#pragma unroll
-                for (int i = 0; i < MAXR; ++i) {
-                    if (r + 16 * i < n[x]) {
-                        float f[VEC];
-                        VecLoad<VEC>::widen(u[x][i], f);
-#pragma unroll
-                        for (int e = 0; e < VEC; ++e) acc[e] = __fadd_rn(acc[e], f[e]);
-                    }
-                }
-                float* part = s_part + (x * 16 + r) * D + cv * VEC;
-#pragma unroll
-                for (int e = 0; e < VEC; e += 4) *reinterpret_cast<float4*>(part + e) = make_float4(acc[e], acc[e + 1], acc[e + 2], acc[e + 3]);
-            }
-            __syncthreads();
-            if (!started) { cluster_wait(); started = true; }
-            for (int e = threadIdx.x; e < C::NB * D; e += C::THREADS) {
-                const int x = e / D, col = e % D, w = w0 + x;
-                if (w < n_mine) {
-                    bool is_q;
-                    const int b = block_of(w, is_q);
-                    const float* part = s_part + x * 16 * D + col;
-                    float tot = part[0];
-#pragma unroll
-                    for (int rr = 1; rr < 16; ++rr) tot = __fadd_rn(tot, part[rr * D]);
-                    put(is_q, b, col, __fdiv_rn(tot, (float)min(BLK, Tc - b * BLK)));
-                }
-            }
+            for (int e = 0; e < VEC; ++e) acc[e] = __fadd_rn(acc[e], f[e]);
         }
     }
-    cp_async_wait<0>();
-    if (nc > 1) { cluster_arrive(); cluster_wait(); }       // every key mean is in place in every thread block
-    else __syncthreads();
-    score_pass<D, R>([&](int j) { return s_k + j * C::LD; }, Tn, s_q, rows, s_sc, Tn, nz);
+    float* part = s_part + (x * 16 + r) * D + cv * VEC;
+#pragma unroll
+    for (int e = 0; e < VEC; e += 4) *reinterpret_cast<float4*>(part + e) = make_float4(acc[e], acc[e + 1], acc[e + 2], acc[e + 3]);
     __syncthreads();
-    finish_rows<KPL, C::G, R>(s_sc, s_mask, bh, i0, rows, Tm, Tn, n_b, keep, o, lists);
+    if (Tm > 1) cluster_wait();
+    if (threadIdx.x < 2 * D) {
+        const int y = threadIdx.x / D, col = threadIdx.x % D;
+        float tot = s_part[y * 16 * D + col];
+#pragma unroll
+        for (int rr = 1; rr < 16; ++rr) tot = __fadd_rn(tot, s_part[(y * 16 + rr) * D + col]);
+        const float mean = __fdiv_rn(tot, (float)n);
+        float* key = s_k + (n_old + b) * LD + col;
+        if (y == 0) s_q[col] = mean;
+        else if (Tm == 1) *key = mean;
+        else for (int z = 0; z < Tm; ++z) cluster_store(smem_u32(key), z, mean);
+    }
+    cp_async_wait<0>();
+    if (Tm > 1) { cluster_arrive(); cluster_wait(); }       // every key mean is in place in every thread block
+    else __syncthreads();
+    score_pass<D, 1>([&](int j) { return s_k + j * LD; }, Tn, s_q, 1, s_sc, Tn, make_float2(neg_zero, neg_zero));
+    __syncthreads();
+    finish_rows<2, 1, 1>(s_sc, nullptr, bh, b, 1, Tm, Tn, Tm, keep, o, UnionOut{nullptr, nullptr, 0, Tc});      // (T_n <= 8 chunks of 5 blocks)
+}
+
+// 16-token blocks, at most eight a head (one unit of the attention kernel).  grid (1, B*H).  Sixteen chains of one token: a thread takes a
+// block's pair of columns, sixteen loads in flight.
+template <int D>
+__global__ void __launch_bounds__(PoolSelect::THREADS) k_pool_select16(ChunkTable tab, const bf16* __restrict__ q, const bf16* __restrict__ k, int Tc,
+                                                                       int Tm, int Tn, int keep, float neg_zero, SelectOut o, UnionOut lists) {
+    constexpr int R = 8, BLK = 16, LD = D + 4, TPB = D / 2, BPS = PoolSelect::THREADS / TPB;
+    extern __shared__ __align__(16) float sel_smem[];
+    float* s_k = sel_smem;                      // [T_n][LD]: key rows, cached chunks' first
+    float* s_q = s_k + Tn * LD;                 // [R][D]
+    float* s_sc = s_q + R * D;                  // [R][Tn]
+    __shared__ uint32_t s_mask[R][32];
+    const int n_old = Tn - Tm, bh = blockIdx.y;
+    pdl_wait();
+    pdl_trigger();
+    load_cached_keys<D, LD>(s_k, tab, n_old, Tm, bh);
+#pragma unroll 1
+    for (int w = threadIdx.x / TPB; w < 2 * Tm; w += BPS) {         // query blocks, then key blocks
+        const int b = w < Tm ? w : w - Tm, n = min(BLK, Tc - b * BLK), col = (threadIdx.x % TPB) * 2;
+        const bf16* src = (w < Tm ? q : k) + ((size_t)bh * Tc + (size_t)b * BLK) * D + col;
+        uint32_t u[16];
+#pragma unroll
+        for (int t = 0; t < 16; ++t) u[t] = t < n ? __ldg(reinterpret_cast<const uint32_t*>(src + (size_t)t * D)) : 0u;
+        float2 tot;
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+            const float2 f = unpack_bf16(u[t]);
+            const float x0 = __fadd_rn(0.f, f.x), x1 = __fadd_rn(0.f, f.y);
+            tot.x = t == 0 ? x0 : __fadd_rn(tot.x, x0);
+            tot.y = t == 0 ? x1 : __fadd_rn(tot.y, x1);
+        }
+        float* at = w < Tm ? s_q + b * D + col : s_k + (n_old + b) * LD + col;
+        at[0] = __fdiv_rn(tot.x, (float)n);
+        at[1] = __fdiv_rn(tot.y, (float)n);
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+    score_pass<D, R>([&](int j) { return s_k + j * LD; }, Tn, s_q, Tm, s_sc, Tn, make_float2(neg_zero, neg_zero));
+    __syncthreads();
+    finish_rows<2, 8, R>(s_sc, s_mask, bh, 0, Tm, Tm, Tn, Tm, keep, o, lists);
 }
