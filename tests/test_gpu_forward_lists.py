@@ -16,7 +16,7 @@ f64 = gen.bf16_bits_to_f64
     (16, 64, 5, 1, 1000), (16, 128, 128, 8, 300), (16, 64, 77, 3, 300), (16, 128, 129, 3, 300), (16, 64, 1021, 3, 250), (16, 128, 520, 8, 330),
     (64, 64, 64, 1, 1000), (64, 128, 65, 3, 340), (64, 64, 1000, 3, 250), (64, 128, 1025, 2, 400), (64, 64, 2048, 4, 300), (64, 128, 2049, 2, 250),
     (128, 64, 1, 2, 500), (128, 128, 128, 8, 300), (128, 64, 300, 4, 250), (128, 128, 513, 3, 200), (128, 64, 640, 8, 60), (128, 128, 640, 1, 1000),
-    (128, 64, 641, 2, 500), (128, 128, 1025, 8, 120),
+    (128, 64, 641, 2, 500), (128, 128, 1024, 8, 120), (128, 64, 1024, 1, 300), (128, 128, 1025, 8, 120),
 ])
 def test_forward_equals_its_parts(block, d, tokens, chunks, permille):
     import torch
