@@ -242,12 +242,15 @@ inline int union_tiles_max(const hf_ctx* c, int keep, int Tn) {
     return (uni + G - 1) / G;
 }
 
-// Whether pooling and selection are one launch: where a head's blocks are few, so that a thread block per query block (128 tokens) or one
-// for all (16 tokens) has little to pool and the launch it spares weighs more.  Forward calls with it and without: 12 heads of 128,
-// 640 queries 15.9 / 16.7 us, 1 000 queries (T_m 8) 19.9 / 19.5, 1 300 (T_m 11) 27.9 / 25.9; 2 heads of 64 queries, 16-token blocks
-// 11.0 / 11.8 us, 12 heads of 300 queries (T_m 19) 29.1 / 28.1.
+// Whether pooling and selection are one launch: where a head's blocks are few, so that a thread block per query block (128 tokens; a cluster
+// has eight) or one for all (16 tokens) has little to pool, and the launch it spares weighs more.  From six blocks a head on, a grid well
+// above the SMs is slower than the other form, which spreads the pooling evenly.  Forward calls without and with it, 3 chunks cached: 128-token
+// blocks, 12 heads of 128, 700 queries (T_m 6) 16.7 / 14.7 us, 1 024 (T_m 8) 18.6 / 17.2; 24 heads of 64, 1 024 queries 23.0 / 20.8, 48
+// heads 32.1 / 32.8; 16-token blocks, 2 heads of 64 queries 11.8 / 11.0, 12 heads of 300 queries (T_m 19) 28.1 / 29.1.
 inline bool pools_and_selects(const hf_ctx* c) {
-    return !c->has_trope && ((c->cfg.block == 128 && c->Tm <= 5) || (c->cfg.block == 16 && c->Tm <= 8));
+    if (c->has_trope) return false;
+    if (c->cfg.block == 16) return c->Tm <= 8;
+    return c->cfg.block == 128 && (c->Tm <= 5 || (c->Tm <= 8 && 2 * c->BH * c->Tm <= 3 * c->sm_count));
 }
 
 // Shared-memory limits of the kernels that a context of this head_dim, block and attention kernel launches: touching a kernel
@@ -265,7 +268,7 @@ hf_status set_attrs(const hf_ctx* c) {
     if (c->cfg.merge == HF_MERGE_FULL_WIDTH)
         HF_CUDA(cudaFuncSetAttribute(k_merge_full<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, MergeFull<D>::SMEM_BYTES));
     HF_TRY((set_select_attr<D, 1>()));
-    if (b == 128 && c->Tm <= 5) HF_CUDA(cudaFuncSetAttribute(k_pool_select<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 128, 5 * HF_MAX_CHUNKS)));
+    if (b == 128 && c->Tm <= 8) HF_CUDA(cudaFuncSetAttribute(k_pool_select<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 128, 8 * HF_MAX_CHUNKS)));
     if (b == 16 && c->Tm <= 8) HF_CUDA(cudaFuncSetAttribute(k_pool_select16<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 16, 8 * HF_MAX_CHUNKS)));
     if (forward_lists(c)) HF_TRY((b == 64 ? set_select_attr<D, 2>() : set_select_attr<D, 8>()));
     return set_state_attr<D>();
