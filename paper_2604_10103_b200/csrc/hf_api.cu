@@ -243,14 +243,14 @@ inline int union_tiles_max(const hf_ctx* c, int keep, int Tn) {
 }
 
 // Whether pooling and selection are one launch: where a head's blocks are few, so that a thread block per query block (128 tokens; a cluster
-// has eight) or one for all (16 tokens) has little to pool, and the launch it spares weighs more.  From six blocks a head on, a grid well
+// has sixteen, above eight by its kernel's attribute) or one for all (16 tokens) has little to pool, and the launch it spares weighs more.  From six blocks a head on, a grid well
 // above the SMs is slower than the other form, which spreads the pooling evenly.  Forward calls without and with it, 3 chunks cached: 128-token
-// blocks, 12 heads of 128, 700 queries (T_m 6) 16.7 / 14.7 us, 1 024 (T_m 8) 18.6 / 17.2; 24 heads of 64, 1 024 queries 23.0 / 20.8, 48
+// blocks, 12 heads of 128, 700 queries (T_m 6) 16.7 / 14.7 us, 1 024 (T_m 8) 18.6 / 17.2, 1 300 (T_m 11) 25.2 / 22.3, 2 048 (T_m 16) 42.2 / 39.1; 24 heads of 64, 1 024 queries 23.0 / 20.8, 48
 // heads 32.1 / 32.8; 16-token blocks, 2 heads of 64 queries 11.8 / 11.0, 12 heads of 300 queries (T_m 19) 28.1 / 29.1.
 inline bool pools_and_selects(const hf_ctx* c) {
     if (c->has_trope) return false;
     if (c->cfg.block == 16) return c->Tm <= 8;
-    return c->cfg.block == 128 && (c->Tm <= 5 || (c->Tm <= 8 && 2 * c->BH * c->Tm <= 3 * c->sm_count));
+    return c->cfg.block == 128 && (c->Tm <= 5 || (c->Tm <= 16 && 2 * c->BH * c->Tm <= 3 * c->sm_count));
 }
 
 // Shared-memory limits of the kernels that a context of this head_dim, block and attention kernel launches: touching a kernel
@@ -268,7 +268,12 @@ hf_status set_attrs(const hf_ctx* c) {
     if (c->cfg.merge == HF_MERGE_FULL_WIDTH)
         HF_CUDA(cudaFuncSetAttribute(k_merge_full<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, MergeFull<D>::SMEM_BYTES));
     HF_TRY((set_select_attr<D, 1>()));
-    if (b == 128 && c->Tm <= 8) HF_CUDA(cudaFuncSetAttribute(k_pool_select<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 128, 8 * HF_MAX_CHUNKS)));
+    if (b == 128 && c->Tm <= 16) {
+        HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 128, 64)));
+        HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 128, 128)));
+        HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 2>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 4>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    }
     if (b == 16 && c->Tm <= 8) HF_CUDA(cudaFuncSetAttribute(k_pool_select16<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 16, 8 * HF_MAX_CHUNKS)));
     if (forward_lists(c)) HF_TRY((b == 64 ? set_select_attr<D, 2>() : set_select_attr<D, 8>()));
     return set_state_attr<D>();
@@ -564,7 +569,7 @@ hf_status launch_select(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_c
         const bool one = c->cfg.block == 16;
         PdlLaunch pl(dim3(one ? 1 : c->Tm, c->BH), dim3(PoolSelect::THREADS), PoolSelect::smem_bytes(D, c->cfg.block, Tn), st, true, one ? 1 : c->Tm);
         if (one) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_pool_select16<D>, tab, q, k_cur, c->Tc, c->Tm, Tn, keep, -0.f, o, lists));
-        else HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_pool_select<D>, tab, q, k_cur, c->Tc, c->Tm, Tn, keep, -0.f, o));
+        else HF_CUDA(cudaLaunchKernelEx(&pl.cfg, Tn <= 64 ? k_pool_select<D, 2> : k_pool_select<D, 4>, tab, q, k_cur, c->Tc, c->Tm, Tn, keep, -0.f, o));
         HF_TRY(post_launch(c, "k_pool_select"));
     } else {
         PoolJobs jobs;

@@ -521,9 +521,9 @@ __device__ __forceinline__ void load_cached_keys(float* s_k, const ChunkTable& t
     cp_async_commit();
 }
 
-// 128-token blocks, at most eight a head.  grid (T_m, B*H), cluster (T_m): a thread block pools its query block (threads 0 .. 255) and the key
+// 128-token blocks, at most sixteen a head (KPL 2: T_n <= 64, 4: <= 128).  grid (T_m, B*H), cluster (T_m): a thread block pools its query block (threads 0 .. 255) and the key
 // block of the same number (the others), hands the key mean round the cluster through distributed shared memory, and ranks its row.
-template <int D>
+template <int D, int KPL>
 __global__ void __launch_bounds__(PoolSelect::THREADS) k_pool_select(ChunkTable tab, const bf16* __restrict__ q, const bf16* __restrict__ k, int Tc,
                                                                      int Tm, int Tn, int keep, float neg_zero, SelectOut o) {
     constexpr int VEC = D / 16, MAXR = 8, LD = D + 4;       // MAXR: rows per chain
@@ -578,7 +578,7 @@ __global__ void __launch_bounds__(PoolSelect::THREADS) k_pool_select(ChunkTable 
     else __syncthreads();
     score_pass<D, 1>([&](int j) { return s_k + j * LD; }, Tn, s_q, 1, s_sc, Tn, make_float2(neg_zero, neg_zero));
     __syncthreads();
-    finish_rows<2, 1, 1>(s_sc, nullptr, bh, b, 1, Tm, Tn, Tm, keep, o, UnionOut{nullptr, nullptr, 0, Tc});      // (T_n <= 8 chunks of 8 blocks)
+    finish_rows<KPL, 1, 1>(s_sc, nullptr, bh, b, 1, Tm, Tn, Tm, keep, o, UnionOut{nullptr, nullptr, 0, Tc});      // (T_n <= 8 chunks of 16 blocks)
 }
 
 // 16-token blocks, at most eight a head (one unit of the attention kernel).  grid (1, B*H).  Sixteen chains of one token: a thread takes a
