@@ -876,9 +876,13 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
     }
     // ---- second pass (rare): the listed units again, with the running maximum.  Every copy and tensor-core operation
     // of the tile stream has completed (the roles above drain before the barrier), so shared memory is free.
+    // Its rows have also been handed to bulk stores, which must not land behind its own: every warp that issued some (a bulk store
+    // belongs to the thread that issued it) waits until they are complete, before a barrier that all threads of the pass are behind.
     const int n_redo = *redo_cnt;
-    if (n_redo > 0 && *abort_flag == 0 && threadIdx.x < 256) {
-        if (lane == 0) bulk_wait_all();                       // the tile stream's bulk stores of these rows come first
+    if (n_redo > 0 && *abort_flag == 0) {                     // (the same for all threads)
+        if (warp < C::NSW && lane == 0) bulk_wait_all();
+        __syncthreads();
+        if (threadIdx.x >= 256) return;
         fence_proxy_async();
         const int total = n_redo > C::REDO_CAP ? my_units : n_redo;
         for (int r = 0; r < total; ++r) {

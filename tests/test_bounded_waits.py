@@ -25,3 +25,12 @@ def test_every_polling_loop_has_a_limit():
     for f, s in sources().items():
         for m in re.finditer(r"while \(!mbar_try_wait[^;{]*", s):
             assert "clock64() - t0 <" in m.group(0), f"{f}: {m.group(0)}"
+
+
+def test_second_pass_is_behind_every_output_store():
+    """A bulk store is complete for the thread that issued it: each warp of the attention kernel that stores output has to wait itself,
+    in front of a barrier of the whole thread block, before rows are written a second time by other threads."""
+    s = sources()["k_swa_tc5.cuh"]
+    end = s[s.index("const int n_redo"):]
+    wait, meet, leave = (end.index(x) for x in ("if (warp < C::NSW && lane == 0) bulk_wait_all();", "__syncthreads();", "threadIdx.x >= 256"))
+    assert wait < meet < leave < end.index("swa_redo_unit<")
