@@ -1,6 +1,7 @@
 // libhf host side: context, validation, ring bookkeeping (Alg. 2) and kernel dispatch.
 #include "../../include/hf.h"
 #include "hf_common.cuh"
+#include "hf_dispatch.h"
 #include "k_pool_select.cuh"
 #include "k_swa_mma.cuh"
 #include "k_swa_tc5.cuh"
@@ -94,6 +95,7 @@ struct hf_ctx {
     uint32_t* union_entries = nullptr;   // small-block tcgen05 attention: merged kept lists [B*H * units, max tiles, G] ...
     int* union_tiles = nullptr;          // ... and tiles per unit
     int union_max_tiles = 0;
+    int pool_clusters = 0;               // clusters of T_m thread blocks of k_pool_select that the device holds at a time
     // dK / dV: g . o_local per query row [B*H, T_c], and the key blocks of the current chunk, most pairs first, with their number
     // [B*H, n_b].  Both live in `hist`, which no call holds across another (one stream per context): nothing is allocated by a
     // backward call, so it can be captured into a graph.
@@ -242,44 +244,11 @@ inline int union_tiles_max(const hf_ctx* c, int keep, int Tn) {
     return (uni + G - 1) / G;
 }
 
-// Whether pooling and selection are one launch: where a head's blocks are few, so that a thread block per query block (128 tokens; a cluster
-// has sixteen, above eight by its kernel's attribute) or one for all (16 tokens) has little to pool, and the launch it spares weighs more.  From six blocks a head on, a grid well
-// above the SMs is slower than the other form, which spreads the pooling evenly.  Forward calls without and with it, 3 chunks cached: 128-token
-// blocks, 12 heads of 128, 700 queries (T_m 6) 16.7 / 14.7 us, 1 024 (T_m 8) 18.6 / 17.2, 1 300 (T_m 11) 25.2 / 22.3, 2 048 (T_m 16) 42.2 / 39.1; 24 heads of 64, 1 024 queries 23.0 / 20.8, 48
-// heads 32.1 / 32.8; 16-token blocks, 2 heads of 64 queries 11.8 / 11.0, 12 heads of 300 queries (T_m 19) 28.1 / 29.1.
 inline bool pools_and_selects(const hf_ctx* c) {
-    if (c->has_trope) return false;
-    if (c->cfg.block == 16) return c->Tm <= 8;
-    return c->cfg.block == 128 && (c->Tm <= 5 || (c->Tm <= 16 && 2 * c->BH * c->Tm <= 3 * c->sm_count));
+    return !c->has_trope && pool_select_one_launch(c->cfg.block, c->Tm, c->BH, c->sm_count, c->pool_clusters);
 }
-
-// Shared-memory limits of the kernels that a context of this head_dim, block and attention kernel launches: touching a kernel
-// loads it, and the first context of a process would pay for all of them.
-template <int D>
-hf_status set_attrs(const hf_ctx* c) {
-    const int b = c->cfg.block;
-    if (c->swa_kernel == HF_SWA_TCGEN05_PINGPONG)
-        HF_CUDA(cudaFuncSetAttribute(k_swa_tc5p<D, HF_TC5P_COLGROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5P<D, HF_TC5P_COLGROUPS>::SMEM_BYTES));
-    else if (c->swa_kernel == HF_SWA_TCGEN05) {
-        HF_TRY((b == 128 ? set_swa_tc5_attr<D, 128, 2>() : b == 64 ? set_swa_tc5_attr<D, 64, 2>() : set_swa_tc5_attr<D, 16, 2>()));
-        if (D == 64 && b == 128) HF_TRY((set_swa_tc5_attr<64, 128, 4>()));
-    } else
-        HF_TRY((b == 128 ? set_swa_attr<128, D>() : b == 64 ? set_swa_attr<64, D>() : set_swa_attr<16, D>()));
-    if (c->cfg.merge == HF_MERGE_FULL_WIDTH)
-        HF_CUDA(cudaFuncSetAttribute(k_merge_full<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, MergeFull<D>::SMEM_BYTES));
-    HF_TRY((set_select_attr<D, 1>()));
-    if (b == 128 && c->Tm <= 16) {
-        HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 128, 64)));
-        HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 128, 128)));
-        HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 2>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 4>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    }
-    if (b == 16 && c->Tm <= 8) HF_CUDA(cudaFuncSetAttribute(k_pool_select16<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 16, 8 * HF_MAX_CHUNKS)));
-    if (forward_lists(c)) HF_TRY((b == 64 ? set_select_attr<D, 2>() : set_select_attr<D, 8>()));
-    return set_state_attr<D>();
-}
-
-#define HF_DISPATCH_D(c, FN, ...) ((c)->d == 128 ? FN<128>(__VA_ARGS__) : FN<64>(__VA_ARGS__))
+// The one-launch form's kernel for 128-token blocks (KPL: T_n <= 32 KPL).
+template <int D> auto pool_select_kernel(int Tn) { return Tn <= 64 ? k_pool_select<D, 2> : k_pool_select<D, 4>; }
 
 // Launch configuration of a kernel that may start while the kernel before it in the stream still runs (programmatic
 // dependent launch); the kernel calls pdl_wait() before it touches anything that kernel wrote.
@@ -299,6 +268,41 @@ struct PdlLaunch {
         }
     }
 };
+
+// Shared-memory limits of the kernels that a context of this head_dim, block and attention kernel launches: touching a kernel
+// loads it, and the first context of a process would pay for all of them.
+template <int D>
+hf_status set_attrs(hf_ctx* c) {
+    const int b = c->cfg.block;
+    if (c->swa_kernel == HF_SWA_TCGEN05_PINGPONG)
+        HF_CUDA(cudaFuncSetAttribute(k_swa_tc5p<D, HF_TC5P_COLGROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5P<D, HF_TC5P_COLGROUPS>::SMEM_BYTES));
+    else if (c->swa_kernel == HF_SWA_TCGEN05) {
+        HF_TRY((b == 128 ? set_swa_tc5_attr<D, 128, 2>() : b == 64 ? set_swa_tc5_attr<D, 64, 2>() : set_swa_tc5_attr<D, 16, 2>()));
+        if (D == 64 && b == 128) HF_TRY((set_swa_tc5_attr<64, 128, 4>()));
+    } else
+        HF_TRY((b == 128 ? set_swa_attr<128, D>() : b == 64 ? set_swa_attr<64, D>() : set_swa_attr<16, D>()));
+    if (c->cfg.merge == HF_MERGE_FULL_WIDTH)
+        HF_CUDA(cudaFuncSetAttribute(k_merge_full<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, MergeFull<D>::SMEM_BYTES));
+    HF_TRY((set_select_attr<D, 1>()));
+    if (b == 128 && c->Tm <= 16) {
+        HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 128, 64)));
+        HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 128, 128)));
+        if (c->Tm > 8) {
+            HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 2>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+            HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 4>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        }
+        PdlLaunch pl(dim3(c->Tm, c->BH), dim3(PoolSelect::THREADS), PoolSelect::smem_bytes(D, 128, c->max_Tn), 0, false, c->Tm);
+        if (c->Tm > 1 && cudaOccupancyMaxActiveClusters(&c->pool_clusters, pool_select_kernel<D>(c->max_Tn), &pl.cfg) != cudaSuccess) {
+            cudaGetLastError();
+            c->pool_clusters = 0;
+        }
+    }
+    if (b == 16 && c->Tm <= 8) HF_CUDA(cudaFuncSetAttribute(k_pool_select16<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 16, 8 * HF_MAX_CHUNKS)));
+    if (forward_lists(c)) HF_TRY((b == 64 ? set_select_attr<D, 2>() : set_select_attr<D, 8>()));
+    return set_state_attr<D>();
+}
+
+#define HF_DISPATCH_D(c, FN, ...) ((c)->d == 128 ? FN<128>(__VA_ARGS__) : FN<64>(__VA_ARGS__))
 
 hf_status post_launch(hf_ctx* c, const char* what, int n = 1) {
     cudaError_t e = cudaGetLastError();
@@ -569,7 +573,7 @@ hf_status launch_select(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_c
         const bool one = c->cfg.block == 16;
         PdlLaunch pl(dim3(one ? 1 : c->Tm, c->BH), dim3(PoolSelect::THREADS), PoolSelect::smem_bytes(D, c->cfg.block, Tn), st, true, one ? 1 : c->Tm);
         if (one) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_pool_select16<D>, tab, q, k_cur, c->Tc, c->Tm, Tn, keep, -0.f, o, lists));
-        else HF_CUDA(cudaLaunchKernelEx(&pl.cfg, Tn <= 64 ? k_pool_select<D, 2> : k_pool_select<D, 4>, tab, q, k_cur, c->Tc, c->Tm, Tn, keep, -0.f, o));
+        else HF_CUDA(cudaLaunchKernelEx(&pl.cfg, pool_select_kernel<D>(Tn), tab, q, k_cur, c->Tc, c->Tm, Tn, keep, -0.f, o));
         HF_TRY(post_launch(c, "k_pool_select"));
     } else {
         PoolJobs jobs;
