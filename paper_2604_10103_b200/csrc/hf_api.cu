@@ -95,7 +95,7 @@ struct hf_ctx {
     uint32_t* union_entries = nullptr;   // small-block tcgen05 attention: merged kept lists [B*H * units, max tiles, G] ...
     int* union_tiles = nullptr;          // ... and tiles per unit
     int union_max_tiles = 0;
-    int pool_clusters = 0;               // clusters of T_m thread blocks of k_pool_select that the device holds at a time
+    int pool_clusters = 0;               // clusters of k_pool_select that the device holds at a time (of pool_select_cluster(T_m) thread blocks)
     // dK / dV: g . o_local per query row [B*H, T_c], and the key blocks of the current chunk, most pairs first, with their number
     // [B*H, n_b].  Both live in `hist`, which no call holds across another (one stream per context): nothing is allocated by a
     // backward call, so it can be captured into a graph.
@@ -245,7 +245,7 @@ inline int union_tiles_max(const hf_ctx* c, int keep, int Tn) {
 }
 
 inline bool pools_and_selects(const hf_ctx* c) {
-    return !c->has_trope && pool_select_one_launch(c->cfg.block, c->Tm, c->BH, c->sm_count, c->pool_clusters);
+    return !c->has_trope && pool_select_one_launch(c->cfg.block, c->Tm, c->BH, c->pool_clusters);
 }
 // The one-launch form's kernel for 128-token blocks (KPL: T_n <= 32 KPL).
 template <int D> auto pool_select_kernel(int Tn) { return Tn <= 64 ? k_pool_select<D, 2> : k_pool_select<D, 4>; }
@@ -287,12 +287,13 @@ hf_status set_attrs(hf_ctx* c) {
     if (b == 128 && c->Tm <= 16) {
         HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 128, 64)));
         HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 128, 128)));
-        if (c->Tm > 8) {
+        const int cluster = pool_select_cluster(c->Tm);
+        if (cluster > 8) {
             HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 2>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
             HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 4>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         }
-        PdlLaunch pl(dim3(c->Tm, c->BH), dim3(PoolSelect::THREADS), PoolSelect::smem_bytes(D, 128, c->max_Tn), 0, false, c->Tm);
-        if (c->Tm > 1 && cudaOccupancyMaxActiveClusters(&c->pool_clusters, pool_select_kernel<D>(c->max_Tn), &pl.cfg) != cudaSuccess) {
+        PdlLaunch pl(dim3(cluster, c->BH), dim3(PoolSelect::THREADS), PoolSelect::smem_bytes(D, 128, c->max_Tn), 0, false, cluster);
+        if (cluster > 1 && cudaOccupancyMaxActiveClusters(&c->pool_clusters, pool_select_kernel<D>(c->max_Tn), &pl.cfg) != cudaSuccess) {
             cudaGetLastError();
             c->pool_clusters = 0;
         }

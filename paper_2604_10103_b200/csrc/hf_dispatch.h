@@ -1,14 +1,24 @@
 // Which of two forms a call takes, where that is a function of numbers alone (host code without CUDA).
 #pragma once
 
-// Whether pooling and selection are one launch: where a head's blocks are few, so that a thread block per query block (128 tokens; a cluster
-// has sixteen, above eight by its kernel's attribute) or one for all (16 tokens) has little to pool, and the launch it spares weighs more.  From six blocks a head on, a grid well
-// above the SMs is slower than the other form, which spreads the pooling evenly.  Forward calls without and with it, 3 chunks cached: 128-token
-// blocks, 12 heads of 128, 700 queries (T_m 6) 16.7 / 14.7 us, 1 024 (T_m 8) 18.6 / 17.2, 1 300 (T_m 11) 25.2 / 22.3, 2 048 (T_m 16) 42.2 / 39.1; 24 heads of 64, 1 024 queries 23.0 / 20.8, 48
-// heads 32.1 / 32.8; 16-token blocks, 2 heads of 64 queries 11.8 / 11.0, 12 heads of 300 queries (T_m 19) 28.1 / 29.1.
-// clusters: how many clusters of T_m thread blocks the device holds at a time.  None (a partition with small groups of SMs): two launches.
-inline bool pool_select_one_launch(int block, int Tm, int BH, int sm_count, int clusters) {
+// Pooling and selection of a head's blocks in one launch: sixteen-token blocks, at most eight a head, by one thread block (faster on any
+// grid: 12 to 1 024 heads 1.11 to 1.38 times); 128-token blocks, at most sixteen a head, by a cluster with a thread block for each (a single
+// block: a thread block alone, faster on any grid).
+//
+// The cluster form spares a launch and the means' way through L2 as long as the clusters of all heads are resident at a time.  Behind
+// the first wave it loses: the two-launch form has shorter thread blocks and spreads the pooling evenly.  `clusters` is how many the
+// device holds by its own count (hf_create asks; 0: none fits, as on a partition with small groups of SMs).  The last tenth of them is not
+// reached in one wave, and clusters of 11 to 15 get the room of 16 (their own counts, 21 to 14, lose from 15 or 17 heads on): those
+// ask for 16.  Forward calls of heads of 128, three chunks cached, two launches / one, at and just past the line (B200: 148 SMs):
+//   T_m 3  (93 clusters)  81 heads 26.0 / 22.8 us,  94 heads 26.8 / 27.0     384 heads 73.0 / 80.1
+//   T_m 5  (56)           49 heads 28.2 / 25.5,     52 heads 28.3 / 28.3    1 024 heads 371 / 431
+//   T_m 8  (33)           28 heads 30.9 / 27.9,     33 heads 31.9 / 32.0    55 heads 43.3 / 43.9
+//   T_m 10 (26)           22 heads 34.2 / 32.1,     24 heads 35.3 / 35.7
+//   T_m 13 (as 16: 14)    14 heads 37.8 / 34.6,     16 heads 38.0 / 39.2    34 heads 54.0 / 58.9
+//   T_m 16 (14)           14 heads 41.7 / 38.9,     15 heads 42.8 / 43.5    27 heads 59.8 / 60.4
+inline int pool_select_cluster(int Tm) { return Tm > 10 ? 16 : Tm; }        // thread blocks of the cluster to ask for
+inline bool pool_select_one_launch(int block, int Tm, int BH, int clusters) {
     if (block == 16) return Tm <= 8;
-    if (block != 128 || (Tm > 1 && clusters < 1)) return false;
-    return Tm <= 5 || (Tm <= 16 && 2 * BH * Tm <= 3 * sm_count);
+    if (block != 128 || Tm > 16) return false;
+    return Tm == 1 || (Tm > 10 ? BH <= clusters : 10 * BH <= 9 * clusters);
 }

@@ -8,7 +8,8 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2604_10103_b200", "csrc")
 SOURCE = """
 #include "hf_dispatch.h"
-extern "C" int one_launch(int block, int Tm, int BH, int sm_count, int clusters) { return pool_select_one_launch(block, Tm, BH, sm_count, clusters); }
+extern "C" int one_launch(int block, int Tm, int BH, int clusters) { return pool_select_one_launch(block, Tm, BH, clusters); }
+extern "C" int cluster_asked_for(int Tm) { return pool_select_cluster(Tm); }
 """
 
 
@@ -24,7 +25,24 @@ def rules(tmp_path_factory):
 def test_pooling_and_selection_without_room_for_a_cluster(rules):
     """Where no cluster of T_m thread blocks can be resident, a head's blocks are pooled and selected in two launches."""
     for Tm in range(1, 40):
-        assert rules.one_launch(128, Tm, 1, 148, 0) == (Tm == 1)          # (one thread block is no cluster)
-        assert rules.one_launch(128, Tm, 1, 148, 1) == (Tm <= 16)
-        assert rules.one_launch(16, Tm, 1, 148, 0) == (Tm <= 8)           # no cluster in this form
-        assert not rules.one_launch(64, Tm, 1, 148, 9)
+        assert rules.one_launch(128, Tm, 1, 0) == (Tm == 1)          # (one thread block is no cluster)
+        assert rules.one_launch(128, Tm, 1, 14) == (Tm <= 16)
+        assert rules.one_launch(16, Tm, 1, 0) == (Tm <= 8)           # no cluster in this form
+        assert not rules.one_launch(64, Tm, 1, 9)
+
+
+# query blocks a head, clusters of the asked size that a B200 holds, most heads measured faster in one launch, fewest measured not faster
+LINE = [(2, 148, 130, 192), (3, 93, 81, 94), (4, 71, 61, 70), (5, 56, 49, 56), (6, 45, 40, 47), (7, 37, 32, 37), (8, 33, 28, 35), (9, 30, 27, 31),
+        (10, 26, 22, 24), (11, 14, 13, 17), (12, 14, 14, 17), (13, 14, 14, 16), (14, 14, 13, 15), (15, 14, 14, 15), (16, 14, 14, 15)]
+
+
+@pytest.mark.parametrize("Tm,clusters,fast,slow", LINE)
+def test_one_launch_up_to_one_wave_of_clusters(rules, Tm, clusters, fast, slow):
+    assert rules.cluster_asked_for(Tm) == (Tm if Tm <= 10 else 16)
+    assert all(rules.one_launch(128, Tm, BH, clusters) for BH in range(1, fast + 1))
+    assert not any(rules.one_launch(128, Tm, BH, clusters) for BH in range(slow, 4096))
+
+
+def test_a_single_block_and_small_blocks_on_any_grid(rules):
+    for BH in (1, 148, 1024, 65535):
+        assert rules.one_launch(128, 1, BH, 0) and rules.one_launch(16, 8, BH, 0) and not rules.one_launch(16, 9, BH, 0)
