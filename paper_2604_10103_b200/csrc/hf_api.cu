@@ -102,8 +102,12 @@ struct hf_ctx {
     float* bwd_delta = nullptr;
     int2* bwd_order = nullptr;
     float* partials = nullptr;       // absorb split partials
-    float* partials_layers = nullptr;    // layer-batched state update: one partial per (layer, batch*head, group)
+    // Layer-batched state update, one partial per (layer, batch*head, group).  Up to as many (layer, batch*head) items as SMs: made with the
+    // context and never moved, since such a call may sit in a graph.  More items: grown on first use, apart from it.
+    float* partials_layers = nullptr;
     size_t partials_layers_count = 0;
+    float* partials_many = nullptr;
+    size_t partials_many_count = 0;
     int nsplit_max = 1;
     float z_scale = 1.f;             // 1 (z = sum of phi(K)) or 1 / tokens_per_frame (per-frame means)
     bf16* stage[4] = {nullptr, nullptr, nullptr, nullptr};   // q, k, v, o staging of the *_host calls
@@ -191,7 +195,7 @@ void free_all(hf_ctx* c) {
     for (auto& L : c->layers) { cudaFree(L.W_full); cudaFree(L.mask); cudaFree(L.idx); }
     cudaFree(c->ring_k_all); cudaFree(c->ring_v_all); cudaFree(c->pooled_k_all); cudaFree(c->S_all); cudaFree(c->z_all);
     cudaFree(c->sf_hi_all); cudaFree(c->sf_lo_all); cudaFree(c->W_all); cudaFree(c->bias_all);
-    cudaFree(c->union_entries); cudaFree(c->union_tiles); cudaFree(c->pooled_q); cudaFree(c->pooled_kcur); cudaFree(c->hist); cudaFree(c->partials); cudaFree(c->partials_layers); cudaFree(c->x_hi); cudaFree(c->x_lo);
+    cudaFree(c->union_entries); cudaFree(c->union_tiles); cudaFree(c->pooled_q); cudaFree(c->pooled_kcur); cudaFree(c->hist); cudaFree(c->partials); cudaFree(c->partials_layers); cudaFree(c->partials_many); cudaFree(c->x_hi); cudaFree(c->x_lo);
     cudaFree(c->dev_status);
     cudaFree(c->rope_q[0]); cudaFree(c->rope_q[1]); cudaFree(c->rope_k[0]); cudaFree(c->rope_k[1]);
     cudaFree(c->trope_tab[0]); cudaFree(c->trope_tab[1]); cudaFree(c->q_rot); cudaFree(c->k_rot);
@@ -428,16 +432,18 @@ hf_status launch_absorb_layers(hf_ctx* c, int first_layer, int n_layers, const C
     p.nsplit = n_tiles < c->nsplit_max ? n_tiles : c->nsplit_max;
     p.ngroup = absorb_groups(p.nsplit);
     p.n_units = n_layers * c->BH * p.ngroup;
-    // scratch for one partial per (item, group), grown on first use (never inside a later call of the same size)
+    // scratch for one partial per (item, group); what the context was made with does not suffice: a buffer that grows on first use
+    // (never inside a later call of the same size)
     const size_t need = (size_t)n_layers * c->BH * p.ngroup * ((size_t)D * D + D);
-    if (need > c->partials_layers_count) {
+    const bool many = need > c->partials_layers_count;
+    if (many && need > c->partials_many_count) {
         HF_CUDA(cudaStreamSynchronize(st));
-        cudaFree(c->partials_layers);
-        c->partials_layers = nullptr; c->partials_layers_count = 0;
-        HF_TRY(dmalloc(&c->partials_layers, need));
-        c->partials_layers_count = need;
+        cudaFree(c->partials_many);
+        c->partials_many = nullptr; c->partials_many_count = 0;
+        HF_TRY(dmalloc(&c->partials_many, need));
+        c->partials_many_count = need;
     }
-    p.partials = c->partials_layers;
+    p.partials = many ? c->partials_many : c->partials_layers;
     for (int l = 0; l < n_layers; ++l) p.slot[l] = slot[l];
     p.cos_k = c->rope_k[0]; p.sin_k = c->rope_k[1]; p.rope_rows = c->Tc; p.dev_status = c->dev_status;
     const int grid = p.n_units < c->sm_count ? p.n_units : c->sm_count;
@@ -448,7 +454,7 @@ hf_status launch_absorb_layers(hf_ctx* c, int first_layer, int n_layers, const C
     unsigned long long has_w = 0;
     for (int l = 0; l < n_layers; ++l) if (c->layers[first_layer + l].has_w) has_w |= 1ull << l;
     PdlLaunch pf(dim3(D / 16, c->BH, n_layers), dim3(2 * D), 0, st, true);
-    HF_CUDA(cudaLaunchKernelEx(&pf.cfg, k_reduce_fold<D, 3>, (const float*)c->partials_layers, p.ngroup, p.ngroup,
+    HF_CUDA(cudaLaunchKernelEx(&pf.cfg, k_reduce_fold<D, 3>, (const float*)p.partials, p.ngroup, p.ngroup,
                                c->S_all + (size_t)first_layer * dd, c->z_all + (size_t)first_layer * dz, c->z_scale,
                                (const bf16*)(c->W_all ? c->W_all + (size_t)first_layer * c->cfg.heads * D * D : nullptr), c->cfg.heads,
                                c->BH, c->sf_hi_all + (size_t)first_layer * dd, c->sf_lo_all + (size_t)first_layer * dd, has_w));
@@ -905,7 +911,7 @@ hf_status hf_create(const hf_config* cfg, int device, hf_ctx** out) {
     if (s == HF_OK && cfg->merge == HF_MERGE_FULL_WIDTH) s = dmalloc(&c->x_hi, c->chunk_elems);
     if (s == HF_OK && cfg->merge == HF_MERGE_FULL_WIDTH) s = dmalloc(&c->x_lo, c->chunk_elems);
     if (s == HF_OK) s = dmalloc(&c->partials, (size_t)c->BH * c->nsplit_max * ((size_t)c->d * c->d + c->d));
-    if (s == HF_OK && c->cfg.layers > 1) {      // the layer-batched update of up to as many items as SMs allocates nothing; larger calls grow it
+    if (s == HF_OK && c->cfg.layers > 1) {      // the layer-batched update of up to as many items as SMs
         const size_t items = (size_t)c->cfg.layers * c->BH < (size_t)c->sm_count ? (size_t)c->cfg.layers * c->BH : (size_t)c->sm_count;
         c->partials_layers_count = items * 2 * ((size_t)c->d * c->d + c->d);
         s = dmalloc(&c->partials_layers, c->partials_layers_count);

@@ -77,6 +77,37 @@ def test_commit_of_few_layers_in_a_graph():
         a.close(); b.close()
 
 
+def test_a_captured_commit_of_few_layers_outlives_an_update_of_many():
+    """A graph holds the commit of two layers; an update of all fourteen (more items than SMs) then needs more scratch than the context was
+    made with.  What the graph writes to must still be there."""
+    import torch
+    from paper_2604_10103_b200 import binding as hf
+    w = gen.Workload("many", batch=1, heads=12, head_dim=64, tokens_per_frame=100, chunk_frames=1, window_frames=2, block=128, topk=0,
+                     keep_permille=500, layers=14, seed=337)
+    assert w.layers * w.heads > torch.cuda.get_device_properties(0).multi_processor_count
+    a, b = (hf.Context(hf.make_config(w)) for _ in range(2))
+    kv = [[[hf.bits_to_cuda(x) for x in gen.clean_kv(w, layer, c)] for layer in range(w.layers)] for c in range(3)]
+    k, v = ([[x[i] for x in chunk] for chunk in kv] for i in range(2))
+    k_ev, v_ev = torch.stack(k[2]), torch.stack(v[2])
+    try:
+        for ctx in (a, b):
+            ctx.hf_kv_append_layers(0, k[0], v[0])
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            a.hf_kv_append_layers(0, k[1][:2], v[1][:2])
+        for ctx in (a, b):
+            ctx.hf_state_absorb_layers(0, w.layers, k_ev, v_ev, w.chunk_tokens)
+        g.replay()
+        b.hf_kv_append_layers(0, k[1][:2], v[1][:2])
+        torch.cuda.synchronize()
+        _same(a, b, w, [hf.bits_to_cuda(x) for x in gen.qkv(w, 0, 9, 0)])
+        assert a.hf_get_device_status() == (0, 0)
+    finally:
+        del g
+        a.close(); b.close()
+
+
 @pytest.mark.parametrize("d,heads", [(64, 1), (128, 3)])
 def test_state_copies(d, heads):
     """Either tensor or both, to this device's memory (a kernel) and to an address that is not 16-byte aligned (a copy)."""
