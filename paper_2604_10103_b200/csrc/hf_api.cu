@@ -138,6 +138,23 @@ hf_status check_ptr(const void* p, const char* name) {
     if (!aligned16(p)) return fail(HF_ERR_INVALID_ARG, "%s is not 16-byte aligned", name);
     return HF_OK;
 }
+// Where a call stands, and what is known of a caller's buffer (hf_dispatch.h).
+Where call_site(const hf_ctx* c, cudaStream_t st) {
+    Where w = {c->device, -1, -1};
+    if (cudaGetDevice(&w.current) != cudaSuccess) { cudaGetLastError(); w.current = -1; }
+    if (st == nullptr || st == cudaStreamLegacy || st == cudaStreamPerThread) w.stream = w.current;
+    else if (cudaStreamGetDevice(st, &w.stream) != cudaSuccess) { cudaGetLastError(); w.stream = -1; }
+    return w;
+}
+CallerMemory caller_memory(const void* p) {
+    CallerMemory m = {p != nullptr, aligned16(p), false, -1};
+    cudaPointerAttributes at;
+    if (!m.given) return m;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return m; }
+    m.device_memory = at.type == cudaMemoryTypeDevice;
+    m.device = at.device;
+    return m;
+}
 hf_status check_layer(hf_ctx* c, int layer) {
     if (c == nullptr) return fail(HF_ERR_INVALID_ARG, "ctx is null");
     if (layer < 0 || layer >= c->cfg.layers) return fail(HF_ERR_INVALID_ARG, "layer %d outside [0, %d)", layer, c->cfg.layers);
@@ -1403,17 +1420,11 @@ hf_status hf_get_state(hf_ctx* c, int layer, float* S, float* z, void* stream) {
     LayerState& L = c->layers[layer];
     cudaStream_t st = (cudaStream_t)stream;
     const size_t n_S = (size_t)c->BH * c->d * c->d, n_z = (size_t)c->BH * c->d;
-    // Memory of this device, aligned: one kernel that may be set up under the tail of the one before.  (Two copies one after the other
-    // ended 8 us behind a read-out, this 1.6: 32 760 tokens absorbed, read and their state taken out 67.5 -> 63.5 us.)  Anything
-    // else: the copies, which take or refuse it as they always have.
-    auto here = [&](const void* p) {
-        cudaPointerAttributes at;
-        if (p == nullptr) return true;
-        if (!aligned16(p)) return false;
-        if (cudaPointerGetAttributes(&at, p) != cudaSuccess) { cudaGetLastError(); return false; }
-        return at.type == cudaMemoryTypeDevice && at.device == c->device;
-    };
-    if ((S || z) && here(S) && here(z)) {
+    // Memory of this device, aligned, this device current and the stream one of its own: one kernel that may be set up under the tail of
+    // the one before.  (Two copies one after the other ended 8 us behind a read-out, this 1.6: 32 760 tokens absorbed, read and their
+    // state taken out 67.5 -> 63.5 us.)  Anything else: the copies, which take or refuse it as they always have.
+    const Where where = call_site(c, st);
+    if ((S || z) && kernel_instead_of_copy(where, caller_memory(S)) && kernel_instead_of_copy(where, caller_memory(z))) {
         const int nS = S ? (int)(n_S / 4) : 0, nz = z ? (int)(n_z / 4) : 0;
         PdlLaunch pl(dim3((nS + nz + 255) / 256), dim3(256), 0, st, true);
         HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_copy_state, (const float4*)L.S, (float4*)S, nS, (const float4*)L.z, (float4*)z, nz));

@@ -22,3 +22,11 @@ inline bool pool_select_one_launch(int block, int Tm, int BH, int clusters) {
     if (block != 128 || Tm > 16) return false;
     return Tm == 1 || (Tm > 10 ? BH <= clusters : 10 * BH <= 9 * clusters);
 }
+
+// Whether a call that could be a copy may launch a kernel instead.  A copy takes any stream and any memory that the runtime can copy
+// between; a kernel runs on the current device only, on a stream of that device, and reaches for certain only memory of its own.
+struct Where { int context, current, stream; };          // devices: the context's, the calling thread's current one, the stream's (-1: unknown)
+struct CallerMemory { bool given, aligned, device_memory; int device; };
+inline bool kernel_instead_of_copy(const Where& w, const CallerMemory& m) {
+    return w.current == w.context && w.stream == w.context && (!m.given || (m.aligned && m.device_memory && m.device == w.context));
+}

@@ -9,6 +9,9 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 SOURCE = """
 #include "hf_dispatch.h"
 extern "C" int one_launch(int block, int Tm, int BH, int clusters) { return pool_select_one_launch(block, Tm, BH, clusters); }
+extern "C" int by_kernel(int context, int current, int stream, int given, int aligned, int device_memory, int device) {
+    return kernel_instead_of_copy(Where{context, current, stream}, CallerMemory{given != 0, aligned != 0, device_memory != 0, device});
+}
 extern "C" int cluster_asked_for(int Tm) { return pool_select_cluster(Tm); }
 """
 
@@ -46,3 +49,17 @@ def test_one_launch_up_to_one_wave_of_clusters(rules, Tm, clusters, fast, slow):
 def test_a_single_block_and_small_blocks_on_any_grid(rules):
     for BH in (1, 148, 1024, 65535):
         assert rules.one_launch(128, 1, BH, 0) and rules.one_launch(16, 8, BH, 0) and not rules.one_launch(16, 9, BH, 0)
+
+
+def test_a_kernel_in_place_of_a_copy_only_at_home(rules):
+    """The state leaves by a kernel where the context's device is current, the stream is one of its own and the buffer is aligned memory of
+    that device; a second device, current or under the stream or under the buffer, takes the copy."""
+    for context in (0, 1):
+        for current in (0, 1):
+            for stream in (-1, 0, 1):
+                home = current == context and stream == context
+                for device in (-1, 0, 1):
+                    assert rules.by_kernel(context, current, stream, 1, 1, 1, device) == (home and device == context)
+                    assert not rules.by_kernel(context, current, stream, 1, 0, 1, device)         # not aligned
+                    assert not rules.by_kernel(context, current, stream, 1, 1, 0, device)         # host, pinned or managed memory
+                assert rules.by_kernel(context, current, stream, 0, 1, 0, -1) == home             # this tensor is not wanted

@@ -131,3 +131,31 @@ def test_state_copies(d, heads):
         assert (S2[:1] == -7).all() and (S2[1 + n_S:] == -7).all() and (z2[:3] == -7).all() and (z2[3 + n_z:] == -7).all()
     finally:
         ctx.close()
+
+
+def test_state_copies_on_a_stream_and_in_a_graph():
+    import torch
+    from paper_2604_10103_b200 import binding as hf
+    w = gen.Workload("state", batch=1, heads=3, head_dim=64, tokens_per_frame=100, chunk_frames=1, window_frames=1, block=128, topk=0,
+                     keep_permille=500, seed=331)
+    ctx = hf.Context(hf.make_config(w))
+    try:
+        ctx.hf_kv_append(0, *[hf.bits_to_cuda(x) for x in gen.clean_kv(w, 0, 0)])
+        new = lambda: (torch.zeros(3, 64, 64, device="cuda"), torch.zeros(3, 64, device="cuda"))  # noqa: E731
+        (S, z), (S1, z1), (S2, z2) = new(), new(), new()
+        ctx.hf_get_state(0, S, z)
+        torch.cuda.synchronize()
+        n, side = ctx.hf_launch_count(), torch.cuda.Stream()
+        with torch.cuda.stream(side):
+            ctx.hf_get_state(0, S1, z1)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            ctx.hf_get_state(0, S2, z2)
+        g.replay()
+        torch.cuda.synchronize()
+        assert ctx.hf_launch_count() - n == 2            # one kernel a call on either stream
+        assert S.abs().sum() > 0 and torch.equal(S, S1) and torch.equal(S, S2) and torch.equal(z, z1) and torch.equal(z, z2)
+    finally:
+        del g
+        ctx.close()
