@@ -1007,12 +1007,14 @@ hf_status hf_set_rope(hf_ctx* c, const float* cos_q, const float* sin_q, const f
     for (int i = 0; i < 4; ++i) {
         if (src[i] == nullptr) continue;
         HF_TRY(check_ptr(src[i], "rotation table"));
-        if (*dst[i] == nullptr) HF_TRY(dmalloc(dst[i], count));
-        if (i >= 2) { HF_CUDA(cudaMemcpyAsync(*dst[i], src[i], count * sizeof(float), cudaMemcpyDeviceToDevice, st)); continue; }
-        // the read-out's threads own a query row each: four pairs of neighbouring rows side by side (k_rope_chunks), by way of the history scratch
-        HF_CUDA(cudaMemcpyAsync(c->hist, src[i], count * sizeof(float), cudaMemcpyDeviceToDevice, st));
+        // the queries' tables are kept twice: as the read-out's threads read them, who own a query row each (four pairs of neighbouring rows
+        // side by side, k_rope_chunks), and behind that as the caller laid them out
+        if (*dst[i] == nullptr) HF_TRY(dmalloc(dst[i], i < 2 ? 2 * count : count));
+        float* copy = i < 2 ? *dst[i] + count : *dst[i];
+        HF_CUDA(cudaMemcpyAsync(copy, src[i], count * sizeof(float), cudaMemcpyDeviceToDevice, st));
+        if (i >= 2) continue;
         const int n4 = (int)(count / 4);
-        k_rope_chunks<<<(n4 + 255) / 256, 256, 0, st>>>(reinterpret_cast<const float4*>(c->hist), reinterpret_cast<float4*>(*dst[i]), c->Tc, c->d / 8);
+        k_rope_chunks<<<(n4 + 255) / 256, 256, 0, st>>>(reinterpret_cast<const float4*>(copy), reinterpret_cast<float4*>(*dst[i]), c->Tc, c->d / 8);
         HF_TRY(post_launch(c, "k_rope_chunks"));
     }
     c->has_rope_q = cos_q != nullptr;

@@ -100,3 +100,32 @@ def test_checkpoint_across_the_cap_continues_bit_for_bit():
         assert np.array_equal(Sa, Sb) and np.array_equal(za, zb)
     finally:
         whole.close(); first.close(); second.close()
+
+
+@pytest.mark.parametrize("d,tokens", [(128, 300), (64, 33)])
+def test_rotation_tables_set_again(d, tokens):
+    """Tables of the history branch that replace others, are switched off and set once more: the numbers of a context that had the last
+    ones from the start."""
+    import torch
+    w = gen.Workload("tables", batch=1, heads=3, head_dim=d, tokens_per_frame=tokens, chunk_frames=1, window_frames=2, block=128, topk=0,
+                     keep_permille=500, seed=419)
+    a, b = hz.GpuStream(w), hz.GpuStream(w)
+    rng = torch.Generator(device="cuda").manual_seed(5)
+    angle = lambda: torch.rand(tokens, d // 2, generator=rng, device="cuda") * 6.0  # noqa: E731
+    old, new = [angle(), angle()], [angle(), angle()]
+    tables = lambda x: [f for t in x for f in (t.cos(), t.sin())]  # noqa: E731
+    try:
+        a.ctx.hf_set_rope(*tables(old))
+        a.ctx.hf_set_rope()
+        for x in (a, b):
+            x.ctx.hf_set_rope(*tables(new))
+        for c in range(3):
+            kc, vc = gen.clean_kv(w, 0, c)
+            a.append(a.up(kc), a.up(vc)); b.append(b.up(kc), b.up(vc))
+        q, k, v = (a.up(x) for x in gen.qkv(w, 0, 3, 0))
+        assert np.array_equal(a.linear(q), b.linear(q)) and np.array_equal(a.forward(q, k, v), b.forward(q, k, v))
+        plain = a.linear(q)
+        a.ctx.hf_set_rope(*tables(old))
+        assert not np.array_equal(a.linear(q), plain)
+    finally:
+        a.close(); b.close()

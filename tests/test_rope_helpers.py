@@ -26,3 +26,13 @@ def test_angle_tables_shape_and_rotation():
     x = np.random.default_rng(0).standard_normal((18, 8))
     y = oa.rotate_pairs(x, cos, sin)
     assert np.allclose(np.linalg.norm(y, axis=1), np.linalg.norm(x, axis=1), rtol=1e-6)
+
+
+def test_setting_the_tables_borrows_no_scratch():
+    """hf_set_rope may be ordered behind other work than the context's: it writes the tables and nothing that a call in flight uses."""
+    import os
+    import re
+    path = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2604_10103_b200", "csrc", "hf_api.cu")
+    s = open(path).read()
+    body = s[s.index("hf_status hf_set_rope("):s.index("hf_status hf_set_temporal_rope(")]
+    assert set(re.findall(r"c->(\w+)", body)) <= {"rope_q", "rope_k", "has_rope_q", "has_rope_k", "Tc", "d", "device"}
