@@ -1004,18 +1004,30 @@ hf_status hf_set_rope(hf_ctx* c, const float* cos_q, const float* sin_q, const f
     float** dst[4] = {&c->rope_q[0], &c->rope_q[1], &c->rope_k[0], &c->rope_k[1]};
     const size_t count = (size_t)c->Tc * (c->d / 2);
     cudaStream_t st = (cudaStream_t)stream;
+    const Where where = call_site(c, st);
     for (int i = 0; i < 4; ++i) {
         if (src[i] == nullptr) continue;
         HF_TRY(check_ptr(src[i], "rotation table"));
         // the queries' tables are kept twice: as the read-out's threads read them, who own a query row each (four pairs of neighbouring rows
         // side by side, k_rope_chunks), and behind that as the caller laid them out
-        if (*dst[i] == nullptr) HF_TRY(dmalloc(dst[i], i < 2 ? 2 * count : count));
+        if (*dst[i] == nullptr) {
+            if (where.current != c->device) HF_CUDA(cudaSetDevice(c->device));
+            const hf_status s = dmalloc(dst[i], i < 2 ? 2 * count : count);
+            if (where.current != c->device && where.current >= 0) cudaSetDevice(where.current);
+            HF_TRY(s);
+        }
         float* copy = i < 2 ? *dst[i] + count : *dst[i];
         HF_CUDA(cudaMemcpyAsync(copy, src[i], count * sizeof(float), cudaMemcpyDeviceToDevice, st));
         if (i >= 2) continue;
-        const int n4 = (int)(count / 4);
-        k_rope_chunks<<<(n4 + 255) / 256, 256, 0, st>>>(reinterpret_cast<const float4*>(copy), reinterpret_cast<float4*>(*dst[i]), c->Tc, c->d / 8);
-        HF_TRY(post_launch(c, "k_rope_chunks"));
+        if (kernel_instead_of_copy(where, CallerMemory{false, true, true, c->device})) {
+            const int n4 = (int)(count / 4);
+            k_rope_chunks<<<(n4 + 255) / 256, 256, 0, st>>>(reinterpret_cast<const float4*>(copy), reinterpret_cast<float4*>(*dst[i]), c->Tc, c->d / 8);
+            HF_TRY(post_launch(c, "k_rope_chunks"));
+        } else {        // from another device's point of view: a strided copy for each four pairs
+            for (int x = 0; x < c->d / 8; ++x)
+                HF_CUDA(cudaMemcpy2DAsync(*dst[i] + (size_t)x * c->Tc * 4, 16, copy + 4 * x, (size_t)c->d / 2 * sizeof(float), 16, c->Tc,
+                                          cudaMemcpyDeviceToDevice, st));
+        }
     }
     c->has_rope_q = cos_q != nullptr;
     c->has_rope_k = cos_k != nullptr;
