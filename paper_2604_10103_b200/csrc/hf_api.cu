@@ -238,13 +238,18 @@ hf_status set_swa_attr() {
     HF_CUDA(cudaFuncSetAttribute(k_swa_mma<BLK, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaMma<BLK, D>::SMEM_BYTES));
     return HF_OK;
 }
-template <int D, int G>
-hf_status set_select_attr() {
-    HF_CUDA(cudaFuncSetAttribute(k_select<D, 4, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G, 4>::smem_bytes(128)));
-    HF_CUDA(cudaFuncSetAttribute(k_select<D, 8, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G, 8>::smem_bytes(256)));
-    HF_CUDA(cudaFuncSetAttribute(k_select<D, 16, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G, 16>::smem_bytes(512)));
-    HF_CUDA(cudaFuncSetAttribute(k_select<D, 32, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G, 32>::smem_bytes(HF_MAX_TN)));
+template <int D, int G, int KPL>
+hf_status set_select_attr_kpl(const hf_ctx* c) {
+    if (!select_uses(KPL, c->n_b, c->max_Tn)) return HF_OK;
+    HF_CUDA(cudaFuncSetAttribute(k_select<D, KPL, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G, KPL>::smem_bytes(32 * KPL)));
     return HF_OK;
+}
+template <int D, int G>
+hf_status set_select_attr(const hf_ctx* c) {
+    HF_TRY((set_select_attr_kpl<D, G, 4>(c)));
+    HF_TRY((set_select_attr_kpl<D, G, 8>(c)));
+    HF_TRY((set_select_attr_kpl<D, G, 16>(c)));
+    return set_select_attr_kpl<D, G, 32>(c);
 }
 template <int D>
 hf_status set_state_attr() {
@@ -298,20 +303,21 @@ hf_status set_attrs(hf_ctx* c) {
     if (c->swa_kernel == HF_SWA_TCGEN05_PINGPONG)
         HF_CUDA(cudaFuncSetAttribute(k_swa_tc5p<D, HF_TC5P_COLGROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5P<D, HF_TC5P_COLGROUPS>::SMEM_BYTES));
     else if (c->swa_kernel == HF_SWA_TCGEN05) {
-        HF_TRY((b == 128 ? set_swa_tc5_attr<D, 128, 2>() : b == 64 ? set_swa_tc5_attr<D, 64, 2>() : set_swa_tc5_attr<D, 16, 2>()));
-        if (D == 64 && b == 128) HF_TRY((set_swa_tc5_attr<64, 128, 4>()));
+        // (kept blocks of the shortest and of the longest window: two column groups, four, or both)
+        if (swa_groups(D, b, keep_for(c, c->n_b)) == 2)
+            HF_TRY((b == 128 ? set_swa_tc5_attr<D, 128, 2>() : b == 64 ? set_swa_tc5_attr<D, 64, 2>() : set_swa_tc5_attr<D, 16, 2>()));
+        if (swa_groups(D, b, keep_for(c, c->max_Tn)) == 4) HF_TRY((set_swa_tc5_attr<64, 128, 4>()));
     } else
         HF_TRY((b == 128 ? set_swa_attr<128, D>() : b == 64 ? set_swa_attr<64, D>() : set_swa_attr<16, D>()));
     if (c->cfg.merge == HF_MERGE_FULL_WIDTH)
         HF_CUDA(cudaFuncSetAttribute(k_merge_full<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, MergeFull<D>::SMEM_BYTES));
-    HF_TRY((set_select_attr<D, 1>()));
+    HF_TRY((set_select_attr<D, 1>(c)));
     if (b == 128 && c->Tm <= 16) {
-        HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 128, 64)));
-        HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 128, 128)));
         const int cluster = pool_select_cluster(c->Tm);
-        if (cluster > 8) {
-            HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 2>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-            HF_CUDA(cudaFuncSetAttribute(k_pool_select<D, 4>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        for (int Tn : {64, 128}) {          // the kernels for up to that many key blocks
+            if (Tn == 128 && c->max_Tn <= 64) continue;
+            HF_CUDA(cudaFuncSetAttribute(pool_select_kernel<D>(Tn), cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 128, Tn)));
+            if (cluster > 8) HF_CUDA(cudaFuncSetAttribute(pool_select_kernel<D>(Tn), cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         }
         PdlLaunch pl(dim3(cluster, c->BH), dim3(PoolSelect::THREADS), PoolSelect::smem_bytes(D, 128, c->max_Tn), 0, false, cluster);
         if (cluster > 1 && cudaOccupancyMaxActiveClusters(&c->pool_clusters, pool_select_kernel<D>(c->max_Tn), &pl.cfg) != cudaSuccess) {
@@ -320,7 +326,7 @@ hf_status set_attrs(hf_ctx* c) {
         }
     }
     if (b == 16 && c->Tm <= 8) HF_CUDA(cudaFuncSetAttribute(k_pool_select16<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 16, 8 * HF_MAX_CHUNKS)));
-    if (forward_lists(c)) HF_TRY((b == 64 ? set_select_attr<D, 2>() : set_select_attr<D, 8>()));
+    if (forward_lists(c)) HF_TRY((b == 64 ? set_select_attr<D, 2>(c) : set_select_attr<D, 8>(c)));
     return set_state_attr<D>();
 }
 
@@ -572,10 +578,12 @@ cudaError_t launch_select_kernel(hf_ctx* c, const ChunkTable& tab, int Tn, int k
 #define HF_SELECT(KPL_) do { typedef Select<D, G, KPL_> S; \
         PdlLaunch pl(dim3((c->Tm + S::R - 1) / S::R, c->BH), dim3(S::THREADS), S::smem_bytes(Tn), st, true); \
         return cudaLaunchKernelEx(&pl.cfg, k_select<D, KPL_, G>, tab, (const float*)c->pooled_q, c->n_b, c->Tm, Tn, keep, -0.f, o, lists); } while (0)
-    if (Tn <= 128) HF_SELECT(4);                    // (registers of the ranking warps: T_n / 32 images per lane)
-    if (Tn <= 256) HF_SELECT(8);
-    if (Tn <= 512) HF_SELECT(16);
-    HF_SELECT(32);
+    switch (select_kpl(Tn)) {
+        case 4: HF_SELECT(4);
+        case 8: HF_SELECT(8);
+        case 16: HF_SELECT(16);
+        default: HF_SELECT(32);
+    }
 #undef HF_SELECT
 }
 

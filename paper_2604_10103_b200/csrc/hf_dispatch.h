@@ -30,3 +30,8 @@ struct CallerMemory { bool given, aligned, device_memory; int device; };
 inline bool kernel_instead_of_copy(const Where& w, const CallerMemory& m) {
     return w.current == w.context && w.stream == w.context && (!m.given || (m.aligned && m.device_memory && m.device == w.context));
 }
+
+// Registers of the selection's ranking warps: T_n / 32 images per lane, in steps.
+inline int select_kpl(int Tn) { return Tn <= 128 ? 4 : Tn <= 256 ? 8 : Tn <= 512 ? 16 : 32; }
+// Whether a context whose windows have n_b .. max_Tn key blocks ever launches the step's kernel.
+inline bool select_uses(int kpl, int n_b, int max_Tn) { return select_kpl(n_b) <= kpl && kpl <= select_kpl(max_Tn); }

@@ -12,6 +12,8 @@ extern "C" int one_launch(int block, int Tm, int BH, int clusters) { return pool
 extern "C" int by_kernel(int context, int current, int stream, int given, int aligned, int device_memory, int device) {
     return kernel_instead_of_copy(Where{context, current, stream}, CallerMemory{given != 0, aligned != 0, device_memory != 0, device});
 }
+extern "C" int kpl(int Tn) { return select_kpl(Tn); }
+extern "C" int uses(int kpl, int n_b, int max_Tn) { return select_uses(kpl, n_b, max_Tn); }
 extern "C" int cluster_asked_for(int Tm) { return pool_select_cluster(Tm); }
 """
 
@@ -63,3 +65,15 @@ def test_a_kernel_in_place_of_a_copy_only_at_home(rules):
                     assert not rules.by_kernel(context, current, stream, 1, 0, 1, device)         # not aligned
                     assert not rules.by_kernel(context, current, stream, 1, 1, 0, device)         # host, pinned or managed memory
                 assert rules.by_kernel(context, current, stream, 0, 1, 0, -1) == home             # this tensor is not wanted
+
+
+def test_a_context_touches_the_selection_kernels_of_its_windows_only(rules):
+    """Touching a kernel loads it: those for longer (or shorter) windows than the context can have stay out, and none that it launches."""
+    for n_b in (1, 5, 37, 128, 129, 256, 300, 512, 1024):
+        for chunks in range(1, 9):
+            if n_b * chunks > 1024:
+                continue
+            launched = {rules.kpl(n_b * x) for x in range(1, chunks + 1)}
+            touched = {k for k in (4, 8, 16, 32) if rules.uses(k, n_b, n_b * chunks)}
+            assert launched <= touched and all(min(launched) <= k <= max(launched) for k in touched)
+            assert all(32 * rules.kpl(n_b * x) >= n_b * x for x in range(1, chunks + 1))
