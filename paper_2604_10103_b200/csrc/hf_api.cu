@@ -138,13 +138,10 @@ hf_status check_ptr(const void* p, const char* name) {
     if (!aligned16(p)) return fail(HF_ERR_INVALID_ARG, "%s is not 16-byte aligned", name);
     return HF_OK;
 }
-// Where a call stands, and what is known of a caller's buffer (hf_dispatch.h).
-Where call_site(const hf_ctx* c, cudaStream_t st) {
-    Where w = {c->device, -1, -1};
-    if (cudaGetDevice(&w.current) != cudaSuccess) { cudaGetLastError(); w.current = -1; }
-    if (st == nullptr || st == cudaStreamLegacy || st == cudaStreamPerThread) w.stream = w.current;
-    else if (cudaStreamGetDevice(st, &w.stream) != cudaSuccess) { cudaGetLastError(); w.stream = -1; }
-    return w;
+int current_device() {
+    int d = -1;
+    if (cudaGetDevice(&d) != cudaSuccess) { cudaGetLastError(); return -1; }
+    return d;
 }
 CallerMemory caller_memory(const void* p) {
     CallerMemory m = {p != nullptr, aligned16(p), false, -1};
@@ -1012,30 +1009,32 @@ hf_status hf_set_rope(hf_ctx* c, const float* cos_q, const float* sin_q, const f
     float** dst[4] = {&c->rope_q[0], &c->rope_q[1], &c->rope_k[0], &c->rope_k[1]};
     const size_t count = (size_t)c->Tc * (c->d / 2);
     cudaStream_t st = (cudaStream_t)stream;
-    const Where where = call_site(c, st);
+    const int cur = current_device();
     for (int i = 0; i < 4; ++i) {
         if (src[i] == nullptr) continue;
         HF_TRY(check_ptr(src[i], "rotation table"));
         // the queries' tables are kept twice: as the read-out's threads read them, who own a query row each (four pairs of neighbouring rows
         // side by side, k_rope_chunks), and behind that as the caller laid them out
         if (*dst[i] == nullptr) {
-            if (where.current != c->device) HF_CUDA(cudaSetDevice(c->device));
+            if (cur != c->device) HF_CUDA(cudaSetDevice(c->device));
             const hf_status s = dmalloc(dst[i], i < 2 ? 2 * count : count);
-            if (where.current != c->device && where.current >= 0) cudaSetDevice(where.current);
+            if (cur != c->device && cur >= 0) cudaSetDevice(cur);
             HF_TRY(s);
         }
         float* copy = i < 2 ? *dst[i] + count : *dst[i];
         HF_CUDA(cudaMemcpyAsync(copy, src[i], count * sizeof(float), cudaMemcpyDeviceToDevice, st));
         if (i >= 2) continue;
-        if (kernel_instead_of_copy(where, CallerMemory{false, true, true, c->device})) {
-            const int n4 = (int)(count / 4);
-            k_rope_chunks<<<(n4 + 255) / 256, 256, 0, st>>>(reinterpret_cast<const float4*>(copy), reinterpret_cast<float4*>(*dst[i]), c->Tc, c->d / 8);
-            HF_TRY(post_launch(c, "k_rope_chunks"));
-        } else {        // from another device's point of view: a strided copy for each four pairs
-            for (int x = 0; x < c->d / 8; ++x)
-                HF_CUDA(cudaMemcpy2DAsync(*dst[i] + (size_t)x * c->Tc * 4, 16, copy + 4 * x, (size_t)c->d / 2 * sizeof(float), 16, c->Tc,
-                                          cudaMemcpyDeviceToDevice, st));
+        if (kernel_instead_of_copy(c->device, cur, CallerMemory{false, true, true, c->device})) {
+            PdlLaunch pl(dim3(((int)(count / 4) + 255) / 256), dim3(256), 0, st, false);
+            if (cudaLaunchKernelEx(&pl.cfg, k_rope_chunks, (const float4*)copy, (float4*)*dst[i], c->Tc, c->d / 8) == cudaSuccess) {
+                HF_TRY(post_launch(c, "k_rope_chunks"));
+                continue;
+            }
+            cudaGetLastError();
         }
+        for (int x = 0; x < c->d / 8; ++x)      // another device current, or its stream: a strided copy for each four pairs
+            HF_CUDA(cudaMemcpy2DAsync(*dst[i] + (size_t)x * c->Tc * 4, 16, copy + 4 * x, (size_t)c->d / 2 * sizeof(float), 16, c->Tc,
+                                      cudaMemcpyDeviceToDevice, st));
     }
     c->has_rope_q = cos_q != nullptr;
     c->has_rope_k = cos_k != nullptr;
@@ -1442,15 +1441,16 @@ hf_status hf_get_state(hf_ctx* c, int layer, float* S, float* z, void* stream) {
     LayerState& L = c->layers[layer];
     cudaStream_t st = (cudaStream_t)stream;
     const size_t n_S = (size_t)c->BH * c->d * c->d, n_z = (size_t)c->BH * c->d;
-    // Memory of this device, aligned, this device current and the stream one of its own: one kernel that may be set up under the tail of
-    // the one before.  (Two copies one after the other ended 8 us behind a read-out, this 1.6: 32 760 tokens absorbed, read and their
-    // state taken out 67.5 -> 63.5 us.)  Anything else: the copies, which take or refuse it as they always have.
-    const Where where = call_site(c, st);
-    if ((S || z) && kernel_instead_of_copy(where, caller_memory(S)) && kernel_instead_of_copy(where, caller_memory(z))) {
+    // Memory of this device, aligned, and this device current: one kernel that may be set up under the tail of the one before.  (Two
+    // copies one after the other ended 8 us behind a read-out, this 1.6: 32 760 tokens absorbed, read and their state taken out
+    // 67.5 -> 63.5 us.)  Anything else, a stream of another device included: the copies, which take or refuse it as they always have.
+    const int cur = current_device();
+    if ((S || z) && kernel_instead_of_copy(c->device, cur, caller_memory(S)) && kernel_instead_of_copy(c->device, cur, caller_memory(z))) {
         const int nS = S ? (int)(n_S / 4) : 0, nz = z ? (int)(n_z / 4) : 0;
         PdlLaunch pl(dim3((nS + nz + 255) / 256), dim3(256), 0, st, true);
-        HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_copy_state, (const float4*)L.S, (float4*)S, nS, (const float4*)L.z, (float4*)z, nz));
-        return post_launch(c, "k_copy_state");
+        if (cudaLaunchKernelEx(&pl.cfg, k_copy_state, (const float4*)L.S, (float4*)S, nS, (const float4*)L.z, (float4*)z, nz) == cudaSuccess)
+            return post_launch(c, "k_copy_state");
+        cudaGetLastError();
     }
     if (S) HF_CUDA(cudaMemcpyAsync(S, L.S, n_S * 4, cudaMemcpyDeviceToDevice, st));
     if (z) HF_CUDA(cudaMemcpyAsync(z, L.z, n_z * 4, cudaMemcpyDeviceToDevice, st));

@@ -23,12 +23,13 @@ inline bool pool_select_one_launch(int block, int Tm, int BH, int clusters) {
     return Tm == 1 || (Tm > 10 ? BH <= clusters : 10 * BH <= 9 * clusters);
 }
 
-// Whether a call that could be a copy may launch a kernel instead.  A copy takes any stream and any memory that the runtime can copy
-// between; a kernel runs on the current device only, on a stream of that device, and reaches for certain only memory of its own.
-struct Where { int context, current, stream; };          // devices: the context's, the calling thread's current one, the stream's (-1: unknown)
+// Whether a call that could be a copy may launch a kernel instead.  A copy takes any memory that the runtime can copy between; a kernel
+// runs on the calling thread's current device, and reaches for certain only memory of its own.  (A copy also takes a stream of another device.
+// A launch refuses that, which a caller of this has to answer with the copy: the runtime's question for a stream's device may not be
+// asked while it is being captured.)
 struct CallerMemory { bool given, aligned, device_memory; int device; };
-inline bool kernel_instead_of_copy(const Where& w, const CallerMemory& m) {
-    return w.current == w.context && w.stream == w.context && (!m.given || (m.aligned && m.device_memory && m.device == w.context));
+inline bool kernel_instead_of_copy(int context_device, int current_device, const CallerMemory& m) {
+    return current_device == context_device && (!m.given || (m.aligned && m.device_memory && m.device == context_device));
 }
 
 // Registers of the selection's ranking warps: T_n / 32 images per lane, in steps.

@@ -9,8 +9,8 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 SOURCE = """
 #include "hf_dispatch.h"
 extern "C" int one_launch(int block, int Tm, int BH, int clusters) { return pool_select_one_launch(block, Tm, BH, clusters); }
-extern "C" int by_kernel(int context, int current, int stream, int given, int aligned, int device_memory, int device) {
-    return kernel_instead_of_copy(Where{context, current, stream}, CallerMemory{given != 0, aligned != 0, device_memory != 0, device});
+extern "C" int by_kernel(int context, int current, int given, int aligned, int device_memory, int device) {
+    return kernel_instead_of_copy(context, current, CallerMemory{given != 0, aligned != 0, device_memory != 0, device});
 }
 extern "C" int kpl(int Tn) { return select_kpl(Tn); }
 extern "C" int uses(int kpl, int n_b, int max_Tn) { return select_uses(kpl, n_b, max_Tn); }
@@ -54,17 +54,16 @@ def test_a_single_block_and_small_blocks_on_any_grid(rules):
 
 
 def test_a_kernel_in_place_of_a_copy_only_at_home(rules):
-    """The state leaves by a kernel where the context's device is current, the stream is one of its own and the buffer is aligned memory of
-    that device; a second device, current or under the stream or under the buffer, takes the copy."""
+    """The state leaves by a kernel where the context's device is current and the buffer is aligned memory of that device; a second device,
+    current or under the buffer, takes the copy."""
     for context in (0, 1):
-        for current in (0, 1):
-            for stream in (-1, 0, 1):
-                home = current == context and stream == context
-                for device in (-1, 0, 1):
-                    assert rules.by_kernel(context, current, stream, 1, 1, 1, device) == (home and device == context)
-                    assert not rules.by_kernel(context, current, stream, 1, 0, 1, device)         # not aligned
-                    assert not rules.by_kernel(context, current, stream, 1, 1, 0, device)         # host, pinned or managed memory
-                assert rules.by_kernel(context, current, stream, 0, 1, 0, -1) == home             # this tensor is not wanted
+        for current in (-1, 0, 1):
+            home = current == context
+            for device in (-1, 0, 1):
+                assert rules.by_kernel(context, current, 1, 1, 1, device) == (home and device == context)
+                assert not rules.by_kernel(context, current, 1, 0, 1, device)         # not aligned
+                assert not rules.by_kernel(context, current, 1, 1, 0, device)         # host, pinned or managed memory
+            assert rules.by_kernel(context, current, 0, 1, 0, -1) == home             # this tensor is not wanted
 
 
 def test_a_context_touches_the_selection_kernels_of_its_windows_only(rules):

@@ -37,5 +37,5 @@ def test_setting_the_tables_borrows_no_scratch():
     body = s[s.index("hf_status hf_set_rope("):s.index("hf_status hf_set_temporal_rope(")]
     assert set(re.findall(r"c->(\w+)", body)) <= {"rope_q", "rope_k", "has_rope_q", "has_rope_k", "Tc", "d", "device"}
     # ... by a kernel only where one may run for the context (test_dispatch_rules.py), by copies elsewhere
-    rule, kernel, copies = (body.index(x) for x in ("kernel_instead_of_copy(where", "k_rope_chunks<<<", "cudaMemcpy2DAsync"))
+    rule, kernel, copies = (body.index(x) for x in ("kernel_instead_of_copy(", "k_rope_chunks,", "cudaMemcpy2DAsync"))
     assert rule < kernel < copies
