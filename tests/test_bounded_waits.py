@@ -10,6 +10,10 @@ NAMED = {
     "k_swa_mma.cuh": 1,     # a unit's warps: no role of it has a wait that can run out
     "k_swa_tc5.cuh": 1,     # the second pass: entered by all its threads, after the roles have met and none has given up
 }
+# barriers of a whole cluster: arrive and wait
+CLUSTER = {
+    "k_pool_select.cuh": 2,     # every thread of every thread block reaches them: nothing in front of them can run out or leave
+}
 
 
 def sources():
@@ -19,6 +23,20 @@ def sources():
 def test_no_named_barrier_between_roles():
     found = {f: len(re.findall(r"\b(?:bar|barrier)(?:\.cta)?\.(?:sync|arrive|red)", s)) for f, s in sources().items()}
     assert {f: n for f, n in found.items() if n} == NAMED
+
+
+def test_no_cluster_barrier_behind_a_way_out():
+    found = {f: len(re.findall(r"\bbarrier\.cluster\.(?:arrive|wait)", s)) for f, s in sources().items()}
+    assert {f: n for f, n in found.items() if n} == CLUSTER
+    for f, s in sources().items():
+        s = re.sub(r"__forceinline__ void cluster_\w+\(\)", "", s)                   # (the definitions)
+        for m in re.finditer(r"__global__[^;{]*?\b(k_\w+)\([^{;]*\{", s, re.S):
+            body = s[m.end():s.find("\n}\n", m.end())]
+            if "cluster_arrive()" not in body and "cluster_wait()" not in body:
+                continue
+            assert f in CLUSTER and "mbar_" not in body and "while" not in body, m.group(1)
+            last = max(body.rfind("cluster_arrive()"), body.rfind("cluster_wait()"))
+            assert "return" not in body[:last], m.group(1)
 
 
 def test_every_polling_loop_has_a_limit():
