@@ -151,8 +151,9 @@ hf_status hf_state_absorb(hf_ctx* ctx, int layer, const void* k_ev, const void* 
  *   k, v   HOST arrays of n_layers DEVICE pointers, bf16 [B,H,T_c,d] each (entry l belongs to layer first_layer + l)
  * Every layer ends up exactly as after hf_kv_append(layer, k[l], v[l]): same cache contents and the same bits in S and
  * z (the token range is cut and summed in the same order).  Layers of the call that are in different phases of the
- * protocol (some still filling the window, some evicting), a window of one chunk, or too few (layer, batch*head) pairs
- * to fill the device are handled layer by layer inside the call. */
+ * protocol (some still filling the window, some evicting), a window of one chunk, the temporal rotation, or two layers of
+ * few heads and long chunks, whose state updates fill the device better one after the other, are handled layer by layer
+ * inside the call. */
 hf_status hf_kv_append_layers(hf_ctx* ctx, int first_layer, int n_layers, const void* const* k, const void* const* v, void* stream);
 
 /* Eq. 3 on caller-supplied tokens for several layers at once: k_ev, v_ev device bf16 [n_layers, B, H, n_tokens, d]
@@ -289,9 +290,9 @@ hf_status hf_query(hf_ctx* ctx, int layer, int what, int64_t* value);
 hf_status hf_get_device_status(hf_ctx* ctx, int* flags, int* detail);
 
 /* Alg. 3 keeps a running row maximum m (m_new = max(m, rowmax S)) and rescales l and O by e^{m - m_new}.  The tcgen05
- * attention kernel (HF_SWA_TCGEN05, what HF_SWA_AUTO resolves to) instead fixes a row's reference after its first kept
- * key block (softmax does not depend on the reference), which covers rows whose later blocks rise up to about 100
- * natural-log units above the first; a (batch*head, query block) unit with a row beyond that is computed a second time
+ * attention kernel (HF_SWA_TCGEN05, what HF_SWA_AUTO resolves to) instead fixes a row's reference after the first kept
+ * key blocks that it walks (128 keys; softmax does not depend on the reference), which covers rows whose later blocks rise
+ * up to about 100 natural-log units above those; a (batch*head, query block) unit with a row beyond that is computed a second time
  * inside the same launch with the running maximum, so o is the softmax of Eq. 6 for every finite input and no status has
  * to be polled.  This call synchronises the device and reports how many units have taken that second pass since the
  * context was created (a diagnostic: such units cost several times a normal one). */

@@ -485,7 +485,10 @@ hf_status launch_absorb_layers(hf_ctx* c, int first_layer, int n_layers, const C
 // layer by layer (k_absorb_tc5: an item cut over several thread blocks, but three launches and the side stream's events per layer).
 // As many items as SMs fill the device either way.  With fewer, in units of a 64-token tile: rounds x tiles of a unit against tiles of a
 // split, plus what a call costs beside its tiles, about ten tiles' time (8 us) either way.  Same bits either way.  The commit of four
-// layers of 8 heads of 128, 300 tokens: 60 us layer by layer, 21 in one launch.
+// layers of 8 heads of 128, 300 tokens: 60 us layer by layer, 21 in one launch.  From four layers on one launch is the faster at any size
+// measured (1 to 64 heads, 64 to 4 680 tokens); the line matters for two.  Their commit, layer by layer / one launch: heads of 64, 1 head of
+// 1 000 tokens 17.3 / 16.2 us, of 1 560 20.3 / 21.3, of 4 680 24.4 / 36.2; 16 heads of 1 560 21.9 / 20.1, of 3 120 31.4 / 29.7 (kept apart all the
+// same); heads of 128, 12 of 3 120 42.0 / 35.3 (apart), 8 of 4 680 44.0 / 43.2 (apart), 5 of 4 680 38.8 / 44.4, 64 of 4 680 166 / 157 (one).
 inline bool layers_in_one_launch(const hf_ctx* c, int n_layers, int n_tokens) {
     if (n_layers < 2) return false;
     if ((long long)n_layers * c->BH >= c->sm_count) return true;
@@ -584,7 +587,6 @@ cudaError_t launch_select_kernel(hf_ctx* c, const ChunkTable& tab, int Tn, int k
 #undef HF_SELECT
 }
 
-// merged: the attention kernel follows in the same call and takes its merged lists from here.
 // merged: the attention kernel follows in the same call and takes its merged lists from here.
 template <int D>
 hf_status launch_select(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_cur,

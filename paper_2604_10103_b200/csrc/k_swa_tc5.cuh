@@ -7,16 +7,17 @@
 // of 128 keys as one stream of tiles t = 0, 1, ...
 //   BLK = 128       unit = query block, tile = kept key block.
 //   BLK = 16, 64    unit = G = 128 / BLK query blocks ("row groups") with a kept list each; tile = G key blocks side by side
-//                   (G boxes of BLK rows, anywhere in the window).  k_union_tiles merges the G lists into one list of key
-//                   blocks, each with the set of row groups that keep it; a (row group, key block) pair that is not kept is
-//                   masked to -inf before the exponential.  k / |union| of the products are wanted: ~57 % for two lists
+//                   (G boxes of BLK rows, anywhere in the window).  The G lists are merged into one list of key blocks
+//                   (k_union.cuh; in a forward call by the selection), each with the set of row groups that keep it; a (row
+//                   group, key block) pair that is not kept is masked to -inf before the exponential.  k / |union| of the products are wanted: ~57 % for two lists
 //                   that keep a random quarter each, ~100 % when neighbouring query blocks keep the same blocks.  A unit's
-//                   first tile holds the first kept block of every row group, so that every row has a finite maximum there.
+//                   first tile holds a kept block of every row group (with 16 tokens its first one), so that every row has a finite
+//                   maximum there.
 //
 // Roles (12 warps, 20 with four column groups):
-//   softmax warps       two column groups of four warps (four at head dim 64, see swa_groups); thread (group g, row r) owns S columns
-//                       [64 g, 64 g + 64) of row r (TMEM lane = row) and half of the O columns.  It takes its share of S into registers (the S buffer is
-//                       free from then on), forms P = exp2(S c - m) and writes it as bf16 to the P buffer.
+//   softmax warps       NG = two column groups of four warps (four at head dim 64, see swa_groups); thread (group g, row r) owns 128 / NG
+//                       columns of S of row r (TMEM lane = row), from 128 g / NG on, and D / NG columns of O.  It takes its share of S into
+//                       registers (the S buffer is free from then on), forms P = exp2(S c - m) and writes it as bf16 to the P buffer.
 //   K loader, V loader  TMA: K tiles (ring of two), V tiles (ring of two), Q, and for HIST the folded state S W^T and z
 //   S warp, P V warp    tcgen05.mma issue, one warp per product.
 //       S_t = Q K_t^T      A = Q (tensor memory), B = K_t (smem, K-major, 128B swizzle)       -> S buffer t & 1
@@ -58,9 +59,13 @@
 
 // NGROUPS: softmax column groups (four warps each), two or four.  At head dim 64 the products leave the softmax warps' chain between two
 // tiles' exponentials as the bound, and four groups of 32 columns overlap more of it: 444 units of 12 heads, 28 kept blocks of 128
-// tokens 85.6 -> 79.7 us, 10 kept 36.7 -> 34.4.  Below five tiles their meetings at a unit's ends weigh more (24 units of one tile 6.4 ->
-// 6.8 us, of three 8.2 either way), and so do the masked segments of smaller blocks (64-token blocks 117 -> 119 us), and head dim 128
-// has no registers for it: two there.
+// tokens 85.6 -> 79.7 us, 10 kept 36.7 -> 34.4.  Below five tiles their meetings at a unit's ends weigh more.  Forward calls, two groups /
+// four, us:                 one tile       three          four           five           eight
+//   1 unit                  7.30 / 7.55    9.09 / 9.22    9.86 / 9.86   10.75 / 10.50   13.1 / 12.7
+//   64 units                8.96 / 9.09    10.9 / 10.9    11.7 / 11.5   12.4 / 12.4     15.1 / 14.6
+//   444 units               22.5 / 23.0    27.8 / 27.9    30.3 / 29.8   32.6 / 32.1     40.3 / 39.2
+// The masked segments of 64-token blocks weigh more too (117 -> 119 us), blocks of 16 tokens have not been tried, and head dim 128 has no
+// registers for it: two there.
 inline constexpr int swa_groups(int d, int blk, int tiles) { return d == 64 && blk == 128 && tiles >= 5 ? 4 : 2; }
 
 template <int D, int NGROUPS>
@@ -76,8 +81,8 @@ struct SwaTc5 {
     static constexpr int H_BYTES = SUB * HSUB_BYTES;
     static constexpr float HEADROOM = 60.f;           // log2 distance of the softmax reference above the first tile's row maximum
     // Tensor memory: two S buffers, P, Q, O.  There is room for one P buffer at head dim 128.  Its halves (keys 0..63 from
-    // column group 0, keys 64..127 from group 1) are products and barriers of their own, so that a group waits only for the
-    // product of its own last half, issued a whole tile earlier.
+    // the lower half of the column groups, keys 64..127 from the upper) are products and barriers of their own, so that a group waits only
+    // for the product of its own last half, issued a whole tile earlier.
     static constexpr int COL_P = 256, COL_Q = COL_P + 64, COL_O = COL_Q + D / 2, TMEM_COLS = 512;
     static_assert(COL_O + D <= TMEM_COLS, "tensor memory layout");
     static constexpr int OFF_Q = 0, OFF_K = TILE_BYTES, OFF_V = OFF_K + 2 * TILE_BYTES;
@@ -113,7 +118,7 @@ struct Tc5Params {
     uint32_t nb_magic;       // ceil(2^32 / n_b) (n_b > 1): x / n_b = high word of x * nb_magic for x <= 1024
     int Tm, n_units;         // query blocks per batch*head; units in all (unit u = bh * upb + i)
     int upb;                 // units per batch*head: T_m, or ceil(T_c / 128) with 16- / 64-token blocks
-    const uint32_t* entries; // 16- / 64-token blocks: [units, max_tiles, G] from k_union_tiles ...
+    const uint32_t* entries; // 16- / 64-token blocks: [units, max_tiles, G] merged lists (k_union.cuh) ...
     const int* tiles;        // ... and tiles per unit
     int max_tiles;
     float scale_log2;
@@ -809,7 +814,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             // overflow (or NaN): a later tile rose too far above the first one.  (After the wait: P V of this unit's last tile
             // needed every warp, so all of them have listed the unit before this one.)
             if (!(l_run < 1e30f)) note_redo(n);
-            // Output through shared memory and one bulk tensor store per warp (32 rows x half of the columns):
+            // Output through shared memory and one bulk tensor store per warp (32 rows x its group's columns):
             // row-per-thread global stores would touch 32 lines per instruction.  The staging tile is the S W^T buffer (free: the
             // history products have completed, or were never asked for); in the map's swizzle of the row width.
             const uint32_t stage_off = C::OFF_H + warp * (32 * C::OCOLS * 2);
@@ -826,8 +831,9 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                 if constexpr (HIST) tmem_ld16(lane_base + (tl & 1) * 128 + grp * C::OCOLS + c * 16, dh);
                 tmem_wait_ld();
                 if (c == C::OCOLS / 16 - 1) {
-                    // The next unit's first P V overwrites O.  It needs P of that tile from the warps of group 0, each of which
-                    // first meets the other warp of its rows in the exchange of the maxima: both are past these loads then.
+                    // The next unit's first P V overwrites O.  It needs the lower half of P of that tile from all warps of the lower half
+                    // of the groups, each of which first meets the warps of its rows in ALL groups in the exchange of the maxima: all
+                    // of them are past these loads then.
                     fence_before_sync();
                     if constexpr (HIST) arrive_t(bar_dr);
                 }

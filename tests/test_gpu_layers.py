@@ -131,8 +131,8 @@ def test_batched_absorb_equals_per_layer_absorbs_bit_for_bit(d, n, zmean, rope):
 
 
 def test_layers_in_different_phases_and_small_calls_fall_back_to_the_per_layer_path():
-    """Layer 0 is one chunk ahead of the others (it evicts while they still fill the window), and a call over two layers
-    has too few items for the persistent launch: both must leave what per-layer commits leave."""
+    """Layer 0 is one chunk ahead of the others (it evicts while they still fill the window): layer by layer.  A call over two
+    layers has fewer items than SMs.  Both must leave what per-layer commits leave."""
     from paper_2604_10103_b200 import binding as hf
     layers = 13
     w = gen.Workload("phases", batch=1, heads=12, head_dim=128, tokens_per_frame=130, chunk_frames=1, window_frames=3,
