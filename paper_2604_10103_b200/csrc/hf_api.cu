@@ -95,7 +95,7 @@ struct hf_ctx {
     uint32_t* union_entries = nullptr;   // small-block tcgen05 attention: merged kept lists [B*H * units, max tiles, G] ...
     int* union_tiles = nullptr;          // ... and tiles per unit
     int union_max_tiles = 0;
-    int pool_clusters = 0;               // clusters of k_pool_select that the device holds at a time (of pool_select_cluster(T_m) thread blocks)
+    int pool_clusters = 0, pool_clusters16 = 0;     // clusters of k_pool_select that the device holds at a time: of T_m thread blocks, of sixteen
     // dK / dV: g . o_local per query row [B*H, T_c], and the key blocks of the current chunk, most pairs first, with their number
     // [B*H, n_b].  Both live in `hist`, which no call holds across another (one stream per context): nothing is allocated by a
     // backward call, so it can be captured into a graph.
@@ -268,7 +268,7 @@ inline int union_tiles_max(const hf_ctx* c, int keep, int Tn) {
 }
 
 inline bool pools_and_selects(const hf_ctx* c) {
-    return !c->has_trope && pool_select_one_launch(c->cfg.block, c->Tm, c->BH, c->pool_clusters);
+    return !c->has_trope && pool_select_one_launch(c->cfg.block, c->d, c->Tm, c->BH, c->pool_clusters, c->pool_clusters16);
 }
 // The one-launch form's kernel for 128-token blocks (KPL: T_n <= 32 KPL).
 template <int D> auto pool_select_kernel(int Tn) { return Tn <= 64 ? k_pool_select<D, 2> : k_pool_select<D, 4>; }
@@ -310,17 +310,19 @@ hf_status set_attrs(hf_ctx* c) {
         HF_CUDA(cudaFuncSetAttribute(k_merge_full<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, MergeFull<D>::SMEM_BYTES));
     HF_TRY((set_select_attr<D, 1>(c)));
     if (b == 128 && c->Tm <= 16) {
-        const int cluster = pool_select_cluster(c->Tm);
         for (int Tn : {64, 128}) {          // the kernels for up to that many key blocks
             if (Tn == 128 && c->max_Tn <= 64) continue;
             HF_CUDA(cudaFuncSetAttribute(pool_select_kernel<D>(Tn), cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 128, Tn)));
-            if (cluster > 8) HF_CUDA(cudaFuncSetAttribute(pool_select_kernel<D>(Tn), cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+            if (c->Tm > 8) HF_CUDA(cudaFuncSetAttribute(pool_select_kernel<D>(Tn), cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         }
-        PdlLaunch pl(dim3(cluster, c->BH), dim3(PoolSelect::THREADS), PoolSelect::smem_bytes(D, 128, c->max_Tn), 0, false, cluster);
-        if (cluster > 1 && cudaOccupancyMaxActiveClusters(&c->pool_clusters, pool_select_kernel<D>(c->max_Tn), &pl.cfg) != cudaSuccess) {
-            cudaGetLastError();
-            c->pool_clusters = 0;
-        }
+        auto resident = [&](int cluster) {
+            PdlLaunch pl(dim3(cluster, c->BH), dim3(PoolSelect::THREADS), PoolSelect::smem_bytes(D, 128, c->max_Tn), 0, false, cluster);
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, pool_select_kernel<D>(c->max_Tn), &pl.cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+            return n;
+        };
+        if (c->Tm > 1) c->pool_clusters = resident(c->Tm);
+        if (c->Tm > 10) c->pool_clusters16 = resident(16);
     }
     if (b == 16 && c->Tm <= 8) HF_CUDA(cudaFuncSetAttribute(k_pool_select16<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, PoolSelect::smem_bytes(D, 16, 8 * HF_MAX_CHUNKS)));
     if (forward_lists(c)) HF_TRY((b == 64 ? set_select_attr<D, 2>(c) : set_select_attr<D, 8>(c)));

@@ -6,21 +6,24 @@
 // block: a thread block alone, faster on any grid).
 //
 // The cluster form spares a launch and the means' way through L2 as long as the clusters of all heads are resident at a time.  Behind
-// the first wave it loses: the two-launch form has shorter thread blocks and spreads the pooling evenly.  `clusters` is how many the
-// device holds by its own count (hf_create asks; 0: none fits, as on a partition with small groups of SMs).  The last tenth of them is not
-// reached in one wave, and clusters of 11 to 15 get the room of 16 (their own counts, 21 to 14, lose from 15 or 17 heads on): those
-// ask for 16.  Forward calls of heads of 128, three chunks cached, two launches / one, at and just past the line (B200: 148 SMs):
-//   T_m 3  (93 clusters)  81 heads 26.0 / 22.8 us,  94 heads 26.8 / 27.0     384 heads 73.0 / 80.1
-//   T_m 5  (56)           49 heads 28.2 / 25.5,     52 heads 28.3 / 28.3    1 024 heads 371 / 431
-//   T_m 8  (33)           28 heads 30.9 / 27.9,     33 heads 31.9 / 32.0    55 heads 43.3 / 43.9
-//   T_m 10 (26)           22 heads 34.2 / 32.1,     24 heads 35.3 / 35.7
-//   T_m 13 (as 16: 14)    14 heads 37.8 / 34.6,     16 heads 38.0 / 39.2    34 heads 54.0 / 58.9
-//   T_m 16 (14)           14 heads 41.7 / 38.9,     15 heads 42.8 / 43.5    27 heads 59.8 / 60.4
-inline int pool_select_cluster(int Tm) { return Tm > 10 ? 16 : Tm; }        // thread blocks of the cluster to ask for
-inline bool pool_select_one_launch(int block, int Tm, int BH, int clusters) {
+// the first wave it loses: the two-launch form has shorter thread blocks and spreads the pooling evenly.  `clusters` is how many of T_m thread
+// blocks the device holds by its own count, `clusters16` how many of sixteen (hf_create asks; 0: none fits, as on a partition with small
+// groups of SMs).  The last tenth of the count is not reached in one wave, and clusters of 11 to 15 get little more than the room of 16: heads
+// of 128 lose from 15 to 17 heads on where the count says 21 to 14, heads of 64 at about four fifths of it.  Forward calls, three chunks
+// cached, two launches / one, up to the line and past it (B200: 148 SMs):
+//   heads of 128, T_m 3  (93 clusters)  81 heads 26.0 / 22.8 us,  94 heads 26.8 / 27.0     384 heads 73.0 / 80.1
+//                 T_m 5  (56)           49 heads 28.2 / 25.5,     52 heads 28.3 / 28.3    1 024 heads 371 / 431
+//                 T_m 8  (33)           28 heads 30.9 / 27.9,     33 heads 31.9 / 32.0    55 heads 43.3 / 43.9
+//                 T_m 10 (26)           22 heads 34.2 / 32.1,     24 heads 35.3 / 35.7
+//                 T_m 13 (as 16: 14)    14 heads 37.8 / 34.6,     16 heads 38.0 / 39.2    34 heads 54.0 / 58.9
+//                 T_m 16 (14)           14 heads 41.7 / 38.9,     15 heads 42.8 / 43.5    27 heads 59.8 / 60.4
+//   heads of 64,  T_m 11 (21)           17 heads 27.5 / 26.0,     19 heads 27.7 / 28.6
+//                 T_m 12 (21)           17 heads 27.7 / 27.0,     19 heads 28.0 / 29.7
+inline bool pool_select_one_launch(int block, int d, int Tm, int BH, int clusters, int clusters16) {
     if (block == 16) return Tm <= 8;
     if (block != 128 || Tm > 16) return false;
-    return Tm == 1 || (Tm > 10 ? BH <= clusters : 10 * BH <= 9 * clusters);
+    if (Tm <= 10) return Tm == 1 || 10 * BH <= 9 * clusters;
+    return BH <= clusters16 || (d == 64 && 5 * BH <= 4 * clusters);
 }
 
 // Whether a call that could be a copy may launch a kernel instead.  A copy takes any memory that the runtime can copy between; a kernel

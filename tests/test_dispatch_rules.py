@@ -8,13 +8,14 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2604_10103_b200", "csrc")
 SOURCE = """
 #include "hf_dispatch.h"
-extern "C" int one_launch(int block, int Tm, int BH, int clusters) { return pool_select_one_launch(block, Tm, BH, clusters); }
+extern "C" int one_launch(int block, int d, int Tm, int BH, int clusters, int clusters16) {
+    return pool_select_one_launch(block, d, Tm, BH, clusters, clusters16);
+}
 extern "C" int by_kernel(int context, int current, int given, int aligned, int device_memory, int device) {
     return kernel_instead_of_copy(context, current, CallerMemory{given != 0, aligned != 0, device_memory != 0, device});
 }
 extern "C" int kpl(int Tn) { return select_kpl(Tn); }
 extern "C" int uses(int kpl, int n_b, int max_Tn) { return select_uses(kpl, n_b, max_Tn); }
-extern "C" int cluster_asked_for(int Tm) { return pool_select_cluster(Tm); }
 """
 
 
@@ -27,30 +28,33 @@ def rules(tmp_path_factory):
     return ctypes.CDLL(str(so))
 
 
-def test_pooling_and_selection_without_room_for_a_cluster(rules):
+@pytest.mark.parametrize("d", [64, 128])
+def test_pooling_and_selection_without_room_for_a_cluster(rules, d):
     """Where no cluster of T_m thread blocks can be resident, a head's blocks are pooled and selected in two launches."""
     for Tm in range(1, 40):
-        assert rules.one_launch(128, Tm, 1, 0) == (Tm == 1)          # (one thread block is no cluster)
-        assert rules.one_launch(128, Tm, 1, 14) == (Tm <= 16)
-        assert rules.one_launch(16, Tm, 1, 0) == (Tm <= 8)           # no cluster in this form
-        assert not rules.one_launch(64, Tm, 1, 9)
+        assert rules.one_launch(128, d, Tm, 1, 0, 0) == (Tm == 1)          # (one thread block is no cluster)
+        assert rules.one_launch(128, d, Tm, 1, 14, 14) == (Tm <= 16)
+        assert rules.one_launch(16, d, Tm, 1, 0, 0) == (Tm <= 8)           # no cluster in this form
+        assert not rules.one_launch(64, d, Tm, 1, 9, 9)
 
 
-# query blocks a head, clusters of the asked size that a B200 holds, most heads measured faster in one launch, fewest measured not faster
-LINE = [(2, 148, 130, 192), (3, 93, 81, 94), (4, 71, 61, 70), (5, 56, 49, 56), (6, 45, 40, 47), (7, 37, 32, 37), (8, 33, 28, 35), (9, 30, 27, 31),
-        (10, 26, 22, 24), (11, 14, 13, 17), (12, 14, 14, 17), (13, 14, 14, 16), (14, 14, 13, 15), (15, 14, 14, 15), (16, 14, 14, 15)]
+# query blocks a head, clusters that a B200 holds, most heads measured faster in one launch, fewest measured not faster (heads of 64; of 128)
+LINE = [(2, 148, 130, 192, 130, 192), (3, 93, 81, 94, 81, 94), (4, 71, 61, 70, 61, 70), (5, 56, 49, 56, 49, 56), (6, 45, 40, 47, 40, 47),
+        (7, 37, 32, 37, 32, 37), (8, 33, 28, 35, 28, 35), (9, 30, 27, 31, 27, 31), (10, 26, 22, 24, 22, 24), (11, 21, 16, 19, 13, 17),
+        (12, 21, 16, 19, 14, 17), (13, 17, 14, 17, 14, 16), (14, 14, 13, 15, 13, 15), (15, 14, 14, 15, 14, 15), (16, 14, 14, 15, 14, 15)]
 
 
-@pytest.mark.parametrize("Tm,clusters,fast,slow", LINE)
-def test_one_launch_up_to_one_wave_of_clusters(rules, Tm, clusters, fast, slow):
-    assert rules.cluster_asked_for(Tm) == (Tm if Tm <= 10 else 16)
-    assert all(rules.one_launch(128, Tm, BH, clusters) for BH in range(1, fast + 1))
-    assert not any(rules.one_launch(128, Tm, BH, clusters) for BH in range(slow, 4096))
+@pytest.mark.parametrize("Tm,clusters,fast64,slow64,fast128,slow128", LINE)
+def test_one_launch_up_to_one_wave_of_clusters(rules, Tm, clusters, fast64, slow64, fast128, slow128):
+    for d, fast, slow in ((64, fast64, slow64), (128, fast128, slow128)):
+        assert all(rules.one_launch(128, d, Tm, BH, clusters, 14) for BH in range(1, fast + 1))
+        assert not any(rules.one_launch(128, d, Tm, BH, clusters, 14) for BH in range(slow, 4096))
 
 
-def test_a_single_block_and_small_blocks_on_any_grid(rules):
+@pytest.mark.parametrize("d", [64, 128])
+def test_a_single_block_and_small_blocks_on_any_grid(rules, d):
     for BH in (1, 148, 1024, 65535):
-        assert rules.one_launch(128, 1, BH, 0) and rules.one_launch(16, 8, BH, 0) and not rules.one_launch(16, 9, BH, 0)
+        assert rules.one_launch(128, d, 1, BH, 0, 0) and rules.one_launch(16, d, 8, BH, 0, 0) and not rules.one_launch(16, d, 9, BH, 0, 0)
 
 
 def test_a_kernel_in_place_of_a_copy_only_at_home(rules):

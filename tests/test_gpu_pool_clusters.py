@@ -24,7 +24,7 @@ def test_large_clusters(d, tokens, chunks, permille):
 
 @pytest.mark.parametrize("d,tokens,heads,launches", [
     (64, 500, 61, 1), (64, 500, 72, 2), (128, 500, 61, 1), (128, 500, 72, 2),            # T_m 4: 71 clusters resident on 148 SMs
-    (64, 1300, 14, 1), (128, 1300, 15, 2),             # T_m 11, which asks for the room of 16
+    (64, 1300, 16, 1), (64, 1300, 19, 2), (128, 1300, 14, 1), (128, 1300, 15, 2),        # T_m 11: about the room of 16
     (64, 77, 600, 1),                                  # a single block a head: any grid
 ])
 def test_both_sides_of_one_wave(d, tokens, heads, launches):
