@@ -246,9 +246,11 @@ __global__ void __launch_bounds__(256, 6) k_pool_copy_layers(const __grid_consta
 // G: the query blocks that share a unit of the attention kernel (blocks of 64 tokens: 2, of 16: 8), whose merged list is formed here
 // from the masks in shared memory, or 1: none is asked for.  A kernel of its own behind this one costs a launch (k_union.cuh).  G = 8
 // takes eight query blocks, one unit, per thread block, with as many threads per score.
-// KPL: key blocks per lane of a ranking warp (T_n <= 32 KPL).  Rows of more than 256 key blocks come in several passes of key rows, and such
-// grids are large: there, too, eight query blocks share a key row's trip through L2 (T_n 259, 48 heads, behind the pooling: 42 us
-// with four query blocks and KPL 32, 24.5 like this).
+// KPL: key blocks per lane of a ranking warp (T_n <= 32 KPL).  Rows of more than 256 key blocks come in several passes of key rows, and their
+// grids are mostly large: there, too, eight query blocks share a key row's trip through L2 (T_n 259, 48 heads, behind the pooling: 42 us
+// with four query blocks and KPL 32, 24.5 like this).  One isolated call, pooling and selection, heads of 128, four / eight query blocks: T_n 296,
+// 48 heads 56.6 / 43.2 us, 12 heads 26.2 / 27.4, 2 heads 18.3 / 20.5; T_n 512, 12 heads 52 / 39.4; T_n 1 024, 1 head 43.2 / 47.0, 12 heads
+// 111 / 107.5.
 template <int D, int G, int KPL>
 struct Select {
     static constexpr int R = G == 8 || KPL > 8 ? 8 : 4, KT = 128;        // query blocks per thread block; key rows per pass
