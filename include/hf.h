@@ -153,7 +153,8 @@ hf_status hf_state_absorb(hf_ctx* ctx, int layer, const void* k_ev, const void* 
  * z (the token range is cut and summed in the same order).  Layers of the call that are in different phases of the
  * protocol (some still filling the window, some evicting), a window of one chunk, the temporal rotation, or two layers of
  * few heads and long chunks, whose state updates fill the device better one after the other, are handled layer by layer
- * inside the call. */
+ * inside the call.  A state update of more (layer, batch*head) pairs than the device has SMs grows its scratch (and waits for
+ * the stream) when no call of that size came before: capture such a call into a graph only after the largest one. */
 hf_status hf_kv_append_layers(hf_ctx* ctx, int first_layer, int n_layers, const void* const* k, const void* const* v, void* stream);
 
 /* Eq. 3 on caller-supplied tokens for several layers at once: k_ev, v_ev device bf16 [n_layers, B, H, n_tokens, d]
