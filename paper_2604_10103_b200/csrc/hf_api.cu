@@ -223,11 +223,11 @@ void free_all(hf_ctx* c) {
 #define HF_TC5P_COLGROUPS 1   // column groups per tile group of the ping-pong attention kernel
 #endif
 
-template <int D, int BLK, int NG>
+template <int D, int BLK, bool TEAMED>
 hf_status set_swa_tc5_attr() {
-    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 0, NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D, NG>::SMEM_BYTES));
-    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 1, NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D, NG>::SMEM_BYTES));
-    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 2, NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D, NG>::SMEM_BYTES));
+    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 0, TEAMED>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D, TEAMED>::SMEM_BYTES));
+    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 1, TEAMED>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D, TEAMED>::SMEM_BYTES));
+    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 2, TEAMED>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D, TEAMED>::SMEM_BYTES));
     return HF_OK;
 }
 template <int BLK, int D>
@@ -300,10 +300,12 @@ hf_status set_attrs(hf_ctx* c) {
     if (c->swa_kernel == HF_SWA_TCGEN05_PINGPONG)
         HF_CUDA(cudaFuncSetAttribute(k_swa_tc5p<D, HF_TC5P_COLGROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5P<D, HF_TC5P_COLGROUPS>::SMEM_BYTES));
     else if (c->swa_kernel == HF_SWA_TCGEN05) {
-        // (kept blocks of the shortest and of the longest window: two column groups, four, or both)
-        if (swa_groups(D, b, keep_for(c, c->n_b)) == 2)
-            HF_TRY((b == 128 ? set_swa_tc5_attr<D, 128, 2>() : b == 64 ? set_swa_tc5_attr<D, 64, 2>() : set_swa_tc5_attr<D, 16, 2>()));
-        if (swa_groups(D, b, keep_for(c, c->max_Tn)) == 4) HF_TRY((set_swa_tc5_attr<64, 128, 4>()));
+        // (128-token blocks: kept blocks of the shortest and of the longest window: column groups, teams, or both)
+        if (b != 128) HF_TRY((b == 64 ? set_swa_tc5_attr<D, 64, D == 64>() : set_swa_tc5_attr<D, 16, D == 64>()));
+        else {
+            if (swa_teams(D, b, keep_for(c, c->max_Tn), false)) HF_TRY((set_swa_tc5_attr<D, 128, true>()));
+            if constexpr (D == 128) { if (!swa_teams(D, b, keep_for(c, c->n_b), true)) HF_TRY((set_swa_tc5_attr<D, 128, false>())); }
+        }
     } else
         HF_TRY((b == 128 ? set_swa_attr<128, D>() : b == 64 ? set_swa_attr<64, D>() : set_swa_attr<16, D>()));
     if (c->cfg.merge == HF_MERGE_FULL_WIDTH)
@@ -642,10 +644,10 @@ hf_status launch_swa_mma_t(hf_ctx* c, const bf16* q, const ChunkTable& tab, cons
 // The tcgen05 attention kernel.  Blocks of 16 or 64 tokens: first the kept lists of the query blocks that share a 128-row unit
 // are merged (k_union_tiles), unless the selection of the same call has done that (merged).  hist_inside: the kernel forms the history term; overlap_prev: it may be launched under the tail
 // of the kernel before it in the stream.
-template <int D, int BLK, int NG>
+template <int D, int BLK, bool TEAMED>
 hf_status launch_swa_tc5_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_cur, const bf16* v_cur, const int32_t* idx,
                            int keep, const float* hist, bf16* o, float* lse, cudaStream_t st, bool hist_inside, bool overlap_prev, bool merged) {
-    typedef SwaTc5<D, NG> C;
+    typedef SwaTc5<D, TEAMED> C;
     Tc5Params p;
     memset(&p, 0, sizeof(p));
     p.upb = (c->Tc + 127) / 128; p.n_units = p.upb * c->BH;
@@ -680,9 +682,9 @@ hf_status launch_swa_tc5_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16* 
     const CUtensorMap& rv = c->R + c->n_sink_max > 0 ? L.tm_vring : tv;
     const int grid = p.n_units < c->sm_count ? p.n_units : c->sm_count;
     PdlLaunch pl(dim3(grid), dim3(C::THREADS), C::SMEM_BYTES, st, overlap_prev);
-    if (hist_inside && c->has_rope_q) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 2, NG>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
-    else if (hist_inside) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 1, NG>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
-    else HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 0, NG>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
+    if (hist_inside && c->has_rope_q) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 2, TEAMED>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
+    else if (hist_inside) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 1, TEAMED>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
+    else HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 0, TEAMED>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
     return post_launch(c, "k_swa_tc5");
 }
 
@@ -713,9 +715,10 @@ hf_status launch_swa(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_cur,
                      int keep, const float* hist, bf16* o, float* lse, cudaStream_t st, bool hist_inside = false, bool overlap_prev = false, bool merged = false) {
     if (c->swa_kernel == HF_SWA_TCGEN05) {
         const int b = c->cfg.block, d = c->d;
-        if (swa_groups(d, b, keep) == 4) return launch_swa_tc5_t<64, 128, 4>(c, L, q, k_cur, v_cur, idx, keep, hist, o, lse, st, hist_inside, overlap_prev, merged);
-#define HF_TC5_CASE(D_, B_) if (d == D_ && b == B_) return launch_swa_tc5_t<D_, B_, 2>(c, L, q, k_cur, v_cur, idx, keep, hist, o, lse, st, hist_inside, overlap_prev, merged)
-        HF_TC5_CASE(128, 128); HF_TC5_CASE(128, 64); HF_TC5_CASE(128, 16); HF_TC5_CASE(64, 128); HF_TC5_CASE(64, 64); HF_TC5_CASE(64, 16);
+#define HF_TC5_CASE(D_, B_, T_) if (d == D_ && b == B_ && teams == T_) return launch_swa_tc5_t<D_, B_, T_>(c, L, q, k_cur, v_cur, idx, keep, hist, o, lse, st, hist_inside, overlap_prev, merged)
+        const bool teams = swa_teams(d, b, keep, hist_inside);
+        HF_TC5_CASE(128, 128, false); HF_TC5_CASE(128, 128, true); HF_TC5_CASE(128, 64, false); HF_TC5_CASE(128, 16, false);
+        HF_TC5_CASE(64, 128, true); HF_TC5_CASE(64, 64, true); HF_TC5_CASE(64, 16, true);
 #undef HF_TC5_CASE
     }
     if (c->swa_kernel == HF_SWA_TCGEN05_PINGPONG) {

@@ -111,3 +111,13 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
 // is below anything the state or the read-out can resolve): the non-flushing form costs several more instructions
 // per value, and the state update is bound by exactly these.
 __device__ __forceinline__ float phi_elu1(float x) { return x > 0.f ? x + 1.f : fast_exp2(x * 1.4426950408889634f); }
+// ... of two values: exp(min(x, 0)) + max(x, 0) is the same number in fewer instructions (a NaN stays one).
+__device__ __forceinline__ float2 phi_elu1(float2 x) {
+    const float2 y = fmul2(x, make_float2(1.4426950408889634f, 1.4426950408889634f));
+    float2 n, p;
+    asm("min.NaN.f32 %0, %1, 0f00000000;" : "=f"(n.x) : "f"(y.x));
+    asm("min.NaN.f32 %0, %1, 0f00000000;" : "=f"(n.y) : "f"(y.y));
+    asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(p.x) : "f"(x.x));
+    asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(p.y) : "f"(x.y));
+    return fadd2(make_float2(fast_exp2(n.x), fast_exp2(n.y)), p);
+}

@@ -39,3 +39,11 @@ inline bool kernel_instead_of_copy(int context_device, int current_device, const
 inline int select_kpl(int Tn) { return Tn <= 128 ? 4 : Tn <= 256 ? 8 : Tn <= 512 ? 16 : 32; }
 // Whether a context whose windows have n_b .. max_Tn key blocks ever launches the step's kernel.
 inline bool select_uses(int kpl, int n_b, int max_Tn) { return select_kpl(n_b) <= kpl && kpl <= select_kpl(max_Tn); }
+
+// Softmax warps of the tcgen05 attention kernel in teams that take turns at the tiles, or in column groups on the same one (k_swa_tc5.cuh).  Head
+// dim 64: teams (1 to 40 tiles, 12 to 320 units: 0.98 to 1.13 times as fast).  Head dim 128, 128-token blocks: teams from 14 tiles on, from
+// 8 without the history term, whose operand they keep in an S buffer; column groups / teams, forward calls (softmax branch alone), us:
+//   132 units, 10 tiles 22.1 / 22.2, 12 tiles 23.9 / 23.7, 14 tiles 25.8 / 25.2, 24 tiles 34.7 / 32.7  (8 tiles 14.4 / 14.4, 12 tiles 18.3 / 16.8)
+//   448 units, 10 tiles 67.1 / 69.3, 12 tiles 73.9 / 75.4, 14 tiles 81.0 / 80.9, 24 tiles 119.9 / 114.8  (8 tiles 44.6 / 41.0, 4 tiles 29.7 / 29.0)
+// and column groups for its blocks of 16 and 64 tokens (0.90 to 0.98 times as fast with teams).
+inline bool swa_teams(int d, int block, int tiles, bool history) { return d == 64 || (block == 128 && tiles >= (history ? 14 : 8)); }

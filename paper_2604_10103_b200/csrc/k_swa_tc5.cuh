@@ -14,15 +14,33 @@
 //                   first tile holds a kept block of every row group (with 16 tokens its first one), so that every row has a finite
 //                   maximum there.
 //
-// Roles (12 warps, 20 with four column groups):
-//   softmax warps       NG = two column groups of four warps (four at head dim 64, see swa_groups); thread (group g, row r) owns 128 / NG
-//                       columns of S of row r (TMEM lane = row), from 128 g / NG on, and D / NG columns of O.  It takes its share of S into
-//                       registers (the S buffer is free from then on), forms P = exp2(S c - m) and writes it as bf16 to the P buffer.
-//   K loader, V loader  TMA: K tiles (ring of two), V tiles (ring of two), Q, and for HIST the folded state S W^T and z
+// Roles (12 warps with column groups, 20 with teams):
+//   softmax warps       Column groups: two of four warps; thread (group g, row r) owns columns 64 g .. 64 g + 63 of S of row r (TMEM lane = row) in every
+//                       tile and D / 2 columns of O.  Teams: two of eight warps, tiles t = team, team + 2, ...; a team's two halves own 32 columns of
+//                       either half of the tile each.  A thread takes its share of S into registers (the S buffer is free from then on), forms
+//                       P = exp2(S c - m) and writes it as bf16 to a P buffer.
+//   K loader, V loader  TMA: K tiles and V tiles (rings of two, of four at head dim 64), Q, and for HIST the folded state S W^T and z
 //   S warp, P V warp    tcgen05.mma issue, one warp per product.
-//       S_t = Q K_t^T      A = Q (tensor memory), B = K_t (smem, K-major, 128B swizzle)       -> S buffer t & 1
+//       S_t = Q K_t^T      A = Q (tensor memory; a unit's first tile: shared memory), B = K_t (smem, K-major, 128B swizzle) -> S buffer t & 1
 //       O  += P_t V_t      A = P (tensor memory), B = V_t (smem, MN-major, 128B swizzle)      -> O, in two halves of 64 keys
 //       D_h = phi(Q) S W^T three products of bf16 hi / lo halves (HIST)                       -> S buffer of the unit's last tile
+//
+// Teams or column groups.  A softmax warp's way through a tile is exponentials (8 clk a warp instruction and scheduler) and about 600 clk of
+// waits, tensor-memory loads and stores and arrivals.  With column groups every warp pays the latter in every tile: 1 640-1 830 clk
+// a tile at head dim 128 with the special-function unit at 56-62 %.  A team pays them in every other one and has two tiles' time for it, four
+// warps on a scheduler cover each other, and no warp of one team waits for the other inside a unit: 1 380-1 450 clk a tile.  A P half of 64
+// keys is written by both halves of a team, so that its product starts in the middle of the tile (with 64 columns in a row for each
+// half it started at the end, and where there is one P buffer the other team waited for it: 1 770 clk).  At a unit's end one team forms phi(Q)
+// while the other has the last tile; that one writes the output while the first has gone on to the next unit's first tile.  Forward calls, two
+// column groups (head dim 64 from five tiles on: four) / teams, us:
+//   head dim 128, 128-token blocks, 444 units of 28 tiles 125.7 / 121.8 (at the power limit), 1 776 units of 130 tiles 1 929 / 1 770; 132 units
+//   of 20 tiles 31.3 / 29.7, of 40 tiles 49.9 / 44.6; 320 units of 20 tiles 79.8 / 76.7, of 40 tiles 134.1 / 122.7
+//   head dim 64, 128-token blocks, 132 units of 8, 20, 40 tiles 16.4 / 16.2, 26.4 / 25.4, 43.3 / 39.4; 320 units of 1, 8, 40 tiles
+//   20.7 / 19.1, 35.8 / 33.7, 113.5 / 103.8; 64-token blocks, 320 units of 10 and 25 kept blocks 41.3 / 37.5, 60.1 / 53.2; 16-token blocks, 12 units
+//   of 4 and 40 kept blocks 14.9 / 14.7, 23.9 / 22.2
+// At head dim 128 the phi(Q) operand has to wait in an S buffer and a unit's ends weigh more than column groups' (all warps share them): those stay
+// for short lists (swa_teams, hf_dispatch.h) and for blocks of 16 and 64 tokens (their masked segments leave the tensor pipe the bound:
+// 64-token blocks, 12 heads, 4 680 queries 158 / 163 us, 16-token blocks 43 / 44).
 //
 // What bounds it, and why it is cut this way (measured with clock stamps and with a loop of the same products alone, 148
 // CTAs, head dim 128, per 128 x 128 tile; 1 024 clk is the tensor pipe's own time):
@@ -36,8 +54,7 @@
 //   - the softmax warps' serial path between two tiles' exponentials (three barrier tests, tensor-memory load and store, two
 //     arrivals): every instruction the convergence unit has to serve costs, so waits are warp-uniform, arrivals predicated, a
 //     tile's tail flag comes from one ballot over 32 list entries, and full, masked and empty tiles are separate code (selects in
-//     every tile: +9 us of a 134 us forward).  Four groups of 32 columns instead of two (16 warps) cover more of it and pay it
-//     twice as often: 132 against 130 us at head dim 128; at 64 they pay (swa_groups).
+//     every tile: +9 us of a 134 us forward).
 //   - power: back to back the kernel runs at the board's limit (990 W, SM clock 1 965 -> 1 610 MHz), where time follows energy;
 //     packing P with one conversion instead of two adds and a permute is worth 2 % there.
 // Measured against the version with one MMA warp, Q in shared memory, three S buffers and a second kernel (plus a separate
@@ -56,50 +73,45 @@
 #include "tc5_common.cuh"
 #include "k_swa_mma.cuh"
 #include "k_union.cuh"
+#include "hf_dispatch.h"
 
-// NGROUPS: softmax column groups (four warps each), two or four.  At head dim 64 the products leave the softmax warps' chain between two
-// tiles' exponentials as the bound, and four groups of 32 columns overlap more of it: 444 units of 12 heads, 28 kept blocks of 128
-// tokens 85.6 -> 79.7 us, 10 kept 36.7 -> 34.4.  Below five tiles their meetings at a unit's ends weigh more.  Forward calls, two groups /
-// four, us:                 one tile       three          four           five           eight
-//   1 unit                  7.30 / 7.55    9.09 / 9.22    9.86 / 9.86   10.75 / 10.50   13.1 / 12.7
-//   64 units                8.96 / 9.09    10.9 / 10.9    11.7 / 11.5   12.4 / 12.4     15.1 / 14.6
-//   444 units               22.5 / 23.0    27.8 / 27.9    30.3 / 29.8   32.6 / 32.1     40.3 / 39.2
-// The masked segments of 64-token blocks weigh more too (117 -> 119 us), blocks of 16 tokens have not been tried, and head dim 128 has no
-// registers for it: two there.
-inline constexpr int swa_groups(int d, int blk, int tiles) { return d == 64 && blk == 128 && tiles >= 5 ? 4 : 2; }
-
-template <int D, int NGROUPS>
+template <int D, bool TEAMED>
 struct SwaTc5 {
-    static constexpr int NG = NGROUPS, NSW = 4 * NG;   // softmax column groups; softmax warps
-    static constexpr long long SKEW_CLK = NG == 2 ? 700 : 300;       // offset between the column groups, in clocks (see the softmax warps)
-    static constexpr int SCOLS = 128 / NG;             // S columns per softmax thread
-    static constexpr int OCOLS = D / NG;               // O columns per softmax thread
+    static constexpr int NSW = TEAMED ? 16 : 8;        // softmax warps: two teams of two halves, or two column groups; four warps each
+    static constexpr int OCOLS = D / 2;                // O columns per softmax warp
     static constexpr int SUB = D / 64;                 // 64-column (128-byte) sub-tiles per operand tile
     static constexpr int SUB_BYTES = 128 * 128;        // 16 KB
     static constexpr int TILE_BYTES = SUB * SUB_BYTES;
     static constexpr int HSUB_BYTES = D * 128;         // S W^T halves: D rows of 64-column sub-tiles
     static constexpr int H_BYTES = SUB * HSUB_BYTES;
     static constexpr float HEADROOM = 60.f;           // log2 distance of the softmax reference above the first tile's row maximum
-    // Tensor memory: two S buffers, P, Q, O.  There is room for one P buffer at head dim 128.  Its halves (keys 0..63 from
-    // the lower half of the column groups, keys 64..127 from the upper) are products and barriers of their own, so that a group waits only
-    // for the product of its own last half, issued a whole tile earlier.
-    static constexpr int COL_P = 256, COL_Q = COL_P + 64, COL_O = COL_Q + D / 2, TMEM_COLS = 512;
+    // Tensor memory: two S buffers (teams: one each), P (a buffer per team at head dim 64; at 128 there is room for one), Q, O.  The halves of a P
+    // buffer (keys 0..63, 64..127) are products and barriers of their own.
+    static constexpr int PBUF = D == 64 ? 2 : 1;
+    // The phi(Q) operand of the history products (D columns): in the P buffer of the team that forms it where there are two, else in that
+    // team's S buffer, where the next unit's first S has to wait for the products.
+    static constexpr bool A_IN_P = PBUF == 2;
+    static constexpr int COL_P = 256, COL_Q = COL_P + 64 * PBUF, COL_O = COL_Q + D / 2, TMEM_COLS = 512;
     static_assert(COL_O + D <= TMEM_COLS, "tensor memory layout");
-    static constexpr int OFF_Q = 0, OFF_K = TILE_BYTES, OFF_V = OFF_K + 2 * TILE_BYTES;
-    static constexpr int OFF_H = OFF_V + 2 * TILE_BYTES;       // S W^T, hi then lo; also the staging tile of the output
+    static constexpr int KV_LOG = D == 64 ? 2 : 1, KV = 1 << KV_LOG;   // stages of the K and of the V ring
+    static constexpr int OFF_Q = 0, OFF_K = TILE_BYTES, OFF_V = OFF_K + KV * TILE_BYTES;
+    static constexpr int OFF_H = OFF_V + KV * TILE_BYTES;       // S W^T, hi then lo; also the staging tile of the output (teams without a history term: one each)
+    static constexpr int END_H = OFF_H + (H_BYTES > TILE_BYTES ? 2 * H_BYTES : 2 * TILE_BYTES);
     // (the second pass keeps its fp32 history tile behind the operand tiles of swa_mma_unit, in front of the barriers)
-    static constexpr int OFF_BAR = OFF_H + 2 * H_BYTES > SwaMma<128, D>::SMEM_BYTES + 128 * D * 4 ? OFF_H + 2 * H_BYTES
-                                                                                                    : SwaMma<128, D>::SMEM_BYTES + 128 * D * 4;
+    static constexpr int END_REDO = SwaMma<128, D>::SMEM_BYTES + 128 * D * 4;
+    static constexpr int OFF_BAR = END_H > END_REDO ? END_H : END_REDO;
     // units whose rows left the range of the fixed reference: count, last unit listed, up to REDO_CAP local unit numbers
     // (more than that: every unit of the thread block is computed again)
-    static constexpr int OFF_REDO = OFF_BAR + 256, REDO_CAP = 8;
+    static constexpr int OFF_REDO = OFF_BAR + 384 + (KV > 2 ? 128 : 0), REDO_CAP = 8;
     static constexpr int OFF_Z = OFF_REDO + 64;        // z [D] of the unit's head
     static_assert((2 + REDO_CAP) * 4 <= OFF_Z - OFF_REDO, "the list must fit");
-    static constexpr int OFF_XM = OFF_Z + 512;         // row maxima of the column groups [NG][128]
-    static constexpr int USED_BYTES = OFF_XM + NG * 128 * 4;
-    // row sums and shares of Eq. 4's denominator [2][NG][128] at a unit's end: beside the staging tile of the output
-    static constexpr int OFF_XS = OFF_H + NSW * 32 * OCOLS * 2;
-    static_assert(OFF_XS + 2 * NG * 128 * 4 <= OFF_BAR, "exchange buffers");
+    static constexpr int OFF_XM = OFF_Z + 512;         // row maxima of the two halves of a unit's first tile [2][128]
+    static constexpr int OFF_XL = OFF_XM + 1024;       // one team's row sums [128] and Eq. 4's denominators [128], for the other
+    static constexpr int USED_BYTES = OFF_XL + 1024;
+    // row sums of the halves of the team that writes the output [2][128]: behind the staging tile; without a history term, which leaves
+    // that to the other team's output, in the places of z and of the denominators
+    __host__ __device__ static constexpr int off_xy(bool hist, int half) { return hist ? OFF_H + TILE_BYTES + 512 * half : half ? OFF_XL + 512 : OFF_Z; }
+    static_assert(OFF_H + TILE_BYTES + 2048 <= OFF_BAR, "exchange buffers");
     static constexpr int MAX_SMEM = 232448;            // 227 KB: the most one thread block can have
     // Slack for the manual 1024-byte alignment of the operand tiles (the kernel checks that it was enough); more than
     // half an SM's shared memory so that one CTA owns the SM (it allocates all 512 TMEM columns)
@@ -168,7 +180,7 @@ __device__ __noinline__ void swa_redo_unit(uint8_t* s_gen, const Tc5Params& p, i
         float* den_t = phi_t + ROWS * PS;                                   // [128]
         float* hist_t = reinterpret_cast<float*>(s_gen + M::SMEM_BYTES);    // [128][D], behind the attention tiles
         static_assert(M::TILE_BYTES + (ROWS * PS + ROWS) * 4 <= M::SMEM_BYTES, "phi(Q) tile must fit in the K / V stages");
-        static_assert(M::SMEM_BYTES + ROWS * D * 4 <= SwaTc5<D, 2>::OFF_BAR, "history tile must fit");
+        static_assert(M::SMEM_BYTES + ROWS * D * 4 <= SwaTc5<D, false>::OFF_BAR, "history tile must fit");
         {   // phi(q) of the unit's rows (zero past the chunk's end): thread = (row, half of the features)
             const int row = tid >> 1, f0 = (tid & 1) * (D / 2);
             const bf16* src = p.q + ((size_t)bh * p.Tc + q0 + row) * D + f0;
@@ -274,15 +286,15 @@ __device__ __forceinline__ float swa_max(const uint32_t* r, int nv) {
 // Persistent: CTA c processes units c, c + gridDim.x, ...
 // HIST 1: the history term is formed here; 2: with its numerator rotated (code of its own: as a branch it cost the plain one
 // 2 % of the call); 0: p.hist, if any, is added.
-template <int D, int BLK, int HIST, int NGROUPS>
-__global__ void __launch_bounds__(SwaTc5<D, NGROUPS>::THREADS, 1)
+template <int D, int BLK, int HIST, bool TEAMED>
+__global__ void __launch_bounds__(SwaTc5<D, TEAMED>::THREADS, 1)
 k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kring,
           const __grid_constant__ CUtensorMap tm_vring, const __grid_constant__ CUtensorMap tm_kcur,
           const __grid_constant__ CUtensorMap tm_vcur, const __grid_constant__ CUtensorMap tm_sh,
           const __grid_constant__ CUtensorMap tm_sl, const __grid_constant__ CUtensorMap tm_o,
           const __grid_constant__ Tc5Params p) {
     using namespace tc5;
-    typedef SwaTc5<D, NGROUPS> C;
+    typedef SwaTc5<D, TEAMED> C;
     constexpr int G = 128 / BLK;                       // key blocks per tile = row groups per unit
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t s_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -295,24 +307,30 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
     const uint32_t bar0 = s_base + C::OFF_BAR;
     // Barriers (pairs: index t & 1, completion t >> 1).  Whoever waits for item t of a pair cannot be passed by item t + 2:
     // producing that one needs the waiter's own step, so a parity test is exact.
-    const uint32_t bar_kf = bar0, bar_vf = bar0 + 16,      // K / V tile t landed
-                   bar_sf = bar0 + 32,                     // S_t complete (its K stage is free)
-                   bar_se = bar0 + 48,                     // S_t is in the softmax warps' registers (all of them)
-                   bar_pf = bar0 + 64,                     // two: a half of P_t written (half of the softmax warps); completion t
-                   bar_pv = bar0 + 80,                     // P V of tile t complete, second half (so its V stage is free)
-                   bar_ph = bar0 + 216,                    // ... first half
-                   // unit n: Q landed / its shared-memory tile is free, which takes the word of both its readers: the copy to tensor
-                   // memory (a commit behind it) and, for HIST, the phi pass of every softmax warp at the unit's last tile.  Neither
-                   // implies the other: in a unit of one tile nothing else orders the phi pass behind the copy, which waits for K.
-                   bar_qf = bar0 + 96, bar_qe = bar0 + 104,
-                   bar_hf = bar0 + 112, bar_he = bar0 + 120,   // unit n: S W^T and z landed / free
-                   bar_af = bar0 + 128,                    // unit n: phi(Q) operand written
-                   bar_ud = bar0 + 136,                    // unit n: history products complete
-                   bar_dr = bar0 + 144,                    // unit n: D_h (and O) read by the epilogue
-                   bar_x = bar0 + 152,                     // four: exchange between the warps that share 32 rows
-                   bar_drain = bar0 + 232;                 // two: each MMA warp's last operations complete
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_gen + C::OFF_BAR + 184);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(s_gen + C::OFF_BAR + 188);
+    const uint32_t bar_kf = bar0 + (C::KV > 2 ? 368 : 0), bar_vf = bar0 + (C::KV > 2 ? 400 : 16),     // K / V tile t landed
+                   bar_sf = bar0 + 32,                     // S_t complete
+                   bar_se = bar0 + 48,                     // S_t is in its team's registers
+                   bar_ph = bar0 + 64,                     // P V of tile t complete, first half
+                   bar_pv = bar0 + 80,                     // ... second half
+                   // the K / V stage of tile t is free: with two stages, S_t and P V of tile t complete
+                   bar_ke = C::KV > 2 ? bar0 + 432 : bar_sf, bar_ve = C::KV > 2 ? bar0 + 464 : bar_pv,
+                   bar_pf = bar0 + 96,                     // two per P buffer: a half of P_t written; completion t (two P buffers: t >> 1)
+                   // unit n: Q landed / copied to tensor memory
+                   bar_qf = bar0 + 128, bar_qe = bar0 + 136,
+                   bar_hf = bar0 + 144, bar_he = bar0 + 152,   // unit n: S W^T and z landed / free
+                   bar_af = bar0 + 160,                    // unit n: phi(Q) operand written
+                   bar_ud = bar0 + 168,                    // unit n: history products complete
+                   bar_drain = bar0 + 184,                 // two: each MMA warp's last operations complete
+                   bar_x = bar0 + 200,                     // four (32 rows each), unit n: one team's sums for the other's epilogue
+                   bar_m = bar0 + 232,                     // four, unit n: row maxima of its first tile written
+                   bar_mr = bar0 + 264,                    // four, unit n: ... and read by all four warps of the rows
+                   bar_h = bar0 + 296,                     // four, unit n: the upper half's sums for the lower half of the same team
+                   bar_y = bar0 + 328;                     // four, unit n: the halves of the team that writes the output meet
+    // unit n: O, D_h and the other team's sums read by the epilogue (two barriers, completion n >> 1: a head-dim-64 unit of one tile may be
+    // through before the next one's first S asks for the unit in front of it)
+    auto bar_dr = [&](int n) -> uint32_t { return bar0 + ((n & 1) ? (C::KV > 2 ? 496 : 368) : 176); };
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_gen + C::OFF_BAR + 360);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(s_gen + C::OFF_BAR + 364);
     int* redo_cnt = reinterpret_cast<int*>(s_gen + C::OFF_REDO);
     int* redo_last = redo_cnt + 1;
     int* redo_list = redo_cnt + 2;
@@ -326,12 +344,19 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) {
-            mbar_init(bar_kf + 8 * s, 1); mbar_init(bar_vf + 8 * s, 1); mbar_init(bar_sf + 8 * s, 1); mbar_init(bar_pv + 8 * s, 1);
-            mbar_init(bar_se + 8 * s, C::NSW); mbar_init(bar_pf + 8 * s, C::NSW / 2); mbar_init(bar_ph + 8 * s, 1); mbar_init(bar_drain + 8 * s, 1);
+            mbar_init(bar_sf + 8 * s, 1); mbar_init(bar_se + 8 * s, 8);
+            mbar_init(bar_ph + 8 * s, 1); mbar_init(bar_pv + 8 * s, 1); mbar_init(bar_drain + 8 * s, 1);
         }
-        for (int s = 0; s < 4; ++s) mbar_init(bar_x + 8 * s, C::NG);
-        mbar_init(bar_qf, 1); mbar_init(bar_qe, HIST ? C::NSW + 1 : 1); mbar_init(bar_hf, 1); mbar_init(bar_he, C::NSW);
-        mbar_init(bar_af, C::NSW); mbar_init(bar_ud, 1); mbar_init(bar_dr, C::NSW);
+        for (int s = 0; s < C::KV; ++s) {
+            mbar_init(bar_kf + 8 * s, 1); mbar_init(bar_vf + 8 * s, 1);
+            if (C::KV > 2) { mbar_init(bar_ke + 8 * s, 1); mbar_init(bar_ve + 8 * s, 1); }
+        }
+        for (int s = 0; s < 4; ++s) {
+            mbar_init(bar_pf + 8 * s, TEAMED ? 8 : 4); mbar_init(bar_x + 8 * s, TEAMED ? 1 : 2); mbar_init(bar_m + 8 * s, 2); mbar_init(bar_mr + 8 * s, 4);
+            mbar_init(bar_h + 8 * s, 1); mbar_init(bar_y + 8 * s, 2);
+        }
+        mbar_init(bar_qf, 1); mbar_init(bar_qe, HIST && !TEAMED ? 9 : 1); mbar_init(bar_hf, 1); mbar_init(bar_he, 8);
+        mbar_init(bar_af, 8); mbar_init(bar_ud, 1); mbar_init(bar_dr(0), 8); mbar_init(bar_dr(1), 8);
         *abort_flag = 0;
         *redo_cnt = 0; *redo_last = -1;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -372,28 +397,29 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         bool ok = true;
         int t = 0;
         const int Tn = p.Tn;
-        const uint32_t tiles = is_k ? sK : sV, full = is_k ? bar_kf : bar_vf, freed = is_k ? bar_sf : bar_pv;
+        const uint32_t tiles = is_k ? sK : sV, full = is_k ? bar_kf : bar_vf, freed = is_k ? bar_ke : bar_ve;
         auto list_of = [&](int u) -> const uint32_t* {
             if constexpr (BLK == 128) return reinterpret_cast<const uint32_t*>(p.idx + (size_t)u * p.keep);
             else return p.entries + (size_t)u * p.max_tiles * G + box;
         };
+        auto load_q = [&](int n) {
+            const int u = blockIdx.x + n * gridDim.x, bh = u / p.upb, i = u - bh * p.upb;
+            if (lane == 0) {
+                mbar_expect_tx(bar_qf, C::TILE_BYTES);
+#pragma unroll
+                for (int s = 0; s < C::SUB; ++s) tma_load_4d(sQ + s * C::SUB_BYTES, &tm_q, s * 64, i * 128, bh, 0, bar_qf);
+            }
+            __syncwarp();
+        };
         uint32_t e_next = my_units > 0 ? __ldg(list_of(blockIdx.x)) : 0u;      // list entry, read one tile ahead
         for (int n = 0; ok && n < my_units; ++n) {
             const int u = blockIdx.x + n * gridDim.x;
-            const int bh = u / p.upb, i = u - bh * p.upb;
+            const int bh = u / p.upb;
             const int cnt = tiles_of(n);
-            if (!is_k) {   // Q of this unit, once the softmax warps are done with the previous one
-                if (n >= 1 && !(ok = wait_w(bar_qe, n - 1, 1))) break;
-                if (lane == 0) {
-                    mbar_expect_tx(bar_qf, C::TILE_BYTES);
-#pragma unroll
-                    for (int s = 0; s < C::SUB; ++s) tma_load_4d(sQ + s * C::SUB_BYTES, &tm_q, s * 64, i * 128, bh, 0, bar_qf);
-                }
-                __syncwarp();
-            }
-            const uint32_t* list = list_of(u);
+            if (!is_k && n == 0) load_q(0);
+           const uint32_t* list = list_of(u);
             for (int j = 0; j < cnt; ++j, ++t) {
-                const uint32_t st = t & 1, dst = tiles + st * C::TILE_BYTES + box * BLK * 128, bar = full + 8 * st;
+                const uint32_t st = t & (C::KV - 1), dst = tiles + st * C::TILE_BYTES + box * BLK * 128, bar = full + 8 * st;
                 int blk;
                 if constexpr (BLK == 128) blk = checked_block((int)e_next, Tn, is_k && lane == 0 ? p.dev_status : nullptr, u);
                 else { blk = (int)(e_next & 1023u); if (blk >= Tn) blk = 0; }          // (the list builder has checked every entry already)
@@ -408,7 +434,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                     else { slot = p.ring_head + c - p.n_sink; if (slot >= p.P) slot -= p.P; }
                 }
                 const CUtensorMap* m = is_k ? (cur ? &tm_kcur : &tm_kring) : (cur ? &tm_vcur : &tm_vring);
-                if (t >= 2 && !(ok = wait_w(freed + 8 * st, (t >> 1) - 1, 2))) break;
+                if (t >= C::KV && !(ok = wait_w(freed + 8 * st, (t >> C::KV_LOG) - 1, 2))) break;
                 if (lane == 0) mbar_expect_tx(bar, C::TILE_BYTES);
                 __syncwarp();
                 if (lane < G) {
@@ -416,7 +442,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                     for (int s = 0; s < C::SUB; ++s) tma_load_4d(dst + s * C::SUB_BYTES, m, s * 64, jb * BLK, bh, slot, bar);
                 }
                 __syncwarp();
-                if (HIST && !is_k && j == (cnt > 1 ? 1 : 0)) {
+                if (HIST && !is_k && j == (cnt >= C::KV ? C::KV - 1 : cnt - 1)) {
                     // For the history term at the unit's end: the head's folded state and z.  The buffer is free once the
                     // previous unit's output, which was staged in it, has been read by the bulk stores.  (Two V tiles of
                     // this unit are on their way by now; the third needs P V of the first, which comes after that.)
@@ -432,6 +458,11 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                     }
                     __syncwarp();
                 }
+                // The next unit's Q, once this unit's is in tensor memory
+                if (!is_k && n + 1 < my_units && j == (cnt > C::KV && !(HIST && !TEAMED) ? C::KV : cnt - 1)) {
+                    if (!(ok = wait_w(bar_qe, n, 1))) break;
+                    load_q(n + 1);
+                }
             }
         }
         if (!ok) {   // gave up: let the copies already in flight land before the CTA leaves
@@ -445,37 +476,45 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         constexpr uint32_t IDESC_S = idesc_bf16(128, false);
         constexpr uint32_t TILE_STEP = C::TILE_BYTES >> 4;      // descriptor address field counts 16-byte units
         const uint64_t dq0 = smem_desc_sw128(sQ, 16, 1024), dk0 = smem_desc_sw128(sK, 16, 1024);
-        const uint32_t k_lo = (uint32_t)dk0, k_hi = (uint32_t)(dk0 >> 32);
+        const uint32_t q_lo = (uint32_t)dq0, k_lo = (uint32_t)dk0, k_hi = (uint32_t)(dk0 >> 32);
         bool ok = true;
-        int x = 0;
+        int x = 0, cnt_prev = 0;
         for (int n = 0; ok && n < my_units; ++n) {
             const int cnt = tiles_of(n);
             for (int j = 0; j < cnt; ++j, ++x) {
-                const uint32_t st = x & 1;
-                if (j == 0) {
-                    // Q of the unit moves from shared to tensor memory, where the previous unit's last S has read it by then
-                    if (!(ok = wait_w(bar_qf, n, 4))) break;
-                    if (n >= 1 && !(ok = wait_w(bar_sf + 8 * ((x - 1) & 1), (x - 1) >> 1, 22))) break;
-                }
-                if (!(ok = wait_w(bar_kf + 8 * st, x >> 1, 5))) break;
-                // The S buffer: free once the softmax warps hold S of two tiles ago in registers.  HIST: at a unit's start the
-                // buffer holds the previous unit's phi(Q) operand, at its second tile the previous unit's D_h.
-                if (HIST && n >= 1 && j == 0) { if (!(ok = wait_w(bar_ud, n - 1, 23))) break; }
-                else if (HIST && n >= 1 && j == 1) { if (!(ok = wait_w(bar_dr, n - 1, 24))) break; }
+                const uint32_t st = x & 1, kv = x & (C::KV - 1);
+                if (j == 0 && !(ok = wait_w(bar_qf, n, 4))) break;
+                if (!(ok = wait_w(bar_kf + 8 * kv, x >> C::KV_LOG, 5))) break;
+                // The S buffer: free once the softmax warps hold S of two tiles ago in registers.  HIST: the buffer of a unit's last tile holds
+                // its D_h afterwards, and (head dim 128) the other one its phi(Q) operand.
+                if (HIST && n >= 1 && j == 1) { if (!(ok = wait_w(bar_dr(n - 1), (n - 1) >> 1, 30))) break; }
+                else if (HIST && !C::A_IN_P && n >= 1 && j == 0) { if (!(ok = wait_w(bar_ud, n - 1, 23))) break; }
+                else if (HIST && C::A_IN_P && n >= 2 && j == 0 && cnt_prev == 1) { if (!(ok = wait_w(bar_dr(n - 2), (n - 2) >> 1, 35))) break; }
                 else if (x >= 2) { if (!(ok = wait_w(bar_se + 8 * st, (x >> 1) - 1, 25))) break; }
                 fence_after_sync();
                 if (elect_one()) {
-                    if (j == 0) {
+                    // a unit's first product takes Q from shared memory, the others from tensor memory
+                    if (j == 0) mma_ss_tile<D>(tmem + st * 128, q_lo, k_lo + kv * TILE_STEP, k_hi, IDESC_S);
+                    else mma_ts_kmajor<D>(tmem + st * 128, tmem + C::COL_Q, k_lo + kv * TILE_STEP, k_hi, IDESC_S);
+                    mma_commit(bar_sf + 8 * st);
+                    if (C::KV > 2) mma_commit(bar_ke + 8 * kv);
+                }
+                __syncwarp();
+                if (j == 0) {
+                    // Q moves to tensor memory once the previous unit's last product, and its phi pass, have read what is there
+                    if (n >= 1 && !(ok = wait_w(bar_sf + 8 * ((x - 1) & 1), (x - 1) >> 1, 22))) break;
+                    if (HIST && C::A_IN_P && n >= 1 && !(ok = wait_w(bar_af, n - 1, 36))) break;
+                    fence_after_sync();
+                    if (elect_one()) {
 #pragma unroll
                         for (int ks = 0; ks < D / 16; ++ks)      // 16 features = 32 bytes of a row = 8 columns
                             tmem_cp_128x256b(tmem + C::COL_Q + 8 * ks, dq0 + (uint64_t)((ks >> 2) * (C::SUB_BYTES >> 4) + (ks & 3) * 2));
                         mma_commit(bar_qe);
                     }
-                    mma_ts_kmajor<D>(tmem + st * 128, tmem + C::COL_Q, k_lo + st * TILE_STEP, k_hi, IDESC_S);
-                    mma_commit(bar_sf + 8 * st);
+                    __syncwarp();
                 }
-                __syncwarp();
             }
+            cnt_prev = cnt;
         }
         // drain: all operations issued by this warp have completed before TMEM is freed
         if (elect_one()) mma_commit(bar_drain);
@@ -497,7 +536,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         for (int n = 0; ok && n < my_units; ++n) {
             const int cnt = tiles_of(n);
             for (int j = 0; j < cnt; ++j, ++t) {
-                const uint32_t st = t & 1;
+                const uint32_t st = t & 1, kv = t & (C::KV - 1);
                 if (HIST && j == cnt - 1) {
                     // D_h = phi(Q) S W^T while the softmax warps work on the unit's last tile: into that tile's S buffer (already
                     // in registers), A from the other S buffer (quarter k of the features: hi half at column 32 k, lo half D / 8 on),
@@ -506,28 +545,37 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                     if (!(ok = wait_w(bar_af, n, 15))) break;
                     if (!(ok = wait_w(bar_se + 8 * st, t >> 1, 26))) break;
                     fence_after_sync();
-                    const uint32_t tD = tmem + st * 128, tA = tmem + (st ^ 1u) * 128;
+                    const uint32_t tD = tmem + st * 128, tA = C::A_IN_P ? tmem + C::COL_P + 64 * (st ^ 1u) : tmem + (st ^ 1u) * 128;
                     if (elect_one()) {
-                        mma_ts_groups<D>(tD, tA, h_lo, h_hi, IDESC_PV, false);                 // hi x hi
-                        mma_ts_groups<D>(tD, tA + D / 8, h_lo, h_hi, IDESC_PV, true);          // lo x hi
-                        mma_ts_groups<D>(tD, tA, h_lo + H_STEP, h_hi, IDESC_PV, true);         // hi x lo
+                        if constexpr (C::A_IN_P) {
+                            mma_ts_half(tD, tA, h_lo, h_hi, IDESC_PV, false);                  // hi x hi
+                            mma_ts_half(tD, tA + D / 2, h_lo, h_hi, IDESC_PV, true);           // lo x hi
+                            mma_ts_half(tD, tA, h_lo + H_STEP, h_hi, IDESC_PV, true);          // hi x lo
+                        } else {
+                            mma_ts_groups<D>(tD, tA, h_lo, h_hi, IDESC_PV, false);
+                            mma_ts_groups<D>(tD, tA + D / 8, h_lo, h_hi, IDESC_PV, true);
+                            mma_ts_groups<D>(tD, tA, h_lo + H_STEP, h_hi, IDESC_PV, true);
+                        }
                         mma_commit(bar_ud);
                     }
                     __syncwarp();
                 }
-                if (!(ok = wait_w(bar_vf + 8 * st, t >> 1, 7))) break;
-                if (!(ok = wait_w(bar_pf, t, 6))) break;
+                if (TEAMED && n >= 1 && j == 0 && !(ok = wait_w(bar_dr(n - 1), (n - 1) >> 1, 24))) break;     // O: the previous unit's has been read
+                if (!(ok = wait_w(bar_vf + 8 * kv, t >> C::KV_LOG, 7))) break;
+                const uint32_t pb = C::PBUF == 2 ? st : 0u, p_par = C::PBUF == 2 ? t >> 1 : t;
+                if (!(ok = wait_w(bar_pf + 16 * pb, p_par, 6))) break;
                 fence_after_sync();
                 if (elect_one()) {
-                    mma_ts_half(tO, tmem + C::COL_P, v_lo + st * TILE_STEP, v_hi, IDESC_PV, j > 0);
+                    mma_ts_half(tO, tmem + C::COL_P + 64 * pb, v_lo + kv * TILE_STEP, v_hi, IDESC_PV, j > 0);
                     mma_commit(bar_ph + 8 * st);
                 }
                 __syncwarp();
-                if (!(ok = wait_w(bar_pf + 8, t, 28))) break;
+                if (!(ok = wait_w(bar_pf + 16 * pb + 8, p_par, 28))) break;
                 fence_after_sync();
                 if (elect_one()) {
-                    mma_ts_half(tO, tmem + C::COL_P + 32, v_lo + st * TILE_STEP + (64 * 128 >> 4), v_hi, IDESC_PV, true);
+                    mma_ts_half(tO, tmem + C::COL_P + 64 * pb + 32, v_lo + kv * TILE_STEP + (64 * 128 >> 4), v_hi, IDESC_PV, true);
                     mma_commit(bar_pv + 8 * st);
+                    if (C::KV > 2) mma_commit(bar_ve + 8 * kv);
                 }
                 __syncwarp();
             }
@@ -540,20 +588,17 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         }
     } else {
         // ================================================================= softmax / epilogue
-        const int grp = warp >> 2;                          // column group: key columns [SCOLS grp, SCOLS grp + SCOLS) of a tile
-        const int half = grp * 2 / C::NG;                   // the half of P they are in
-        const int row = (warp & 3) * 32 + lane;             // query row of the unit = TMEM lane
+        // Teams: the team's tiles are t = team, team + 2, ...; the half's columns of a tile 32 half + [0, 32) and 64 on.  Column groups (half):
+        // every tile, columns 64 half + [0, 64).
+        const int team = TEAMED ? warp >> 3 : 0, half = (warp >> 2) & 1, wq = warp & 3;
+        const int row = wq * 32 + lane;                     // query row of the unit = TMEM lane
         const int rg = row / BLK;                           // row group (query block within the unit)
-        const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-        constexpr int EPT = BLK >= C::SCOLS ? 1 : C::SCOLS / BLK;  // list entries (key blocks) under this thread's columns
-        const int col0 = grp * C::SCOLS % BLK;                     // first column within its key block (0 where it has several)
-        const uint32_t bar_xw = bar_x + 8 * (warp & 3);     // partners: the warps with the same rows in the other groups
+        const uint32_t lane_base = tmem + ((uint32_t)(wq * 32) << 16);
+        const uint32_t tS = lane_base + 128 * team, pb = C::PBUF == 2 ? team : 0, tP = lane_base + C::COL_P + 64 * pb;
+        constexpr int EPT = BLK == 128 ? 1 : BLK == 64 ? (TEAMED ? 2 : 1) : 4;     // list entries (key blocks) under the warp's columns
         float* x_m = reinterpret_cast<float*>(s_gen + C::OFF_XM);
-        float* x_l = reinterpret_cast<float*>(s_gen + C::OFF_XS);
-        float* x_d = x_l + C::NG * 128;
         const bool ragged = p.Tc % BLK != 0;                // every chunk's last block is short
         bool ok = true;
-        int t = 0;
         auto wait_s = [&](uint32_t bar, uint32_t parity, int where) -> bool {
             return mbar_wait_warp(bar, parity & 1u, abort_flag, p.dev_status, where);
         };
@@ -562,10 +607,6 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         const bool lane0 = lane == 0;
         auto arrive_t = [&](uint32_t bar) { mbar_arrive_if(bar, lane0); };
         auto arrive_w = [&](uint32_t bar) { __syncwarp(); mbar_arrive_if(bar, lane0); };
-        // Exchange number e of the kernel between partner warps: what a caller wrote to shared memory before is visible to the
-        // others after.  Two per unit (maxima, then sums): a buffer written at one is read by the partners before they arrive
-        // at the next, so each buffer is free again one exchange later.
-        auto exchange = [&](uint32_t e, int where) -> bool { arrive_w(bar_xw); return wait_s(bar_xw, e, where); };
         auto note_redo = [&](int n) {                       // list unit n once
             if (atomicMax(redo_last, n) < n) {
                 const int slot = atomicAdd(redo_cnt, 1);
@@ -576,274 +617,152 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         // unit are read during the current one
         const int dbh = gridDim.x / p.upb, di = gridDim.x - dbh * p.upb;
         int u = blockIdx.x, bh = u / p.upb, i = u - bh * p.upb, cnt_next = tiles_of(0);
-        const uint32_t bar_own = half == 0 ? bar_ph : bar_pv;      // product of its half of P
-        // BLK 16, 64: list entries, read one tile ahead.  BLK 128: all that matters here is whether a tile is a chunk's short last
+        // BLK 16, 64: list entries of the next tile.  BLK 128: all that matters here is whether a tile is a chunk's short last
         // block; one bit per tile from a ballot over 32 list entries at a time (lane = entry), read one window ahead.  An entry
         // outside [0, T_n) is block 0 here as for the loader, which reports it.
         auto entries_of = [&](int unit) -> const uint32_t* {
             if constexpr (BLK == 128) return reinterpret_cast<const uint32_t*>(p.idx + (size_t)unit * p.keep);
-            else return p.entries + (size_t)unit * p.max_tiles * G + grp * C::SCOLS / BLK;
+            else return p.entries + (size_t)unit * p.max_tiles * G;
         };
         uint32_t e_next[EPT], tails = 0;
 #pragma unroll
         for (int x = 0; x < EPT; ++x) e_next[x] = 0u;
-        if (my_units > 0) {
-            if constexpr (BLK == 128) { if (ragged && lane < p.keep) e_next[0] = __ldg(entries_of(u) + lane); }
-            else {
-#pragma unroll
-                for (int x = 0; x < EPT; ++x) e_next[x] = __ldg(entries_of(u) + x);
-            }
-        }
-        for (int n = 0; ok && n < my_units; ++n) {
-            const int q0 = i * 128;
-            const int nq = min(128, p.Tc - q0);
-            const int cnt = cnt_next;
-            cnt_next = n + 1 < my_units ? tiles_of(n + 1) : 0;
-            float m_used = 0.f, l_run = 0.f, dsum = 0.f;    // l_run, dsum: this thread's shares
-            const uint32_t* ent = entries_of(u);
-            // The previous unit's output was staged where S W^T lives, and z where its denominators were exchanged: the loader
-            // may refill both once this warp's bulk store has read its part.  (Said after the unit's first tile, when the store
-            // has long done so; in a unit of one tile, before it.)
-            auto release_h = [&] {
+        auto read_entries = [&](const uint32_t* src) {
+            if constexpr (BLK == 16) {
+                const uint2* src2 = reinterpret_cast<const uint2*>(src) + (TEAMED ? half : 2 * half);
+                const uint2 a = __ldg(src2), b = __ldg(src2 + (TEAMED ? 2 : 1));
+                e_next[0] = a.x; e_next[1] = a.y; e_next[2] = b.x; e_next[3] = b.y;
+            } else if constexpr (BLK == 64 && TEAMED) {
+                const uint2 a = __ldg(reinterpret_cast<const uint2*>(src));
+                e_next[0] = a.x; e_next[1] = a.y;
+            } else if constexpr (BLK == 64) e_next[0] = __ldg(src + half);
+        };
+        auto first_entries = [&](int unit, int pj, int cnt) {      // of a unit: its first window, or the team's first tile
+            if constexpr (BLK == 128) { if (ragged && lane < p.keep) e_next[0] = __ldg(entries_of(unit) + lane); }
+            else if (pj < cnt) read_entries(entries_of(unit) + pj * G);
+        };
+        if (my_units > 0) first_entries(u, team, cnt_next);
+        bool staged = false;                                // this warp's last output is on its way out of shared memory
+        // The previous unit's output was staged where S W^T lives: the loader may refill it, and z, once every warp's bulk store has read
+        // its part.  (Said after the warp's next tile, when the store has long done so, or before its phi pass.)
+        auto release_h = [&] {
+            if (HIST && staged) {
                 if (lane == 0) bulk_wait_read();
                 arrive_w(bar_he);
-            };
-            if (HIST && n >= 1 && cnt == 1) release_h();
-            for (int j = 0; j < cnt; ++j, ++t) {
-                const uint32_t st = t & 1;
-                uint32_t e_cur[EPT];
-                if constexpr (BLK == 128) {
-                    if (ragged && (j & 31) == 0) {
-                        const uint32_t x1 = (e_next[0] < (uint32_t)p.Tn ? e_next[0] : 0u) + 1u;     // last block of a chunk: its index + 1 is a multiple of n_b (no division)
-                        tails = __ballot_sync(0xffffffffu, p.n_b == 1 || __umulhi(x1, p.nb_magic) * p.n_b == x1);
-                        const int j2 = j + 32 < cnt ? j + 32 : 0;
-                        if (j2 + lane < p.keep) e_next[0] = __ldg(entries_of(j2 || n + 1 >= my_units ? u : u + (int)gridDim.x) + j2 + lane);
-                    }
-                } else {
-                    const uint32_t* src = j + 1 < cnt ? ent + (j + 1) * G : entries_of(n + 1 < my_units ? u + (int)gridDim.x : u);
-#pragma unroll
-                    for (int x = 0; x < EPT; ++x) { e_cur[x] = e_next[x]; e_next[x] = __ldg(src + x); }
-                }
-                if (HIST && j == cnt - 1) {
-                    // ---- history term (Eq. 4): A = phi(q) as bf16 hi + lo, this group's share of the features, into the other
-                    // S buffer: this thread's own S columns of it, which it has read (last tile's share).  In a unit of one tile
-                    // the buffer holds the last unit's D_h instead, which other groups may still be reading at head dim 64.
-                    // (columns: quarter k of the features at column 32 k, hi half first)
-                    constexpr int FPT = D / 4;              // features per quarter
-                    if (D == 64 && cnt == 1 && n >= 1) ok = wait_s(bar_dr, n - 1, 29);
-                    ok = ok && wait_s(bar_qf, n, 21) && wait_s(bar_hf, n, 27);
-                    if (!ok) break;
-#pragma unroll 1
-                    for (int k = grp * (4 / C::NG); k < (grp + 1) * (4 / C::NG); ++k) {
-                        const uint8_t* qrow = s_gen + C::OFF_Q + (D == 128 ? (k >> 1) * C::SUB_BYTES : 0) + row * 128;
-                        const float* zs = reinterpret_cast<const float*>(s_gen + C::OFF_Z) + k * FPT;
-                        const uint32_t tA = lane_base + (st ^ 1u) * 128 + k * 32;
-                        uint32_t hi[FPT / 2], lo[FPT / 2];
-#pragma unroll
-                        for (int c = 0; c < FPT / 8; ++c) {
-                            const int ch = (D == 128 ? 4 * (k & 1) : 2 * k) + c;           // 16-byte chunk of the row, 128-byte swizzle
-                            const uint4 qv = *reinterpret_cast<const uint4*>(qrow + ((ch ^ (row & 7)) << 4));
-                            const float4 z0 = *reinterpret_cast<const float4*>(zs + c * 8), z1 = *reinterpret_cast<const float4*>(zs + c * 8 + 4);
-                            const float zz[8] = {z0.x, z0.y, z0.z, z0.w, z1.x, z1.y, z1.z, z1.w};
-                            const uint32_t ws[4] = {qv.x, qv.y, qv.z, qv.w};
-                            float cs[4] = {1.f, 1.f, 1.f, 1.f}, sn[4] = {0.f, 0.f, 0.f, 0.f};
-                            if constexpr (HIST == 2) {      // the pairs' angles belong to the query's row
-                                const int at = (k * (FPT / 8) + c) * p.Tc + min(q0 + row, p.Tc - 1);
-                                const float4 c4 = __ldg(reinterpret_cast<const float4*>(p.cos_q) + at), s4 = __ldg(reinterpret_cast<const float4*>(p.sin_q) + at);
-                                cs[0] = c4.x; cs[1] = c4.y; cs[2] = c4.z; cs[3] = c4.w;
-                                sn[0] = s4.x; sn[1] = s4.y; sn[2] = s4.z; sn[3] = s4.w;
-                            }
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const float2 xq = unpack_bf16(ws[e]);
-                                float f0 = phi_elu1(xq.x), f1 = phi_elu1(xq.y);
-                                dsum = fmaf(f0, zz[2 * e], fmaf(f1, zz[2 * e + 1], dsum));      // (the denominator is not rotated)
-                                if constexpr (HIST == 2) {
-                                    const float r0 = fmaf(-f1, sn[e], f0 * cs[e]), r1 = fmaf(f0, sn[e], f1 * cs[e]);
-                                    f0 = r0; f1 = r1;
-                                }
-                                const uint32_t hp = pack_bf16(f0, f1);
-                                const float2 hf = unpack_bf16(hp);
-                                hi[c * 4 + e] = hp;
-                                lo[c * 4 + e] = pack_bf16(f0 - hf.x, f1 - hf.y);
-                            }
-                        }
-                        if constexpr (D == 128) { tmem_st16(tA, hi); tmem_st16(tA + 16, lo); }
-                        else { tmem_st8(tA, hi); tmem_st8(tA + 8, lo); }
-                    }
-                    tmem_wait_st();
-                    fence_before_sync();
-                    arrive_w(bar_af);
-                    arrive_t(bar_qe);
-                }
-                ok = wait_s(bar_sf + 8 * st, t >> 1, 8);
-                if (!ok) break;
-                fence_after_sync();
-                // ---- this thread's share of the S row in registers
-                uint32_t r[C::SCOLS];
-#pragma unroll
-                for (int c = 0; c < C::SCOLS / 32; ++c) tmem_ld32(lane_base + st * 128 + grp * C::SCOLS + c * 32, *reinterpret_cast<uint32_t(*)[32]>(r + 32 * c));
-                tmem_wait_ld();
-                // ---- columns of this thread that count: all, or the first nv of a segment (a short block; 0: its row group does not
-                // keep the block).  Full and masked segments are separate code: selects on 32 registers in every tile cost 9 us of
-                // a 134 us forward.
-                constexpr int W = C::SCOLS / EPT;
-                int nv[EPT];
-#pragma unroll
-                for (int x = 0; x < EPT; ++x) {
-                    nv[x] = W;
-                    if constexpr (BLK == 128) {
-                        if ((tails >> (j & 31)) & 1u) nv[0] = p.Tc - (p.n_b - 1) * BLK - col0;
-                    } else {
-                        const bool kept = (e_cur[x] >> (10 + rg)) & 1u;
-                        nv[x] = kept ? (int)((e_cur[x] >> 18) & 127u) - col0 : 0;
-                    }
-                }
-                if (j == 0) {
-                    // ---- the reference exponent of the row for the whole unit: the maximum of its first tile plus HEADROOM.  No
-                    // running maximum, no rescaling and no exchange between the column groups after this.  P of the first tile is
-                    // <= 2^-60; a later tile may rise above the first one by a factor of up to ~2^150 (about 100 natural-log
-                    // units) before the row sum passes 2^100, which the end of the unit detects (fp32 overflows at 2^128; rows
-                    // that fall below the first tile lose nothing: what flushes to zero is 2^-66 of the largest term).  Floating
-                    // point is scale invariant, so the result is the one the exact running maximum gives.
-                    float mine = -INFINITY;
-#pragma unroll
-                    for (int x = 0; x < EPT; ++x) mine = fmaxf(mine, swa_max<W, true>(r + x * W, nv[x]));
-                    x_m[grp * 128 + row] = mine;
-                    ok = exchange(0, 11);
-                    if (!ok) break;
-                    float mrow = x_m[row];
-#pragma unroll
-                    for (int g = 1; g < C::NG; ++g) mrow = fmaxf(mrow, x_m[g * 128 + row]);
-                    // rows of a row group past the last query block keep nothing at all: any finite reference will do
-                    m_used = mrow == -INFINITY ? 0.f : fmaf(mrow, p.scale_log2, C::HEADROOM);
-                    if (grp > 0) {
-                        // The exchange has put the two warps that share a scheduler (same rows, different column groups) in step;
-                        // they would run their exponentials at the same time and their waits at the same time, and the
-                        // special-function unit would idle through the latter.  Set back by part of a tile, one group's waits
-                        // fall into the other's exponentials.  Nothing couples the groups until the end of the unit.
-                        const long long t_skew = clock64();
-                        while (clock64() - t_skew < grp * C::SKEW_CLK) {}
-                    }
-                }
-                // ---- P = exp2(S*c - m), row sum, bf16 pairs, 32 columns at a time
-                float2 rsum[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-                auto store_p = [&](int c, const uint32_t (&pk)[16]) {
-                    if (c == 0) {                           // S is in registers: its buffer is free (said here, off the critical path)
-                        fence_before_sync();
-                        arrive_t(bar_se + 8 * st);
-                    }
-                    if (c == 0 && t >= 1) {                 // its half of the P buffer: the product of the tile before has read it
-                        ok = wait_s(bar_own + 8 * ((t - 1) & 1), (t - 1) >> 1, 9);
-                        fence_after_sync();
-                    }
-                    tmem_st16(lane_base + C::COL_P + (C::SCOLS / 2) * grp + 16 * c, pk);
-                };
-                if constexpr (BLK == 16) {
-#pragma unroll
-                    for (int c = 0; c < C::SCOLS / 32; ++c) {
-                        uint32_t pk[16];
-#pragma unroll
-                        for (int x = 2 * c; x < 2 * c + 2; ++x) {
-                            if (__all_sync(0xffffffffu, nv[x] >= W)) swa_weights<W, false>(r + x * W, W, p.scale_log2, m_used, rsum, pk + (x & 1) * (W / 2));
-                            else if (__any_sync(0xffffffffu, nv[x] > 0)) swa_weights<W, true>(r + x * W, nv[x], p.scale_log2, m_used, rsum, pk + (x & 1) * (W / 2));
-                            else {
-#pragma unroll
-                                for (int e = 0; e < W / 2; ++e) pk[(x & 1) * (W / 2) + e] = 0u;
-                            }
-                        }
-                        store_p(c, pk);
-                    }
-                } else if (nv[0] >= W) {                    // (the same for the whole warp)
-#pragma unroll
-                    for (int c = 0; c < C::SCOLS / 32; ++c) {
-                        uint32_t pk[16];
-                        swa_weights<32, false>(r + 32 * c, 32, p.scale_log2, m_used, rsum, pk);
-                        store_p(c, pk);
-                    }
-                } else if (BLK == 128 || nv[0] > 0) {
-#pragma unroll
-                    for (int c = 0; c < C::SCOLS / 32; ++c) {
-                        uint32_t pk[16];
-                        swa_weights<32, true>(r + 32 * c, nv[0] - 32 * c, p.scale_log2, m_used, rsum, pk);
-                        store_p(c, pk);
-                    }
-                } else {
-#pragma unroll
-                    for (int c = 0; c < C::SCOLS / 32; ++c) {
-                        uint32_t pk[16];
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) pk[e] = 0u;
-                        store_p(c, pk);
-                    }
-                }
-                if (!ok) break;
-                l_run += ((rsum[0].x + rsum[0].y) + (rsum[1].x + rsum[1].y)) + ((rsum[2].x + rsum[2].y) + (rsum[3].x + rsum[3].y));
-                tmem_wait_st();
-                fence_before_sync();
-                arrive_t(bar_pf + 8 * half);
-                if (HIST && n >= 1 && j == 0 && cnt > 1) release_h();
+                staged = false;
             }
-            if (!ok) break;
-            // (a thread block that leaves room beside it lets the next kernel in only now: that one waits, but its blocks take slots)
-            if (C::SMEM_BYTES <= 200 * 1024 && n + 1 == my_units) pdl_trigger();
-            // ---- end of the unit: row sums (and the shares of Eq. 4's denominator) of the column groups, range test, output
-            const bf16* bias_row = (HIST && p.bias) ? p.bias + (size_t)(bh % p.heads) * D + grp * C::OCOLS : nullptr;
-            uint4 bw[C::OCOLS / 8];
-#pragma unroll
-            for (int c = 0; c < C::OCOLS / 8; ++c) bw[c] = bias_row ? __ldg(reinterpret_cast<const uint4*>(bias_row) + c) : make_uint4(0, 0, 0, 0);
-            if constexpr (HIST) {
-                ok = wait_s(bar_ud, n, 19);                 // D_h complete: the buffer of S W^T is free
-                if (!ok) break;
-                x_d[grp * 128 + row] = dsum;
-            }
-            x_l[grp * 128 + row] = l_run;
-            ok = exchange(1, 12);
-            if (!ok) break;
-            l_run = x_l[row];
-            float den = HIST ? x_d[row] : 0.f;
-#pragma unroll
-            for (int g = 1; g < C::NG; ++g) { l_run += x_l[g * 128 + row]; if constexpr (HIST) den += x_d[g * 128 + row]; }
-            const float inv = 1.f / l_run, inv_den = 1.f / (p.eps + den);
-            const size_t g_row = (size_t)bh * p.Tc + q0 + row;
-            if (grp == 0 && row < nq && p.lse) p.lse[g_row] = (m_used + log2f(l_run)) * 0.6931471805599453f;
-            const uint32_t tl = t - 1;                      // the unit's last tile
-            ok = wait_s(bar_pv + 8 * (tl & 1), tl >> 1, 10);
-            if (!ok) break;
+        };
+        // one bit per tile of the window of 32 that starts at tile j: the short last block of a chunk
+        auto next_tails = [&](const uint32_t* ent, int j, int cnt) {
+            const uint32_t x1 = (e_next[0] < (uint32_t)p.Tn ? e_next[0] : 0u) + 1u;     // last block of a chunk: its index + 1 is a multiple of n_b (no division)
+            tails = __ballot_sync(0xffffffffu, p.n_b == 1 || __umulhi(x1, p.nb_magic) * p.n_b == x1);
+            const int j2 = (j | 31) + 1 + lane;
+            if (j2 < cnt) e_next[0] = __ldg(ent + j2);
+        };
+        // The reference exponent of the row for the whole unit: the maximum of its first tile plus HEADROOM.  No running maximum and no
+        // rescaling after this.  P of the first tile is <= 2^-60; a later tile may rise above the first one by a factor of up to ~2^150
+        // (about 100 natural-log units) before the row sum passes 2^100, which the end of the unit detects (fp32 overflows at 2^128; rows
+        // that fall below the first tile lose nothing: what flushes to zero is 2^-66 of the largest term).  Floating point is scale
+        // invariant, so the result is the one the exact running maximum gives.  Rows of a row group past the last query block keep nothing
+        // at all: any finite reference will do.
+        auto reference = [&](const float* xm) -> float {
+            const float mrow = fmaxf(xm[row], xm[128 + row]);
+            return mrow == -INFINITY ? 0.f : fmaf(mrow, p.scale_log2, C::HEADROOM);
+        };
+        // History term (Eq. 4) of unit n: this warp's quarters of the features of A = phi(q), as bf16 hi + lo, to tensor memory from ta on (quarter k
+        // at column 32 k, hi half first; in a P buffer all of hi, then all of lo); returns its share of the denominator in dsum.
+        auto form_phi = [&](int n, int q0, uint32_t ta, float& dsum) -> bool {
+            constexpr int FPT = D / 4;              // features per quarter
+            // (S columns 32 k on are the warp's own: a half's, or a column group's)
+            const int k0 = TEAMED ? half : 2 * half, dk = TEAMED ? 2 : 1;
+            if (!wait_s(TEAMED ? bar_qe : bar_qf, n, 21) || !wait_s(bar_hf, n, 27)) return false;
             fence_after_sync();
-            // overflow (or NaN): a later tile rose too far above the first one.  (After the wait: P V of this unit's last tile
-            // needed every warp, so all of them have listed the unit before this one.)
-            if (!(l_run < 1e30f)) note_redo(n);
-            // Output through shared memory and one bulk tensor store per warp (32 rows x its group's columns):
-            // row-per-thread global stores would touch 32 lines per instruction.  The staging tile is the S W^T buffer (free: the
-            // history products have completed, or were never asked for); in the map's swizzle of the row width.
-            const uint32_t stage_off = C::OFF_H + warp * (32 * C::OCOLS * 2);
+            float2 ds = make_float2(0.f, 0.f);
+#pragma unroll 1
+            for (int k = k0; k < (TEAMED ? 4 : 2 * half + 2); k += dk) {
+                uint32_t qw[FPT / 2];
+                if constexpr (!TEAMED) {                    // q from shared memory
+                    const uint8_t* qrow = s_gen + C::OFF_Q + (D == 128 ? (k >> 1) * C::SUB_BYTES : 0) + row * 128;
+#pragma unroll
+                    for (int c = 0; c < FPT / 8; ++c) {
+                        const uint4 qv = *reinterpret_cast<const uint4*>(qrow + (((D == 128 ? 4 * (k & 1) + c : 2 * k + c) ^ (row & 7)) << 4));
+                        qw[4 * c] = qv.x; qw[4 * c + 1] = qv.y; qw[4 * c + 2] = qv.z; qw[4 * c + 3] = qv.w;
+                    }
+                } else {                                    // q from tensor memory
+                    if constexpr (D == 128) tmem_ld16(lane_base + C::COL_Q + k * (FPT / 2), qw);
+                    else tmem_ld8(lane_base + C::COL_Q + k * (FPT / 2), qw);
+                    tmem_wait_ld();
+                }
+                const float* zs = reinterpret_cast<const float*>(s_gen + C::OFF_Z) + k * FPT;
+                const uint32_t tA = ta + k * (C::A_IN_P ? FPT / 2 : 32);
+                uint32_t hi[FPT / 2], lo[FPT / 2];
+#pragma unroll
+                for (int c = 0; c < FPT / 8; ++c) {
+                    const float4 z0 = *reinterpret_cast<const float4*>(zs + c * 8), z1 = *reinterpret_cast<const float4*>(zs + c * 8 + 4);
+                    const float zz[8] = {z0.x, z0.y, z0.z, z0.w, z1.x, z1.y, z1.z, z1.w};
+                    float cs[4] = {1.f, 1.f, 1.f, 1.f}, sn[4] = {0.f, 0.f, 0.f, 0.f};
+                    if constexpr (HIST == 2) {      // the pairs' angles belong to the query's row
+                        const int at = (k * (FPT / 8) + c) * p.Tc + min(q0 + row, p.Tc - 1);
+                        const float4 c4 = __ldg(reinterpret_cast<const float4*>(p.cos_q) + at), s4 = __ldg(reinterpret_cast<const float4*>(p.sin_q) + at);
+                        cs[0] = c4.x; cs[1] = c4.y; cs[2] = c4.z; cs[3] = c4.w;
+                        sn[0] = s4.x; sn[1] = s4.y; sn[2] = s4.z; sn[3] = s4.w;
+                    }
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        float2 f = phi_elu1(unpack_bf16(qw[4 * c + e]));
+                        ds = ffma2(f, make_float2(zz[2 * e], zz[2 * e + 1]), ds);       // (the denominator is not rotated)
+                        if constexpr (HIST == 2) f = make_float2(fmaf(-f.y, sn[e], f.x * cs[e]), fmaf(f.x, sn[e], f.y * cs[e]));
+                        const uint32_t hp = pack_bf16(f.x, f.y);
+                        const float2 r = ffma2(unpack_bf16(hp), make_float2(-1.f, -1.f), f);
+                        hi[c * 4 + e] = hp;
+                        lo[c * 4 + e] = pack_bf16(r.x, r.y);
+                    }
+                }
+                if constexpr (D == 128) { tmem_st16(tA, hi); tmem_st16(tA + 16, lo); }
+                else { tmem_st8(tA, hi); tmem_st8(tA + D / 2, lo); }
+            }
+            tmem_wait_st();
+            fence_before_sync();
+            arrive_w(bar_af);
+            if (!TEAMED) arrive_t(bar_qe);
+            dsum = ds.x + ds.y;
+            return true;
+        };
+        // This warp's columns of the head's bias (read ahead of the waits at a unit's end: one at a time between them they are a trip to L2 each)
+        auto read_bias = [&](uint4 (&bw)[C::OCOLS / 8]) {
+            const uint4* b = HIST && p.bias ? reinterpret_cast<const uint4*>(p.bias + (size_t)(bh % p.heads) * D + half * C::OCOLS) : nullptr;
+#pragma unroll
+            for (int c = 0; c < C::OCOLS / 8; ++c) bw[c] = b ? __ldg(b + c) : make_uint4(0, 0, 0, 0);
+        };
+        // Output of unit n, D_h at tD.
+        auto write_output = [&](int n, int q0, uint32_t tD, float inv, float inv_den, const uint4 (&bw)[C::OCOLS / 8]) {
+            // Output through shared memory and one bulk tensor store per warp (32 rows x half of the columns): row-per-thread global stores
+            // would touch 32 lines per instruction.  The staging tile is the S W^T buffer (free: the history products have completed;
+            // where there are none each team has its own), in the map's swizzle of the row width.
+            const uint32_t stage_off = C::OFF_H + (HIST ? 0 : team * C::TILE_BYTES) + (half * 4 + wq) * (32 * C::OCOLS * 2);
             uint8_t* stage = s_gen + stage_off + lane * (C::OCOLS * 2);
-            const int swz = C::OCOLS == 64 ? lane & 7 : C::OCOLS == 32 ? (lane >> 1) & 3 : (lane >> 2) & 1;
-            if (!HIST && n >= 1) {
-                if (lane == 0) bulk_wait_read();            // this warp's previous store has read its part
+            const int swz = C::OCOLS == 64 ? lane & 7 : (lane >> 1) & 3;
+            if (!HIST && staged) {
+                if (lane == 0) bulk_wait_read();        // this warp's previous store has read its part
                 __syncwarp();
             }
 #pragma unroll
             for (int c = 0; c < C::OCOLS / 16; ++c) {
                 uint32_t o[16], dh[16];
-                tmem_ld16(lane_base + C::COL_O + grp * C::OCOLS + c * 16, o);
-                if constexpr (HIST) tmem_ld16(lane_base + (tl & 1) * 128 + grp * C::OCOLS + c * 16, dh);
+                tmem_ld16(lane_base + C::COL_O + half * C::OCOLS + c * 16, o);
+                if constexpr (HIST != 0) tmem_ld16(tD + half * C::OCOLS + c * 16, dh);
                 tmem_wait_ld();
                 if (c == C::OCOLS / 16 - 1) {
-                    // The next unit's first P V overwrites O.  It needs the lower half of P of that tile from all warps of the lower half
-                    // of the groups, each of which first meets the warps of its rows in ALL groups in the exchange of the maxima: all
-                    // of them are past these loads then.
                     fence_before_sync();
-                    if constexpr (HIST) arrive_t(bar_dr);
+                    if (TEAMED) arrive_w(bar_dr(n)); else if (HIST) arrive_t(bar_dr(n));
                 }
-                const float* hsrc = !HIST && p.hist ? p.hist + g_row * D + grp * C::OCOLS + c * 16 : nullptr;
+                const float* hsrc = !HIST && p.hist ? p.hist + ((size_t)bh * p.Tc + q0 + row) * D + half * C::OCOLS + c * 16 : nullptr;
 #pragma unroll
                 for (int v = 0; v < 2; ++v) {
                     float x[8];
 #pragma unroll
                     for (int e = 0; e < 8; ++e) x[e] = __uint_as_float(o[v * 8 + e]) * inv;
-                    if constexpr (HIST) {
+                    if constexpr (HIST != 0) {
 #pragma unroll
                         for (int e = 0; e < 8; ++e) x[e] = fmaf(__uint_as_float(dh[v * 8 + e]), inv_den, x[e]);
                         // Eq. 4's Linear: its matrix is folded into the state, its bias is added here
@@ -851,7 +770,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                         const float2 b0 = unpack_bf16(b.x), b1 = unpack_bf16(b.y), b2 = unpack_bf16(b.z), b3 = unpack_bf16(b.w);
                         x[0] += b0.x; x[1] += b0.y; x[2] += b1.x; x[3] += b1.y;
                         x[4] += b2.x; x[5] += b2.y; x[6] += b3.x; x[7] += b3.y;
-                    } else if (hsrc && row < nq) {
+                    } else if (hsrc && q0 + row < p.Tc) {
                         const float4 h0 = *reinterpret_cast<const float4*>(hsrc + v * 8);
                         const float4 h1 = *reinterpret_cast<const float4*>(hsrc + v * 8 + 4);
                         x[0] += h0.x; x[1] += h0.y; x[2] += h0.z; x[3] += h0.w;
@@ -865,12 +784,327 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             }
             fence_proxy_async();
             __syncwarp();
-            if (lane == 0 && q0 + (warp & 3) * 32 < p.Tc) {     // rows past the chunk's end are clipped by the map
-                tma_store_4d(&tm_o, s_base + stage_off, grp * C::OCOLS, q0 + (warp & 3) * 32, bh, 0);
+            if (lane == 0 && q0 + wq * 32 < p.Tc) {     // rows past the chunk's end are clipped by the map
+                tma_store_4d(&tm_o, s_base + stage_off, half * C::OCOLS, q0 + wq * 32, bh, 0);
                 bulk_commit();
             }
-            u += gridDim.x; bh += dbh; i += di;
-            if (i >= p.upb) { i -= p.upb; ++bh; }
+            staged = true;
+        };
+        if constexpr (TEAMED) {
+            float* x_l = reinterpret_cast<float*>(s_gen + C::OFF_XL);
+            float* x_d = x_l + 128;
+            int t0 = 0;                                         // first tile of the unit
+            for (int n = 0; ok && n < my_units; ++n) {
+                const int q0 = i * 128;
+                const int nq = min(128, p.Tc - q0);
+                const int cnt = cnt_next;
+                cnt_next = n + 1 < my_units ? tiles_of(n + 1) : 0;
+                const int pj = (t0 ^ team) & 1;                 // own tiles of the unit: pj, pj + 2, ...
+                float m_used = 0.f, l_run = 0.f, dsum = 0.f;    // l_run, dsum: this thread's shares
+                const uint32_t* ent = entries_of(u);
+                for (int j = pj; j < cnt; j += 2) {
+                    const int t = t0 + j;
+                    uint32_t e_cur[EPT];
+                    if constexpr (BLK == 128) {
+                        if (ragged && (j & 31) == pj) {
+                            next_tails(ent, j, cnt);
+                        }
+                    } else {
+#pragma unroll
+                        for (int x = 0; x < EPT; ++x) e_cur[x] = e_next[x];
+                        if (j + 2 < cnt) read_entries(ent + (j + 2) * G);
+                    }
+                    // valid columns of entry x for this row: all, or the first nv (a short block; 0: its row group does not keep the block)
+                    auto valid = [&](int x) -> int {
+                        if constexpr (BLK == 128) return (tails >> (j & 31)) & 1u ? p.Tc - (p.n_b - 1) * BLK : BLK;
+                        else return (e_cur[x] >> (10 + rg)) & 1u ? (int)((e_cur[x] >> 18) & 127u) : 0;
+                    };
+                    // ... of the 32 columns 64 c + 32 half on (blocks of 64 and 128 tokens)
+                    auto valid32 = [&](int c) -> int { return BLK == 128 ? valid(0) - 64 * c - 32 * half : valid(c) - 32 * half; };
+                    if (!(ok = wait_s(bar_sf + 8 * team, t >> 1, 8))) break;
+                    fence_after_sync();
+                    if (j == 0) {
+                        // row maxima for the reference exponent
+                        float mine = -INFINITY;
+                        uint32_t r[2][32];
+                        tmem_ld32(tS + 32 * half, r[0]);
+                        tmem_ld32(tS + 64 + 32 * half, r[1]);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            if constexpr (BLK == 16) mine = fmaxf(mine, fmaxf(swa_max<16, true>(r[c], valid(2 * c)), swa_max<16, true>(r[c] + 16, valid(2 * c + 1))));
+                            else if (valid32(c) >= 32) mine = fmaxf(mine, swa_max<32, false>(r[c], 32));
+                            else if (valid32(c) > 0) mine = fmaxf(mine, swa_max<32, true>(r[c], valid32(c)));
+                        }
+                        if (n >= 1 && !(ok = wait_s(bar_mr + 8 * wq, n - 1, 32))) break;       // the unit before: read
+                        x_m[half * 128 + row] = mine;
+                        arrive_w(bar_m + 8 * wq);
+                    }
+                    if (j <= 1) {
+                        if (!(ok = wait_s(bar_m + 8 * wq, n, 11))) break;
+                        m_used = reference(x_m);
+                        arrive_w(bar_mr + 8 * wq);
+                    }
+                    // ---- P = exp2(S*c - m), row sum, bf16 pairs
+                    float2 rsum[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        uint32_t r[32], pk[16];
+                        tmem_ld32(tS + 64 * c + 32 * half, r);
+                        tmem_wait_ld();
+                        if (c == 1) {                           // S is in registers: its buffer is free
+                            fence_before_sync();
+                            arrive_t(bar_se + 8 * team);
+                        }
+                        // Full, masked and empty segments are separate code: selects on 32 registers in every tile cost 9 us of a 134 us
+                        // forward.  (BLK 64, 128: the same for the whole warp.)
+                        if constexpr (BLK == 16) {
+#pragma unroll
+                            for (int x = 0; x < 2; ++x) {
+                                const int nv = valid(2 * c + x);
+                                if (__all_sync(0xffffffffu, nv >= 16)) swa_weights<16, false>(r + 16 * x, 16, p.scale_log2, m_used, rsum, pk + 8 * x);
+                                else if (__any_sync(0xffffffffu, nv > 0)) swa_weights<16, true>(r + 16 * x, nv, p.scale_log2, m_used, rsum, pk + 8 * x);
+                                else {
+#pragma unroll
+                                    for (int e = 0; e < 8; ++e) pk[8 * x + e] = 0u;
+                                }
+                            }
+                        } else {
+                            const int nv = valid32(c);
+                            if (nv >= 32) swa_weights<32, false>(r, 32, p.scale_log2, m_used, rsum, pk);
+                            else if (nv > 0) swa_weights<32, true>(r, nv, p.scale_log2, m_used, rsum, pk);
+                            else {
+#pragma unroll
+                                for (int e = 0; e < 16; ++e) pk[e] = 0u;
+                            }
+                        }
+                        if (HIST && C::A_IN_P && c == 0 && j == 0 && n >= 1) {      // the P buffer held the unit before's phi(Q) operand
+                            if (!(ok = wait_s(bar_ud, n - 1, 37))) break;
+                        }
+                        if (t >= C::PBUF) {                     // its half of the P buffer: the product that last read it is complete
+                            const int tr = t - C::PBUF;
+                            if (!(ok = wait_s((c == 0 ? bar_ph : bar_pv) + 8 * (tr & 1), tr >> 1, 9))) break;
+                            fence_after_sync();
+                        }
+                        tmem_st16(tP + 32 * c + 16 * half, pk);
+                        tmem_wait_st();
+                        fence_before_sync();
+                        arrive_t(bar_pf + 16 * pb + 8 * c);
+                    }
+                    if (!ok) break;
+                    l_run += ((rsum[0].x + rsum[0].y) + (rsum[1].x + rsum[1].y)) + ((rsum[2].x + rsum[2].y) + (rsum[3].x + rsum[3].y));
+                    release_h();
+                }
+                if (!ok) break;
+                if (n + 1 < my_units) first_entries(u + (int)gridDim.x, (t0 + cnt ^ team) & 1, cnt_next);
+                if (((cnt - 1) & 1) != pj) {
+                    // ---- the other team has the unit's last tile, and its output: this one hands over its row sums and goes on to the next unit
+                    if constexpr (HIST != 0) {
+                        release_h();
+                        if (C::A_IN_P) {                        // its P buffer: the product of its last tile is complete
+                            const int tx = t0 + cnt - 2;
+                            if (tx >= 0) ok = wait_s(bar_pv + 8 * (tx & 1), tx >> 1, 29);
+                        } else if (cnt == 1 && n >= 1) ok = wait_s(bar_dr(n - 1), (n - 1) >> 1, 29);
+                        if (!(ok = ok && form_phi(n, q0, C::A_IN_P ? tP : tS, dsum))) break;
+                    }
+                    if (cnt == 1) arrive_t(bar_mr + 8 * wq);                    // (nothing to read)
+                    if (half == 1) {
+                        if (n >= 1 && !(ok = wait_s(bar_dr(n - 1), (n - 1) >> 1, 31))) break; // the sums of the unit before have been read
+                        x_l[row] = l_run;
+                        if constexpr (HIST != 0) x_d[row] = dsum;
+                        arrive_w(bar_h + 8 * wq);
+                    } else {
+                        if (!(ok = wait_s(bar_h + 8 * wq, n, 33))) break;
+                        x_l[row] += l_run;
+                        if constexpr (HIST != 0) x_d[row] += dsum;
+                        arrive_w(bar_x + 8 * wq);
+                    }
+                } else {
+                    // (a thread block that leaves room beside it lets the next kernel in only now: that one waits, but its blocks take slots)
+                    if (C::SMEM_BYTES <= 200 * 1024 && n + 1 == my_units) pdl_trigger();
+                    // ---- output of the unit
+                    uint4 bw[C::OCOLS / 8];
+                    read_bias(bw);
+                    if constexpr (HIST != 0) {
+                        if (!(ok = wait_s(bar_ud, n, 19))) break;           // D_h complete: the buffer of S W^T is free
+                    }
+                    if (!(ok = wait_s(bar_x + 8 * wq, n, 12))) break;
+                    float* x_y = reinterpret_cast<float*>(s_gen + C::off_xy(HIST != 0, half));
+                    x_y[row] = l_run;
+                    arrive_w(bar_y + 8 * wq);
+                    if (!(ok = wait_s(bar_y + 8 * wq, n, 34))) break;
+                    {   // (the same order in both halves: the same bits)
+                        const float other = reinterpret_cast<const float*>(s_gen + C::off_xy(HIST != 0, half ^ 1))[row];
+                        l_run = x_l[row] + (half ? other + l_run : l_run + other);
+                    }
+                    const float inv = 1.f / l_run, inv_den = HIST ? 1.f / (p.eps + x_d[row]) : 0.f;
+                    const size_t g_row = (size_t)bh * p.Tc + q0 + row;
+                    if (half == 0 && row < nq && p.lse) p.lse[g_row] = (m_used + log2f(l_run)) * 0.6931471805599453f;
+                    const uint32_t tl = t0 + cnt - 1;           // the unit's last tile
+                    if (!(ok = wait_s(bar_pv + 8 * (tl & 1), tl >> 1, 10))) break;
+                    fence_after_sync();
+                    // overflow (or NaN): a later tile rose too far above the first one.  (The next unit's first P V waits for all of this team's
+                    // warps below: a unit is listed before the next one can be.)
+                    if (!(l_run < 1e30f)) note_redo(n);
+                    write_output(n, q0, tS, inv, inv_den, bw);
+                }
+                t0 += cnt;
+                u += gridDim.x; bh += dbh; i += di;
+                if (i >= p.upb) { i -= p.upb; ++bh; }
+            }
+        } else {
+            // ---- column groups    : all warps on the same tile
+            static_assert(TEAMED || C::PBUF == 1, "one P buffer");
+            // Exchange number e of the kernel between partner warps: what a caller wrote to shared memory before is visible to the
+            // others after.  Two per unit (maxima, then sums): a buffer written at one is read by the partners before they arrive
+            // at the next, so each buffer is free again one exchange later.
+            auto exchange = [&](uint32_t e, int where) -> bool { arrive_w(bar_x + 8 * wq); return wait_s(bar_x + 8 * wq, e, where); };
+            float* x_l = reinterpret_cast<float*>(s_gen + C::off_xy(true, 0));      // [2][128], behind the staging tile of the output
+            float* x_d = x_l + 256;
+            const uint32_t bar_own = half == 0 ? bar_ph : bar_pv;      // product of its half of P
+            const uint32_t tPh = tP + 32 * half;
+            const int col0 = 64 * half % BLK;                   // first column within its key block (0 where it has several)
+            int t = 0;
+            for (int n = 0; ok && n < my_units; ++n) {
+                const int q0 = i * 128;
+                const int nq = min(128, p.Tc - q0);
+                const int cnt = cnt_next;
+                cnt_next = n + 1 < my_units ? tiles_of(n + 1) : 0;
+                float m_used = 0.f, l_run = 0.f, dsum = 0.f;    // l_run, dsum: this thread's shares
+                const uint32_t* ent = entries_of(u);
+                if (cnt == 1) release_h();
+                for (int j = 0; j < cnt; ++j, ++t) {
+                    const uint32_t st = t & 1;
+                    uint32_t e_cur[EPT];
+                    if constexpr (BLK == 128) {
+                        if (ragged && (j & 31) == 0) next_tails(ent, j, cnt);
+                    } else {
+#pragma unroll
+                        for (int x = 0; x < EPT; ++x) e_cur[x] = e_next[x];
+                        if (j + 1 < cnt) read_entries(ent + (j + 1) * G);
+                    }
+                    if (HIST && j == cnt - 1) {
+                        // history term's operand into the other S buffer: this thread's own S columns of it, which it has read (last tile's share),
+                        // or its columns of the last unit's D_h
+                        if (!(ok = form_phi(n, q0, lane_base + (st ^ 1u) * 128, dsum))) break;
+                    }
+                    if (!(ok = wait_s(bar_sf + 8 * st, t >> 1, 8))) break;
+                    fence_after_sync();
+                    // ---- this thread's share of the S row in registers
+                    uint32_t r[64];
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) tmem_ld32(lane_base + st * 128 + half * 64 + c * 32, *reinterpret_cast<uint32_t(*)[32]>(r + 32 * c));
+                    tmem_wait_ld();
+                    // ---- columns of this thread that count: all, or the first nv of a segment (a short block; 0: its row group does not
+                    // keep the block)
+                    constexpr int W = 64 / EPT;
+                    int nv[EPT];
+#pragma unroll
+                    for (int x = 0; x < EPT; ++x) {
+                        nv[x] = W;
+                        if constexpr (BLK == 128) {
+                            if ((tails >> (j & 31)) & 1u) nv[0] = p.Tc - (p.n_b - 1) * BLK - col0;
+                        } else {
+                            const bool kept = (e_cur[x] >> (10 + rg)) & 1u;
+                            nv[x] = kept ? (int)((e_cur[x] >> 18) & 127u) - col0 : 0;
+                        }
+                    }
+                    if (j == 0) {
+                        float mine = -INFINITY;
+#pragma unroll
+                        for (int x = 0; x < EPT; ++x) mine = fmaxf(mine, swa_max<W, true>(r + x * W, nv[x]));
+                        x_m[half * 128 + row] = mine;
+                        if (!(ok = exchange(0, 11))) break;
+                        m_used = reference(x_m);
+                        if (half > 0) {
+                            // The exchange has put the two warps that share a scheduler (same rows, different column groups) in step;
+                            // they would run their exponentials at the same time and their waits at the same time, and the
+                            // special-function unit would idle through the latter.  Set back by part of a tile, one group's waits
+                            // fall into the other's exponentials.  Nothing couples the groups until the end of the unit.
+                            const long long t_skew = clock64();
+                            while (clock64() - t_skew < 700) {}
+                        }
+                    }
+                    // ---- P = exp2(S*c - m), row sum, bf16 pairs, 32 columns at a time
+                    float2 rsum[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+                    auto store_p = [&](int c, const uint32_t (&pk)[16]) {
+                        if (c == 0) {                           // S is in registers: its buffer is free (said here, off the critical path)
+                            fence_before_sync();
+                            arrive_t(bar_se + 8 * st);
+                        }
+                        if (c == 0 && t >= 1) {                 // its half of the P buffer: the product of the tile before has read it
+                            ok = wait_s(bar_own + 8 * ((t - 1) & 1), (t - 1) >> 1, 9);
+                            fence_after_sync();
+                        }
+                        tmem_st16(tPh + 16 * c, pk);
+                    };
+                    if constexpr (BLK == 16) {
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            uint32_t pk[16];
+#pragma unroll
+                            for (int x = 2 * c; x < 2 * c + 2; ++x) {
+                                if (__all_sync(0xffffffffu, nv[x] >= W)) swa_weights<W, false>(r + x * W, W, p.scale_log2, m_used, rsum, pk + (x & 1) * (W / 2));
+                                else if (__any_sync(0xffffffffu, nv[x] > 0)) swa_weights<W, true>(r + x * W, nv[x], p.scale_log2, m_used, rsum, pk + (x & 1) * (W / 2));
+                                else {
+#pragma unroll
+                                    for (int e = 0; e < W / 2; ++e) pk[(x & 1) * (W / 2) + e] = 0u;
+                                }
+                            }
+                            store_p(c, pk);
+                        }
+                    } else if (nv[0] >= W) {                    // (the same for the whole warp)
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            uint32_t pk[16];
+                            swa_weights<32, false>(r + 32 * c, 32, p.scale_log2, m_used, rsum, pk);
+                            store_p(c, pk);
+                        }
+                    } else if (BLK == 128 || nv[0] > 0) {
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            uint32_t pk[16];
+                            swa_weights<32, true>(r + 32 * c, nv[0] - 32 * c, p.scale_log2, m_used, rsum, pk);
+                            store_p(c, pk);
+                        }
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            uint32_t pk[16];
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) pk[e] = 0u;
+                            store_p(c, pk);
+                        }
+                    }
+                    if (!ok) break;
+                    l_run += ((rsum[0].x + rsum[0].y) + (rsum[1].x + rsum[1].y)) + ((rsum[2].x + rsum[2].y) + (rsum[3].x + rsum[3].y));
+                    tmem_wait_st();
+                    fence_before_sync();
+                    arrive_t(bar_pf + 8 * half);
+                    if (cnt > 1) release_h();
+                }
+                if (!ok) break;
+                if (n + 1 < my_units) first_entries(u + (int)gridDim.x, 0, cnt_next);
+                // ---- end of the unit: row sums (and the shares of Eq. 4's denominator) of the column groups, range test, output
+                uint4 bw[C::OCOLS / 8];
+                read_bias(bw);
+                if constexpr (HIST != 0) {
+                    if (!(ok = wait_s(bar_ud, n, 19))) break;   // D_h complete: the buffer of S W^T is free
+                    x_d[half * 128 + row] = dsum;
+                }
+                x_l[half * 128 + row] = l_run;
+                if (!(ok = exchange(1, 12))) break;
+                l_run = x_l[row] + x_l[128 + row];
+                const float inv = 1.f / l_run, inv_den = HIST ? 1.f / (p.eps + (x_d[row] + x_d[128 + row])) : 0.f;
+                if (half == 0 && row < nq && p.lse) p.lse[(size_t)bh * p.Tc + q0 + row] = (m_used + log2f(l_run)) * 0.6931471805599453f;
+                const uint32_t tl = t - 1;                      // the unit's last tile
+                if (!(ok = wait_s(bar_pv + 8 * (tl & 1), tl >> 1, 10))) break;
+                fence_after_sync();
+                if (!(l_run < 1e30f)) note_redo(n);
+                write_output(n, q0, lane_base + (tl & 1) * 128, inv, inv_den, bw);
+                u += gridDim.x; bh += dbh; i += di;
+                if (i >= p.upb) { i -= p.upb; ++bh; }
+            }
         }
     }
     if (warp < C::NSW && lane == 0) bulk_wait_read();    // output tiles still on their way out of shared memory

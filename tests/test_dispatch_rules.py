@@ -16,6 +16,7 @@ extern "C" int by_kernel(int context, int current, int given, int aligned, int d
 }
 extern "C" int kpl(int Tn) { return select_kpl(Tn); }
 extern "C" int uses(int kpl, int n_b, int max_Tn) { return select_uses(kpl, n_b, max_Tn); }
+extern "C" int teams(int d, int block, int tiles, int history) { return swa_teams(d, block, tiles, history != 0); }
 """
 
 
@@ -80,3 +81,15 @@ def test_a_context_touches_the_selection_kernels_of_its_windows_only(rules):
             touched = {k for k in (4, 8, 16, 32) if rules.uses(k, n_b, n_b * chunks)}
             assert launched <= touched and all(min(launched) <= k <= max(launched) for k in touched)
             assert all(32 * rules.kpl(n_b * x) >= n_b * x for x in range(1, chunks + 1))
+
+
+def test_softmax_teams(rules):
+    """Teams at head dim 64; at 128 for long lists of 128-token blocks, shorter ones without the history term (a context loads both kernels
+    of the lists between, so that the rule must grow with the tiles and shrink with the history term)."""
+    for tiles in range(1, 1025):
+        for block in (16, 64, 128):
+            assert rules.teams(64, block, tiles, 0) and rules.teams(64, block, tiles, 1)
+            for history in (0, 1):
+                t = rules.teams(128, block, tiles, history)
+                assert t == (block == 128 and tiles >= (14 if history else 8))
+                assert rules.teams(128, block, tiles + 1, history) >= t >= rules.teams(128, block, tiles, 1)
