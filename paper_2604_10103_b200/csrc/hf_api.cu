@@ -225,9 +225,10 @@ void free_all(hf_ctx* c) {
 
 template <int D, int BLK, bool TEAMED>
 hf_status set_swa_tc5_attr() {
-    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 0, TEAMED>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D, TEAMED>::SMEM_BYTES));
-    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 1, TEAMED>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D, TEAMED>::SMEM_BYTES));
-    HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, 2, TEAMED>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D, TEAMED>::SMEM_BYTES));
+#define HF_TC5_ATTR(HIST_, AHEAD_) HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, HIST_, TEAMED, AHEAD_>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D, TEAMED>::SMEM_BYTES))
+    HF_TC5_ATTR(0, false); HF_TC5_ATTR(1, false); HF_TC5_ATTR(2, false);
+    if (!TEAMED) { HF_TC5_ATTR(1, !TEAMED); HF_TC5_ATTR(2, !TEAMED); }
+#undef HF_TC5_ATTR
     return HF_OK;
 }
 template <int BLK, int D>
@@ -267,6 +268,13 @@ inline int union_tiles_max(const hf_ctx* c, int keep, int Tn) {
     return (uni + G - 1) / G;
 }
 
+inline bool pools_and_selects(const hf_ctx* c);
+// Thread blocks of a forward call's last kernel before the attention kernel.
+inline int select_blocks(const hf_ctx* c) {
+    if (pools_and_selects(c)) return c->cfg.block == 16 ? c->BH : c->Tm * c->BH;
+    const int R = c->cfg.block == 16 ? 8 : 4;
+    return (c->Tm + R - 1) / R * c->BH;
+}
 inline bool pools_and_selects(const hf_ctx* c) {
     return !c->has_trope && pool_select_one_launch(c->cfg.block, c->d, c->Tm, c->BH, c->pool_clusters, c->pool_clusters16);
 }
@@ -682,9 +690,16 @@ hf_status launch_swa_tc5_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16* 
     const CUtensorMap& rv = c->R + c->n_sink_max > 0 ? L.tm_vring : tv;
     const int grid = p.n_units < c->sm_count ? p.n_units : c->sm_count;
     PdlLaunch pl(dim3(grid), dim3(C::THREADS), C::SMEM_BYTES, st, overlap_prev);
-    if (hist_inside && c->has_rope_q) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 2, TEAMED>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
-    else if (hist_inside) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 1, TEAMED>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
-    else HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, 0, TEAMED>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p));
+#define HF_TC5_LAUNCH(HIST_, AHEAD_) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, HIST_, TEAMED, AHEAD_>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p))
+    // Ahead: q, the folded state and z are older than the kernel before this one (the selection, whose pooling kernel lets it in behind its own
+    // wait; k_union_tiles likewise), but not the rotated copy of q that the pooling kernel itself writes.
+    if (!hist_inside) HF_TC5_LAUNCH(0, false);
+    else if (!TEAMED && !c->has_trope && swa_history_ahead(BLK, p.n_units, select_blocks(c), c->sm_count)) {
+        if (c->has_rope_q) HF_TC5_LAUNCH(2, !TEAMED);
+        else HF_TC5_LAUNCH(1, !TEAMED);
+    } else if (c->has_rope_q) HF_TC5_LAUNCH(2, false);
+    else HF_TC5_LAUNCH(1, false);
+#undef HF_TC5_LAUNCH
     return post_launch(c, "k_swa_tc5");
 }
 

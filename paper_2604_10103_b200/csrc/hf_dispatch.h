@@ -47,3 +47,13 @@ inline bool select_uses(int kpl, int n_b, int max_Tn) { return select_kpl(n_b) <
 //   448 units, 10 tiles 67.1 / 69.3, 12 tiles 73.9 / 75.4, 14 tiles 81.0 / 80.9, 24 tiles 119.9 / 114.8  (8 tiles 44.6 / 41.0, 4 tiles 29.7 / 29.0)
 // and column groups for its blocks of 16 and 64 tokens (0.90 to 0.98 times as fast with teams).
 inline bool swa_teams(int d, int block, int tiles, bool history) { return d == 64 || (block == 128 && tiles >= (history ? 14 : 8)); }
+
+// Whether the attention kernel's column groups form their first unit's history term ahead of the selection's end.  It is for nothing where the
+// thread block is resident early, which takes an SM that the selection leaves free, and on the chain in front of the first tile where it is not;
+// with several units a thread block the one makes up for the other.  Forward calls, heads of 128, behind / ahead, us: 128-token blocks, 12 units
+// (12 selection blocks) of 1, 3, 8 tiles 10.8 / 10.0, 12.6 / 11.6, 16.6 / 15.6; 132 units (36) 14.5 / 15.1, 16.3 / 16.9, 20.5 / 21.1; 320 units
+// 28.3 / 27.9, 34.0 / 33.6, 47.9 / 47.6.  64-token blocks, whose selection also merges the lists: 12 units 14.4 / 13.4, 132 units of
+// 2, 10, 25 kept blocks 18.7 / 17.9, 23.0 / 22.1, 31.5 / 31.1, 320 units 34.0 / 33.5, 49.7 / 49.4.
+inline bool swa_history_ahead(int block, int units, int selection_blocks, int sms) {
+    return block == 64 || units > sms || units + selection_blocks <= sms;
+}

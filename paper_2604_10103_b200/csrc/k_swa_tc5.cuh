@@ -42,6 +42,11 @@
 // for short lists (swa_teams, hf_dispatch.h) and for blocks of 16 and 64 tokens (their masked segments leave the tensor pipe the bound:
 // 64-token blocks, 12 heads, 4 680 queries 158 / 163 us, 16-token blocks 43 / 44).
 //
+// The first unit ahead.  A thread block waits for the lists for 2 us and more after it is resident (launched under the selection's tail), and q, the folded
+// state and z are there all the while.  Column groups form their first unit's history term in that time (form_ahead; AHEAD): the chain behind
+// the unit's last tile is shorter by phi(Q) and the products.  Where this pays: swa_history_ahead (hf_dispatch.h); 16 forwards of 8 heads of 128, 300 queries and
+// their commit 242.6 -> 228.5 us.  With teams the same code cost the tile loop more registers than it had (132 units of 40 tiles 44.9 -> 47.2 us): not there.
+//
 // What bounds it, and why it is cut this way (measured with clock stamps and with a loop of the same products alone, 148
 // CTAs, head dim 128, per 128 x 128 tile; 1 024 clk is the tensor pipe's own time):
 //   - one warp issuing both products: every barrier test in its loop is ~70-90 clk in which the pipe runs dry (1 170 clk per
@@ -97,6 +102,9 @@ struct SwaTc5 {
     static constexpr int OFF_Q = 0, OFF_K = TILE_BYTES, OFF_V = OFF_K + KV * TILE_BYTES;
     static constexpr int OFF_H = OFF_V + KV * TILE_BYTES;       // S W^T, hi then lo; also the staging tile of the output (teams without a history term: one each)
     static constexpr int END_H = OFF_H + (H_BYTES > TILE_BYTES ? 2 * H_BYTES : 2 * TILE_BYTES);
+    // D_h of a thread block's first unit, formed ahead of the tiles (column groups), in place of S W^T: fp32 [OCOLS][32 rows] for each warp
+    static constexpr int DH_WARP = OCOLS * 32 * 4;
+    static_assert(TEAMED || OFF_H + 8 * DH_WARP <= END_H, "buffers of the history term");
     // (the second pass keeps its fp32 history tile behind the operand tiles of swa_mma_unit, in front of the barriers)
     static constexpr int END_REDO = SwaMma<128, D>::SMEM_BYTES + 128 * D * 4;
     static constexpr int OFF_BAR = END_H > END_REDO ? END_H : END_REDO;
@@ -286,7 +294,9 @@ __device__ __forceinline__ float swa_max(const uint32_t* r, int nv) {
 // Persistent: CTA c processes units c, c + gridDim.x, ...
 // HIST 1: the history term is formed here; 2: with its numerator rotated (code of its own: as a branch it cost the plain one
 // 2 % of the call); 0: p.hist, if any, is added.
-template <int D, int BLK, int HIST, bool TEAMED>
+// AHEAD (column groups with a history term): the first unit's is formed ahead of the wait for the kernel before this one; q has to be older than that
+// one (code of its own: as a branch it cost the other calls 2 %).
+template <int D, int BLK, int HIST, bool TEAMED, bool AHEAD>
 __global__ void __launch_bounds__(SwaTc5<D, TEAMED>::THREADS, 1)
 k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kring,
           const __grid_constant__ CUtensorMap tm_vring, const __grid_constant__ CUtensorMap tm_kcur,
@@ -329,6 +339,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
     // unit n: O, D_h and the other team's sums read by the epilogue (two barriers, completion n >> 1: a head-dim-64 unit of one tile may be
     // through before the next one's first S asks for the unit in front of it)
     auto bar_dr = [&](int n) -> uint32_t { return bar0 + ((n & 1) ? (C::KV > 2 ? 496 : 368) : 176); };
+    const uint32_t bar_d0 = bar0 + (C::KV > 2 ? 504 : 376);     // the first unit's D_h, formed ahead, has been read from O's columns
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_gen + C::OFF_BAR + 360);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(s_gen + C::OFF_BAR + 364);
     int* redo_cnt = reinterpret_cast<int*>(s_gen + C::OFF_REDO);
@@ -356,11 +367,15 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             mbar_init(bar_h + 8 * s, 1); mbar_init(bar_y + 8 * s, 2);
         }
         mbar_init(bar_qf, 1); mbar_init(bar_qe, HIST && !TEAMED ? 9 : 1); mbar_init(bar_hf, 1); mbar_init(bar_he, 8);
-        mbar_init(bar_af, 8); mbar_init(bar_ud, 1); mbar_init(bar_dr(0), 8); mbar_init(bar_dr(1), 8);
+        mbar_init(bar_af, 8); mbar_init(bar_ud, 1); mbar_init(bar_dr(0), 8); mbar_init(bar_dr(1), 8); mbar_init(bar_d0, 8);
         *abort_flag = 0;
         *redo_cnt = 0; *redo_last = -1;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
+    static_assert(!AHEAD || (HIST && !TEAMED), "column groups form a history term ahead");
+    constexpr bool early = AHEAD;
+    float* x_den = reinterpret_cast<float*>(s_gen + C::OFF_XL) + 128;      // ... its denominators [128]
+    if (early && threadIdx.x < 128) x_den[threadIdx.x] = 0.f;
     if (warp == C::WARP_S) {
         tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS);
         tmem_relinquish();
@@ -375,13 +390,8 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
     __syncthreads();
     fence_after_sync();
     const uint32_t tmem = *tmem_slot;
-    // Everything above (barriers, tensor memory) may overlap the tail of the kernel before this one in the stream when the
-    // launch allows it; the lists it wrote are read from here on.
-    pdl_wait();
-    // The next kernel in the stream may be made resident on SMs this grid has left (it waits itself) -- only where a thread
-    // block of this kernel takes all of an SM's shared memory, so that no waiting block of the dependent grid ever sits
-    // beside a working block of this one.
-    if (C::SMEM_BYTES > 200 * 1024) pdl_trigger();
+    // Everything above (barriers, tensor memory), and the first unit's history term, may overlap the tail of the kernel before this one in
+    // the stream when the launch allows it: every role waits for that kernel itself, before it reads the lists that one wrote.
 
     auto wait_w = [&](uint32_t bar, uint32_t parity, int where) -> bool {      // a warp's wait, warp-uniform result
         return mbar_wait_warp<true>(bar, parity & 1u, abort_flag, p.dev_status, where);
@@ -393,6 +403,18 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         // their list entries' loads between them, they bounded the tile loop: 16-token blocks, 12 heads, 1 300 queries, 62 of 246 blocks
         // kept 53 -> 32.5 us at head dim 64, 69 -> 41 at 128).  The loops are the warp's.
         const bool is_k = (warp == C::WARP_LOAD_K);
+        auto load_h = [&](int bh) {                             // folded state and z of a head
+            if (lane == 0) {
+                mbar_expect_tx(bar_hf, 2 * C::H_BYTES + D * 4);
+#pragma unroll
+                for (int s = 0; s < C::SUB; ++s) {
+                    tma_load_4d(sH + s * C::HSUB_BYTES, &tm_sh, s * 64, 0, bh, 0, bar_hf);
+                    tma_load_4d(sH + C::H_BYTES + s * C::HSUB_BYTES, &tm_sl, s * 64, 0, bh, 0, bar_hf);
+                }
+                bulk_load(s_base + C::OFF_Z, p.z + (size_t)bh * D, D * 4, bar_hf);
+            }
+            __syncwarp();
+        };
         const int box = lane < G ? lane : 0;
         bool ok = true;
         int t = 0;
@@ -411,12 +433,18 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             }
             __syncwarp();
         };
+        if (!is_k && early) { load_q(0); load_h(blockIdx.x / p.upb); }
+        pdl_wait();
+        // The next kernel in the stream may be made resident on SMs this grid has left (it waits itself) -- only where a thread
+        // block of this kernel takes all of an SM's shared memory, so that no waiting block of the dependent grid ever sits
+        // beside a working block of this one.
+        if (is_k && C::SMEM_BYTES > 200 * 1024) pdl_trigger();
         uint32_t e_next = my_units > 0 ? __ldg(list_of(blockIdx.x)) : 0u;      // list entry, read one tile ahead
         for (int n = 0; ok && n < my_units; ++n) {
             const int u = blockIdx.x + n * gridDim.x;
             const int bh = u / p.upb;
             const int cnt = tiles_of(n);
-            if (!is_k && n == 0) load_q(0);
+            if (!is_k && n == 0 && !early) load_q(0);
            const uint32_t* list = list_of(u);
             for (int j = 0; j < cnt; ++j, ++t) {
                 const uint32_t st = t & (C::KV - 1), dst = tiles + st * C::TILE_BYTES + box * BLK * 128, bar = full + 8 * st;
@@ -442,21 +470,12 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                     for (int s = 0; s < C::SUB; ++s) tma_load_4d(dst + s * C::SUB_BYTES, m, s * 64, jb * BLK, bh, slot, bar);
                 }
                 __syncwarp();
-                if (HIST && !is_k && j == (cnt >= C::KV ? C::KV - 1 : cnt - 1)) {
+                if (HIST && !is_k && !(early && n == 0) && j == (cnt >= C::KV ? C::KV - 1 : cnt - 1)) {
                     // For the history term at the unit's end: the head's folded state and z.  The buffer is free once the
                     // previous unit's output, which was staged in it, has been read by the bulk stores.  (Two V tiles of
                     // this unit are on their way by now; the third needs P V of the first, which comes after that.)
                     if (n >= 1 && !(ok = wait_w(bar_he, n - 1, 13))) break;
-                    if (lane == 0) {
-                        mbar_expect_tx(bar_hf, 2 * C::H_BYTES + D * 4);
-#pragma unroll
-                        for (int s = 0; s < C::SUB; ++s) {
-                            tma_load_4d(sH + s * C::HSUB_BYTES, &tm_sh, s * 64, 0, bh, 0, bar_hf);
-                            tma_load_4d(sH + C::H_BYTES + s * C::HSUB_BYTES, &tm_sl, s * 64, 0, bh, 0, bar_hf);
-                        }
-                        bulk_load(s_base + C::OFF_Z, p.z + (size_t)bh * D, D * 4, bar_hf);
-                    }
-                    __syncwarp();
+                    load_h(bh);
                 }
                 // The next unit's Q, once this unit's is in tensor memory
                 if (!is_k && n + 1 < my_units && j == (cnt > C::KV && !(HIST && !TEAMED) ? C::KV : cnt - 1)) {
@@ -479,6 +498,18 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         const uint32_t q_lo = (uint32_t)dq0, k_lo = (uint32_t)dk0, k_hi = (uint32_t)(dk0 >> 32);
         bool ok = true;
         int x = 0, cnt_prev = 0;
+        auto copy_q = [&] {                                 // the unit's Q from shared to tensor memory
+            fence_after_sync();
+            if (elect_one()) {
+#pragma unroll
+                for (int ks = 0; ks < D / 16; ++ks)         // 16 features = 32 bytes of a row = 8 columns
+                    tmem_cp_128x256b(tmem + C::COL_Q + 8 * ks, dq0 + (uint64_t)((ks >> 2) * (C::SUB_BYTES >> 4) + (ks & 3) * 2));
+                mma_commit(bar_qe);
+            }
+            __syncwarp();
+        };
+        if (early && (ok = wait_w(bar_qf, 0, 4))) copy_q();
+        pdl_wait();
         for (int n = 0; ok && n < my_units; ++n) {
             const int cnt = tiles_of(n);
             for (int j = 0; j < cnt; ++j, ++x) {
@@ -486,32 +517,26 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                 if (j == 0 && !(ok = wait_w(bar_qf, n, 4))) break;
                 if (!(ok = wait_w(bar_kf + 8 * kv, x >> C::KV_LOG, 5))) break;
                 // The S buffer: free once the softmax warps hold S of two tiles ago in registers.  HIST: the buffer of a unit's last tile holds
-                // its D_h afterwards, and (head dim 128) the other one its phi(Q) operand.
+                // its D_h afterwards, and (head dim 128) the other one its phi(Q) operand; the first unit's, formed ahead, was in the second buffer.
                 if (HIST && n >= 1 && j == 1) { if (!(ok = wait_w(bar_dr(n - 1), (n - 1) >> 1, 30))) break; }
-                else if (HIST && !C::A_IN_P && n >= 1 && j == 0) { if (!(ok = wait_w(bar_ud, n - 1, 23))) break; }
+                else if (HIST && !C::A_IN_P && n >= 1 && j == 0 && !(early && n == 1)) { if (!(ok = wait_w(bar_ud, n - 1, 23))) break; }
                 else if (HIST && C::A_IN_P && n >= 2 && j == 0 && cnt_prev == 1) { if (!(ok = wait_w(bar_dr(n - 2), (n - 2) >> 1, 35))) break; }
                 else if (x >= 2) { if (!(ok = wait_w(bar_se + 8 * st, (x >> 1) - 1, 25))) break; }
+                else if (early && x == 1) { if (!(ok = wait_w(bar_ud, 0, 40))) break; }
                 fence_after_sync();
                 if (elect_one()) {
-                    // a unit's first product takes Q from shared memory, the others from tensor memory
-                    if (j == 0) mma_ss_tile<D>(tmem + st * 128, q_lo, k_lo + kv * TILE_STEP, k_hi, IDESC_S);
+                    // a unit's first product takes Q from shared memory (unless it is in tensor memory already), the others from tensor memory
+                    if (j == 0 && !(early && n == 0)) mma_ss_tile<D>(tmem + st * 128, q_lo, k_lo + kv * TILE_STEP, k_hi, IDESC_S);
                     else mma_ts_kmajor<D>(tmem + st * 128, tmem + C::COL_Q, k_lo + kv * TILE_STEP, k_hi, IDESC_S);
                     mma_commit(bar_sf + 8 * st);
                     if (C::KV > 2) mma_commit(bar_ke + 8 * kv);
                 }
                 __syncwarp();
-                if (j == 0) {
+                if (j == 0 && !(early && n == 0)) {
                     // Q moves to tensor memory once the previous unit's last product, and its phi pass, have read what is there
                     if (n >= 1 && !(ok = wait_w(bar_sf + 8 * ((x - 1) & 1), (x - 1) >> 1, 22))) break;
                     if (HIST && C::A_IN_P && n >= 1 && !(ok = wait_w(bar_af, n - 1, 36))) break;
-                    fence_after_sync();
-                    if (elect_one()) {
-#pragma unroll
-                        for (int ks = 0; ks < D / 16; ++ks)      // 16 features = 32 bytes of a row = 8 columns
-                            tmem_cp_128x256b(tmem + C::COL_Q + 8 * ks, dq0 + (uint64_t)((ks >> 2) * (C::SUB_BYTES >> 4) + (ks & 3) * 2));
-                        mma_commit(bar_qe);
-                    }
-                    __syncwarp();
+                    copy_q();
                 }
             }
             cnt_prev = cnt;
@@ -531,35 +556,40 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         const uint64_t dv0 = smem_desc_sw128(sV, C::SUB_BYTES, 1024);
         const uint64_t dh0 = smem_desc_sw128(sH, C::HSUB_BYTES, 1024);    // S W^T tiles: laid out like a V tile (rows = contraction index)
         const uint32_t v_lo = (uint32_t)dv0, v_hi = (uint32_t)(dv0 >> 32), h_lo = (uint32_t)dh0, h_hi = (uint32_t)(dh0 >> 32);
+        // D_h = phi(Q) S W^T: A in quarters of the features (quarter k at column 32 k, hi half first; in a P buffer all of hi, then all of lo), B = the hi
+        // and lo tiles of S W^T; three products, the lo x lo one is below fp32 resolution
+        auto history = [&](uint32_t tD, uint32_t tA) {
+            fence_after_sync();
+            if (elect_one()) {
+                if constexpr (C::A_IN_P) {
+                    mma_ts_half(tD, tA, h_lo, h_hi, IDESC_PV, false);                  // hi x hi
+                    mma_ts_half(tD, tA + D / 2, h_lo, h_hi, IDESC_PV, true);           // lo x hi
+                    mma_ts_half(tD, tA, h_lo + H_STEP, h_hi, IDESC_PV, true);          // hi x lo
+                } else {
+                    mma_ts_groups<D>(tD, tA, h_lo, h_hi, IDESC_PV, false);
+                    mma_ts_groups<D>(tD, tA + D / 8, h_lo, h_hi, IDESC_PV, true);
+                    mma_ts_groups<D>(tD, tA, h_lo + H_STEP, h_hi, IDESC_PV, true);
+                }
+                mma_commit(bar_ud);
+            }
+            __syncwarp();
+        };
         bool ok = true;
         int t = 0;
+        if (early && (ok = wait_w(bar_hf, 0, 14) && wait_w(bar_af, 0, 15)))
+            history(tO, tmem + 128);
+        pdl_wait();
         for (int n = 0; ok && n < my_units; ++n) {
             const int cnt = tiles_of(n);
             for (int j = 0; j < cnt; ++j, ++t) {
                 const uint32_t st = t & 1, kv = t & (C::KV - 1);
-                if (HIST && j == cnt - 1) {
-                    // D_h = phi(Q) S W^T while the softmax warps work on the unit's last tile: into that tile's S buffer (already
-                    // in registers), A from the other S buffer (quarter k of the features: hi half at column 32 k, lo half D / 8 on),
-                    // B = the hi and lo tiles of S W^T; three products, the lo x lo one is below fp32 resolution
-                    if (!(ok = wait_w(bar_hf, n, 14))) break;
-                    if (!(ok = wait_w(bar_af, n, 15))) break;
-                    if (!(ok = wait_w(bar_se + 8 * st, t >> 1, 26))) break;
-                    fence_after_sync();
-                    const uint32_t tD = tmem + st * 128, tA = C::A_IN_P ? tmem + C::COL_P + 64 * (st ^ 1u) : tmem + (st ^ 1u) * 128;
-                    if (elect_one()) {
-                        if constexpr (C::A_IN_P) {
-                            mma_ts_half(tD, tA, h_lo, h_hi, IDESC_PV, false);                  // hi x hi
-                            mma_ts_half(tD, tA + D / 2, h_lo, h_hi, IDESC_PV, true);           // lo x hi
-                            mma_ts_half(tD, tA, h_lo + H_STEP, h_hi, IDESC_PV, true);          // hi x lo
-                        } else {
-                            mma_ts_groups<D>(tD, tA, h_lo, h_hi, IDESC_PV, false);
-                            mma_ts_groups<D>(tD, tA + D / 8, h_lo, h_hi, IDESC_PV, true);
-                            mma_ts_groups<D>(tD, tA, h_lo + H_STEP, h_hi, IDESC_PV, true);
-                        }
-                        mma_commit(bar_ud);
-                    }
-                    __syncwarp();
+                // while the softmax warps work on the unit's last tile: into that tile's S buffer (already in registers), A from the other
+                if (HIST && j == cnt - 1 && !(early && n == 0)) {
+                    ok = wait_w(bar_hf, n, 14) && wait_w(bar_af, n, 15) && wait_w(bar_se + 8 * st, t >> 1, 26);
+                    if (!ok) break;
+                    history(tmem + st * 128, C::A_IN_P ? tmem + C::COL_P + 64 * (st ^ 1u) : tmem + (st ^ 1u) * 128);
                 }
+                if (early && t == 0 && !(ok = wait_w(bar_d0, 0, 41))) break;            // O: the first unit's D_h has been read
                 if (TEAMED && n >= 1 && j == 0 && !(ok = wait_w(bar_dr(n - 1), (n - 1) >> 1, 24))) break;     // O: the previous unit's has been read
                 if (!(ok = wait_w(bar_vf + 8 * kv, t >> C::KV_LOG, 7))) break;
                 const uint32_t pb = C::PBUF == 2 ? st : 0u, p_par = C::PBUF == 2 ? t >> 1 : t;
@@ -616,7 +646,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
         // (batch*head, position) of a unit without a division per unit; the tile count and the first list entries of the next
         // unit are read during the current one
         const int dbh = gridDim.x / p.upb, di = gridDim.x - dbh * p.upb;
-        int u = blockIdx.x, bh = u / p.upb, i = u - bh * p.upb, cnt_next = tiles_of(0);
+        int u = blockIdx.x, bh = u / p.upb, i = u - bh * p.upb;
         // BLK 16, 64: list entries of the next tile.  BLK 128: all that matters here is whether a tile is a chunk's short last
         // block; one bit per tile from a ballot over 32 list entries at a time (lane = entry), read one window ahead.  An entry
         // outside [0, T_n) is block 0 here as for the loader, which reports it.
@@ -641,7 +671,6 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             if constexpr (BLK == 128) { if (ragged && lane < p.keep) e_next[0] = __ldg(entries_of(unit) + lane); }
             else if (pj < cnt) read_entries(entries_of(unit) + pj * G);
         };
-        if (my_units > 0) first_entries(u, team, cnt_next);
         bool staged = false;                                // this warp's last output is on its way out of shared memory
         // The previous unit's output was staged where S W^T lives: the loader may refill it, and z, once every warp's bulk store has read
         // its part.  (Said after the warp's next tile, when the store has long done so, or before its phi pass.)
@@ -734,12 +763,24 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
 #pragma unroll
             for (int c = 0; c < C::OCOLS / 8; ++c) bw[c] = b ? __ldg(b + c) : make_uint4(0, 0, 0, 0);
         };
-        // Output of unit n, D_h at tD.
+        // Output of unit n, D_h at tD, or in shared memory (first unit, formed ahead).
         auto write_output = [&](int n, int q0, uint32_t tD, float inv, float inv_den, const uint4 (&bw)[C::OCOLS / 8]) {
             // Output through shared memory and one bulk tensor store per warp (32 rows x half of the columns): row-per-thread global stores
             // would touch 32 lines per instruction.  The staging tile is the S W^T buffer (free: the history products have completed;
             // where there are none each team has its own), in the map's swizzle of the row width.
-            const uint32_t stage_off = C::OFF_H + (HIST ? 0 : team * C::TILE_BYTES) + (half * 4 + wq) * (32 * C::OCOLS * 2);
+            const bool ahead = early && n == 0;
+            // (D_h in shared memory: 8 KB a warp, the staging tile in front of it)
+            const uint32_t dh_off = C::OFF_H + warp * C::DH_WARP;
+            const uint32_t stage_off = ahead ? dh_off : C::OFF_H + (HIST ? 0 : team * C::TILE_BYTES) + (half * 4 + wq) * (32 * C::OCOLS * 2);
+            const float* dh_s = reinterpret_cast<const float*>(s_gen + dh_off) + lane;
+            uint32_t dh0[TEAMED ? 1 : 32];                  // D_h where the staging tile goes
+            if constexpr (HIST != 0 && !TEAMED) {
+                if (ahead) {
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) dh0[e] = __float_as_uint(dh_s[e * 32]);
+                    __syncwarp();
+                }
+            }
             uint8_t* stage = s_gen + stage_off + lane * (C::OCOLS * 2);
             const int swz = C::OCOLS == 64 ? lane & 7 : (lane >> 1) & 3;
             if (!HIST && staged) {
@@ -750,7 +791,12 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             for (int c = 0; c < C::OCOLS / 16; ++c) {
                 uint32_t o[16], dh[16];
                 tmem_ld16(lane_base + C::COL_O + half * C::OCOLS + c * 16, o);
-                if constexpr (HIST != 0) tmem_ld16(tD + half * C::OCOLS + c * 16, dh);
+                if constexpr (HIST != 0) {
+                    if (ahead) {
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) dh[e] = c < 2 ? dh0[(16 * c + e) % (TEAMED ? 1 : 32)] : __float_as_uint(dh_s[(16 * c + e) * 32]);
+                    } else tmem_ld16(tD + half * C::OCOLS + c * 16, dh);
+                }
                 tmem_wait_ld();
                 if (c == C::OCOLS / 16 - 1) {
                     fence_before_sync();
@@ -790,6 +836,33 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
             }
             staged = true;
         };
+        // The first unit's history term ahead of its tiles, and ahead of the wait for the kernel before this one (q, the folded state, z and
+        // the bias are older than that one): phi(Q), its products into O's columns, D_h from there to shared memory, the denominators
+        // to x_den (the groups' shares added to zero: the same sum in either order).  A thread block of a small grid is resident 2 us and more before
+        // the lists are there, and the chain behind its unit's last tile is shorter by phi and the products (3 000-4 000 clk).
+        auto form_ahead = [&]() -> bool {
+            float ds;
+            if (!form_phi(0, i * 128, lane_base + 128, ds)) return false;
+            atomicAdd(x_den + row, ds);
+            if (!wait_s(bar_ud, 0, 42)) return false;
+            fence_after_sync();
+            float* dh = reinterpret_cast<float*>(s_gen + C::OFF_H + warp * C::DH_WARP) + lane;
+#pragma unroll
+            for (int c = 0; c < C::OCOLS / 16; ++c) {
+                uint32_t o[16];
+                tmem_ld16(lane_base + C::COL_O + half * C::OCOLS + c * 16, o);
+                tmem_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 16; ++e) dh[(c * 16 + e) * 32] = __uint_as_float(o[e]);
+            }
+            fence_before_sync();
+            arrive_w(bar_d0);
+            return true;
+        };
+        if (early) ok = form_ahead();
+        pdl_wait();
+        int cnt_next = tiles_of(0);
+        if (my_units > 0) first_entries(u, team, cnt_next);
         if constexpr (TEAMED) {
             float* x_l = reinterpret_cast<float*>(s_gen + C::OFF_XL);
             float* x_d = x_l + 128;
@@ -953,7 +1026,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                 if (i >= p.upb) { i -= p.upb; ++bh; }
             }
         } else {
-            // ---- column groups    : all warps on the same tile
+            // ---- column groups: all warps on the same tile
             static_assert(TEAMED || C::PBUF == 1, "one P buffer");
             // Exchange number e of the kernel between partner warps: what a caller wrote to shared memory before is visible to the
             // others after.  Two per unit (maxima, then sums): a buffer written at one is read by the partners before they arrive
@@ -983,7 +1056,7 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                         for (int x = 0; x < EPT; ++x) e_cur[x] = e_next[x];
                         if (j + 1 < cnt) read_entries(ent + (j + 1) * G);
                     }
-                    if (HIST && j == cnt - 1) {
+                    if (HIST && j == cnt - 1 && !(early && n == 0)) {
                         // history term's operand into the other S buffer: this thread's own S columns of it, which it has read (last tile's share),
                         // or its columns of the last unit's D_h
                         if (!(ok = form_phi(n, q0, lane_base + (st ^ 1u) * 128, dsum))) break;
@@ -1088,14 +1161,18 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                 // ---- end of the unit: row sums (and the shares of Eq. 4's denominator) of the column groups, range test, output
                 uint4 bw[C::OCOLS / 8];
                 read_bias(bw);
-                if constexpr (HIST != 0) {
+                // (first unit, history term formed ahead: D_h is where the sums go otherwise)
+                const bool ahead = early && n == 0;
+                float* l0 = ahead ? x_den - 128 : x_l;
+                float* l1 = ahead ? reinterpret_cast<float*>(s_gen + C::OFF_Z) : x_l + 128;
+                if (HIST && !ahead) {
                     if (!(ok = wait_s(bar_ud, n, 19))) break;   // D_h complete: the buffer of S W^T is free
                     x_d[half * 128 + row] = dsum;
                 }
-                x_l[half * 128 + row] = l_run;
+                (half ? l1 : l0)[row] = l_run;
                 if (!(ok = exchange(1, 12))) break;
-                l_run = x_l[row] + x_l[128 + row];
-                const float inv = 1.f / l_run, inv_den = HIST ? 1.f / (p.eps + (x_d[row] + x_d[128 + row])) : 0.f;
+                l_run = l0[row] + l1[row];
+                const float inv = 1.f / l_run, inv_den = HIST ? 1.f / (p.eps + (ahead ? x_den[row] : x_d[row] + x_d[128 + row])) : 0.f;
                 if (half == 0 && row < nq && p.lse) p.lse[(size_t)bh * p.Tc + q0 + row] = (m_used + log2f(l_run)) * 0.6931471805599453f;
                 const uint32_t tl = t - 1;                      // the unit's last tile
                 if (!(ok = wait_s(bar_pv + 8 * (tl & 1), tl >> 1, 10))) break;

@@ -16,6 +16,7 @@ extern "C" int by_kernel(int context, int current, int given, int aligned, int d
 }
 extern "C" int kpl(int Tn) { return select_kpl(Tn); }
 extern "C" int uses(int kpl, int n_b, int max_Tn) { return select_uses(kpl, n_b, max_Tn); }
+extern "C" int ahead(int block, int units, int selection_blocks, int sms) { return swa_history_ahead(block, units, selection_blocks, sms); }
 extern "C" int teams(int d, int block, int tiles, int history) { return swa_teams(d, block, tiles, history != 0); }
 """
 
@@ -93,3 +94,11 @@ def test_softmax_teams(rules):
                 t = rules.teams(128, block, tiles, history)
                 assert t == (block == 128 and tiles >= (14 if history else 8))
                 assert rules.teams(128, block, tiles + 1, history) >= t >= rules.teams(128, block, tiles, 1)
+
+
+def test_history_term_ahead_of_the_selections_end(rules):
+    """Where the selection leaves an SM for every thread block, where there are several units for each of them, and with 64-token blocks."""
+    for block in (16, 128):
+        assert rules.ahead(block, 12, 12, 148) and rules.ahead(block, 100, 48, 148) and not rules.ahead(block, 101, 48, 148)
+        assert not rules.ahead(block, 148, 1, 148) and rules.ahead(block, 149, 40, 148)
+    assert rules.ahead(64, 132, 72, 148)
