@@ -236,18 +236,21 @@ hf_status set_swa_attr() {
     HF_CUDA(cudaFuncSetAttribute(k_swa_mma<BLK, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaMma<BLK, D>::SMEM_BYTES));
     return HF_OK;
 }
-template <int D, int G, int KPL>
+template <int D, int G, int KPL, int R>
 hf_status set_select_attr_kpl(const hf_ctx* c) {
-    if (!select_uses(KPL, c->n_b, c->max_Tn)) return HF_OK;
-    HF_CUDA(cudaFuncSetAttribute(k_select<D, KPL, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G, KPL>::smem_bytes(32 * KPL)));
+    if (!select_uses(KPL, c->n_b, c->max_Tn) || select_rows(KPL, G, c->Tm, c->BH, c->sm_count) != R) return HF_OK;
+    HF_CUDA(cudaFuncSetAttribute(k_select<D, KPL, G, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G, KPL, R>::smem_bytes(32 * KPL)));
     return HF_OK;
 }
 template <int D, int G>
 hf_status set_select_attr(const hf_ctx* c) {
-    HF_TRY((set_select_attr_kpl<D, G, 4>(c)));
-    HF_TRY((set_select_attr_kpl<D, G, 8>(c)));
-    HF_TRY((set_select_attr_kpl<D, G, 16>(c)));
-    return set_select_attr_kpl<D, G, 32>(c);
+    if constexpr (G != 8) {
+        HF_TRY((set_select_attr_kpl<D, G, 4, 4>(c)));
+        HF_TRY((set_select_attr_kpl<D, G, 8, 4>(c)));
+    } else HF_TRY((set_select_attr_kpl<D, G, 4, 8>(c)));
+    HF_TRY((set_select_attr_kpl<D, G, 8, 8>(c)));
+    HF_TRY((set_select_attr_kpl<D, G, 16, 8>(c)));
+    return set_select_attr_kpl<D, G, 32, 8>(c);
 }
 template <int D>
 hf_status set_state_attr() {
@@ -270,9 +273,9 @@ inline int union_tiles_max(const hf_ctx* c, int keep, int Tn) {
 
 inline bool pools_and_selects(const hf_ctx* c);
 // Thread blocks of a forward call's last kernel before the attention kernel.
-inline int select_blocks(const hf_ctx* c) {
+inline int select_blocks(const hf_ctx* c, int Tn) {
     if (pools_and_selects(c)) return c->cfg.block == 16 ? c->BH : c->Tm * c->BH;
-    const int R = c->cfg.block == 16 ? 8 : 4;
+    const int R = select_rows(select_kpl(Tn), c->cfg.block == 128 ? 1 : 128 / c->cfg.block, c->Tm, c->BH, c->sm_count);
     return (c->Tm + R - 1) / R * c->BH;
 }
 inline bool pools_and_selects(const hf_ctx* c) {
@@ -587,14 +590,20 @@ ChunkTable make_table(hf_ctx* c, LayerState& L, const bf16* k_cur, const bf16* v
 template <int D, int G>
 cudaError_t launch_select_kernel(hf_ctx* c, const ChunkTable& tab, int Tn, int keep, const SelectOut& o, const UnionOut& lists, cudaStream_t st) {
     // follows the pooling kernel
-#define HF_SELECT(KPL_) do { typedef Select<D, G, KPL_> S; \
+#define HF_SELECT(KPL_, R_) do { typedef Select<D, G, KPL_, R_> S; \
         PdlLaunch pl(dim3((c->Tm + S::R - 1) / S::R, c->BH), dim3(S::THREADS), S::smem_bytes(Tn), st, true); \
-        return cudaLaunchKernelEx(&pl.cfg, k_select<D, KPL_, G>, tab, (const float*)c->pooled_q, c->n_b, c->Tm, Tn, keep, -0.f, o, lists); } while (0)
-    switch (select_kpl(Tn)) {
-        case 4: HF_SELECT(4);
-        case 8: HF_SELECT(8);
-        case 16: HF_SELECT(16);
-        default: HF_SELECT(32);
+        return cudaLaunchKernelEx(&pl.cfg, k_select<D, KPL_, G, R_>, tab, (const float*)c->pooled_q, c->n_b, c->Tm, Tn, keep, -0.f, o, lists); } while (0)
+    const int kpl = select_kpl(Tn);
+    if constexpr (G != 8) {
+        if (select_rows(kpl, G, c->Tm, c->BH, c->sm_count) == 4) {
+            if (kpl == 4) HF_SELECT(4, 4);
+            HF_SELECT(8, 4);
+        }
+    } else if (kpl == 4) HF_SELECT(4, 8);
+    switch (kpl) {
+        case 8: HF_SELECT(8, 8);
+        case 16: HF_SELECT(16, 8);
+        default: HF_SELECT(32, 8);
     }
 #undef HF_SELECT
 }
@@ -694,7 +703,7 @@ hf_status launch_swa_tc5_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16* 
     // Ahead: q, the folded state and z are older than the kernel before this one (the selection, whose pooling kernel lets it in behind its own
     // wait; k_union_tiles likewise), but not the rotated copy of q that the pooling kernel itself writes.
     if (!hist_inside) HF_TC5_LAUNCH(0, false);
-    else if (!TEAMED && !c->has_trope && swa_history_ahead(BLK, p.n_units, select_blocks(c), c->sm_count)) {
+    else if (!TEAMED && !c->has_trope && swa_history_ahead(BLK, p.n_units, select_blocks(c, p.Tn), c->sm_count)) {
         if (c->has_rope_q) HF_TC5_LAUNCH(2, !TEAMED);
         else HF_TC5_LAUNCH(1, !TEAMED);
     } else if (c->has_rope_q) HF_TC5_LAUNCH(2, false);

@@ -40,6 +40,13 @@ inline int select_kpl(int Tn) { return Tn <= 128 ? 4 : Tn <= 256 ? 8 : Tn <= 512
 // Whether a context whose windows have n_b .. max_Tn key blocks ever launches the step's kernel.
 inline bool select_uses(int kpl, int n_b, int max_Tn) { return select_kpl(n_b) <= kpl && kpl <= select_kpl(max_Tn); }
 
+// Query blocks that a thread block of the selection takes: eight where they share a unit's list (G 8: 16-token blocks) and for more than 256 key
+// blocks; with 129 to 256 eight where four would give more thread blocks than SMs, of which only one fits an SM with all key rows.
+inline int select_rows(int kpl, int G, int Tm, int BH, int sms) {
+    if (G == 8 || kpl > 8) return 8;
+    return kpl == 8 && (Tm + 3) / 4 * BH > sms ? 8 : 4;
+}
+
 // Softmax warps of the tcgen05 attention kernel in teams that take turns at the tiles, or in column groups on the same one (k_swa_tc5.cuh).  Head
 // dim 64: teams (1 to 40 tiles, 12 to 320 units: 0.98 to 1.13 times as fast).  Head dim 128, 128-token blocks: teams from 14 tiles on, from
 // 8 without the history term, whose operand they keep in an S buffer; column groups / teams, forward calls (softmax branch alone), us:

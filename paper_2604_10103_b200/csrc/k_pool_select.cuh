@@ -228,8 +228,8 @@ __global__ void __launch_bounds__(256, 6) k_pool_copy_layers(const __grid_consta
 }
 
 // A[i][j] = Mean(q_i) . Mean(k_j) in the canonical order, and the top-K of every row under the total order (score descending,
-// block index ascending): bit mask and ascending index list.  grid (ceil(T_m / 4), B*H), 256 threads: four query blocks of a
-// head per thread block.
+// block index ascending): bit mask and ascending index list.  grid (ceil(T_m / R), B*H), 64 R threads: R = four query
+// blocks of a head per thread block, or eight.
 //
 // Scores: one THREAD per (query block, key block).  The butterfly of the canonical order is a plain tree, so a thread that walks
 // the columns in the order l, l + 16, l + 8, l + 24 (l = 0..3, then 4..7) needs four running values and no shuffle: 2 D - 1
@@ -251,9 +251,14 @@ __global__ void __launch_bounds__(256, 6) k_pool_copy_layers(const __grid_consta
 // with four query blocks and KPL 32, 24.5 like this).  One isolated call, pooling and selection, heads of 128, four / eight query blocks: T_n 296,
 // 48 heads 56.6 / 43.2 us, 12 heads 26.2 / 27.4, 2 heads 18.3 / 20.5; T_n 512, 12 heads 52 / 39.4; T_n 1 024, 1 head 43.2 / 47.0, 12 heads
 // 111 / 107.5.
-template <int D, int G, int KPL>
+// RQ: query blocks per thread block.  Rows of 129 to 256 key blocks (KPL 8) have all their key rows in shared memory at once and four scores per thread,
+// so that a key row is read once for four query blocks (the scores are bound by shared-memory reads) and no pass waits for the next one's rows: from the
+// pooled rows' arrival to the scores, 12 heads of 128, T_n 222 12 100 -> 8 300 clk, heads of 64, T_n 246 7 300 -> 5 300; with the ranking's two bits a step and its
+// words before the stores the forward of 64-token blocks 158 -> 155 us, of 16-token blocks at head dim 64 35.6 -> 33.4, 12 heads of 16-token blocks, T_n 176 45.0 -> 40.5;
+// eight query blocks where four would be more thread blocks than SMs (hf_dispatch.h).
+template <int D, int G, int KPL, int RQ>
 struct Select {
-    static constexpr int R = G == 8 || KPL > 8 ? 8 : 4, KT = 128;        // query blocks per thread block; key rows per pass
+    static constexpr int R = RQ, KT = KPL == 8 ? 256 : 128;       // query blocks per thread block; key rows per pass
     static constexpr int THREADS = 64 * R;
     static constexpr int LD = D + 4;            // floats per key row in shared memory
     static int smem_bytes(int Tn) { const int kt = Tn < KT ? Tn : KT; return (kt * LD + R * D + R * Tn) * (int)sizeof(float); }
@@ -338,6 +343,7 @@ __device__ __forceinline__ uint32_t rank_row(const float* sc, size_t row, int Tn
     int ahead[KPL <= 2 ? KPL : 1];
     uint32_t thr = 0;           // more keys: largest value with at least `keep` images at or above it
     int ties = Tn;              // ... and blocks at the threshold still to be kept, lowest index first
+    bool exact = false;
     if constexpr (KPL <= 2) {
 #pragma unroll
         for (int x = 0; x < KPL; ++x) ahead[x] = 0;
@@ -352,14 +358,22 @@ __device__ __forceinline__ uint32_t rank_row(const float* sc, size_t row, int Tn
             }
         }
     } else {
-        bool exact = keep >= Tn;    // exactly `keep` images at or above the threshold: no ties to cut (all blocks kept: every image counts)
-        for (uint32_t bit = 0x80000000u; bit != 0u && !exact; bit >>= 1) {
-            const uint32_t cand = thr | bit;
-            int n = 0;
+        // Two bits a step, the three counts of a step side by side in one word (T_n <= 512; two words above): a step is a chain, mostly the sum
+        // over the warp (3 300 -> 2 300 clk with 222 key blocks; votes and population counts instead 3 400).
+        exact = keep >= Tn;         // exactly `keep` images at or above the threshold: no ties to cut (all blocks kept: every image counts)
+        for (int sh = 30; sh >= 0 && !exact; sh -= 2) {
+            const uint32_t c1 = thr | (1u << sh), c2 = thr | (2u << sh), c3 = thr | (3u << sh);
+            uint32_t a1[2] = {0, 0}, a2[2] = {0, 0}, a3[2] = {0, 0};
 #pragma unroll
-            for (int x = 0; x < KPL; ++x) n += key[x] >= cand;
+            for (int x = 0; x < KPL; ++x) { a1[x & 1] += key[x] >= c1; a2[x & 1] += key[x] >= c2; a3[x & 1] += key[x] >= c3; }
+            uint32_t n = a1[0] + a1[1] + ((a2[0] + a2[1]) << (KPL < 32 ? 10 : 16)), m = a3[0] + a3[1];
+            if (KPL < 32) n += m << 20;
             n = __reduce_add_sync(0xffffffffu, n);
-            if (n >= keep) { thr = cand; exact = n == keep; }
+            const int n3 = (int)(KPL < 32 ? n >> 20 : __reduce_add_sync(0xffffffffu, m));
+            const int n1 = (int)(n & (KPL < 32 ? 1023u : 65535u)), n2 = (int)(KPL < 32 ? n >> 10 & 1023u : n >> 16);
+            if (n3 >= keep) { thr = c3; exact = n3 == keep; }
+            else if (n2 >= keep) { thr = c2; exact = n2 == keep; }
+            else if (n1 >= keep) { thr = c1; exact = n1 == keep; }
         }
         if (!exact) {
             int n = 0;
@@ -369,29 +383,30 @@ __device__ __forceinline__ uint32_t rank_row(const float* sc, size_t row, int Tn
         }
     }
     const uint32_t below = (1u << lane) - 1u;
-    int pos = 0;
-    uint32_t my_word = 0;
+    uint32_t word[KPL];             // the row's mask
+    if (KPL <= 2 || exact) {
 #pragma unroll
-    for (int x = 0; x < KPL; ++x) {
-        const int j = x * 32 + lane;
-        bool kept;
-        if constexpr (KPL <= 2) {
-            kept = j < Tn && ahead[x] < keep;
-        } else {
-            const uint32_t eq = __ballot_sync(0xffffffffu, j < Tn && key[x] == thr);
-            kept = j < Tn && (key[x] > thr || (key[x] == thr && __popc(eq & below) < ties));
+        for (int x = 0; x < KPL; ++x) word[x] = __ballot_sync(0xffffffffu, x * 32 + lane < Tn && (KPL <= 2 ? ahead[x % (KPL <= 2 ? KPL : 1)] < keep : key[x] >= thr));
+    } else {
+#pragma unroll
+        for (int x = 0; x < KPL; ++x) {
+            const uint32_t eq = __ballot_sync(0xffffffffu, x * 32 + lane < Tn && key[x] == thr);
+            word[x] = __ballot_sync(0xffffffffu, x * 32 + lane < Tn && (key[x] > thr || (key[x] == thr && __popc(eq & below) < ties)));
             ties -= __popc(eq);
         }
-        const uint32_t word = __ballot_sync(0xffffffffu, kept);
-        if (lane == x) my_word = word;
-        if (kept) {
-            const int at = pos + __popc(word & below);
-            if (at < keep) {    // (always true under the total order above; the store never leaves the row)
-                o.idx[row * keep + at] = j;
-                if (o.idx_out) o.idx_out[row * keep + at] = j;
-            }
+    }
+    int pos = 0;
+    uint32_t my_word = 0;
+    int32_t* list = o.idx + row * keep;
+#pragma unroll
+    for (int x = 0; x < KPL; ++x) {
+        if (lane == x) my_word = word[x];
+        const int at = pos + __popc(word[x] & below);
+        if ((word[x] >> lane & 1u) && at < keep) {      // (always true under the total order above; the store never leaves the row)
+            list[at] = x * 32 + lane;
+            if (o.idx_out) o.idx_out[row * keep + at] = x * 32 + lane;
         }
-        pos += __popc(word);
+        pos += __popc(word[x]);
     }
     if (lane < o.mask_words) {
         o.mask[row * o.mask_words + lane] = my_word;
@@ -422,6 +437,18 @@ __device__ __forceinline__ void score_pass(KeyRow key_row, int n, const float* s
         }
     }
 }
+// ... of up to 256 key rows, four scores per thread (64 threads a query row).
+template <int D>
+__device__ __forceinline__ void score_quads(const float* s_k, int ld, int n, const float* s_q, int rows, float* sc, int Tn, float2 nz) {
+    const int j = threadIdx.x & 255, r = (threadIdx.x >> 8) * 4;
+    if (j < n && r < rows) {
+        float v[4];
+        canonical_scores<D, 4>(s_k + j * ld, s_q + r * D, nz, v);      // (rows past T_m: stale shared memory, not stored)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (r + e < rows) sc[(r + e) * Tn + j] = v[e];
+    }
+}
 // The end of a selection: scores out, top-K of every row, and (G > 1, lists.entries set) the merged lists of the units of these rows.
 template <int KPL, int G, int R>
 __device__ __forceinline__ void finish_rows(const float* s_sc, uint32_t (*s_mask)[32], int bh, int i0, int rows, int Tm, int Tn, int n_b, int keep,
@@ -443,10 +470,10 @@ __device__ __forceinline__ void finish_rows(const float* s_sc, uint32_t (*s_mask
     }
 }
 
-template <int D, int KPL, int G>
-__global__ void __launch_bounds__(Select<D, G, KPL>::THREADS) k_select(ChunkTable tab, const float* __restrict__ pooled_q,
+template <int D, int KPL, int G, int RQ>
+__global__ void __launch_bounds__(Select<D, G, KPL, RQ>::THREADS) k_select(ChunkTable tab, const float* __restrict__ pooled_q,
                                                 int n_b, int Tm, int Tn, int keep, float neg_zero, SelectOut o, UnionOut lists) {
-    typedef Select<D, G, KPL> C;
+    typedef Select<D, G, KPL, RQ> C;
     const float2 nz = make_float2(neg_zero, neg_zero);
     extern __shared__ __align__(16) float sel_smem[];
     const int kt = min(Tn, C::KT);
@@ -484,7 +511,8 @@ __global__ void __launch_bounds__(Select<D, G, KPL>::THREADS) k_select(ChunkTabl
         }
         cp_async_wait<0>();
         __syncthreads();
-        score_pass<D, C::R>([&](int j) { return s_k + j * C::LD; }, n, s_q, rows, s_sc + base, Tn, nz);
+        if constexpr (KPL == 8) score_quads<D>(s_k, C::LD, n, s_q, rows, s_sc + base, Tn, nz);
+        else score_pass<D, C::R>([&](int j) { return s_k + j * C::LD; }, n, s_q, rows, s_sc + base, Tn, nz);
     }
     __syncthreads();
     finish_rows<KPL, G, C::R>(s_sc, s_mask, bh, i0, rows, Tm, Tn, n_b, keep, o, lists);

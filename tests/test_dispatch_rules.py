@@ -16,6 +16,7 @@ extern "C" int by_kernel(int context, int current, int given, int aligned, int d
 }
 extern "C" int kpl(int Tn) { return select_kpl(Tn); }
 extern "C" int uses(int kpl, int n_b, int max_Tn) { return select_uses(kpl, n_b, max_Tn); }
+extern "C" int rows(int kpl, int G, int Tm, int BH, int sms) { return select_rows(kpl, G, Tm, BH, sms); }
 extern "C" int ahead(int block, int units, int selection_blocks, int sms) { return swa_history_ahead(block, units, selection_blocks, sms); }
 extern "C" int teams(int d, int block, int tiles, int history) { return swa_teams(d, block, tiles, history != 0); }
 """
@@ -102,3 +103,12 @@ def test_history_term_ahead_of_the_selections_end(rules):
         assert rules.ahead(block, 12, 12, 148) and rules.ahead(block, 100, 48, 148) and not rules.ahead(block, 101, 48, 148)
         assert not rules.ahead(block, 148, 1, 148) and rules.ahead(block, 149, 40, 148)
     assert rules.ahead(64, 132, 72, 148)
+
+
+def test_query_blocks_per_thread_block_of_the_selection(rules):
+    for G in (1, 2, 8):
+        for Tm in (1, 3, 4, 5, 37, 74, 100):
+            for BH in (1, 4, 12, 48):
+                assert rules.rows(4, G, Tm, BH, 148) == (8 if G == 8 else 4)
+                assert rules.rows(16, G, Tm, BH, 148) == rules.rows(32, G, Tm, BH, 148) == 8
+                assert rules.rows(8, G, Tm, BH, 148) == (8 if G == 8 or -(-Tm // 4) * BH > 148 else 4)
