@@ -56,11 +56,14 @@ inline int select_rows(int kpl, int G, int Tm, int BH, int sms) {
 inline bool swa_teams(int d, int block, int tiles, bool history) { return d == 64 || (block == 128 && tiles >= (history ? 14 : 8)); }
 
 // Whether the attention kernel's column groups form their first unit's history term ahead of the selection's end.  It is for nothing where the
-// thread block is resident early, which takes an SM that the selection leaves free, and on the chain in front of the first tile where it is not;
-// with several units a thread block the one makes up for the other.  Forward calls, heads of 128, behind / ahead, us: 128-token blocks, 12 units
-// (12 selection blocks) of 1, 3, 8 tiles 10.8 / 10.0, 12.6 / 11.6, 16.6 / 15.6; 132 units (36) 14.5 / 15.1, 16.3 / 16.9, 20.5 / 21.1; 320 units
-// 28.3 / 27.9, 34.0 / 33.6, 47.9 / 47.6.  64-token blocks, whose selection also merges the lists: 12 units 14.4 / 13.4, 132 units of
-// 2, 10, 25 kept blocks 18.7 / 17.9, 23.0 / 22.1, 31.5 / 31.1, 320 units 34.0 / 33.5, 49.7 / 49.4.
+// thread block is resident early, which takes an SM that the selection leaves free, and on the chain in front of the first tile where it is not.  What
+// counts are the thread blocks of the last round, the first on the device and the last to finish.  Forward calls, heads of 128, behind / ahead, us:
+//   128-token blocks, 12 units (12 selection blocks) of 1, 3, 8 tiles 10.8 / 10.0, 12.6 / 11.6, 16.6 / 15.6; 132 units (36) 14.5 / 15.1, 16.3 / 16.9,
+//   20.5 / 21.1; 320 units, 24 in the last round (80) 29.1 / 27.1, 33.8 / 33.4, 47.0 / 46.6; 444 units, 148 in the last round 30.7 / 31.2, 35.6 / 36.8,
+//   50.1 / 50.5
+//   64-token blocks, 132 units of 2, 8, 20 kept blocks, T_n 84 (72) 18.4 / 17.4, 22.2 / 21.2, 28.3 / 27.5; 444 units 46.4 / 47.2, 62.3 / 63.1, 80.2 / 81.3; 1 776
+//   units, T_n 74 141.6 / 145.5
 inline bool swa_history_ahead(int block, int units, int selection_blocks, int sms) {
-    return block == 64 || units > sms || units + selection_blocks <= sms;
+    const int last = units % sms ? units % sms : sms;
+    return last + selection_blocks <= sms || (block == 64 && units < sms);
 }

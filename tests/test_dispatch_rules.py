@@ -98,11 +98,13 @@ def test_softmax_teams(rules):
 
 
 def test_history_term_ahead_of_the_selections_end(rules):
-    """Where the selection leaves an SM for every thread block, where there are several units for each of them, and with 64-token blocks."""
-    for block in (16, 128):
-        assert rules.ahead(block, 12, 12, 148) and rules.ahead(block, 100, 48, 148) and not rules.ahead(block, 101, 48, 148)
-        assert not rules.ahead(block, 148, 1, 148) and rules.ahead(block, 149, 40, 148)
-    assert rules.ahead(64, 132, 72, 148)
+    """Where the selection leaves an SM for every thread block of the last round of units, and with one round of 64-token blocks."""
+    for block in (16, 64, 128):
+        assert rules.ahead(block, 12, 12, 148) and rules.ahead(block, 100, 48, 148)
+        assert rules.ahead(block, 149, 147, 148) and not rules.ahead(block, 149, 148, 148)
+        assert rules.ahead(block, 320, 80, 148) and not rules.ahead(block, 444, 1, 148) and not rules.ahead(block, 148, 1, 148)
+        assert rules.ahead(block, 101, 48, 148) == (block == 64)
+    assert rules.ahead(64, 132, 72, 148) and not rules.ahead(64, 1776, 76, 148)
 
 
 def test_query_blocks_per_thread_block_of_the_selection(rules):
