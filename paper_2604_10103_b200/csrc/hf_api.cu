@@ -665,6 +665,7 @@ template <int D, int BLK, bool TEAMED>
 hf_status launch_swa_tc5_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16* k_cur, const bf16* v_cur, const int32_t* idx,
                            int keep, const float* hist, bf16* o, float* lse, cudaStream_t st, bool hist_inside, bool overlap_prev, bool merged) {
     typedef SwaTc5<D, TEAMED> C;
+    const bool behind_selection = overlap_prev;     // (else lists that were there before the call)
     Tc5Params p;
     memset(&p, 0, sizeof(p));
     p.upb = (c->Tc + 127) / 128; p.n_units = p.upb * c->BH;
@@ -700,10 +701,10 @@ hf_status launch_swa_tc5_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16* 
     const int grid = p.n_units < c->sm_count ? p.n_units : c->sm_count;
     PdlLaunch pl(dim3(grid), dim3(C::THREADS), C::SMEM_BYTES, st, overlap_prev);
 #define HF_TC5_LAUNCH(HIST_, AHEAD_) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, HIST_, TEAMED, AHEAD_>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p))
-    // Ahead: q, the folded state and z are older than the kernel before this one (the selection, whose pooling kernel lets it in behind its own
-    // wait; k_union_tiles likewise), but not the rotated copy of q that the pooling kernel itself writes.
+    // Ahead: q, the folded state and z are older than the selection before this kernel, whose pooling kernel lets it in behind its own wait, but
+    // not the rotated copy of q that the pooling kernel itself writes.
     if (!hist_inside) HF_TC5_LAUNCH(0, false);
-    else if (!TEAMED && !c->has_trope && swa_history_ahead(BLK, p.n_units, select_blocks(c, p.Tn), c->sm_count)) {
+    else if (!TEAMED && !c->has_trope && swa_history_ahead(BLK, p.n_units, behind_selection ? select_blocks(c, p.Tn) : 0, c->sm_count)) {
         if (c->has_rope_q) HF_TC5_LAUNCH(2, !TEAMED);
         else HF_TC5_LAUNCH(1, !TEAMED);
     } else if (c->has_rope_q) HF_TC5_LAUNCH(2, false);

@@ -63,7 +63,13 @@ inline bool swa_teams(int d, int block, int tiles, bool history) { return d == 6
 //   50.1 / 50.5
 //   64-token blocks, 132 units of 2, 8, 20 kept blocks, T_n 84 (72) 18.4 / 17.4, 22.2 / 21.2, 28.3 / 27.5; 444 units 46.4 / 47.2, 62.3 / 63.1, 80.2 / 81.3; 1 776
 //   units, T_n 74 141.6 / 145.5
+// No selection in front (selection_blocks 0: attention on lists that are there before the call): nothing to wait for, the term is only in the way of
+// the first tile, and behind k_union_tiles there is less time than it takes.  hf_sparse_swa_merged, behind / ahead, us:
+//   128-token blocks, 12 units of 1, 3, 8 tiles 8.4 / 9.3, 9.9 / 10.9, 14.0 / 15.1; 300 units 19.9 / 20.9, 22.6 / 23.9, 35.6 / 36.8
+//   64-token blocks, 12 units of 2 and 8 kept blocks 9.7 / 10.0, 13.1 / 13.6; 156 units of 2, 8, 20 16.0 / 16.6, 23.9 / 24.9, 39.0 / 40.2
+//   16-token blocks, 12 units of 4 and 30 kept blocks 12.0 / 12.5, 18.5 / 19.1; 132 units 14.7 / 14.0, 36.9 / 36.4
 inline bool swa_history_ahead(int block, int units, int selection_blocks, int sms) {
+    if (selection_blocks == 0) return false;
     const int last = units % sms ? units % sms : sms;
     return last + selection_blocks <= sms || (block == 64 && units < sms);
 }
