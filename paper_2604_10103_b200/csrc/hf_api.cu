@@ -238,7 +238,7 @@ hf_status set_swa_attr() {
 }
 template <int D, int G, int KPL, int R>
 hf_status set_select_attr_kpl(const hf_ctx* c) {
-    if (!select_uses(KPL, c->n_b, c->max_Tn) || select_rows(KPL, G, c->Tm, c->BH, c->sm_count) != R) return HF_OK;
+    if (!select_uses_rows(KPL, R, G, D, c->n_b, c->max_Tn, c->Tm, c->BH, c->sm_count)) return HF_OK;
     HF_CUDA(cudaFuncSetAttribute(k_select<D, KPL, G, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, Select<D, G, KPL, R>::smem_bytes(32 * KPL)));
     return HF_OK;
 }
@@ -275,7 +275,7 @@ inline bool pools_and_selects(const hf_ctx* c);
 // Thread blocks of a forward call's last kernel before the attention kernel.
 inline int select_blocks(const hf_ctx* c, int Tn) {
     if (pools_and_selects(c)) return c->cfg.block == 16 ? c->BH : c->Tm * c->BH;
-    const int R = select_rows(select_kpl(Tn), c->cfg.block == 128 ? 1 : 128 / c->cfg.block, c->Tm, c->BH, c->sm_count);
+    const int R = select_rows_of(select_kpl(Tn), c->cfg.block == 128 ? 1 : 128 / c->cfg.block, c->d, Tn, c->Tm, c->BH, c->sm_count);
     return (c->Tm + R - 1) / R * c->BH;
 }
 inline bool pools_and_selects(const hf_ctx* c) {
@@ -595,7 +595,7 @@ cudaError_t launch_select_kernel(hf_ctx* c, const ChunkTable& tab, int Tn, int k
         return cudaLaunchKernelEx(&pl.cfg, k_select<D, KPL_, G, R_>, tab, (const float*)c->pooled_q, c->n_b, c->Tm, Tn, keep, -0.f, o, lists); } while (0)
     const int kpl = select_kpl(Tn);
     if constexpr (G != 8) {
-        if (select_rows(kpl, G, c->Tm, c->BH, c->sm_count) == 4) {
+        if (select_rows_of(kpl, G, D, Tn, c->Tm, c->BH, c->sm_count) == 4) {
             if (kpl == 4) HF_SELECT(4, 4);
             HF_SELECT(8, 4);
         }

@@ -41,10 +41,36 @@ inline int select_kpl(int Tn) { return Tn <= 128 ? 4 : Tn <= 256 ? 8 : Tn <= 512
 inline bool select_uses(int kpl, int n_b, int max_Tn) { return select_kpl(n_b) <= kpl && kpl <= select_kpl(max_Tn); }
 
 // Query blocks that a thread block of the selection takes: eight where they share a unit's list (G 8: 16-token blocks) and for more than 256 key
-// blocks; with 129 to 256 eight where four would give more thread blocks than SMs, of which only one fits an SM with all key rows.
+// blocks; with 129 to 256, which are all in shared memory at once, eight where four would give more thread blocks than SMs ...
 inline int select_rows(int kpl, int G, int Tm, int BH, int sms) {
     if (G == 8 || kpl > 8) return 8;
     return kpl == 8 && (Tm + 3) / 4 * BH > sms ? 8 : 4;
+}
+inline constexpr int select_smem_bytes(int d, int rows, int key_rows, int Tn) { return (key_rows * (d + 4) + rows * d + rows * Tn) * 4; }
+// ... unless those are through in fewer rounds: an SM holds up to three thread blocks of four by registers (72 or 80 of 256 threads), by shared memory
+// three at head dim 64 and up to 136 key blocks at 128, two up to 208, then one; of eight it holds one (76 or 86 registers of 512 threads).
+// Pooling and selection of 64-token blocks, four / eight, us (forward calls: the same differences):
+//   head dim 64, thread blocks of four in one round, of eight in two: T_n 130, 24 heads 12.0 / 15.6; 148, 16 heads 10.9 / 13.1; 180, 16 heads 12.3 / 15.6;
+//   208, 12 and 16 heads 12.4 / 15.3, 13.9 / 17.1; 222, 16 heads 12.3 / 14.1; 250, 12 heads 13.9 / 17.1; two rounds, three of eight: 208, 24 heads 21.2 / 24.1;
+//   250, 24 heads 25.3 / 26.7; as many: 130, 8, 12, 16 heads 7.7 / 8.0, 8.7 / 8.8, 10.2 / 9.5; 180, 8, 12, 24 heads 9.3 / 9.0, 11.2 / 9.8, 19.0 / 17.9; 222, 8, 12, 24
+//   heads 9.8 / 9.0, 10.8 / 9.6, 17.6 / 17.5; 250, 8, 16 heads 11.5 / 10.3, 19.8 / 18.7
+//   head dim 128, one round, two: 130, 24 heads 17.2 / 21.1; as many: 130, 12, 16 heads 13.5 / 11.8, 14.7 / 12.7; 148, 8 to 24 heads 11.2 / 11.4, 12.6 / 12.7, 18.3 / 18.0,
+//   22.7 / 22.5; 180 13.0 / 12.2, 14.6 / 13.4, 21.4 / 21.6, 27.0 / 25.0; 208 14.1 / 13.0, 21.4 / 21.6, 23.7 / 23.5, 35.8 / 34.7; fewer of eight: 222 16.8 / 11.9, 18.8 / 13.5,
+//   26.1 / 19.8, 35.0 / 24.2; 250 19.8 / 14.7, 28.8 / 23.8, 37.8 / 26.3, 56.9 / 40.7
+// (The form with its key rows in two passes had three thread blocks to an SM at head dim 128 too: where that was one round and this is two, 148 to 250 key
+// blocks with 304 to 416 thread blocks of four, pooling and selection alone take up to 1.07 times as long as they did, a forward call as long.)
+inline int select_rows_of(int kpl, int G, int d, int Tn, int Tm, int BH, int sms) {
+    const int rows = select_rows(kpl, G, Tm, BH, sms);
+    if (G == 8 || kpl != 8 || rows == 4) return rows;
+    const int fit = (228 << 10) / (select_smem_bytes(d, 4, Tn, Tn) + (G > 1 ? 512 : 128) + 1024), resident = fit < 3 ? fit : 3;
+    const int rounds4 = ((Tm + 3) / 4 * BH + resident * sms - 1) / (resident * sms), rounds8 = ((Tm + 7) / 8 * BH + sms - 1) / sms;
+    return rounds8 <= rounds4 ? 8 : 4;
+}
+// Whether some window of a context, n_b, 2 n_b .. max_Tn key blocks, launches the step's kernel with that many.
+inline bool select_uses_rows(int kpl, int rows, int G, int d, int n_b, int max_Tn, int Tm, int BH, int sms) {
+    for (int Tn = n_b; Tn <= max_Tn && select_uses(kpl, n_b, max_Tn); Tn += n_b)
+        if (select_kpl(Tn) == kpl && select_rows_of(kpl, G, d, Tn, Tm, BH, sms) == rows) return true;
+    return false;
 }
 
 // Softmax warps of the tcgen05 attention kernel in teams that take turns at the tiles, or in column groups on the same one (k_swa_tc5.cuh).  Head

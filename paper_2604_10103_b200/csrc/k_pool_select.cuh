@@ -255,13 +255,13 @@ __global__ void __launch_bounds__(256, 6) k_pool_copy_layers(const __grid_consta
 // so that a key row is read once for four query blocks (the scores are bound by shared-memory reads) and no pass waits for the next one's rows: from the
 // pooled rows' arrival to the scores, 12 heads of 128, T_n 222 12 100 -> 8 300 clk, heads of 64, T_n 246 7 300 -> 5 300; with the ranking's two bits a step and its
 // words before the stores the forward of 64-token blocks 158 -> 155 us, of 16-token blocks at head dim 64 35.6 -> 33.4, 12 heads of 16-token blocks, T_n 176 45.0 -> 40.5;
-// eight query blocks where four would be more thread blocks than SMs (hf_dispatch.h).
+// four query blocks or eight: select_rows_of (hf_dispatch.h).
 template <int D, int G, int KPL, int RQ>
 struct Select {
     static constexpr int R = RQ, KT = KPL == 8 ? 256 : 128;       // query blocks per thread block; key rows per pass
     static constexpr int THREADS = 64 * R;
     static constexpr int LD = D + 4;            // floats per key row in shared memory
-    static int smem_bytes(int Tn) { const int kt = Tn < KT ? Tn : KT; return (kt * LD + R * D + R * Tn) * (int)sizeof(float); }
+    static int smem_bytes(int Tn) { return select_smem_bytes(D, R, Tn < KT ? Tn : KT, Tn); }
 };
 struct Quad { float2 a, b; };                   // four neighbouring columns
 __device__ __forceinline__ Quad quad_add(const Quad& x, const Quad& y) { return {fadd2(x.a, y.a), fadd2(x.b, y.b)}; }
