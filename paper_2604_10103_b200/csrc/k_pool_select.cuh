@@ -8,6 +8,7 @@
 #pragma once
 #include "hf_common.cuh"
 #include "k_union.cuh"
+#include "hf_dispatch.h"
 
 template <int VEC> struct VecLoad;
 template <> struct VecLoad<8> {
