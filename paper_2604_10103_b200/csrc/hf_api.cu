@@ -5,6 +5,7 @@
 #include "k_pool_select.cuh"
 #include "k_swa_mma.cuh"
 #include "k_swa_tc5.cuh"
+#include "hf_swa_tc5.h"
 #include "k_swa_tc5p.cuh"
 #include "k_swa_bwd.cuh"
 #include "k_readout_bwd.cuh"
@@ -223,12 +224,12 @@ void free_all(hf_ctx* c) {
 #define HF_TC5P_COLGROUPS 1   // column groups per tile group of the ping-pong attention kernel
 #endif
 
-template <int D, int BLK, bool TEAMED>
-hf_status set_swa_tc5_attr() {
-#define HF_TC5_ATTR(HIST_, AHEAD_) HF_CUDA(cudaFuncSetAttribute(k_swa_tc5<D, BLK, HIST_, TEAMED, AHEAD_>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D, TEAMED>::SMEM_BYTES))
-    HF_TC5_ATTR(0, false); HF_TC5_ATTR(1, false); HF_TC5_ATTR(2, false);
-    if (!TEAMED) { HF_TC5_ATTR(1, !TEAMED); HF_TC5_ATTR(2, !TEAMED); }
-#undef HF_TC5_ATTR
+template <int D, bool TEAMED>
+hf_status set_swa_tc5_attr(int block) {
+    for (int ahead = 0; ahead < 2; ++ahead)
+        for (int history = 0; history < 3; ++history)
+            if (const void* kernel = swa_tc5_kernel(D, block, history, TEAMED, ahead != 0))
+                HF_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5<D, TEAMED>::SMEM_BYTES));
     return HF_OK;
 }
 template <int BLK, int D>
@@ -312,10 +313,10 @@ hf_status set_attrs(hf_ctx* c) {
         HF_CUDA(cudaFuncSetAttribute(k_swa_tc5p<D, HF_TC5P_COLGROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SwaTc5P<D, HF_TC5P_COLGROUPS>::SMEM_BYTES));
     else if (c->swa_kernel == HF_SWA_TCGEN05) {
         // (128-token blocks: kept blocks of the shortest and of the longest window: column groups, teams, or both)
-        if (b != 128) HF_TRY((b == 64 ? set_swa_tc5_attr<D, 64, D == 64>() : set_swa_tc5_attr<D, 16, D == 64>()));
+        if (b != 128) HF_TRY((set_swa_tc5_attr<D, D == 64>(b)));
         else {
-            if (swa_teams(D, b, keep_for(c, c->max_Tn), false)) HF_TRY((set_swa_tc5_attr<D, 128, true>()));
-            if constexpr (D == 128) { if (!swa_teams(D, b, keep_for(c, c->n_b), true)) HF_TRY((set_swa_tc5_attr<D, 128, false>())); }
+            if (swa_teams(D, b, keep_for(c, c->max_Tn), false)) HF_TRY((set_swa_tc5_attr<D, true>(128)));
+            if constexpr (D == 128) { if (!swa_teams(D, b, keep_for(c, c->n_b), true)) HF_TRY((set_swa_tc5_attr<D, false>(128))); }
         }
     } else
         HF_TRY((b == 128 ? set_swa_attr<128, D>() : b == 64 ? set_swa_attr<64, D>() : set_swa_attr<16, D>()));
@@ -700,16 +701,12 @@ hf_status launch_swa_tc5_t(hf_ctx* c, LayerState& L, const bf16* q, const bf16* 
     const CUtensorMap& rv = c->R + c->n_sink_max > 0 ? L.tm_vring : tv;
     const int grid = p.n_units < c->sm_count ? p.n_units : c->sm_count;
     PdlLaunch pl(dim3(grid), dim3(C::THREADS), C::SMEM_BYTES, st, overlap_prev);
-#define HF_TC5_LAUNCH(HIST_, AHEAD_) HF_CUDA(cudaLaunchKernelEx(&pl.cfg, k_swa_tc5<D, BLK, HIST_, TEAMED, AHEAD_>, tq, rk, rv, tk, tv, L.tm_sfhi, L.tm_sflo, to, p))
     // Ahead: q, the folded state and z are older than the selection before this kernel, whose pooling kernel lets it in behind its own wait, but
     // not the rotated copy of q that the pooling kernel itself writes.
-    if (!hist_inside) HF_TC5_LAUNCH(0, false);
-    else if (!TEAMED && !c->has_trope && swa_history_ahead(BLK, p.n_units, behind_selection ? select_blocks(c, p.Tn) : 0, c->sm_count)) {
-        if (c->has_rope_q) HF_TC5_LAUNCH(2, !TEAMED);
-        else HF_TC5_LAUNCH(1, !TEAMED);
-    } else if (c->has_rope_q) HF_TC5_LAUNCH(2, false);
-    else HF_TC5_LAUNCH(1, false);
-#undef HF_TC5_LAUNCH
+    const bool ahead = hist_inside && !TEAMED && !c->has_trope && swa_history_ahead(BLK, p.n_units, behind_selection ? select_blocks(c, p.Tn) : 0, c->sm_count);
+    const void* kernel = swa_tc5_kernel(D, BLK, !hist_inside ? 0 : c->has_rope_q ? 2 : 1, TEAMED, ahead);
+    const void* args[] = {&tq, &rk, &rv, &tk, &tv, &L.tm_sfhi, &L.tm_sflo, &to, &p};
+    HF_CUDA(cudaLaunchKernelExC(&pl.cfg, kernel, const_cast<void**>(args)));
     return post_launch(c, "k_swa_tc5");
 }
 
