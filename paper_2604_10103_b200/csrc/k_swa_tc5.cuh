@@ -121,11 +121,12 @@ struct SwaTc5 {
     __host__ __device__ static constexpr int off_xy(bool hist, int half) { return hist ? OFF_H + TILE_BYTES + 512 * half : half ? OFF_XL + 512 : OFF_Z; }
     static_assert(OFF_H + TILE_BYTES + 2048 <= OFF_BAR, "exchange buffers");
     static constexpr int MAX_SMEM = 232448;            // 227 KB: the most one thread block can have
-    // Slack for the manual 1024-byte alignment of the operand tiles (the kernel checks that it was enough); more than
-    // half an SM's shared memory so that one CTA owns the SM (it allocates all 512 TMEM columns)
+    // The window of a kernel without static shared memory starts on a 1 KB boundary, as the operand tiles have to (the kernel checks it, with what slack there
+    // is: 64 bytes at head dim 128).  With a static array it would not, but then the runtime refuses MAX_SMEM, and hf_create fails with its error.
+    // More than half an SM's shared memory, so that one CTA owns the SM (it allocates all 512 TMEM columns).
     static constexpr int WANT_BYTES = (USED_BYTES + 1024) > 120 * 1024 ? (USED_BYTES + 1024) : 120 * 1024;
     static constexpr int SMEM_BYTES = WANT_BYTES < MAX_SMEM ? WANT_BYTES : MAX_SMEM;
-    static_assert(USED_BYTES <= MAX_SMEM, "shared memory layout does not fit");
+    static_assert(USED_BYTES <= MAX_SMEM && (SMEM_BYTES == MAX_SMEM || SMEM_BYTES >= USED_BYTES + 1024), "shared memory layout does not fit");
     static constexpr int THREADS = 32 * NSW + 128;
     static constexpr int WARP_LOAD_K = NSW, WARP_LOAD_V = NSW + 1, WARP_S = NSW + 2, WARP_PV = NSW + 3;
 };
