@@ -79,7 +79,7 @@ inline bool select_uses_rows(int kpl, int rows, int G, int d, int n_b, int max_T
 //   132 units, 10 tiles 22.1 / 22.2, 12 tiles 23.9 / 23.7, 14 tiles 25.8 / 25.2, 24 tiles 34.7 / 32.7  (8 tiles 14.4 / 14.4, 12 tiles 18.3 / 16.8)
 //   448 units, 10 tiles 67.1 / 69.3, 12 tiles 73.9 / 75.4, 14 tiles 81.0 / 80.9, 24 tiles 119.9 / 114.8  (8 tiles 44.6 / 41.0, 4 tiles 29.7 / 29.0)
 // and column groups for its blocks of 16 and 64 tokens (0.90 to 0.98 times as fast with teams).
-inline bool swa_teams(int d, int block, int tiles, bool history) { return d == 64 || (block == 128 && tiles >= (history ? 14 : 8)); }
+inline constexpr bool swa_teams(int d, int block, int tiles, bool history) { return d == 64 || (block == 128 && tiles >= (history ? 14 : 8)); }
 
 // Whether the attention kernel's column groups form their first unit's history term ahead of the selection's end.  It is for nothing where the
 // thread block is resident early, which takes an SM that the selection leaves free, and on the chain in front of the first tile where it is not.  What

@@ -96,6 +96,7 @@ struct SwaTc5 {
     // The phi(Q) operand of the history products (D columns): in the P buffer of the team that forms it where there are two, else in that
     // team's S buffer, where the next unit's first S has to wait for the products.
     static constexpr bool A_IN_P = PBUF == 2;
+    static_assert(!TEAMED || A_IN_P || !swa_teams(D, 128, 1, true), "a unit of one tile would have its operand where the unit before has D_h");
     static constexpr int COL_P = 256, COL_Q = COL_P + 64 * PBUF, COL_O = COL_Q + D / 2, TMEM_COLS = 512;
     static_assert(COL_O + D <= TMEM_COLS, "tensor memory layout");
     static constexpr int KV_LOG = D == 64 ? 2 : 1, KV = 1 << KV_LOG;   // stages of the K and of the V ring
@@ -975,10 +976,10 @@ k_swa_tc5(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUte
                     // ---- the other team has the unit's last tile, and its output: this one hands over its row sums and goes on to the next unit
                     if constexpr (HIST != 0) {
                         release_h();
-                        if (C::A_IN_P) {                        // its P buffer: the product of its last tile is complete
+                        if constexpr (C::A_IN_P) {              // its P buffer: the product of its last tile is complete
                             const int tx = t0 + cnt - 2;
                             if (tx >= 0) ok = wait_s(bar_pv + 8 * (tx & 1), tx >> 1, 29);
-                        } else if (cnt == 1 && n >= 1) ok = wait_s(bar_dr(n - 1), (n - 1) >> 1, 29);
+                        }
                         if (!(ok = ok && form_phi(n, q0, C::A_IN_P ? tP : tS, dsum))) break;
                     }
                     if (cnt == 1) arrive_t(bar_mr + 8 * wq);                    // (nothing to read)
