@@ -74,7 +74,14 @@ inline bool select_uses_rows(int kpl, int rows, int G, int d, int n_b, int max_T
 }
 
 // Softmax warps of the tcgen05 attention kernel in teams that take turns at the tiles, or in column groups on the same one (k_swa_tc5.cuh).  Head
-// dim 64: teams (1 to 40 tiles, 12 to 320 units: 0.98 to 1.13 times as fast).  Head dim 128, 128-token blocks: teams from 14 tiles on, from
+// dim 64: teams.  Several units a thread block, 1 to 40 tiles: 1.01 to 1.13 times as fast.  One unit of few tiles has none to take turns at and pays for
+// the hand-overs; two column groups (from five tiles on: four) / teams, forward calls (softmax branch alone), us:
+//   12 units, 1, 3, 6 tiles 7.5 / 7.5, 9.3 / 9.2, 11.3 / 11.4  (5.8 / 6.1, 7.4 / 7.4, 9.6 / 9.6)
+//   36 units, 1, 3, 6, 12 tiles 8.3 / 8.5, 10.1 / 10.1, 12.4 / 12.4, 16.9 / 16.5  (6.0 / 6.1, 7.6 / 7.5, 9.8 / 9.5, 14.0 / 13.6)
+//   132 units, 1, 3, 6, 12, 16 tiles 9.9 / 10.3, 11.8 / 12.1, 14.1 / 14.3, 19.0 / 19.0, 22.4 / 22.2  (6.1 / 6.6, 7.8 / 8.1, 10.0 / 10.5, 14.5 / 15.3, 17.4 / 18.3)
+//   156 units, 1, 3, 8 tiles 13.0 / 12.4, 16.2 / 15.3, 23.5 / 22.2  (8.2 / 7.3, 11.5 / 10.5, 18.6 / 17.7)
+// The line cannot lie at the number of units: the two forms add a row's weights in another order, and the same head would not have the same bits in a call
+// with other heads beside it.  Head dim 128, 128-token blocks: teams from 14 tiles on, from
 // 8 without the history term, whose operand they keep in an S buffer; column groups / teams, forward calls (softmax branch alone), us:
 //   132 units, 10 tiles 22.1 / 22.2, 12 tiles 23.9 / 23.7, 14 tiles 25.8 / 25.2, 24 tiles 34.7 / 32.7  (8 tiles 14.4 / 14.4, 12 tiles 18.3 / 16.8)
 //   448 units, 10 tiles 67.1 / 69.3, 12 tiles 73.9 / 75.4, 14 tiles 81.0 / 80.9, 24 tiles 119.9 / 114.8  (8 tiles 44.6 / 41.0, 4 tiles 29.7 / 29.0)
@@ -89,6 +96,8 @@ inline constexpr bool swa_teams(int d, int block, int tiles, bool history) { ret
 //   50.1 / 50.5
 //   64-token blocks, 132 units of 2, 8, 20 kept blocks, T_n 84 (72) 18.4 / 17.4, 22.2 / 21.2, 28.3 / 27.5; 444 units 46.4 / 47.2, 62.3 / 63.1, 80.2 / 81.3; 1 776
 //   units, T_n 74 141.6 / 145.5
+//   16-token blocks (a thread block of the selection for each unit), 2 units of 2 and 8 kept blocks 12.8 / 11.5, 13.7 / 12.4; 12 units 13.3 / 12.1, 14.5 / 13.2; 36 units of 2,
+//   8, 30 16.3 / 15.2, 20.9 / 20.4, 24.6 / 24.0; 132 units 22.8 / 23.3, 28.9 / 30.3, 42.8 / 44.3; 320 units 43.9 / 44.3, 57.0 / 57.3, 81.9 / 82.4
 // No selection in front (selection_blocks 0: attention on lists that are there before the call): nothing to wait for, the term is only in the way of
 // the first tile, and behind k_union_tiles there is less time than it takes.  hf_sparse_swa_merged, behind / ahead, us:
 //   128-token blocks, 12 units of 1, 3, 8 tiles 8.4 / 9.3, 9.9 / 10.9, 14.0 / 15.1; 300 units 19.9 / 20.9, 22.6 / 23.9, 35.6 / 36.8

@@ -360,7 +360,9 @@ __device__ __forceinline__ uint32_t rank_row(const float* sc, size_t row, int Tn
         }
     } else {
         // Two bits a step, the three counts of a step side by side in one word (T_n <= 512; two words above): a step is a chain, mostly the sum
-        // over the warp (3 300 -> 2 300 clk with 222 key blocks; votes and population counts instead 3 400).
+        // over the warp (3 300 -> 2 300 clk with 222 key blocks; votes and population counts instead 3 400).  Pooling and selection with a bit a step and the
+        // stores between the words' votes / like this, us: T_n 72 and 120 in one launch 5.3 / 5.1, 6.1 / 5.9; T_n 80 9.6 / 9.0; 370 30.3 / 29.9, 400 22.7 / 22.1; in two words 592,
+        // 720 (head dim 128, 64) 31.6 / 28.0, 70.7 / 64.1, 30.3 / 25.6.
         exact = keep >= Tn;         // exactly `keep` images at or above the threshold: no ties to cut (all blocks kept: every image counts)
         for (int sh = 30; sh >= 0 && !exact; sh -= 2) {
             const uint32_t c1 = thr | (1u << sh), c2 = thr | (2u << sh), c3 = thr | (3u << sh);

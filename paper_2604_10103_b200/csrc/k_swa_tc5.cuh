@@ -31,7 +31,8 @@
 // warps on a scheduler cover each other, and no warp of one team waits for the other inside a unit: 1 380-1 450 clk a tile.  A P half of 64
 // keys is written by both halves of a team, so that its product starts in the middle of the tile (with 64 columns in a row for each
 // half it started at the end, and where there is one P buffer the other team waited for it: 1 770 clk).  At a unit's end one team forms phi(Q)
-// while the other has the last tile; that one writes the output while the first has gone on to the next unit's first tile.  Forward calls, two
+// while the other has the last tile; that one writes the output while the first has gone on to the next unit's first tile.  Twenty warps leave 96 registers a
+// thread; what is spilt lies outside the tile loop (132 units, 20 and 40 tiles alike: 52 loads and 40 to 80 stores of local memory a thread block).  Forward calls, two
 // column groups (head dim 64 from five tiles on: four) / teams, us:
 //   head dim 128, 128-token blocks, 444 units of 28 tiles 125.7 / 121.8 (at the power limit), 1 776 units of 130 tiles 1 929 / 1 770; 132 units
 //   of 20 tiles 31.3 / 29.7, of 40 tiles 49.9 / 44.6; 320 units of 20 tiles 79.8 / 76.7, of 40 tiles 134.1 / 122.7
